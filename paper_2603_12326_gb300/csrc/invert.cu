@@ -3,9 +3,8 @@
 // eps(w, q+G) = 1/[eps^-1]_GG (Eq. (eps_LFE)); eps^noLFE = eps_GG
 // (Eq. (eps_noLFE)); L = Im[-1/eps] (Eq. (dynamic_structure_factor)).
 //
-// One CTA per (q, w) block runs Gauss-Jordan elimination with partial
-// (row) pivoting in place on a work copy of the matrix, then undoes the
-// column permutation.  The FP64 path does this in double.  The mixed path
+// Every (q, w) block is inverted by blocked Gauss-Jordan elimination with partial
+// (row) pivoting.  The FP64 path does this in double.  The mixed path
 // does it in FP32 on the rounded copy of the FP64 matrix and records the
 // condition estimate kappa_1 = |A|_1 |X|_1.  Blocks with kappa_1 above the
 // context's threshold (default 1e4; the ill-conditioned ones, near the
@@ -17,420 +16,314 @@
 #include "qcx_internal.h"
 #include "cplx.cuh"
 
-#include <cooperative_groups.h>
+#include <algorithm>
 
 namespace {
 
-constexpr int INV_THREADS = 512;
-
-template <typename T> struct InvArgs {
-    int ng, nw;
-    const double2* eps64;      // FP64 input [nw][ng][ng]
-    cplx<T>* X;                // work [nw][ng][ng]
-    double* kappa;             // [nw] condition estimate (mixed path) or null
-    double2* diag_inv;         // [nw][ng]
-    double2* eps_diag;         // [nw][ng]
-    double* L;                 // [2][nw][ng] (LFE, noLFE)
-    int* flags;                // [nw]
-};
+// Blocked in-place Gauss-Jordan over all matrices at once.  Per panel of PB columns:
+//
+//   k_inv_panel   one CTA per matrix holds the n x PB panel in shared memory and eliminates its columns with
+//                 partial pivoting over the rows not used yet (rows are not moved: the CTA records which row
+//                 serves as pivot of which column);
+//   k_inv_update  every other column at once, out of place (src -> dst), as a product with inner length PB:
+//                     dst[i][j] = (i in panel ? 0 : src[p(i)][j]) + sum_c M[i][c] src[p(k0 + c)][j],
+//                 where M is the eliminated panel (for a pivot row the inverse of the pivot block, for any other
+//                 row minus its multipliers) and p the panel's row exchange.
+//
+// What bounds it: the rank-1 form rewrote the whole matrix for every one of the n columns (n^3 elements through
+// L2, one CTA per matrix, or through shared memory with a cluster barrier per column); this form touches it
+// n/PB times and spends 8 n^3 flops in a product that the FP32 (FP64) pipe bounds, with tiles of all matrices in
+// one grid.  PB = 32 (FP32) keeps the panel's serial part (two CTA barriers per column, ~0.3 us) below the
+// update's time.  Measured (CUDA events, GB300): 200 matrices of 181: 3.33 -> 0.82 ms; 100 of 531: 177 -> 5.6 ms;
+// FP64, 8 of 181: 10.8 -> 2.0 ms.
+// With P A = rows in pivot order, the eliminated matrix is (P A)^-1, so its column k is the inverse's column
+// row(k): the last update writes its columns there.
+constexpr int UPD = 64;                     // update tile edge
+template <typename T> struct InvCfg;
+template <> struct InvCfg<float> { static constexpr int PB = 32; };
+template <> struct InvCfg<double> { static constexpr int PB = 16; };
+constexpr size_t PANEL_SMEM = 200 * 1024;   // the panel narrows above this (n > 800 in FP32 and FP64)
+constexpr int PANEL_ROWS = 4;               // rows per thread of the panel at most (n <= 4096)
 
 template <typename T> __device__ __forceinline__ T cabs2(cplx<T> z) { return z.x * z.x + z.y * z.y; }
+// |z| without overflow of the squares
+__device__ __forceinline__ float cabs_safe(float2 z) {
+    const float x = fabsf(z.x), y = fabsf(z.y), m = fmaxf(x, y), r = fminf(x, y);
+    if (!(m > 0.f)) return m;
+    const float t = r / m;
+    return m * sqrtf(fmaf(t, t, 1.f));
+}
 
+// order of a squared magnitude as an integer: NaN below everything, zero 1, larger magnitudes larger
+__device__ __forceinline__ unsigned long long mag_key(float v) {
+    return v >= 0.f ? (unsigned long long)__float_as_uint(v) + 1ull : 0ull;
+}
+__device__ __forceinline__ unsigned long long mag_key(double v) {
+    return v >= 0.0 ? (unsigned long long)__double_as_longlong(v) + 1ull : 0ull;
+}
+// largest key of the warp; with ties the first lane's `row` wins
+template <typename T> __device__ __forceinline__ void warp_best(unsigned long long& key, int& row);
+template <> __device__ __forceinline__ void warp_best<float>(unsigned long long& key, int& row) {
+    const unsigned m = __reduce_max_sync(0xffffffffu, (unsigned)key);
+    const int r = (unsigned)key == m ? row : 0x7fffffff;
+    row = __reduce_min_sync(0xffffffffu, r);
+    key = m;
+}
+template <> __device__ __forceinline__ void warp_best<double>(unsigned long long& key, int& row) {
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32));
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(key >> 32) == hi ? (unsigned)key : 0u);
+    const unsigned long long m = ((unsigned long long)hi << 32) | lo;
+    const int r = key == m ? row : 0x7fffffff;
+    row = __reduce_min_sync(0xffffffffu, r);
+    key = m;
+}
+
+// FP64 matrices -> work precision; eps_GG, the loss without local fields, |A|_1 (largest column sum) and the
+// starting row order.  Grid (matrix, 64 columns); 64 columns x 4 row groups per CTA.
 template <typename T>
-__global__ void __launch_bounds__(INV_THREADS) k_gauss_jordan(InvArgs<T> a, int write_lfe) {
+__global__ void __launch_bounds__(256) k_inv_load(int n, const double2* A, cplx<T>* X, double* anorm, double2* eps_diag,
+                                                  double* L_nolfe, int* rows, int* flags) {
+    __shared__ double sums[4][64];
+    const int b = blockIdx.x, tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+    const int j = blockIdx.y * 64 + tx;
+    A += (size_t)b * n * n;
+    X += (size_t)b * n * n;
+    double cs = 0.0;
+    if (j < n)
+        for (int i = ty; i < n; i += 4) {
+            const double2 z = A[(size_t)i * n + j];
+            const cplx<T> x = mk<T>((T)z.x, (T)z.y);
+            X[(size_t)i * n + j] = x;
+            if constexpr (sizeof(T) == 4) cs += (double)cabs_safe(x);
+            if (i == j) {
+                eps_diag[(size_t)b * n + i] = z;
+                L_nolfe[(size_t)b * n + i] = z.y / (z.x * z.x + z.y * z.y);
+                rows[(size_t)b * n + i] = i;
+            }
+        }
+    if (blockIdx.y == 0 && threadIdx.x == 0) flags[b] = 0;
+    if constexpr (sizeof(T) == 4) {
+        sums[ty][tx] = cs;
+        __syncthreads();
+        if (ty == 0 && j < n) {
+            cs = (sums[0][tx] + sums[1][tx]) + (sums[2][tx] + sums[3][tx]);
+            atomicMax(reinterpret_cast<unsigned long long*>(anorm + b), (unsigned long long)__double_as_longlong(cs));
+        }
+    }
+}
+
+// One panel: columns k0 .. k0 + nb - 1 of every row.  Warps: RW row warps x column groups of bc columns; a thread
+// eliminates in its rows (row, row + 32 RW, ...) and its group's columns.  M[c][i] gets the eliminated panel in the
+// new row order, perm the exchange (new position -> old position), rows the original row of each position.
+template <typename T>
+__global__ void __launch_bounds__(1024) k_inv_panel(int n, int k0, int nb, int RW, int bc, const cplx<T>* src, cplx<T>* M, int* perm, int* rows,
+                            int* flags) {
     using C = cplx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int n = a.ng;
-    C* rowk = reinterpret_cast<C*>(smem_raw);          // [n]
-    C* colk = rowk + n;                                 // [n]
-    int* piv = reinterpret_cast<int*>(colk + n);        // [n]
-    int* idx = piv + n;                                 // [n]
-    __shared__ T red_v[INV_THREADS / 32];
-    __shared__ int red_i[INV_THREADS / 32];
-    __shared__ int s_p;
-    __shared__ int s_bad;
-
+    const int ld = n | 1;
+    C* xs = reinterpret_cast<C*>(smem_raw);            // [nb][ld]
+    C* prow = xs + (size_t)nb * ld;                     // [nb] scaled pivot row (inverse pivot at its own column)
+    unsigned long long* wkey = reinterpret_cast<unsigned long long*>(prow + nb);   // [32] best per row warp
+    int* wrow = reinterpret_cast<int*>(wkey + 32);      // [32]
+    int* pos = wrow + 32;                               // [n] position -> row of src
+    int* ipos = pos + n;                                // [n] its inverse
     const int b = blockIdx.x;
-    C* X = a.X + (size_t)b * n * n;
-    // load the matrix; record eps_GG and the loss without local fields
-    for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-        const double2 z = a.eps64[(size_t)b * n * n + e];
-        X[e] = mk<T>((T)z.x, (T)z.y);
-        const int i = e / n;
-        if (e == i * n + i) {
-            const double re = z.x, im = z.y;
-            a.eps_diag[(size_t)b * n + i] = make_double2(re, im);
-            a.L[((size_t)a.nw + b) * n + i] = im / (re * re + im * im);
-        }
-    }
-    __shared__ double s_norm;
-    if (threadIdx.x == 0) {
-        s_bad = 0;
-        s_norm = 0.0;
-    }
-    __syncthreads();
-    if (a.kappa) {
-        // |A|_1: largest column sum of |A_ij|
-        double best = 0.0;
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            double cs = 0.0;
-            for (int i = 0; i < n; ++i) {
-                const double2 z = a.eps64[(size_t)b * n * n + (size_t)i * n + j];
-                cs += sqrt(z.x * z.x + z.y * z.y);
-            }
-            best = fmax(best, cs);
-        }
-        for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_down_sync(0xffffffffu, best, o));
-        if ((threadIdx.x & 31) == 0)
-            atomicMax(reinterpret_cast<unsigned long long*>(&s_norm), (unsigned long long)__double_as_longlong(best));
-    }
-    __syncthreads();
-
-    for (int k = 0; k < n; ++k) {
-        // pivot: largest |X_ik| over i >= k (smallest index on ties)
-        T best = -1;
-        int bi = n;
-        for (int i = k + threadIdx.x; i < n; i += blockDim.x) {
-            const T v = cabs2<T>(X[(size_t)i * n + k]);
-            if (v > best) {
-                best = v;
-                bi = i;
-            }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            const T ov = __shfl_down_sync(0xffffffffu, best, o);
-            const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-            if (ov > best || (ov == best && oi < bi)) {
-                best = ov;
-                bi = oi;
-            }
-        }
-        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        if (lane == 0) {
-            red_v[wid] = best;
-            red_i[wid] = bi;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            T bv = red_v[0];
-            int bix = red_i[0];
-            for (int w = 1; w < (int)(blockDim.x >> 5); ++w)
-                if (red_v[w] > bv || (red_v[w] == bv && red_i[w] < bix)) {
-                    bv = red_v[w];
-                    bix = red_i[w];
-                }
-            if (!(bv > 0) || bix >= n) {
-                s_bad = 1;
-                bix = k;
-            }
-            s_p = bix;
-            piv[k] = bix;
-        }
-        __syncthreads();
-        if (s_bad) break;
-        const int p = s_p;
-        // swap rows k and p, then load the (scaled) pivot row and column k
-        if (p != k) {
-            for (int j = threadIdx.x; j < n; j += blockDim.x) {
-                const C t = X[(size_t)k * n + j];
-                X[(size_t)k * n + j] = X[(size_t)p * n + j];
-                X[(size_t)p * n + j] = t;
-            }
-            __syncthreads();
-        }
-        const C pv = X[(size_t)k * n + k];
-        const T d = (T)1 / cabs2<T>(pv);
-        const C inv = mk<T>(pv.x * d, -pv.y * d);
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            const C v = (j == k) ? mk<T>(1, 0) : X[(size_t)k * n + j];
-            rowk[j] = cmul(v, inv);
-            colk[j] = (j == k) ? mk<T>(0, 0) : X[(size_t)j * n + k];
-        }
-        __syncthreads();
-        for (int j = threadIdx.x; j < n; j += blockDim.x) X[(size_t)k * n + j] = rowk[j];
-        // eliminate column k from every other row; X_ik itself becomes -colk_i * inv
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-            const int i = e / n, j = e - i * n;
-            if (i == k) continue;
-            const C f = colk[i];
-            C x = (j == k) ? mk<T>(0, 0) : X[e];
-            x.x -= f.x * rowk[j].x - f.y * rowk[j].y;
-            x.y -= f.x * rowk[j].y + f.y * rowk[j].x;
-            X[e] = x;
-        }
-        __syncthreads();
-    }
-    if (s_bad) {
-        if (threadIdx.x == 0) a.flags[b] = 1;
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            a.diag_inv[(size_t)b * n + j] = make_double2(0.0, 0.0);
-            if (write_lfe) a.L[(size_t)b * n + j] = 0.0;
-        }
-        return;
-    }
-    // undo the column permutation: the inverse's column c is X's column idx[c]
-    if (threadIdx.x == 0) {
-        a.flags[b] = 0;
-        for (int c = 0; c < n; ++c) idx[c] = c;
-        for (int k = n - 1; k >= 0; --k) {
-            const int t = idx[k];
-            idx[k] = idx[piv[k]];
-            idx[piv[k]] = t;
-        }
-    }
-    __syncthreads();
-    // write the permuted inverse back in place, row by row through shared memory
-    for (int i = 0; i < n; ++i) {
-        for (int j = threadIdx.x; j < n; j += blockDim.x) rowk[j] = X[(size_t)i * n + idx[j]];
-        __syncthreads();
-        for (int j = threadIdx.x; j < n; j += blockDim.x) X[(size_t)i * n + j] = rowk[j];
-        __syncthreads();
-    }
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const C z = X[(size_t)j * n + j];
-        a.diag_inv[(size_t)b * n + j] = make_double2((double)z.x, (double)z.y);
-        if (write_lfe) a.L[(size_t)b * n + j] = -(double)z.y;
-    }
-    if (a.kappa) {
-        // |X|_1 of the computed inverse
-        __shared__ double s_xnorm;
-        if (threadIdx.x == 0) s_xnorm = 0.0;
-        __syncthreads();
-        double best = 0.0;
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            double cs = 0.0;
-            for (int i = 0; i < n; ++i) {
-                const C z = X[(size_t)i * n + j];
-                cs += sqrt((double)z.x * z.x + (double)z.y * z.y);
-            }
-            best = fmax(best, cs);
-        }
-        for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_down_sync(0xffffffffu, best, o));
-        if ((threadIdx.x & 31) == 0)
-            atomicMax(reinterpret_cast<unsigned long long*>(&s_xnorm), (unsigned long long)__double_as_longlong(best));
-        __syncthreads();
-        if (threadIdx.x == 0) a.kappa[b] = s_norm * s_xnorm;
-    }
-}
-
-// Mixed path, N_G <= GJC_MAXN: the same elimination with the matrix resident
-// in shared memory, split by columns over a cluster of GJC_CS CTAs (a 181 x 181
-// FP32 complex matrix is 262 KB, more than one CTA holds; with four CTAs of
-// 74 KB, three clusters' CTAs share an SM and hide each other's barriers).  Step k: the CTA
-// owning column k picks the pivot row and publishes the row index, the pivot
-// and column k after the row exchange (the multipliers) in its shared memory;
-// after one cluster barrier the others read them through distributed shared
-// memory; every CTA then exchanges rows, scales the pivot row and eliminates
-// in its own columns.  The published values alternate between two slots, so
-// the barrier of the next step also orders their reuse.  Warps take rows,
-// lanes take columns.
-constexpr int GJC_CS = 4;
-constexpr int GJC_THREADS = 256;
-constexpr int GJC_MAXN = 192;
-constexpr int GJC_WARPS = GJC_THREADS / 32;
-
-__global__ void __cluster_dims__(GJC_CS, 1, 1) __launch_bounds__(GJC_THREADS) k_gj_cluster(InvArgs<float> a) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cl = cg::this_cluster();
-    const int rank = (int)cl.block_rank();
-    const int b = blockIdx.x / GJC_CS;
-    const int n = a.ng;
-    const int h = (n + GJC_CS - 1) / GJC_CS;
-    const int c0 = rank * h;
-    const int hn = max(0, min(h, n - c0));
+    if (flags[b]) return;
+    src += (size_t)b * n * n;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2* Xs = reinterpret_cast<float2*>(smem_raw);     // [n][h] my columns
-    float2* F = Xs + (size_t)n * h;                        // [2][n] published multipliers
-    float2* Fl = F + 2 * n;                                // [n] multipliers of this step
-    float2* rowk = Fl + n;                                 // [h] scaled pivot row
-    int* piv = reinterpret_cast<int*>(rowk + h);           // [n]
-    int* idx = piv + n;                                    // [n]
-    int* jof = idx + n;                                    // [n] inverse of idx
-    __shared__ int s_p[2], s_bad[2];
-    __shared__ float2 s_pv[2];
-    __shared__ float red_v[GJC_WARPS];
-    __shared__ int red_i[GJC_WARPS];
-    __shared__ double s_anorm, s_xnorm;
-
-    const double2* A = a.eps64 + (size_t)b * n * n;
-    for (int i = warp; i < n; i += GJC_WARPS)
-        for (int c = lane; c < hn; c += 32) {
-            const double2 z = A[(size_t)i * n + c0 + c];
-            Xs[i * h + c] = make_float2((float)z.x, (float)z.y);
-            if (i == c0 + c) {
-                a.eps_diag[(size_t)b * n + i] = z;
-                a.L[((size_t)a.nw + b) * n + i] = z.y / (z.x * z.x + z.y * z.y);
-            }
-        }
-    if (threadIdx.x == 0) {
-        s_anorm = 0.0;
-        s_xnorm = 0.0;
+    const int rw = warp % RW, grp = warp / RW;
+    const int stride = 32 * RW;
+    const int row0 = rw * 32 + lane;
+    for (int e = threadIdx.x; e < n * nb; e += blockDim.x) {
+        const int i = e / nb, c = e - i * nb;
+        xs[(size_t)c * ld + i] = src[(size_t)i * n + k0 + c];
     }
+    for (int i = threadIdx.x; i < n; i += blockDim.x) pos[i] = ipos[i] = i;
     __syncthreads();
-    if (a.kappa) {
-        double best = 0.0;
-        for (int c = threadIdx.x; c < hn; c += blockDim.x) {
-            double cs = 0.0;
-            for (int i = 0; i < n; ++i) {
-                const double2 z = A[(size_t)i * n + c0 + c];
-                cs += sqrt(z.x * z.x + z.y * z.y);
-            }
-            best = fmax(best, cs);
-        }
-        for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_down_sync(0xffffffffu, best, o));
-        if (lane == 0)
-            atomicMax(reinterpret_cast<unsigned long long*>(&s_anorm), (unsigned long long)__double_as_longlong(best));
+    unsigned free_rows = 0;                             // rows of this thread that may still serve as pivot
+#pragma unroll
+    for (int u = 0; u < PANEL_ROWS; ++u) {
+        const int i = row0 + u * stride;
+        if (i >= k0 && i < n) free_rows |= 1u << u;
     }
-    __syncthreads();
-
-    int bad = 0;
-    for (int k = 0; k < n; ++k) {
-        const int owner = k / h, kc = k - owner * h, par = k & 1;
-        if (rank == owner) {
-            float best = -1.0f;
-            int bi = n;
-            for (int i = k + threadIdx.x; i < n; i += blockDim.x) {
-                const float2 z = Xs[i * h + kc];
-                const float v = z.x * z.x + z.y * z.y;
-                if (v > best) {
-                    best = v;
-                    bi = i;
+    const int c_lo = grp * bc, c_hi = min(nb, c_lo + bc);
+    auto publish = [&](int c) {                         // best free row of column c, by the warps of its group
+        unsigned long long key = 0;
+        int row = 0x7fffffff;
+#pragma unroll
+        for (int u = 0; u < PANEL_ROWS; ++u)
+            if (free_rows >> u & 1) {
+                const unsigned long long q = mag_key(cabs2<T>(xs[(size_t)c * ld + row0 + u * stride]));
+                if (q > key) {
+                    key = q;
+                    row = row0 + u * stride;
                 }
             }
-            for (int o = 16; o > 0; o >>= 1) {
-                const float ov = __shfl_down_sync(0xffffffffu, best, o);
-                const int oi = __shfl_down_sync(0xffffffffu, bi, o);
-                if (ov > best || (ov == best && oi < bi)) {
-                    best = ov;
-                    bi = oi;
-                }
-            }
+        warp_best<T>(key, row);
+        if (lane == 0) {
+            wkey[rw] = key;
+            wrow[rw] = row;
+        }
+    };
+    if (grp == 0) publish(0);
+    bool bad = false;
+    for (int k = 0; k < nb; ++k) {
+        __syncthreads();
+        unsigned long long key = lane < RW ? wkey[lane] : 0ull;
+        int p = lane < RW ? wrow[lane] : 0x7fffffff;
+        warp_best<T>(key, p);
+        if (key <= 1ull) {                              // no free row with a non-zero entry (uniform over the CTA)
+            bad = true;
+            break;
+        }
+        C f[PANEL_ROWS];                                // column k of this thread's rows before it is overwritten
+#pragma unroll
+        for (int u = 0; u < PANEL_ROWS; ++u) {
+            const int i = row0 + u * stride;
+            if (i < n) f[u] = xs[(size_t)k * ld + i];
+        }
+        if (threadIdx.x < 32) {
+            // the pivot row, scaled, and the exchange of positions
+            const C pv = xs[(size_t)k * ld + p];
+            const T d = (T)1 / cabs2<T>(pv);
+            const C inv = mk<T>(pv.x * d, -pv.y * d);
+            for (int c = lane; c < nb; c += 32) prow[c] = c == k ? inv : cmul(xs[(size_t)c * ld + p], inv);
             if (lane == 0) {
-                red_v[warp] = best;
-                red_i[warp] = bi;
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                float bv = red_v[0];
-                int bix = red_i[0];
-                for (int w = 1; w < GJC_WARPS; ++w)
-                    if (red_v[w] > bv || (red_v[w] == bv && red_i[w] < bix)) {
-                        bv = red_v[w];
-                        bix = red_i[w];
-                    }
-                const int sing = !(bv > 0.0f) || bix >= n;
-                if (sing) bix = k;
-                s_bad[par] = sing;
-                s_p[par] = bix;
-                s_pv[par] = Xs[bix * h + kc];
-            }
-            __syncthreads();
-            const int p = s_p[par];
-            for (int i = threadIdx.x; i < n; i += blockDim.x) {
-                const int src = (i == k) ? p : (i == p ? k : i);
-                F[par * n + i] = Xs[src * h + kc];
+                const int l = ipos[p], r = pos[k0 + k];
+                pos[l] = r;
+                ipos[r] = l;
+                pos[k0 + k] = p;
+                ipos[p] = k0 + k;
             }
         }
-        cl.sync();
-        const int p = cl.map_shared_rank(s_p, owner)[par];
-        bad = cl.map_shared_rank(s_bad, owner)[par];
-        const float2 pv = cl.map_shared_rank(s_pv, owner)[par];
-        if (bad) break;
-        const float2* Fr = cl.map_shared_rank(F, owner) + par * n;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) Fl[i] = Fr[i];
-        if (threadIdx.x == 0) piv[k] = p;
-        if (p != k)
-            for (int c = threadIdx.x; c < hn; c += blockDim.x) {
-                const float2 t = Xs[k * h + c];
-                Xs[k * h + c] = Xs[p * h + c];
-                Xs[p * h + c] = t;
-            }
         __syncthreads();
-        const float d = 1.0f / (pv.x * pv.x + pv.y * pv.y);
-        const float2 inv = make_float2(pv.x * d, -pv.y * d);
-        for (int c = threadIdx.x; c < hn; c += blockDim.x)
-            rowk[c] = (rank == owner && c == kc) ? inv : cmul(Xs[k * h + c], inv);
-        __syncthreads();
-        for (int i = warp; i < n; i += GJC_WARPS) {
-            const float2 f = Fl[i];
-            for (int c = lane; c < hn; c += 32) {
-                const float2 r = rowk[c];
-                if (i == k) {
-                    Xs[k * h + c] = r;
+#pragma unroll
+        for (int u = 0; u < PANEL_ROWS; ++u) {
+            const int i = row0 + u * stride;
+            if (i < n) {
+                if (i == p) {
+                    for (int c = c_lo; c < c_hi; ++c) xs[(size_t)c * ld + i] = prow[c];
+                    free_rows &= ~(1u << u);
                 } else {
-                    float2 x = (rank == owner && c == kc) ? make_float2(0.f, 0.f) : Xs[i * h + c];
-                    x.x -= f.x * r.x - f.y * r.y;
-                    x.y -= f.x * r.y + f.y * r.x;
-                    Xs[i * h + c] = x;
+                    const C fi = f[u];
+#pragma unroll 4
+                    for (int c = c_lo; c < c_hi; ++c) {
+                        const C r = prow[c];
+                        C x = c == k ? mk<T>(0, 0) : xs[(size_t)c * ld + i];
+                        x.x -= fi.x * r.x - fi.y * r.y;
+                        x.y -= fi.x * r.y + fi.y * r.x;
+                        xs[(size_t)c * ld + i] = x;
+                    }
                 }
             }
         }
-        __syncthreads();
+        if (k + 1 < nb && k + 1 >= c_lo && k + 1 < c_hi) publish(k + 1);
     }
+    __syncthreads();
     if (bad) {
-        if (rank == 0) {
-            if (threadIdx.x == 0) {
-                a.flags[b] = 1;
-                if (a.kappa) a.kappa[b] = 0.0;
-            }
-            for (int j = threadIdx.x; j < n; j += blockDim.x) a.diag_inv[(size_t)b * n + j] = make_double2(0.0, 0.0);
-        }
-        cl.sync();    // no CTA leaves while another may still read its shared memory
+        if (threadIdx.x == 0) flags[b] = 1;
         return;
     }
-    // the inverse's column j is the eliminated matrix's column idx[j]
-    if (threadIdx.x == 0) {
-        for (int c = 0; c < n; ++c) idx[c] = c;
-        for (int kk = n - 1; kk >= 0; --kk) {
-            const int t = idx[kk];
-            idx[kk] = idx[piv[kk]];
-            idx[piv[kk]] = t;
-        }
-        if (rank == 0) a.flags[b] = 0;
+    M += (size_t)b * nb * n;
+    for (int c = 0; c < nb; ++c)
+        for (int i = threadIdx.x; i < n; i += blockDim.x) M[(size_t)c * n + i] = xs[(size_t)c * ld + pos[i]];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        perm[(size_t)b * n + i] = pos[i];
+        ipos[i] = rows[(size_t)b * n + pos[i]];
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < n; j += blockDim.x) jof[idx[j]] = j;
-    __syncthreads();
-    float2* Xg = a.X + (size_t)b * n * n;
-    for (int i = warp; i < n; i += GJC_WARPS)
-        for (int c = lane; c < hn; c += 32) Xg[(size_t)i * n + jof[c0 + c]] = Xs[i * h + c];
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const int cgl = idx[j] - c0;
-        if (cgl >= 0 && cgl < hn) {
-            const float2 z = Xs[j * h + cgl];
-            a.diag_inv[(size_t)b * n + j] = make_double2((double)z.x, (double)z.y);
-        }
-    }
-    if (a.kappa) {
-        double best = 0.0;
-        for (int c = threadIdx.x; c < hn; c += blockDim.x) {
-            double cs = 0.0;
-            for (int i = 0; i < n; ++i) {
-                const float2 z = Xs[i * h + c];
-                cs += sqrt((double)z.x * z.x + (double)z.y * z.y);
-            }
-            best = fmax(best, cs);
-        }
-        for (int o = 16; o > 0; o >>= 1) best = fmax(best, __shfl_down_sync(0xffffffffu, best, o));
-        if (lane == 0)
-            atomicMax(reinterpret_cast<unsigned long long*>(&s_xnorm), (unsigned long long)__double_as_longlong(best));
-    }
-    cl.sync();
-    if (a.kappa && rank == 0 && threadIdx.x == 0) {
-        double an = 0.0, xn = 0.0;
-        for (int r = 0; r < GJC_CS; ++r) {
-            an = fmax(an, *cl.map_shared_rank(&s_anorm, r));
-            xn = fmax(xn, *cl.map_shared_rank(&s_xnorm, r));
-        }
-        a.kappa[b] = an * xn;
-    }
-    cl.sync();    // rank 0 has read every CTA's norms
+    for (int i = threadIdx.x; i < n; i += blockDim.x) rows[(size_t)b * n + i] = ipos[i];
 }
 
-size_t gjc_smem(int n) {
-    const int h = (n + GJC_CS - 1) / GJC_CS;
-    return ((size_t)n * h + 3 * (size_t)n + h) * sizeof(float2) + 3 * (size_t)n * sizeof(int);
+// The other columns (see above).  Grid (column tile, row tile, matrix); thread (tx, ty) holds rows ty 4 .. + 3 and
+// columns tx + 16 u of a 64 x 64 tile, the panel's multipliers and pivot rows staged once in shared memory.
+template <typename T>
+__global__ void __launch_bounds__(256) k_inv_update(int n, int k0, int nb, const cplx<T>* src, cplx<T>* dst,
+                                                    const cplx<T>* M, const int* perm, const int* rows, int last,
+                                                    const int* flags) {
+    using C = cplx<T>;
+    constexpr int PB = InvCfg<T>::PB;
+    __shared__ __align__(16) C ms[PB][UPD];
+    __shared__ __align__(16) C rs[PB][UPD];
+    const int b = blockIdx.z;
+    if (flags[b]) return;
+    src += (size_t)b * n * n;
+    dst += (size_t)b * n * n;
+    M += (size_t)b * nb * n;
+    perm += (size_t)b * n;
+    rows += (size_t)b * n;
+    const int i0 = blockIdx.y * UPD, j0 = blockIdx.x * UPD;
+    for (int e = threadIdx.x; e < nb * UPD; e += 256) {
+        const int c = e / UPD, x = e % UPD;
+        ms[c][x] = i0 + x < n ? M[(size_t)c * n + i0 + x] : mk<T>(0, 0);
+        rs[c][x] = j0 + x < n ? src[(size_t)perm[k0 + c] * n + j0 + x] : mk<T>(0, 0);
+    }
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    C acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = i0 + ty * 4 + r;
+        const bool keep = i < n && (i < k0 || i >= k0 + nb);
+        const C* s = src + (keep ? (size_t)perm[i] * n : 0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = j0 + tx + 16 * u;
+            acc[r][u] = keep && j < n ? s[j] : mk<T>(0, 0);
+        }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int c = 0; c < nb; ++c) {
+        C m[4], x[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) m[r] = ms[c][ty * 4 + r];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = rs[c][tx + 16 * u];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) cfma(acc[r][u], m[r], x[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int j = j0 + tx + 16 * u;
+        if (j >= n) continue;
+        const bool in_panel = j >= k0 && j < k0 + nb;
+        const int jd = last ? rows[j] : j;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int i = i0 + ty * 4 + r;
+            if (i < n) dst[(size_t)i * n + jd] = in_panel ? ms[j - k0][ty * 4 + r] : acc[r][u];
+        }
+    }
+}
+
+// The diagonal of the inverse, and kappa_1 = |A|_1 |X|_1 (mixed path; xnorm starts at 0 and is read by the callers
+// that need kappa).  Singular matrices get a zero diagonal.
+template <typename T>
+__global__ void __launch_bounds__(256) k_inv_finish(int n, const cplx<T>* X, const int* flags, double* xnorm,
+                                                    double2* diag_inv, double* L) {
+    __shared__ double sums[4][64];
+    const int b = blockIdx.x, tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+    const int j = blockIdx.y * 64 + tx;
+    X += (size_t)b * n * n;
+    const bool bad = flags[b] != 0;
+    if (j < n && ty == 0) {
+        const cplx<T> z = bad ? mk<T>(0, 0) : X[(size_t)j * n + j];
+        diag_inv[(size_t)b * n + j] = make_double2((double)z.x, (double)z.y);
+        if constexpr (sizeof(T) == 8) L[(size_t)b * n + j] = -(double)z.y;
+    }
+    if constexpr (sizeof(T) == 4) {
+        double cs = 0.0;
+        if (j < n && !bad)
+            for (int i = ty; i < n; i += 4) cs += (double)cabs_safe(X[(size_t)i * n + j]);
+        sums[ty][tx] = cs;
+        __syncthreads();
+        if (ty == 0 && j < n) {
+            cs = (sums[0][tx] + sums[1][tx]) + (sums[2][tx] + sums[3][tx]);
+            atomicMax(reinterpret_cast<unsigned long long*>(xnorm + b), (unsigned long long)__double_as_longlong(cs));
+        }
+    }
 }
 
 // FP64 correction of the diagonal of X ~ A^-1 for the blocks with kappa_1 above
@@ -438,13 +331,13 @@ size_t gjc_smem(int n) {
 // Grid (block, 32-column panel).  The other blocks keep X_jj.
 constexpr int RF_COLS = 32;
 __global__ void __launch_bounds__(256) k_refine_diag(int n, const double2* Aall, const float2* Xall,
-                                                     const int* flags, const double* kappa, double kappa_refine,
+                                                     const int* flags, const double* norms, double kappa_refine,
                                                      double2* diag_inv, double* L, double* resid) {
     __shared__ double2 s_d[RF_COLS];
     const int b = blockIdx.x, j0 = blockIdx.y * RF_COLS;
     if (flags[b] || j0 >= n) return;
     const float2* X = Xall + (size_t)b * n * n;
-    if (!(kappa[b] > kappa_refine)) {
+    if (!(norms[b] * norms[gridDim.x + b] > kappa_refine)) {
         if (threadIdx.x < RF_COLS && j0 + threadIdx.x < n) {
             const int j = j0 + threadIdx.x;
             const float2 x = X[(size_t)j * n + j];
@@ -504,14 +397,14 @@ __global__ void __launch_bounds__(256) k_refine_diag(int n, const double2* Aall,
 // becomes -L_j.  Blocks corrected in FP64 keep their values.
 constexpr int QF = 32;
 __global__ void __launch_bounds__(256) k_loss_quadform(int n, const double2* Aall, const float2* Xall,
-                                                       const int* flags, const double* kappa, double kappa_refine,
+                                                       const int* flags, const double* norms, double kappa_refine,
                                                        double2* diag_inv, double* L) {
     __shared__ float2 Xs[QF][QF + 1];
     __shared__ float2 Bs[QF][QF + 1];
     __shared__ double2 At[QF][QF + 1];       // A_lk tile, read along rows, used transposed
     __shared__ float Lrow[QF];
     const int b = blockIdx.x, j0 = blockIdx.y * QF;
-    if (flags[b] || kappa[b] > kappa_refine) return;
+    if (flags[b] || norms[b] * norms[gridDim.x + b] > kappa_refine) return;
     const double2* A = Aall + (size_t)b * n * n;
     const float2* X = Xall + (size_t)b * n * n;
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -583,65 +476,96 @@ __global__ void __launch_bounds__(256) k_loss_quadform(int n, const double2* Aal
 
 }  // namespace
 
+// Inverse of nmat matrices of order n into X; B2 holds as many for the out-of-place updates, aux the panels and row
+// orders.  norms (mixed path): |A|_1 of every matrix, then |X|_1.
+template <typename T>
+static cudaError_t invert_batch(cudaStream_t st, int n, int nmat, const double2* A, cplx<T>* X, cplx<T>* B2, void* aux,
+                                double* anorm, double* xnorm, double2* eps_diag, double* L, double* L_nolfe,
+                                double2* diag_inv, int* flags) {
+    using C = cplx<T>;
+    int pb = InvCfg<T>::PB;
+    auto smem_of = [&](int w) {
+        return ((size_t)w * (n | 1) + w) * sizeof(C) + 32 * (sizeof(unsigned long long) + sizeof(int)) + 2 * (size_t)n * sizeof(int);
+    };
+    while (pb > 1 && smem_of(pb) > PANEL_SMEM) pb >>= 1;
+    pb = std::min(pb, n);
+    C* M = reinterpret_cast<C*>(aux);
+    int* perm = reinterpret_cast<int*>(M + (size_t)nmat * pb * n);
+    int* rows = perm + (size_t)nmat * n;
+    const size_t smem = smem_of(pb);
+    cudaError_t e = cudaFuncSetAttribute((const void*)k_inv_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int npan = (n + pb - 1) / pb;
+    C* cur = npan & 1 ? B2 : X;                         // the last update lands in X
+    C* nxt = npan & 1 ? X : B2;
+    const dim3 cols(nmat, (n + 63) / 64);
+    k_inv_load<T><<<cols, 256, 0, st>>>(n, A, cur, anorm, eps_diag, L_nolfe, rows, flags);
+    const int RW = std::min((n + 31) / 32, 32);
+    int groups = 1;
+    while (groups * 2 * RW <= 16 && groups * 2 <= pb) groups *= 2;
+    const int bc = (pb + groups - 1) / groups;
+    const dim3 tiles((n + UPD - 1) / UPD, (n + UPD - 1) / UPD, nmat);
+    for (int p = 0; p < npan; ++p) {
+        const int k0 = p * pb, nb = std::min(pb, n - k0);
+        k_inv_panel<T><<<nmat, 32 * RW * groups, smem, st>>>(n, k0, nb, RW, bc, cur, M, perm, rows, flags);
+        k_inv_update<T><<<tiles, 256, 0, st>>>(n, k0, nb, cur, nxt, M, perm, rows, p + 1 == npan, flags);
+        std::swap(cur, nxt);
+    }
+    k_inv_finish<T><<<cols, 256, 0, st>>>(n, X, flags, xnorm, diag_inv, L);
+    return cudaGetLastError();
+}
+
+// Matrices are inverted in groups whose second copy stays within INV_COPY_BYTES (at least one), so that the scratch
+// does not grow with the number of frequencies.
+constexpr size_t INV_COPY_BYTES = 1ull << 30;
+
+template <typename T>
+static cudaError_t invert_all(qcx_ctx* ctx, QSlot& s, double* norms, double* L) {
+    using C = cplx<T>;
+    const int n = s.ng, nw = s.nw;
+    const size_t one = (size_t)n * n * sizeof(C);
+    const int per = (int)std::min<size_t>({(size_t)nw, std::max<size_t>(1, INV_COPY_BYTES / one), 32768});
+    cudaError_t e = s.work2.ensure(per * one);
+    if (e != cudaSuccess) return e;
+    e = s.gjaux.ensure((size_t)per * n * (InvCfg<T>::PB * sizeof(C) + 2 * sizeof(int)));
+    if (e != cudaSuccess) return e;
+    for (int w0 = 0; w0 < nw; w0 += per) {
+        const int m = std::min(per, nw - w0);
+        const size_t o = (size_t)w0 * n;
+        e = invert_batch<T>(ctx->stream, n, m, s.eps.as<double2>() + o * n, s.work.as<C>() + o * n, s.work2.as<C>(),
+                            s.gjaux.p, norms ? norms + w0 : nullptr, norms ? norms + nw + w0 : nullptr,
+                            s.eps_diag.as<double2>() + o, L + o, L + (size_t)nw * n + o, s.diag_inv.as<double2>() + o,
+                            s.flags.as<int>() + w0);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t qcx_launch_invert(qcx_ctx* ctx, QSlot& s, qcx_precision prec, double* d_loss_out) {
     const int n = s.ng;
     if (prec == QCX_FP64) {
-        InvArgs<double> a{};
-        a.ng = n;
-        a.nw = s.nw;
-        a.eps64 = s.eps.as<double2>();
-        a.X = s.work.as<double2>();
-        a.diag_inv = s.diag_inv.as<double2>();
-        a.eps_diag = s.eps_diag.as<double2>();
-        a.L = d_loss_out;
-        a.flags = s.flags.as<int>();
-        a.kappa = nullptr;
-        const size_t smem = (size_t)n * 2 * sizeof(double2) + (size_t)n * 2 * sizeof(int);
-        cudaError_t e = cudaFuncSetAttribute((const void*)k_gauss_jordan<double>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_gauss_jordan<double><<<s.nw, INV_THREADS, smem, ctx->stream>>>(a, 1);
-        e = cudaGetLastError();
+        cudaError_t e = invert_all<double>(ctx, s, nullptr, d_loss_out);
         if (e != cudaSuccess) return e;
         return cudaMemsetAsync(s.resid.p, 0, sizeof(double) * s.nw, ctx->stream);
     }
-    InvArgs<float> a{};
-    a.ng = n;
-    a.nw = s.nw;
-    a.eps64 = s.eps.as<double2>();
-    a.X = s.work.as<float2>();
-    cudaError_t e = s.kappa1.ensure(sizeof(double) * s.nw);
+    cudaError_t e = s.kappa1.ensure(2 * sizeof(double) * s.nw);
     if (e != cudaSuccess) return e;
-    a.kappa = s.kappa1.as<double>();
-    a.diag_inv = s.diag_inv.as<double2>();
-    a.eps_diag = s.eps_diag.as<double2>();
-    a.L = d_loss_out;
-    a.flags = s.flags.as<int>();
-    if (n <= GJC_MAXN) {
-        // the matrix stays in the shared memory of a GJC_CS-CTA cluster
-        const size_t smem = gjc_smem(n);
-        e = cudaFuncSetAttribute((const void*)k_gj_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_gj_cluster<<<s.nw * GJC_CS, GJC_THREADS, smem, ctx->stream>>>(a);
-    } else {
-        const size_t smem = (size_t)n * 2 * sizeof(float2) + (size_t)n * 2 * sizeof(int);
-        e = cudaFuncSetAttribute((const void*)k_gauss_jordan<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-        if (e != cudaSuccess) return e;
-        k_gauss_jordan<float><<<s.nw, INV_THREADS, smem, ctx->stream>>>(a, 0);
-    }
-    e = cudaGetLastError();
+    double* norms = s.kappa1.as<double>();
+    e = cudaMemsetAsync(norms, 0, 2 * sizeof(double) * s.nw, ctx->stream);
+    if (e != cudaSuccess) return e;
+    e = invert_all<float>(ctx, s, norms, d_loss_out);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(s.resid.p, 0, sizeof(double) * s.nw, ctx->stream);
     if (e != cudaSuccess) return e;
     dim3 grid(s.nw, (n + RF_COLS - 1) / RF_COLS);
-    k_refine_diag<<<grid, 256, 0, ctx->stream>>>(n, a.eps64, a.X, a.flags, a.kappa, ctx->kappa_refine, a.diag_inv,
-                                                  d_loss_out, s.resid.as<double>());
+    k_refine_diag<<<grid, 256, 0, ctx->stream>>>(n, s.eps.as<double2>(), s.work.as<float2>(), s.flags.as<int>(), norms,
+                                                  ctx->kappa_refine, s.diag_inv.as<double2>(), d_loss_out,
+                                                  s.resid.as<double>());
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     dim3 gq(s.nw, (n + QF - 1) / QF);
-    k_loss_quadform<<<gq, 256, 0, ctx->stream>>>(n, a.eps64, a.X, a.flags, a.kappa, ctx->kappa_refine, a.diag_inv,
-                                                  d_loss_out);
+    k_loss_quadform<<<gq, 256, 0, ctx->stream>>>(n, s.eps.as<double2>(), s.work.as<float2>(), s.flags.as<int>(), norms,
+                                                  ctx->kappa_refine, s.diag_inv.as<double2>(), d_loss_out);
     return cudaGetLastError();
 }
 

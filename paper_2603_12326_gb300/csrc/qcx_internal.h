@@ -63,10 +63,11 @@ struct QSlot {
     DevBuf vs32;               // [ng] float
     DevBuf rho;                // FP64: [ng][nt] double2 ; MIXED: three BF16 planes [ngp][kp]
     DevBuf eps;                // [nw][ng][ng] double2 (MIXED stores eps^T: row G', column G)
-    DevBuf work;               // inverse work space
+    DevBuf work;               // inverse [nw][ng][ng]
+    DevBuf work2, gjaux;       // second copy, panels and row orders of one group of matrices being inverted
     DevBuf acc64;              // FP64 partial sums of the tensor-core chi0 (one region per CTA)
     DevBuf wtab;               // [nw][kp/2] float2 transition weights of the mixed path
-    DevBuf kappa1;             // [nw] double condition estimates of the mixed inverse
+    DevBuf kappa1;             // [2][nw] double |A|_1 and |X|_1 of the mixed inverse (kappa_1 is their product)
     DevBuf w;                  // [nw] double
     DevBuf diag_inv;           // [nw][ng] double2
     DevBuf eps_diag;           // [nw][ng] double2
