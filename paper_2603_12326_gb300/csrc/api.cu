@@ -419,15 +419,18 @@ qcx_status qcx_chi0(qcx_ctx* ctx, int iq, int nw, const double* w, double eta, q
             chi = ctx->scratch.as<double2>();
         }
     }
+    CUDA_OR_FAIL(s.flags.ensure(sizeof(int) * (nw > 4 ? nw : 4)), "alloc");
+    CUDA_OR_FAIL(cudaMemsetAsync(s.flags.p, 0, sizeof(int), ctx->stream), "clear status");
+    bool tensor = prec == QCX_MIXED;
     if (prec == QCX_FP64) {
-        CUDA_OR_FAIL(qcx_launch_chi0_fp64(ctx, s, iq, chi), "chi0 fp64 kernel");
+        CUDA_OR_FAIL(qcx_launch_chi0_fp64(ctx, s, iq, chi, s.flags.as<int>(), &tensor), "chi0 fp64 kernel");
     } else {
-        CUDA_OR_FAIL(s.flags.ensure(sizeof(int) * (nw > 4 ? nw : 4)), "alloc");
-        CUDA_OR_FAIL(cudaMemsetAsync(s.flags.p, 0, sizeof(int), ctx->stream), "clear status");
         cudaError_t e = qcx_launch_chi0_mixed(ctx, s, iq, chi, s.flags.as<int>());
         if (e == cudaErrorNotSupported)
             return ctx->fail(QCX_ERR_UNSUPPORTED, "chi0: this G-set size is not handled by the tensor-core kernel");
         CUDA_OR_FAIL(e, "chi0 tensor-core kernel");
+    }
+    if (tensor) {
         int st = 0;
         CUDA_OR_FAIL(cudaMemcpyAsync(&st, s.flags.p, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), "status");
         CUDA_OR_FAIL(cudaStreamSynchronize(ctx->stream), "sync");

@@ -16,6 +16,7 @@ namespace {
 constexpr int TG = 32;   // G tile
 constexpr int TK = 16;   // transitions per stage
 constexpr int TW = 4;    // frequencies per CTA
+constexpr long long TC_MIN_NT = 32;
 
 struct Chi64Args {
     const double2* R;     // [ng][nt]
@@ -126,7 +127,8 @@ __global__ void __launch_bounds__(256) k_chi0_fp64(Chi64Args a) {
 
 }  // namespace
 
-cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out) {
+cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out, int* d_status, bool* used_tc) {
+    *used_tc = false;
     Chi64Args a;
     a.R = s.rho.as<double2>();
     a.nt = (long long)ctx->nk * ctx->nv * ctx->nc;
@@ -145,6 +147,19 @@ cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0
     a.vs = s.vs.as<double>();
     a.eps = s.eps.as<double2>();
     a.chi = d_chi0_out;
+    // The tensor-core route, except for a handful of transitions, when its work space does not fit, or while the
+    // stream is being captured (the status word could not be read).  This kernel walks the transitions serially
+    // at ~5.2 us each whatever N_G and N_w up to a full GPU (measured 425 us at N_t = 80, 15.8 ms at 3072); the
+    // tensor-core route starts at ~120 us for its launches.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (a.nt >= TC_MIN_NT && cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+        const cudaError_t e = qcx_launch_chi0_fp64_tc(ctx, s, iq, a.pref, d_chi0_out, d_status);
+        if (e != cudaErrorMemoryAllocation) {
+            *used_tc = true;
+            return e;
+        }
+        cudaGetLastError();
+    }
     dim3 grid((s.ng + TG - 1) / TG, (s.ng + TG - 1) / TG, (s.nw + TW - 1) / TW);
     k_chi0_fp64<<<grid, 256, 0, ctx->stream>>>(a);
     return cudaGetLastError();

@@ -135,6 +135,12 @@ struct OpticalBufs {
     int nk = 0;
 };
 
+// Digit planes and partial sums of the FP64 chi0 on the tensor cores (chi0_fp64_tc.cu).
+struct OzBufs {
+    DevBuf a, b;               // digits of rho and of W rho
+    DevBuf w, e, part;         // weights of a group of frequencies, row exponents, FP64 sums per K split
+};
+
 // Work space of the spectral route to chi0 (one q at a time, either precision).
 struct SpecBufs {
     DevBuf bin, x;             // [nt] grid point and hat weight of each transition
@@ -216,6 +222,7 @@ struct qcx_ctx {
     int withhold_copies = 0;       // fault injection (tests): the per-q tensor-core kernel issues no copies
     MlpState* mlp = nullptr;       // surrogate network (parameters, Adam moments, work buffers)
     SpecBufs spec;                 // spectral route work space
+    OzBufs oz;                     // FP64 chi0 on the tensor cores
     OpticalBufs optical;           // optical-limit work space
     int spec_chunk_bins = 0;       // grid points per chunk of the spectral route (0: from a 4 GiB budget)
     int spec_cuda_cores = 0;       // mixed spectral contraction on the CUDA cores (FP32) instead of tcgen05
@@ -287,7 +294,9 @@ cudaError_t qcx_spec_tc_contract(cudaStream_t st, const CUtensorMap* kmaps, cons
                                  long long wait_limit);
 
 // chi0 (chi0_fp64.cu, chi0_tc.cu)
-cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out);
+// FP64: sets *used_tc when the tensor-core route ran (its status word is then to be read)
+cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out, int* d_status, bool* used_tc);
+cudaError_t qcx_launch_chi0_fp64_tc(qcx_ctx* ctx, QSlot& s, int iq, double pref, double2* chi, int* d_status);
 cudaError_t qcx_launch_chi0_mixed(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out, int* d_status);
 // 2-D tensor map over one BF16 plane [rows][kp], box {box_k, box_rows} (box_k 16: 32-byte
 // swizzle, 32: 64-byte swizzle)
