@@ -214,12 +214,14 @@ qcx_status qcx_overlap(qcx_ctx* ctx, int nk, const double* kpts, qcx_c64* out_S)
     const size_t nout = (size_t)nk * ctx->nb * ctx->nb * sizeof(double2);
     CUDA_OR_FAIL(ctx->scratch2.ensure(3 * sizeof(double) * nk), "alloc");
     CUDA_OR_FAIL(qcx_copy_in(ctx, ctx->scratch2.p, kpts, 3 * sizeof(double) * nk), "copy kpts");
+    std::vector<double> kh;
+    CUDA_OR_FAIL(fetch(ctx, kh, kpts, 3 * (size_t)nk), "overlap kpts");
     double2* dst = qcx_is_device_ptr(out_S) ? reinterpret_cast<double2*>(out_S) : nullptr;
     if (!dst) {
         CUDA_OR_FAIL(ctx->scratch.ensure(nout), "alloc");
         dst = ctx->scratch.as<double2>();
     }
-    CUDA_OR_FAIL(qcx_launch_overlap(ctx, nk, ctx->scratch2.as<double>(), dst), "overlap kernel");
+    CUDA_OR_FAIL(qcx_launch_overlap(ctx, nk, ctx->scratch2.as<double>(), kh.data(), dst), "overlap kernel");
     if (dst != reinterpret_cast<double2*>(out_S)) CUDA_OR_FAIL(qcx_copy_out(ctx, out_S, dst, nout), "copy out");
     return QCX_OK;
 }
@@ -296,10 +298,10 @@ qcx_status qcx_pair_density(qcx_ctx* ctx, int iq, int ng, const int* G_int, qcx_
     CUDA_OR_FAIL(ctx->scratch2.ensure(3 * sizeof(int) * ng), "alloc");
     CUDA_OR_FAIL(qcx_copy_in(ctx, ctx->scratch2.p, G_int, 3 * sizeof(int) * ng), "copy G");
     CUDA_OR_FAIL(qcx_launch_qsetup(ctx, s, ctx->scratch2.as<int>(), ng, &ctx->qpts[3 * iq]), "q setup");
-    if (prec == QCX_MIXED) {
+    {
         std::vector<int> Gh;
         CUDA_OR_FAIL(fetch(ctx, Gh, G_int, 3 * (size_t)ng), "G list");
-        CUDA_OR_FAIL(qcx_pd_tab_prepare(ctx, s, Gh.data(), ng, iq), "pair-density tables");
+        CUDA_OR_FAIL(qcx_pd_tab_prepare(ctx, s, Gh.data(), ng, iq, prec), "pair-density tables");
     }
     if (prec == QCX_FP64) {
         CUDA_OR_FAIL(s.rho.ensure((size_t)ng * nt * sizeof(double2)), "alloc rho");

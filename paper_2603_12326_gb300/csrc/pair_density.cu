@@ -23,6 +23,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 namespace {
 
@@ -55,10 +56,8 @@ template <typename T> struct PDArgs {
     __nv_bfloat162* R2;      // x2 = bf16(x - x0 - x1)
     long long kp2;           // row length of the BF16 planes in bf16x2 units
     cplx<T>* Sout;           // overlap mode: [nk][nb][nb]
-    // tables of the mixed path (PdTab): one-dimensional factors per (pair, axis, k class, q+G
-    // class) and the factor of (pair, G)
-    const float2* ptab;      // [entries][NCH][4]
-    const float2* pcmn;      // [npair][ng]
+    // tables (PdTab): one-dimensional factors per (pair, axis, k class, q+G class)
+    const cplx<T>* ptab;     // [entries][NCH][4], or null
     const int* kidx;         // [nk][3]
     const int* gidx;         // [ng][3]
     int nkx[3], nqx[3];
@@ -206,28 +205,35 @@ __device__ __forceinline__ void store_split3(float re, float im, __nv_bfloat162*
     R2[o] = __floats2bfloat162_rn(rr - mf.x, ri - mf.y);
 }
 
-// Arguments of the table kernels (arithmetic in T, FP32 results).
 template <typename T> struct PdTabArgs {
-    const T* par;            // [npair][8]
+    const double* par;       // [npair][8]
     const cplx<T>* tab;      // lattice terms {w_n, d_n}
     const int* dir_off;
     const int* dir_cnt;
     const int* dir_nlo;
-    T h;
+    double h;
     T charre[4][3], charim[4][3];
     const double* kval;      // k classes, axes concatenated
     const double* qval;      // q+G classes, axes concatenated
-    const T* kappa;          // [ng][3] q + G
     int nkx[3], nqx[3], kofs[3], qofs[3];
     long long tbase[4];
-    int npair, ng;
-    float2* out;             // [entries][NCH][4]
-    float2* cmn;             // [npair][ng]
+    cplx<T>* out;            // [entries][NCH][4]
 };
+
+__device__ __forceinline__ void sincos_reduced(double x, double* s, double* c) { sincos(x, s, c); }
+// FP32: the angle is reduced to [-pi, pi] in FP64 first, so its error is that of the FP32 angle there and not
+// 2^-24 of the whole angle
+__device__ __forceinline__ void sincos_reduced(double x, float* s, float* c) {
+    const double r = fma(-rint(x * 0.15915494309189535), 6.283185307179586, x);
+    sincosf((float)r, s, c);
+}
 
 // One entry of the one-dimensional table: for shell-group pair ip, axis x, the k component of
 // class ik and the q+G component of class iq, the factors E(0,0), E(1,0), E(0,1), E(1,1) of every
-// character, by the lattice sum of pair_block_vals (same operations, same order) in T.
+// character by the lattice sum of pair_block_vals, times the axis's share of the pair's factor
+// e^{-kappa_x^2/4p} e^{i kappa_x P_x} (the x axis also carries pref / number of characters) and the
+// p normalisations 2 sqrt(alpha), 2 sqrt(beta): a component of the block is then a plain product of
+// three entries.
 template <typename T, int NCH> __global__ void k_pd_axis_table(PdTabArgs<T> a) {
     using C = cplx<T>;
     const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -238,18 +244,22 @@ template <typename T, int NCH> __global__ void k_pd_axis_table(PdTabArgs<T> a) {
     r /= a.nqx[x];
     const int ik = (int)(r % a.nkx[x]);
     const int ip = (int)(r / a.nkx[x]);
-    const T kk = (T)a.kval[a.kofs[x] + ik], kap = (T)a.qval[a.qofs[x] + iq];
-    const T* par = a.par + (size_t)ip * 8;
-    const T p = par[0], ap = par[1], bp = par[2];
+    const double kd = a.kval[a.kofs[x] + ik], qd = a.qval[a.qofs[x] + iq];
+    const double* par = a.par + (size_t)ip * 8;
+    const T kap = (T)qd, p = (T)par[0], ap = (T)par[1], bp = (T)par[2];
     const T inv2p = T(0.5) / p;
     const int di = ip * 3 + x;
     const int off = a.dir_off[di], cnt = a.dir_cnt[di], nlo = a.dir_nlo[di];
-    const T theta = (kk + bp * kap) * a.h;
     const T tk = kap * inv2p;
     T zs, zc;
-    sincos_t(theta, &zs, &zc);
+    sincos_reduced((kd + par[2] * qd) * a.h, &zs, &zc);
     const C z = mk<T>(zc, zs);
-    float4* out = reinterpret_cast<float4*>(a.out + e * (NCH * 4));
+    sincos_reduced(qd * par[4 + x], &zs, &zc);
+    T amp = exp_t(-kap * kap * T(0.25) / p);
+    if (x == 0) amp *= (T)par[3] / T(NCH);
+    const C f0 = mk<T>(amp * zc, amp * zs);
+    const T na = T(2) * sqrt(ap * p), nb = T(2) * sqrt(bp * p);
+    C* out = a.out + e * (NCH * 4);
 #pragma unroll
     for (int ch = 0; ch < NCH; ++ch) {
         const C zch = ch ? cmul(z, mk<T>(a.charre[ch][x], a.charim[ch][x])) : z;
@@ -269,47 +279,54 @@ template <typename T, int NCH> __global__ void k_pd_axis_table(PdTabArgs<T> a) {
         const C e10 = cadd(cscale(M1, -bp), itkM0);
         const C e01 = cadd(cscale(M1, ap), itkM0);
         const C e11 = cadd(cadd(cscale(M2, -ap * bp), cscale(itkM1, ap - bp)), cscale(M0, inv2p - tk * tk));
-        out[2 * ch] = make_float4((float)M0.x, (float)M0.y, (float)e10.x, (float)e10.y);
-        out[2 * ch + 1] = make_float4((float)e01.x, (float)e01.y, (float)e11.x, (float)e11.y);
+        out[4 * ch] = cmul(M0, f0);
+        out[4 * ch + 1] = cscale(cmul(e10, f0), na);
+        out[4 * ch + 2] = cscale(cmul(e01, f0), nb);
+        out[4 * ch + 3] = cscale(cmul(e11, f0), na * nb);
     }
 }
 
-// The factor of pair ip and G: pref e^{-|q+G|^2/4p} e^{i (q+G).P} / (number of characters), in T.
-template <typename T, int NCH> __global__ void k_pd_common(PdTabArgs<T> a) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= (long long)a.npair * a.ng) return;
-    const int ip = (int)(i / a.ng), g = (int)(i - (long long)ip * a.ng);
-    const T* par = a.par + (size_t)ip * 8;
-    const T kap[3] = {a.kappa[3 * g], a.kappa[3 * g + 1], a.kappa[3 * g + 2]};
-    const T k2 = kap[0] * kap[0] + kap[1] * kap[1] + kap[2] * kap[2];
-    T s, c;
-    sincos_t(kap[0] * par[4] + kap[1] * par[5] + kap[2] * par[6], &s, &c);
-    const T amp = par[3] * exp_t(-k2 * T(0.25) / par[0]) / T(NCH);
-    a.cmn[i] = make_float2((float)(amp * c), (float)(amp * s));
+// B += the 4 x 4 block of one character from its table entries (index 0: E(0,0), 1: E(1,0), 2: E(0,1),
+// 3: E(1,1) per axis): the nine y-z products are formed once, 25 complex multiplications for 16 components.
+template <typename C>
+__device__ __forceinline__ void add_character(const C (&x)[4], const C (&y)[4], const C (&z)[4], C (&B)[4][4]) {
+    C t = cmul(y[0], z[0]);
+    cfma(B[0][0], x[0], t);
+    cfma(B[1][0], x[1], t);
+    cfma(B[0][1], x[2], t);
+    cfma(B[1][1], x[3], t);
+    t = cmul(y[1], z[0]);
+    cfma(B[2][0], x[0], t);
+    cfma(B[2][1], x[2], t);
+    t = cmul(y[2], z[0]);
+    cfma(B[0][2], x[0], t);
+    cfma(B[1][2], x[1], t);
+    t = cmul(y[3], z[0]);
+    cfma(B[2][2], x[0], t);
+    t = cmul(y[0], z[1]);
+    cfma(B[3][0], x[0], t);
+    cfma(B[3][1], x[2], t);
+    t = cmul(y[0], z[2]);
+    cfma(B[0][3], x[0], t);
+    cfma(B[1][3], x[1], t);
+    t = cmul(y[0], z[3]);
+    cfma(B[3][3], x[0], t);
+    t = cmul(y[1], z[2]);
+    cfma(B[2][3], x[0], t);
+    t = cmul(y[2], z[1]);
+    cfma(B[3][2], x[0], t);
 }
 
-// One group pair's block from the tables (k classes kx, q+G classes gx of this thread's G).
-template <int NCH>
-__device__ __forceinline__ void pair_block_tab(const PDArgs<float>& a, int ip, int ga, int gb, const int (&kx)[3],
-                                               const int (&gx)[3], int g, cplx<float> (&out)[4][4]) {
-    using C = cplx<float>;
-    const float* par = a.par + (size_t)ip * 8;
-    const float2 cm = a.pcmn[(size_t)ip * a.ng + g];
-    C E[3][NCH][4];
+__device__ __forceinline__ void load4(const float2* p, float2 (&v)[4]) {
+    const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+    v[0] = make_float2(a.x, a.y);
+    v[1] = make_float2(a.z, a.w);
+    v[2] = make_float2(b.x, b.y);
+    v[3] = make_float2(b.z, b.w);
+}
+__device__ __forceinline__ void load4(const double2* p, double2 (&v)[4]) {
 #pragma unroll
-    for (int x = 0; x < 3; ++x) {
-        const float4* src = reinterpret_cast<const float4*>(
-            a.ptab + (a.tbase[x] + ((long long)ip * a.nkx[x] + kx[x]) * a.nqx[x] + gx[x]) * (NCH * 4));
-#pragma unroll
-        for (int ch = 0; ch < NCH; ++ch) {
-            const float4 u = src[2 * ch], v = src[2 * ch + 1];
-            E[x][ch][0] = mk<float>(u.x, u.y);
-            E[x][ch][1] = mk<float>(u.z, u.w);
-            E[x][ch][2] = mk<float>(v.x, v.y);
-            E[x][ch][3] = mk<float>(v.z, v.w);
-        }
-    }
-    assemble_block<float, NCH>(a, ga, gb, par[0], par[1], par[2], mk<float>(cm.x, cm.y), E, out);
+    for (int i = 0; i < 4; ++i) v[i] = p[i];
 }
 
 template <typename T, int NCH>
@@ -368,14 +385,11 @@ __global__ void __launch_bounds__(PD_THREADS) k_pair_density(PDArgs<T> a) {
 // memory.  Threads are ordered G fastest, so a warp holds one or two groups a
 // and every thread of it runs the same pair's lattice sums.  Y then goes to
 // shared memory and rho = C_kq^H Y is formed per (G, v, c).  The sums run in
-// the same order as in k_pair_density.  With the tables of PdTab (TAB) the
-// one-dimensional lattice sums and the (pair, G) factor are read, not formed
-// per (k, G).
+// the same order as in k_pair_density.  For point sets whose components do not repeat
+// (no tables).
 template <int NV> constexpr int pdf_maxt() { return NV <= 4 ? PDF_MAXT : (NV <= 8 ? 256 : 192); }
 
-// TAB: the one-dimensional factors and the common factor come from the tables of this q (PdTab)
-// instead of being formed per (k, G).
-template <int NCH, int NV, bool TAB>
+template <int NCH, int NV>
 __global__ void __launch_bounds__(pdf_maxt<NV>()) k_pair_density_fused(PDArgs<float> a) {
     using C = cplx<float>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -396,14 +410,6 @@ __global__ void __launch_bounds__(pdf_maxt<NV>()) k_pair_density_fused(PDArgs<fl
         const int g = g0 + gl;
         const float kap[3] = {a.kappa[3 * g], a.kappa[3 * g + 1], a.kappa[3 * g + 2]};
         const float k2 = kap[0] * kap[0] + kap[1] * kap[1] + kap[2] * kap[2];
-        int kx[3] = {0, 0, 0}, gx[3] = {0, 0, 0};
-        if (TAB) {
-#pragma unroll
-            for (int x = 0; x < 3; ++x) {
-                kx[x] = a.kidx[3 * k + x];
-                gx[x] = a.gidx[3 * g + x];
-            }
-        }
         C Y[4][NV];
 #pragma unroll
         for (int ca = 0; ca < 4; ++ca)
@@ -411,10 +417,7 @@ __global__ void __launch_bounds__(pdf_maxt<NV>()) k_pair_density_fused(PDArgs<fl
             for (int v = 0; v < NV; ++v) Y[ca][v] = mk<float>(0, 0);
         for (int gb = 0; gb < a.ngrp; ++gb) {
             C blk[4][4];
-            if (TAB)
-                pair_block_tab<NCH>(a, ga * a.ngrp + gb, ga, gb, kx, gx, g, blk);
-            else
-                pair_block_vals<float, NCH>(a, ga * a.ngrp + gb, kk, kap, k2, blk);
+            pair_block_vals<float, NCH>(a, ga * a.ngrp + gb, kk, kap, k2, blk);
             const int mb = a.grp_mask[gb];
             const int nu0 = a.grp_mu0[gb] - ((mb & 1) ? 0 : 1);
 #pragma unroll
@@ -453,6 +456,154 @@ __global__ void __launch_bounds__(pdf_maxt<NV>()) k_pair_density_fused(PDArgs<fl
         const long long t = ((long long)k * nv + v) * nc + c;
         store_split3(acc.x, acc.y, a.R0, a.R1, a.R2, (long long)(g0 + l) * a.kp2 + t);
     }
+}
+
+// The pair densities from the tables of PdTab, either precision.  One thread per (G, group a), threads ordered G
+// fastest (a warp reads the entries of one or two pairs, a few hundred bytes each); per group b it adds up the 4 x 4
+// pair block from three table entries per character and multiplies it into its rows of Y = B C_k for NV bands at a
+// time.  Y goes to shared memory (bands padded to a multiple of 4) and rho = C_kq^H Y takes four bands per thread.
+//
+// What bounds it: the FP32 (FP64) pipe: per (k, G, pair) 100 multiply-adds per character for the block and 64 per
+// four bands for Y, where the form with a common factor and unshared y-z products took 192 per character and 96 more.
+// Measured (one q: 512 k x 181 G, 24 groups, 4 x 32 bands): FP32 2.54 -> 1.70 ms; FP64, which formed the lattice
+// sums per (k, G) before, 252 -> 51 ms.
+template <typename T, int NV> constexpr int pdt_threads() { return sizeof(T) == 8 ? 192 : pdf_maxt<NV>(); }
+template <typename T, int NCH, int NV>
+__global__ void __launch_bounds__(pdt_threads<T, NV>()) k_pair_density_tab(PDArgs<T> a) {
+    using C = cplx<T>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int nb = a.nb, nv = a.nv, nc = a.nc, gc = a.g_per_cta;
+    const int nvp = (nv + NV - 1) / NV * NV;
+    C* Cks = reinterpret_cast<C*>(smem_raw);       // [nb][nvp], zero for v >= nv
+    C* Ys = Cks + (size_t)nb * nvp;                // [gc][nb][nvp]
+    C* Ckqs = Ys + (size_t)gc * nb * nvp;          // [nb][nc]
+    const int k = blockIdx.x;
+    const int g0 = blockIdx.y * gc;
+    const int ngl = min(gc, a.ng - g0);
+    for (int i = threadIdx.x; i < nb * nvp; i += blockDim.x) {
+        const int mu = i / nvp, v = i - mu * nvp;
+        Cks[i] = v < nv ? a.Ck[((size_t)k * nb + mu) * nv + v] : mk<T>(0, 0);
+    }
+    for (int i = threadIdx.x; i < nb * nc; i += blockDim.x) Ckqs[i] = a.Ckq[(size_t)k * nb * nc + i];
+    __syncthreads();
+
+    const int ga = threadIdx.x / gc, gl = threadIdx.x - ga * gc;
+    if (ga < a.ngrp && gl < ngl) {
+        const C* t0[3];
+        int stride[3];
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            stride[x] = a.nkx[x] * a.nqx[x] * (NCH * 4);
+            t0[x] = a.ptab + (a.tbase[x] + ((long long)ga * a.ngrp * a.nkx[x] + a.kidx[3 * k + x]) * a.nqx[x] +
+                              a.gidx[3 * (g0 + gl) + x]) * (NCH * 4);
+        }
+        const int ma = a.grp_mask[ga];
+        const int mu0 = a.grp_mu0[ga] - ((ma & 1) ? 0 : 1);
+        C* yrow = Ys + (size_t)gl * nb * nvp;
+        for (int v0 = 0; v0 < nvp; v0 += NV) {
+            C Y[4][NV];
+#pragma unroll
+            for (int ca = 0; ca < 4; ++ca)
+#pragma unroll
+                for (int v = 0; v < NV; ++v) Y[ca][v] = mk<T>(0, 0);
+            for (int gb = 0; gb < a.ngrp; ++gb) {
+                C B[4][4];
+#pragma unroll
+                for (int ca = 0; ca < 4; ++ca)
+#pragma unroll
+                    for (int cb = 0; cb < 4; ++cb) B[ca][cb] = mk<T>(0, 0);
+#pragma unroll
+                for (int ch = 0; ch < NCH; ++ch) {
+                    C x[4], y[4], z[4];
+                    load4(t0[0] + (size_t)gb * stride[0] + 4 * ch, x);
+                    load4(t0[1] + (size_t)gb * stride[1] + 4 * ch, y);
+                    load4(t0[2] + (size_t)gb * stride[2] + 4 * ch, z);
+                    add_character(x, y, z, B);
+                }
+                const int mb = a.grp_mask[gb];
+                const int nu0 = a.grp_mu0[gb] - ((mb & 1) ? 0 : 1);
+#pragma unroll
+                for (int cb = 0; cb < 4; ++cb) {
+                    if (!(cb == 0 ? (mb & 1) : (mb & 2))) continue;
+                    const C* ck = Cks + (size_t)(nu0 + cb) * nvp + v0;
+#pragma unroll
+                    for (int v = 0; v < NV; v += 4) {
+                        C c[4];
+                        load4(ck + v, c);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int ca = 0; ca < 4; ++ca) cfma(Y[ca][v + u], B[ca][cb], c[u]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int ca = 0; ca < 4; ++ca) {
+                if (!(ca == 0 ? (ma & 1) : (ma & 2))) continue;
+#pragma unroll
+                for (int v = 0; v < NV; ++v) yrow[(size_t)(mu0 + ca) * nvp + v0 + v] = Y[ca][v];
+            }
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < ngl * nc * (nvp / 4); i += blockDim.x) {
+        const int c = i % nc, r = i / nc;
+        const int l = r % ngl, v0 = r / ngl * 4;
+        if (v0 >= nv) continue;
+        const C* y = Ys + (size_t)l * nb * nvp + v0;
+        C acc[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[u] = mk<T>(0, 0);
+        for (int mu = 0; mu < nb; ++mu) {
+            C yv[4];
+            load4(y + (size_t)mu * nvp, yv);
+            const C q = Ckqs[mu * nc + c];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) cfmac(acc[u], q, yv[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (v0 + u >= nv) continue;
+            const long long t = ((long long)k * nv + v0 + u) * nc + c;
+            if constexpr (sizeof(T) == 8)
+                a.R64[(long long)(g0 + l) * a.nt + t] = acc[u];
+            else
+                store_split3(acc[u].x, acc[u].y, a.R0, a.R1, a.R2, (long long)(g0 + l) * a.kp2 + t);
+        }
+    }
+}
+
+// S(k) = B(k; 0) from the tables: one thread per (k, pair).  Bound by the FP64 pipe (200 multiply-adds per 16
+// elements); measured for 512 k, N_b = 96: 0.12 ms (1.46 with the lattice sums formed per k).
+template <int NCH> __global__ void __launch_bounds__(128) k_overlap_tab(PDArgs<double> a) {
+    const int ip = blockIdx.x * 128 + threadIdx.x, k = blockIdx.y;
+    if (ip >= a.ngrp * a.ngrp) return;
+    const int ga = ip / a.ngrp, gb = ip - ga * a.ngrp;
+    double2 B[4][4];
+#pragma unroll
+    for (int ca = 0; ca < 4; ++ca)
+#pragma unroll
+        for (int cb = 0; cb < 4; ++cb) B[ca][cb] = make_double2(0.0, 0.0);
+    const double2* t0[3];
+#pragma unroll
+    for (int x = 0; x < 3; ++x)
+        t0[x] = a.ptab + (a.tbase[x] + ((long long)ip * a.nkx[x] + a.kidx[3 * k + x]) * a.nqx[x]) * (NCH * 4);
+#pragma unroll
+    for (int ch = 0; ch < NCH; ++ch) {
+        double2 x[4], y[4], z[4];
+        load4(t0[0] + 4 * ch, x);
+        load4(t0[1] + 4 * ch, y);
+        load4(t0[2] + 4 * ch, z);
+        add_character(x, y, z, B);
+    }
+    const int ma = a.grp_mask[ga], mb = a.grp_mask[gb];
+    const int mu0 = a.grp_mu0[ga] - ((ma & 1) ? 0 : 1), nu0 = a.grp_mu0[gb] - ((mb & 1) ? 0 : 1);
+#pragma unroll
+    for (int ca = 0; ca < 4; ++ca)
+#pragma unroll
+        for (int cb = 0; cb < 4; ++cb)
+            if ((ca == 0 ? (ma & 1) : (ma & 2)) && (cb == 0 ? (mb & 1) : (mb & 2)))
+                a.Sout[((size_t)k * a.nb + mu0 + ca) * a.nb + nu0 + cb] = B[ca][cb];
 }
 
 // S(k) = B(k; 0): one CTA per k, full matrix written to Sout.
@@ -559,20 +710,78 @@ template <typename T, int NCH> cudaError_t launch_pd(qcx_ctx* ctx, PDArgs<T>& a,
 }
 
 template <int NCH, int NV> cudaError_t launch_fused(qcx_ctx* ctx, PDArgs<float>& a, size_t smem, dim3 grid, int nthr) {
-    cudaError_t e;
-    if (a.ptab) {
-        if ((e = set_smem<float>((const void*)k_pair_density_fused<NCH, NV, true>, smem)) != cudaSuccess) return e;
-        k_pair_density_fused<NCH, NV, true><<<grid, nthr, smem, ctx->stream>>>(a);
-        return cudaGetLastError();
-    }
-    if ((e = set_smem<float>((const void*)k_pair_density_fused<NCH, NV, false>, smem)) != cudaSuccess) return e;
-    k_pair_density_fused<NCH, NV, false><<<grid, nthr, smem, ctx->stream>>>(a);
+    const cudaError_t e = set_smem<float>((const void*)k_pair_density_fused<NCH, NV>, smem);
+    if (e != cudaSuccess) return e;
+    k_pair_density_fused<NCH, NV><<<grid, nthr, smem, ctx->stream>>>(a);
     return cudaGetLastError();
 }
 template <int NCH> cudaError_t launch_fused_nv(qcx_ctx* ctx, PDArgs<float>& a, size_t smem, dim3 grid, int nthr) {
     if (a.nv <= 4) return launch_fused<NCH, 4>(ctx, a, smem, grid, nthr);
     if (a.nv <= 8) return launch_fused<NCH, 8>(ctx, a, smem, grid, nthr);
     return launch_fused<NCH, 16>(ctx, a, smem, grid, nthr);
+}
+
+// Table kernel with NV bands in registers; cudaErrorInvalidConfiguration when its shared-memory plan does not fit (the
+// caller then takes the kernels without tables).
+template <typename T, int NCH, int NV> cudaError_t launch_tab(qcx_ctx* ctx, PDArgs<T>& a) {
+    const int nvp = (a.nv + NV - 1) / NV * NV;
+    int gc = std::min(16, pdt_threads<T, NV>() / a.ngrp);
+    auto need = [&](int g) {
+        return sizeof(cplx<T>) * ((size_t)(g + 1) * a.nb * nvp + (size_t)a.nb * a.nc);
+    };
+    while (gc > 1 && need(gc) > 200 * 1024) --gc;
+    if (gc < 1 || need(gc) > 200 * 1024) return cudaErrorInvalidConfiguration;
+    a.g_per_cta = gc;
+    const cudaError_t e = set_smem<T>((const void*)k_pair_density_tab<T, NCH, NV>, need(gc));
+    if (e != cudaSuccess) return e;
+    k_pair_density_tab<T, NCH, NV><<<dim3(a.nk, (a.ng + gc - 1) / gc), gc * a.ngrp, need(gc), ctx->stream>>>(a);
+    return cudaGetLastError();
+}
+
+template <typename T, int NCH> cudaError_t build_table(qcx_ctx* ctx, PDArgs<T>& a, const PdTab& t) {
+    PdTabArgs<T> ta{};
+    ta.par = ctx->pairs.par64.as<double>();
+    ta.tab = sizeof(T) == 8 ? reinterpret_cast<const cplx<T>*>(ctx->pairs.tab64.p)
+                            : reinterpret_cast<const cplx<T>*>(ctx->pairs.tab32.p);
+    ta.dir_off = a.dir_off;
+    ta.dir_cnt = a.dir_cnt;
+    ta.dir_nlo = a.dir_nlo;
+    ta.h = ctx->h;
+    std::memcpy(ta.charre, a.charre, sizeof(ta.charre));
+    std::memcpy(ta.charim, a.charim, sizeof(ta.charim));
+    ta.kval = t.kval.as<double>();
+    ta.qval = t.qval.as<double>();
+    for (int x = 0; x < 3; ++x) {
+        ta.nkx[x] = a.nkx[x] = t.nkx[x];
+        ta.nqx[x] = a.nqx[x] = t.nqx[x];
+        ta.kofs[x] = t.kofs[x];
+        ta.qofs[x] = t.qofs[x];
+    }
+    for (int x = 0; x < 4; ++x) ta.tbase[x] = a.tbase[x] = t.tbase[x];
+    ta.out = t.tab.as<cplx<T>>();
+    a.ptab = ta.out;
+    a.kidx = t.kidx.as<int>();
+    a.gidx = t.gidx.as<int>();
+    k_pd_axis_table<T, NCH><<<(unsigned)((t.tbase[3] + 127) / 128), 128, 0, ctx->stream>>>(ta);
+    return cudaGetLastError();
+}
+
+// FP64 keeps four bands in registers (a fifth would spill), FP32 up to sixteen
+template <typename T, int NCH> cudaError_t run_tab(qcx_ctx* ctx, PDArgs<T>& a, const PdTab& t) {
+    const cudaError_t e = build_table<T, NCH>(ctx, a, t);
+    if (e != cudaSuccess) return e;
+    if constexpr (sizeof(T) == 4) {
+        if (a.nv > 8) return launch_tab<T, NCH, 16>(ctx, a);
+        if (a.nv > 4) return launch_tab<T, NCH, 8>(ctx, a);
+    }
+    return launch_tab<T, NCH, 4>(ctx, a);
+}
+template <typename T> cudaError_t run_tab_nch(qcx_ctx* ctx, PDArgs<T>& a, const PdTab& t) {
+    switch (ctx->nchar) {
+        case 1: return run_tab<T, 1>(ctx, a, t);
+        case 2: return run_tab<T, 2>(ctx, a, t);
+        default: return run_tab<T, 4>(ctx, a, t);
+    }
 }
 
 template <typename T, int NCH> cudaError_t launch_ov(qcx_ctx* ctx, PDArgs<T>& a, size_t smem, int nk) {
@@ -766,11 +975,56 @@ static void axis_classes(const double* v, int n, int x, std::vector<double>& val
     }
 }
 
-cudaError_t qcx_pd_tab_prepare(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng, int iq) {
-    PdTab& t = s.pdt;
+// Classes and buffers of the tables for nk k points and ng values of q+G (host arrays); leaves t invalid when the
+// tables would not save work or exceed their memory budget.
+static cudaError_t tab_prepare(qcx_ctx* ctx, PdTab& t, const double* kpts, int nk, const double* kap, int ng,
+                               size_t elem) {
     t.valid = false;
-    const int nk = ctx->nk, npair = ctx->ngrp * ctx->ngrp;
-    if ((int)ctx->kpts_h.size() != 3 * nk || npair < 1) return cudaSuccess;
+    for (int i = 0; i < 3 * nk; ++i)
+        if (!std::isfinite(kpts[i])) return cudaSuccess;
+    for (int i = 0; i < 3 * ng; ++i)
+        if (!std::isfinite(kap[i])) return cudaSuccess;
+    const int npair = ctx->ngrp * ctx->ngrp;
+    std::vector<double> kval, qval;
+    std::vector<int> kidx(3 * (size_t)nk), gidx(3 * (size_t)ng);
+    long long cells = 0;
+    for (int x = 0; x < 3; ++x) {
+        t.kofs[x] = (int)kval.size();
+        t.qofs[x] = (int)qval.size();
+        axis_classes(kpts, nk, x, kval, kidx);
+        axis_classes(kap, ng, x, qval, gidx);
+        t.nkx[x] = (int)kval.size() - t.kofs[x];
+        t.nqx[x] = (int)qval.size() - t.qofs[x];
+        cells += (long long)t.nkx[x] * t.nqx[x];
+    }
+    // worth it only when the classes repeat (regular k grids, G shells); bounded memory
+    const size_t tab_bytes = (size_t)npair * cells * ctx->nchar * 4 * elem;
+    if (4 * cells > 3LL * 3 * nk * ng || tab_bytes > ((size_t)512 << 20)) return cudaSuccess;
+    for (int x = 0; x < 3; ++x) t.tbase[x + 1] = t.tbase[x] + (long long)npair * t.nkx[x] * t.nqx[x];
+    cudaError_t e;
+    if ((e = t.tab.ensure(tab_bytes)) != cudaSuccess) {
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();                       // no room for the tables: the kernels without them serve
+        return cudaSuccess;
+    }
+    if ((e = t.kidx.ensure(kidx.size() * sizeof(int))) != cudaSuccess) return e;
+    if ((e = t.gidx.ensure(gidx.size() * sizeof(int))) != cudaSuccess) return e;
+    if ((e = t.kval.ensure(kval.size() * sizeof(double))) != cudaSuccess) return e;
+    if ((e = t.qval.ensure(qval.size() * sizeof(double))) != cudaSuccess) return e;
+    const cudaMemcpyKind h2d = cudaMemcpyHostToDevice;
+    if ((e = cudaMemcpyAsync(t.kidx.p, kidx.data(), kidx.size() * sizeof(int), h2d, ctx->stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(t.gidx.p, gidx.data(), gidx.size() * sizeof(int), h2d, ctx->stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(t.kval.p, kval.data(), kval.size() * sizeof(double), h2d, ctx->stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(t.qval.p, qval.data(), qval.size() * sizeof(double), h2d, ctx->stream)) != cudaSuccess)
+        return e;
+    t.valid = true;
+    return cudaSuccess;
+}
+
+cudaError_t qcx_pd_tab_prepare(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng, int iq, qcx_precision prec) {
+    s.pdt.valid = false;
+    const int nk = ctx->nk;
+    if ((int)ctx->kpts_h.size() != 3 * nk || ctx->ngrp < 1) return cudaSuccess;
     // q + G in Cartesian components (reciprocal basis b_i = 2 pi inv(A)^T rows)
     const double* A = ctx->lattice;
     const double det = A[0] * (A[4] * A[8] - A[5] * A[7]) - A[1] * (A[3] * A[8] - A[5] * A[6]) +
@@ -788,38 +1042,8 @@ cudaError_t qcx_pd_tab_prepare(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng
             for (int i = 0; i < 3; ++i) v += G_host[3 * g + i] * 2.0 * M_PI * inv[3 * x + i];
             kap[3 * g + x] = v;
         }
-    std::vector<double> kval, qval;
-    std::vector<int> kidx(3 * (size_t)nk), gidx(3 * (size_t)ng);
-    long long cells = 0;
-    for (int x = 0; x < 3; ++x) {
-        t.kofs[x] = (int)kval.size();
-        t.qofs[x] = (int)qval.size();
-        axis_classes(ctx->kpts_h.data(), nk, x, kval, kidx);
-        axis_classes(kap.data(), ng, x, qval, gidx);
-        t.nkx[x] = (int)kval.size() - t.kofs[x];
-        t.nqx[x] = (int)qval.size() - t.qofs[x];
-        cells += (long long)t.nkx[x] * t.nqx[x];
-    }
-    // worth it only when the classes repeat (regular k grids, G shells); bounded memory
-    const int nch = ctx->nchar;
-    const size_t tab_bytes = (size_t)npair * cells * nch * 4 * sizeof(float2);
-    if (4 * cells > 3LL * 3 * nk * ng || tab_bytes > ((size_t)512 << 20)) return cudaSuccess;
-    for (int x = 0; x < 3; ++x) t.tbase[x + 1] = t.tbase[x] + (long long)npair * t.nkx[x] * t.nqx[x];
-    cudaError_t e;
-    if ((e = t.tab.ensure(tab_bytes)) != cudaSuccess) return e;
-    if ((e = t.cmn.ensure((size_t)npair * ng * sizeof(float2))) != cudaSuccess) return e;
-    if ((e = t.kidx.ensure(kidx.size() * sizeof(int))) != cudaSuccess) return e;
-    if ((e = t.gidx.ensure(gidx.size() * sizeof(int))) != cudaSuccess) return e;
-    if ((e = t.kval.ensure(kval.size() * sizeof(double))) != cudaSuccess) return e;
-    if ((e = t.qval.ensure(qval.size() * sizeof(double))) != cudaSuccess) return e;
-    const cudaMemcpyKind h2d = cudaMemcpyHostToDevice;
-    if ((e = cudaMemcpyAsync(t.kidx.p, kidx.data(), kidx.size() * sizeof(int), h2d, ctx->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(t.gidx.p, gidx.data(), gidx.size() * sizeof(int), h2d, ctx->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(t.kval.p, kval.data(), kval.size() * sizeof(double), h2d, ctx->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(t.qval.p, qval.data(), qval.size() * sizeof(double), h2d, ctx->stream)) != cudaSuccess)
-        return e;
-    t.valid = true;
-    return cudaSuccess;
+    return tab_prepare(ctx, s.pdt, ctx->kpts_h.data(), nk, kap.data(), ng,
+                       prec == QCX_FP64 ? sizeof(double2) : sizeof(float2));
 }
 
 cudaError_t qcx_launch_pair_density(qcx_ctx* ctx, QSlot& s, int iq, qcx_precision prec) {
@@ -844,6 +1068,10 @@ cudaError_t qcx_launch_pair_density(qcx_ctx* ctx, QSlot& s, int iq, qcx_precisio
         a.Ck = ctx->d_Ck64.as<double2>();
         a.Ckq = ctx->d_Ckq64.as<double2>() + (size_t)iq * ctx->nk * ctx->nb * ctx->nc;
         a.R64 = s.rho.as<double2>();
+        if (s.pdt.valid) {
+            const cudaError_t e = run_tab_nch<double>(ctx, a, s.pdt);
+            if (e != cudaErrorInvalidConfiguration) return e;
+        }
         switch (ctx->nchar) {
             case 1: return launch_pd<double, 1>(ctx, a, smem, grid);
             case 2: return launch_pd<double, 2>(ctx, a, smem, grid);
@@ -885,62 +1113,8 @@ cudaError_t qcx_launch_pair_density(qcx_ctx* ctx, QSlot& s, int iq, qcx_precisio
     a.R2 = a.R1 + (size_t)s.ngp * (s.kp / 2);
     a.kp2 = s.kp / 2;
     if (gcf && s.pdt.valid) {
-        // tables of this q first (FP32, the operations of pair_block_vals: FP64 tables were no more
-        // accurate in the loss and cost ~2 ms per mid q at the GB300's FP64 rate): the one-dimensional
-        // factors, then the factor of (pair, G)
-        const PdTab& t = s.pdt;
-        PdTabArgs<float> ta{};
-        ta.par = ctx->pairs.par32.as<float>();
-        ta.tab = ctx->pairs.tab32.as<float2>();
-        ta.dir_off = ctx->pairs.dir_off.as<int>();
-        ta.dir_cnt = ctx->pairs.dir_cnt.as<int>();
-        ta.dir_nlo = ctx->pairs.dir_nlo.as<int>();
-        ta.h = (float)ctx->h;
-        for (int c = 0; c < 4; ++c)
-            for (int x = 0; x < 3; ++x) {
-                ta.charre[c][x] = (float)cos(2.0 * M_PI * ctx->chars[c][x]);
-                ta.charim[c][x] = (float)sin(2.0 * M_PI * ctx->chars[c][x]);
-            }
-        ta.kval = t.kval.as<double>();
-        ta.qval = t.qval.as<double>();
-        ta.kappa = s.kappa32.as<float>();
-        for (int x = 0; x < 3; ++x) {
-            ta.nkx[x] = t.nkx[x];
-            ta.nqx[x] = t.nqx[x];
-            ta.kofs[x] = t.kofs[x];
-            ta.qofs[x] = t.qofs[x];
-        }
-        for (int x = 0; x < 4; ++x) ta.tbase[x] = t.tbase[x];
-        ta.npair = ctx->ngrp * ctx->ngrp;
-        ta.ng = s.ng;
-        ta.out = t.tab.as<float2>();
-        ta.cmn = t.cmn.as<float2>();
-        const unsigned gt = (unsigned)((t.tbase[3] + 255) / 256);
-        const unsigned gcm = (unsigned)(((long long)ta.npair * s.ng + 255) / 256);
-        switch (ctx->nchar) {
-            case 1:
-                k_pd_axis_table<float, 1><<<gt, 256, 0, ctx->stream>>>(ta);
-                k_pd_common<float, 1><<<gcm, 256, 0, ctx->stream>>>(ta);
-                break;
-            case 2:
-                k_pd_axis_table<float, 2><<<gt, 256, 0, ctx->stream>>>(ta);
-                k_pd_common<float, 2><<<gcm, 256, 0, ctx->stream>>>(ta);
-                break;
-            default:
-                k_pd_axis_table<float, 4><<<gt, 256, 0, ctx->stream>>>(ta);
-                k_pd_common<float, 4><<<gcm, 256, 0, ctx->stream>>>(ta);
-        }
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        a.ptab = t.tab.as<float2>();
-        a.pcmn = t.cmn.as<float2>();
-        a.kidx = t.kidx.as<int>();
-        a.gidx = t.gidx.as<int>();
-        for (int x = 0; x < 3; ++x) {
-            a.nkx[x] = t.nkx[x];
-            a.nqx[x] = t.nqx[x];
-        }
-        for (int x = 0; x < 4; ++x) a.tbase[x] = t.tbase[x];
+        const cudaError_t e = run_tab_nch<float>(ctx, a, s.pdt);
+        if (e != cudaErrorInvalidConfiguration) return e;
     }
     if (gcf) {
         a.g_per_cta = gcf;
@@ -959,7 +1133,8 @@ cudaError_t qcx_launch_pair_density(qcx_ctx* ctx, QSlot& s, int iq, qcx_precisio
     }
 }
 
-cudaError_t qcx_launch_overlap(qcx_ctx* ctx, int nk, const double* d_kpts, double2* d_out) {
+// k_host: the k points on the host (for the tables' classes)
+cudaError_t qcx_launch_overlap(qcx_ctx* ctx, int nk, const double* d_kpts, const double* k_host, double2* d_out) {
     PDArgs<double> a{};
     fill_common(ctx, a);
     size_t smem = 0;
@@ -968,6 +1143,29 @@ cudaError_t qcx_launch_overlap(qcx_ctx* ctx, int nk, const double* d_kpts, doubl
     a.tab = ctx->pairs.tab64.as<double2>();
     a.kpts = d_kpts;
     a.Sout = d_out;
+    const double zero[3] = {0.0, 0.0, 0.0};
+    if (nk <= 65535) {
+        const cudaError_t e = tab_prepare(ctx, ctx->overlap_tab, k_host, nk, zero, 1, sizeof(double2));
+        if (e != cudaSuccess) return e;
+        if (ctx->overlap_tab.valid) {
+            const dim3 grid((ctx->ngrp * ctx->ngrp + 127) / 128, nk);
+            cudaError_t e2;
+            switch (ctx->nchar) {
+                case 1:
+                    if ((e2 = build_table<double, 1>(ctx, a, ctx->overlap_tab)) != cudaSuccess) return e2;
+                    k_overlap_tab<1><<<grid, 128, 0, ctx->stream>>>(a);
+                    break;
+                case 2:
+                    if ((e2 = build_table<double, 2>(ctx, a, ctx->overlap_tab)) != cudaSuccess) return e2;
+                    k_overlap_tab<2><<<grid, 128, 0, ctx->stream>>>(a);
+                    break;
+                default:
+                    if ((e2 = build_table<double, 4>(ctx, a, ctx->overlap_tab)) != cudaSuccess) return e2;
+                    k_overlap_tab<4><<<grid, 128, 0, ctx->stream>>>(a);
+            }
+            return cudaGetLastError();
+        }
+    }
     switch (ctx->nchar) {
         case 1: return launch_ov<double, 1>(ctx, a, smem, nk);
         case 2: return launch_ov<double, 2>(ctx, a, smem, nk);
