@@ -552,6 +552,11 @@ bool qcx_make_bf16_map(CUtensorMap* m, void* base, long long kp, int rows, int b
 }
 
 cudaError_t qcx_launch_chi0_mixed(qcx_ctx* ctx, QSlot& s, int iq, double2* chi, int* d_status) {
+    bool panels = false;                         // many frequencies: through energy panels
+    {
+        const cudaError_t ep = qcx_launch_chi0_panels(ctx, s, iq, chi, d_status, &panels);
+        if (panels || ep != cudaSuccess) return ep;
+    }
     const int ng = s.ng;
     const long long nt = (long long)ctx->nk * ctx->nv * ctx->nc;
     TcArgs a{};

@@ -140,6 +140,18 @@ struct OzBufs {
     DevBuf w, e, part;         // weights of a group of frequencies, row exponents, FP64 sums per K split
 };
 
+// Work space of the mixed chi0 through energy panels (chi0_panels.cu).
+struct PanelBufs {
+    DevBuf small;              // energy range, totals
+    DevBuf keys, perm, cnt;    // sort of the transitions by panel
+    DevBuf seg;                // segments, then the column tiles
+    DevBuf tr, Lw;             // transition and Lagrange weights of every stage slot
+    DevBuf tiles, r2;          // gathered rho~ stage tiles (two planes), |rho|^2
+    DevBuf ktab, kplanes;      // W at the nodes: FP32, BF16 planes
+    DevBuf S, splanes, tp;     // S of one chunk, its BF16 planes, 32-tile pairs
+    DevBuf Sd, part, chi;      // diagonal of S, its frequency sums; chi0 [nw][ng][ng]
+};
+
 // Work space of the spectral route to chi0 (one q at a time, either precision).
 struct SpecBufs {
     DevBuf bin, x;             // [nt] grid point and hat weight of each transition
@@ -223,6 +235,7 @@ struct qcx_ctx {
     MlpState* mlp = nullptr;       // surrogate network (parameters, Adam moments, work buffers)
     SpecBufs spec;                 // spectral route work space
     OzBufs oz;                     // FP64 chi0 on the tensor cores
+    PanelBufs panels;              // mixed chi0 through energy panels
     OpticalBufs optical;           // optical-limit work space
     int spec_chunk_bins = 0;       // grid points per chunk of the spectral route (0: from a 4 GiB budget)
     int spec_cuda_cores = 0;       // mixed spectral contraction on the CUDA cores (FP32) instead of tcgen05
@@ -293,7 +306,13 @@ cudaError_t qcx_spec_tc_contract(cudaStream_t st, const CUtensorMap* kmaps, cons
                                  __nv_bfloat16* splanes, const int2* tp, int accumulate, double2* chi, int* status,
                                  long long wait_limit);
 
-// chi0 (chi0_fp64.cu, chi0_tc.cu)
+// the contraction alone, on planes already split
+cudaError_t qcx_spec_tc_kk(cudaStream_t st, const CUtensorMap* kmaps, const CUtensorMap* smaps, int mtiles, int ntiles, int nw,
+                           int ng, int nb, int kb0, const int2* tp, int accumulate, double2* chi, int* status,
+                           long long wait_limit);
+
+// chi0 (chi0_fp64.cu, chi0_tc.cu, chi0_panels.cu)
+cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi, int* d_status, bool* used);
 // FP64: sets *used_tc when the tensor-core route ran (its status word is then to be read)
 cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out, int* d_status, bool* used_tc);
 cudaError_t qcx_launch_chi0_fp64_tc(qcx_ctx* ctx, QSlot& s, int iq, double pref, double2* chi, int* d_status);

@@ -9,18 +9,19 @@
 //   n = 2 X + c      B = (Re S, Im S)_b at the upper (G, G') pair X  (c = 0, 1)
 // so that with Ar = D[2w][2X], Bi = D[2w+1][2X+1], Cs = D[2w][2X+1], Dr = D[2w+1][2X]
 //   chi0[G][G'] = (Ar - Bi) + i (Cs + Dr),   chi0[G'][G] = (Ar + Bi) + i (Dr - Cs)
-// (S_b is Hermitian; X runs over the 32 x 32 tiles with G-tile <= G'-tile, X = p 1024 + 32 r + c).
+// (S_b is Hermitian; X runs over the 32 x 32 tiles of one triangle, X = p 1024 + 32 r + c).
 //
 // Both operands are split into three BF16 terms (the six products of order <= 2 are
 // accumulated, as in the direct route's kernel) and stored K-major: the K table as
 // [2 N_w (padded)][grid points], the weights of one chunk as [2 x 1024 x tile pairs][chunk
-// points], both loaded by TMA into 64-byte-swizzled stages.  FP32 accumulation in TMEM is
-// restarted every two K stages (24 MMAs; the tensor core's FP32 sums truncate) and the window
-// sums are added in FP32 registers, so a chunk is summed in two levels; chunks are added into
+// points], both loaded by TMA into 64-byte-swizzled stages.  The tensor core's FP32 sums
+// truncate with every MMA: the leading product has its own accumulator, restarted every two K
+// stages (4 MMAs) and added in FP32 registers, so a chunk is summed in two levels; the five
+// smaller products (2^-8 of it and less) share one for the whole chunk.  Chunks are added into
 // an FP64 chi0 in the epilogue.
 //
 // CTA: one 128-row M tile (64 frequencies) x one 128-column N tile (64 pairs).  Warps: 0 TMA
-// producer; 1 and 10 MMA issuers on alternate accumulation windows (TMEM buffers 0 and 1);
+// producer; 1 and 10 MMA issuers on alternate accumulation windows (each its own pair of TMEM sums);
 // 2-9 drain the accumulators and run the epilogue; 11 idles.  Every wait is bounded: on
 // timeout the kernel records an error status, lets its own copies and MMAs finish, frees
 // TMEM and returns.
@@ -81,7 +82,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1)
         *abort_flag = 0;
         fence_barrier_init();
     }
-    if (warp == 1) tmem_alloc(tmem_slot, 2 * SK_N);
+    if (warp == 1) tmem_alloc(tmem_slot, 4 * SK_N);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -137,16 +138,16 @@ __global__ void __launch_bounds__(SK_THREADS, 1)
                     unsigned char* st = base + s * SK_STAGE;
                     const uint32_t a0 = smem_u32(st), a1 = a0 + SK_TILE, a2 = a1 + SK_TILE;
                     const uint32_t b0 = a2 + SK_TILE, b1 = b0 + SK_TILE, b2 = b1 + SK_TILE;
-                    const uint32_t d = tmem + (uint32_t)(b * SK_N);
+                    const uint32_t d = tmem + (uint32_t)(b * SK_N), dl = d + 2 * SK_N;
 #pragma unroll
                     for (int kk = 0; kk < KSTEP / 16; ++kk) {
                         const uint32_t off = kk * 32;
                         umma_bf16(d, sw64_desc(a0 + off), sw64_desc(b0 + off), idesc, (first && kk == 0) ? 0u : 1u);
-                        umma_bf16(d, sw64_desc(a0 + off), sw64_desc(b1 + off), idesc, 1u);
-                        umma_bf16(d, sw64_desc(a1 + off), sw64_desc(b0 + off), idesc, 1u);
-                        umma_bf16(d, sw64_desc(a0 + off), sw64_desc(b2 + off), idesc, 1u);
-                        umma_bf16(d, sw64_desc(a1 + off), sw64_desc(b1 + off), idesc, 1u);
-                        umma_bf16(d, sw64_desc(a2 + off), sw64_desc(b0 + off), idesc, 1u);
+                        umma_bf16(dl, sw64_desc(a0 + off), sw64_desc(b1 + off), idesc, (win < 2 && first && kk == 0) ? 0u : 1u);
+                        umma_bf16(dl, sw64_desc(a1 + off), sw64_desc(b0 + off), idesc, 1u);
+                        umma_bf16(dl, sw64_desc(a0 + off), sw64_desc(b2 + off), idesc, 1u);
+                        umma_bf16(dl, sw64_desc(a1 + off), sw64_desc(b1 + off), idesc, 1u);
+                        umma_bf16(dl, sw64_desc(a2 + off), sw64_desc(b0 + off), idesc, 1u);
                     }
                     umma_commit(&empty[s]);
                 }
@@ -168,17 +169,21 @@ __global__ void __launch_bounds__(SK_THREADS, 1)
             const int b = wd & 1;
             if (!(ok = warp_wait(&acc_full[b], (uint32_t)(wd >> 1) & 1u, abort_flag, a.status, a.wait_limit))) break;
             tc_fence_after();
-            const uint32_t tb = tmem + lane_off + (uint32_t)(b * SK_N + hc * SK_HALF);
+            // with an issuer's last window, its low-order sums too
+            const int nsum = wd + 2 >= nwin ? 2 : 1;
+            for (int z = 0; z < nsum; ++z) {
+                const uint32_t tb = tmem + lane_off + (uint32_t)((b + 2 * z) * SK_N + hc * SK_HALF);
 #pragma unroll
-            for (int grp = 0; grp < SK_HALF / 16; ++grp) {
-                uint32_t r[2][8];
-                tmem_ld8(tb + (uint32_t)(grp * 16), r[0]);
-                tmem_ld8(tb + (uint32_t)(grp * 16 + 8), r[1]);
-                tmem_wait_ld();
+                for (int grp = 0; grp < SK_HALF / 16; ++grp) {
+                    uint32_t r[2][8];
+                    tmem_ld8(tb + (uint32_t)(grp * 16), r[0]);
+                    tmem_ld8(tb + (uint32_t)(grp * 16 + 8), r[1]);
+                    tmem_wait_ld();
 #pragma unroll
-                for (int u = 0; u < 2; ++u)
+                    for (int u = 0; u < 2; ++u)
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) part[grp * 16 + u * 8 + i] += __uint_as_float(r[u][i]);
+                        for (int i = 0; i < 8; ++i) part[grp * 16 + u * 8 + i] += __uint_as_float(r[u][i]);
+                }
             }
             tc_fence_before();
             __syncwarp();
@@ -207,6 +212,9 @@ __global__ void __launch_bounds__(SK_THREADS, 1)
                 const int2 pr = a.tp[p];
                 const int G = pr.x * 32 + (X >> 5), H = pr.y * 32 + (X & 31);
                 if (w >= a.nw || G >= a.ng || H >= a.ng) continue;
+                // within a diagonal tile the elements below the diagonal serve both triangles too: with two
+                // roundings of the same S, Re K would carry their difference into the anti-Hermitian part of chi0
+                if (pr.x == pr.y && G < H) continue;
                 double2* d = a.chi + ((size_t)w * a.ng + G) * a.ng + H;
                 const double2 gh = make_double2(Ar - Bi, Cs + Dr);
                 if (a.accumulate) {
@@ -215,7 +223,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1)
                 } else {
                     *d = gh;
                 }
-                if (pr.x != pr.y) {
+                if (G != H) {
                     double2* e = a.chi + ((size_t)w * a.ng + H) * a.ng + G;
                     const double2 hg = make_double2(Ar + Bi, Dr - Cs);
                     if (a.accumulate) {
@@ -232,7 +240,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1)
     __syncthreads();
     if (warp == 1) {
         tc_fence_after();
-        tmem_dealloc(tmem, 2 * SK_N);
+        tmem_dealloc(tmem, 4 * SK_N);
     }
 }
 
@@ -317,6 +325,12 @@ cudaError_t qcx_spec_tc_contract(cudaStream_t st, const CUtensorMap* kmaps, cons
     k_spec_s_split<<<sg, dim3(32, 8), 0, st>>>(nbc, nb, sld, S, splanes, splanes + n, splanes + 2 * n);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    return qcx_spec_tc_kk(st, kmaps, smaps, mtiles, ntiles, nw, ng, nb, kb0, tp, accumulate, chi, status, wait_limit);
+}
+
+cudaError_t qcx_spec_tc_kk(cudaStream_t st, const CUtensorMap* kmaps, const CUtensorMap* smaps, int mtiles, int ntiles, int nw,
+                           int ng, int nb, int kb0, const int2* tp, int accumulate, double2* chi, int* status,
+                           long long wait_limit) {
     SkArgs a;
     a.nw = nw;
     a.ng = ng;
@@ -328,7 +342,7 @@ cudaError_t qcx_spec_tc_contract(cudaStream_t st, const CUtensorMap* kmaps, cons
     a.status = status;
     a.wait_limit = wait_limit;
     const size_t smem = qcx_spec_tc_smem();
-    e = cudaFuncSetAttribute((const void*)k_spec_kk_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute((const void*)k_spec_kk_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k_spec_kk_tc<<<dim3(mtiles, ntiles), SK_THREADS, smem, st>>>(kmaps[0], kmaps[1], kmaps[2], smaps[0], smaps[1],
                                                                    smaps[2], a);
