@@ -597,12 +597,17 @@ __global__ void __launch_bounds__(pdt_threads<T, NV>()) k_pair_density_tab(PDArg
     }
 }
 
-// S(k) = B(k; 0) from the tables: one thread per (k, pair).  Bound by the FP64 pipe (200 multiply-adds per 16
-// elements); measured for 512 k, N_b = 96: 0.12 ms (1.46 with the lattice sums formed per k).
+// S(k) = B(k; 0) from the tables: one thread per (k, pair of groups a <= b), the block written to both triangles (S is
+// Hermitian).  Bound by the FP64 pipe (200 multiply-adds per 16 elements); measured for 512 k, N_b = 96: 0.08 ms (1.46
+// with the lattice sums formed per k, 0.12 with all pairs).  Pair number p walks rows r and n - 1 - r of the triangle
+// together, n + 1 pairs each.
 template <int NCH> __global__ void __launch_bounds__(128) k_overlap_tab(PDArgs<double> a) {
-    const int ip = blockIdx.x * 128 + threadIdx.x, k = blockIdx.y;
-    if (ip >= a.ngrp * a.ngrp) return;
-    const int ga = ip / a.ngrp, gb = ip - ga * a.ngrp;
+    const int p = blockIdx.x * 128 + threadIdx.x, k = blockIdx.y, n = a.ngrp;
+    const int r = p / (n + 1), c = p - r * (n + 1);
+    if (r >= (n + 1) / 2) return;
+    const int ga = c < n - r ? r : n - 1 - r, gb = c < n - r ? r + c : c - 1;
+    if (c >= n - r && ga == r) return;                 // the middle row of an odd n, already walked
+    const int ip = ga * n + gb;
     double2 B[4][4];
 #pragma unroll
     for (int ca = 0; ca < 4; ++ca)
@@ -626,8 +631,11 @@ template <int NCH> __global__ void __launch_bounds__(128) k_overlap_tab(PDArgs<d
     for (int ca = 0; ca < 4; ++ca)
 #pragma unroll
         for (int cb = 0; cb < 4; ++cb)
-            if ((ca == 0 ? (ma & 1) : (ma & 2)) && (cb == 0 ? (mb & 1) : (mb & 2)))
+            if ((ca == 0 ? (ma & 1) : (ma & 2)) && (cb == 0 ? (mb & 1) : (mb & 2))) {
                 a.Sout[((size_t)k * a.nb + mu0 + ca) * a.nb + nu0 + cb] = B[ca][cb];
+                if (ga != gb)
+                    a.Sout[((size_t)k * a.nb + nu0 + cb) * a.nb + mu0 + ca] = make_double2(B[ca][cb].x, -B[ca][cb].y);
+            }
 }
 
 // S(k) = B(k; 0): one CTA per k, full matrix written to Sout.
@@ -1173,7 +1181,7 @@ cudaError_t qcx_launch_overlap(qcx_ctx* ctx, int nk, const double* d_kpts, const
         const cudaError_t e = tab_prepare(ctx, ctx->overlap_tab, k_host, nk, zero, 1, sizeof(double2));
         if (e != cudaSuccess) return e;
         if (ctx->overlap_tab.valid) {
-            const dim3 grid((ctx->ngrp * ctx->ngrp + 127) / 128, nk);
+            const dim3 grid(((ctx->ngrp + 1) / 2 * (ctx->ngrp + 1) + 127) / 128, nk);
             cudaError_t e2;
             switch (ctx->nchar) {
                 case 1:
