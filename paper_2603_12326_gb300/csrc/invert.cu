@@ -392,85 +392,106 @@ __global__ void __launch_bounds__(256) k_refine_diag(int n, const double2* Aall,
 // |[A^-1]_jj| (Im of an O(1) diagonal) the imaginary part of the FP32 diagonal
 // loses its relative accuracy; the form builds L from the small B itself
 // (B from the FP64 matrix in FP64, rounded once), so its relative error is
-// that of X.  One CTA per (block, 32 rows j): T = X B in 32 x 32 tiles, then
-// L_j = Re sum_l T_jl conj(X_jl); the imaginary part of the reported diagonal
-// becomes -L_j.  Blocks corrected in FP64 keep their values.
-constexpr int QF = 32;
-__global__ void __launch_bounds__(256) k_loss_quadform(int n, const double2* Aall, const float2* Xall,
-                                                       const int* flags, const double* norms, double kappa_refine,
-                                                       double2* diag_inv, double* L) {
-    __shared__ float2 Xs[QF][QF + 1];
-    __shared__ float2 Bs[QF][QF + 1];
-    __shared__ double2 At[QF][QF + 1];       // A_lk tile, read along rows, used transposed
-    __shared__ float Lrow[QF];
-    const int b = blockIdx.x, j0 = blockIdx.y * QF;
-    if (flags[b] || norms[b] * norms[gridDim.x + b] > kappa_refine) return;
+// that of X.  The imaginary part of the reported diagonal becomes -L_j.  Blocks
+// corrected in FP64 keep their values.
+//
+// B is formed once per matrix (k_form_b, tile and transposed tile), then a CTA of
+// k_loss_quadform takes 64 rows j: T = X B in 64 x 64 tiles of l, L_j += Re sum_l T_jl
+// conj(X_jl).  B being Hermitian, the k tiles above an l tile's own count twice and those
+// below it are left out, half the product.  Bound by the FP32 pipe; with 32 x 32 tiles, all
+// of B and its FP64 source read again by every row block: 200 matrices of 181 660 -> 280 us,
+// 100 of 531 7.0 -> 2.3 ms.
+constexpr int QF = 64, QK = 16;
+__global__ void __launch_bounds__(256) k_form_b(int n, const double2* Aall, const int* flags, const double* norms,
+                                                const double* xnorms, double kappa_refine, float2* Ball) {
+    __shared__ double2 At[32][33];
+    const int b = blockIdx.z;
+    if (flags[b] || norms[b] * xnorms[b] > kappa_refine) return;
     const double2* A = Aall + (size_t)b * n * n;
-    const float2* X = Xall + (size_t)b * n * n;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    if (threadIdx.x < QF) Lrow[threadIdx.x] = 0.0f;
-    for (int l0 = 0; l0 < n; l0 += QF) {
-        float2 acc[2][2];
-#pragma unroll
-        for (int r = 0; r < 2; ++r)
-#pragma unroll
-            for (int c = 0; c < 2; ++c) acc[r][c] = make_float2(0.f, 0.f);
-        for (int k0 = 0; k0 < n; k0 += QF) {
-            for (int e = threadIdx.x; e < QF * QF; e += blockDim.x) {
-                const int r = e / QF, c = e % QF;
-                At[r][c] = (l0 + r < n && k0 + c < n) ? A[(size_t)(l0 + r) * n + k0 + c] : make_double2(0.0, 0.0);
-            }
-            __syncthreads();
-            for (int e = threadIdx.x; e < QF * QF; e += blockDim.x) {
-                const int r = e / QF, c = e % QF;
-                const int j = j0 + r, kk = k0 + c;
-                Xs[r][c] = (j < n && kk < n) ? X[(size_t)j * n + kk] : make_float2(0.f, 0.f);
-                const int kr = k0 + r, lc = l0 + c;
-                float2 bv = make_float2(0.f, 0.f);
-                if (kr < n && lc < n) {
-                    const double2 akl = A[(size_t)kr * n + lc], alk = At[c][r];
-                    bv = make_float2((float)(0.5 * (akl.y + alk.y)), (float)(-0.5 * (akl.x - alk.x)));
-                }
-                Bs[r][c] = bv;
-            }
-            __syncthreads();
-#pragma unroll 8
-            for (int kk = 0; kk < QF; ++kk) {
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    const float2 x = Xs[ty + 16 * r][kk];
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        const float2 bb = Bs[kk][tx + 16 * c];
-                        acc[r][c].x = fmaf(x.x, bb.x, fmaf(-x.y, bb.y, acc[r][c].x));
-                        acc[r][c].y = fmaf(x.x, bb.y, fmaf(x.y, bb.x, acc[r][c].y));
-                    }
-                }
-            }
-            __syncthreads();
+    float2* B = Ball + (size_t)b * n * n;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int k0 = blockIdx.y * 32, l0 = blockIdx.x * 32;
+    for (int r = ty; r < 32; r += 8)
+        if (l0 + r < n && k0 + tx < n) At[r][tx] = A[(size_t)(l0 + r) * n + k0 + tx];
+    __syncthreads();
+    for (int r = ty; r < 32; r += 8) {
+        const int k = k0 + r, l = l0 + tx;
+        if (k < n && l < n) {
+            const double2 akl = A[(size_t)k * n + l], alk = At[tx][r];
+            B[(size_t)k * n + l] = make_float2((float)(0.5 * (akl.y + alk.y)), (float)(-0.5 * (akl.x - alk.x)));
         }
-        // L_j += Re sum_l T_jl conj(X_jl) over this column tile
+    }
+}
+
+__global__ void __launch_bounds__(256) k_loss_quadform(int n, const float2* Xall, const float2* Ball, const int* flags,
+                                                       const double* norms, const double* xnorms, double kappa_refine,
+                                                       double2* diag_inv, double* L) {
+    __shared__ __align__(16) float2 Xs[QK][QF + 2];        // [k][j]
+    __shared__ __align__(16) float2 Bs[QK][QF];            // [k][l]
+    const int b = blockIdx.x, j0 = blockIdx.y * QF;
+    if (flags[b] || norms[b] * xnorms[b] > kappa_refine) return;
+    const float2* X = Xall + (size_t)b * n * n;
+    const float2* B = Ball + (size_t)b * n * n;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // rows 4 ty .. + 3, columns tx + 16 u
+    float part[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int l0 = 0; l0 < n; l0 += QF) {
+        float2 acc[4][4];
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-            const int j = j0 + ty + 16 * r;
-            float part = 0.0f;
+        for (int r = 0; r < 4; ++r)
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                const int l = l0 + tx + 16 * c;
+            for (int u = 0; u < 4; ++u) acc[r][u] = make_float2(0.f, 0.f);
+        for (int k0 = 0; k0 < l0 + QF && k0 < n; k0 += QK) {
+            if (k0 == l0) {                                    // the tiles before count for their mirror images too
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) acc[r][u] = make_float2(2.f * acc[r][u].x, 2.f * acc[r][u].y);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int v = 0; v < QF * QK / 256; ++v) {
+                const int e = threadIdx.x + 256 * v;
+                const int kx = e % QK, jx = e / QK;            // rows of X along k
+                Xs[kx][jx] = j0 + jx < n && k0 + kx < n ? X[(size_t)(j0 + jx) * n + k0 + kx] : make_float2(0.f, 0.f);
+                const int lb = e % QF, kb = e / QF;
+                Bs[kb][lb] = k0 + kb < n && l0 + lb < n ? B[(size_t)(k0 + kb) * n + l0 + lb] : make_float2(0.f, 0.f);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < QK; ++k) {
+                const float4 xa = *reinterpret_cast<const float4*>(&Xs[k][ty * 4]);
+                const float4 xb = *reinterpret_cast<const float4*>(&Xs[k][ty * 4 + 2]);
+                const float2 x[4] = {make_float2(xa.x, xa.y), make_float2(xa.z, xa.w), make_float2(xb.x, xb.y),
+                                     make_float2(xb.z, xb.w)};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float2 v = Bs[k][tx + 16 * u];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) cfma(acc[r][u], x[r], v);
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = j0 + ty * 4 + r, l = l0 + tx + 16 * u;
                 if (j < n && l < n) {
                     const float2 x = X[(size_t)j * n + l];
-                    part = fmaf(acc[r][c].x, x.x, fmaf(acc[r][c].y, x.y, part));
+                    part[r] = fmaf(acc[r][u].x, x.x, fmaf(acc[r][u].y, x.y, part[r]));
                 }
             }
-            for (int o = 8; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o, 16);
-            if (tx == 0) Lrow[ty + 16 * r] += part;
-        }
-        __syncthreads();
     }
-    if (threadIdx.x < QF && j0 + threadIdx.x < n) {
-        const size_t o = (size_t)b * n + j0 + threadIdx.x;
-        L[o] = (double)Lrow[threadIdx.x];
-        diag_inv[o].y = -(double)Lrow[threadIdx.x];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        float s = part[r];
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, 16);
+        const int j = j0 + ty * 4 + r;
+        if (tx == 0 && j < n) {
+            const size_t o = (size_t)b * n + j;
+            L[o] = (double)s;
+            diag_inv[o].y = -(double)s;
+        }
     }
 }
 
@@ -518,14 +539,16 @@ static cudaError_t invert_batch(cudaStream_t st, int n, int nmat, const double2*
 // Matrices are inverted in groups whose second copy stays within INV_COPY_BYTES (at least one), so that the scratch
 // does not grow with the number of frequencies.
 constexpr size_t INV_COPY_BYTES = 1ull << 30;
+template <typename C> static int inv_group(int n, int nw) {
+    return (int)std::min<size_t>({(size_t)nw, std::max<size_t>(1, INV_COPY_BYTES / ((size_t)n * n * sizeof(C))), 32768});
+}
 
 template <typename T>
 static cudaError_t invert_all(qcx_ctx* ctx, QSlot& s, double* norms, double* L) {
     using C = cplx<T>;
     const int n = s.ng, nw = s.nw;
-    const size_t one = (size_t)n * n * sizeof(C);
-    const int per = (int)std::min<size_t>({(size_t)nw, std::max<size_t>(1, INV_COPY_BYTES / one), 32768});
-    cudaError_t e = s.work2.ensure(per * one);
+    const int per = inv_group<C>(n, nw);
+    cudaError_t e = s.work2.ensure((size_t)per * n * n * sizeof(C));
     if (e != cudaSuccess) return e;
     e = s.gjaux.ensure((size_t)per * n * (InvCfg<T>::PB * sizeof(C) + 2 * sizeof(int)));
     if (e != cudaSuccess) return e;
@@ -563,10 +586,20 @@ cudaError_t qcx_launch_invert(qcx_ctx* ctx, QSlot& s, qcx_precision prec, double
                                                   s.resid.as<double>());
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    dim3 gq(s.nw, (n + QF - 1) / QF);
-    k_loss_quadform<<<gq, 256, 0, ctx->stream>>>(n, s.eps.as<double2>(), s.work.as<float2>(), s.flags.as<int>(), norms,
-                                                  ctx->kappa_refine, s.diag_inv.as<double2>(), d_loss_out);
-    return cudaGetLastError();
+    const int per = inv_group<float2>(n, s.nw);          // B takes the inverse's second copy, group by group
+    const int t32 = (n + 31) / 32;
+    for (int w0 = 0; w0 < s.nw; w0 += per) {
+        const int m = std::min(per, s.nw - w0);
+        const size_t o = (size_t)w0 * n;
+        k_form_b<<<dim3(t32, t32, m), 256, 0, ctx->stream>>>(n, s.eps.as<double2>() + o * n, s.flags.as<int>() + w0, norms + w0,
+                                                              norms + s.nw + w0, ctx->kappa_refine, s.work2.as<float2>());
+        k_loss_quadform<<<dim3(m, (n + QF - 1) / QF), 256, 0, ctx->stream>>>(
+            n, s.work.as<float2>() + o * n, s.work2.as<float2>(), s.flags.as<int>() + w0, norms + w0, norms + s.nw + w0,
+            ctx->kappa_refine, s.diag_inv.as<double2>() + o, d_loss_out + o);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 extern "C" qcx_status qcx_set_refine_threshold(qcx_ctx* ctx, double kappa1) {
