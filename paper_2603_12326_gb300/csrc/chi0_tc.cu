@@ -36,7 +36,7 @@
 // buffer and eps is stored in FP64.
 //
 // CTA work item: one 64-row G' block, one frequency (a 128 x N accumulator:
-// 64 re rows and 64 im rows), one N chunk of G.  Warp roles (five warpgroups):
+// 64 re rows and 64 im rows), one N chunk of G, one split of K.  Warp roles (five warpgroups):
 // warp 0 issues TMA loads of the B tiles (and, when the G range is split, of the
 // A-source rows); warp 1 owns TMEM; one thread of warp 1 issues the MMAs of the
 // even accumulation windows and one thread of warp 2 those of the odd windows;
@@ -81,12 +81,13 @@ struct TcArgs {
     int ng, nw, nv, nc;
     long long nt;
     int n_tile, n_gb, kstages, src_from_b;
+    int kper;                         // K stages per split (gridDim.z splits)
     uint32_t acc_off, tmem_cols;      // second TMEM buffer column, columns allocated
     const float2* wtab;   // [nw][kp/2] W_t(w) in FP32 (tabulated with FP64 dE)
     long long wld;        // row length of wtab
     double pref;
     const double* vs;
-    double* acc64;    // [grid][n_tile][128] FP64 partial sums, one region per CTA (column-major, so a
+    double* acc64;    // [split][grid][n_tile][128] FP64 partial sums, one region per CTA (column-major, so a
                       // warp's 32 accumulator rows are contiguous)
     double2* eps;     // [nw][ng][ng], eps^T: row G', column G (FP64)
     double2* chi;     // optional [nw][ng][ng], row G, column G'
@@ -103,6 +104,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gb = blockIdx.x / a.nw, iw = blockIdx.x % a.nw;
     const int n0 = blockIdx.y * a.n_tile;
+    const int k_off = blockIdx.z * a.kper, kst = min(a.kper, a.kstages - k_off);   // this split's K stages
     const uint32_t bbytes = (uint32_t)a.n_tile * ROWB;          // one B piece
     const uint32_t spiece = (uint32_t)GBLK * ROWB;              // one A-source piece
     const uint32_t sbytes = a.src_from_b ? 0u : NPB * spiece;
@@ -145,7 +147,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int nwin = (a.kstages + PROMOTE - 1) / PROMOTE;
+    const int nwin = (kst + PROMOTE - 1) / PROMOTE;
 
     if (warp < AGEN_WARP0) {
         regs_dec<REG_CTRL>();
@@ -154,34 +156,34 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             if (lane == 0) {
                 // a stage's lines are requested into L2 a few stages before its copy is issued
                 auto prefetch = [&](int it) {
-                    bulk_prefetch(a.wtab + (size_t)iw * a.wld + (size_t)it * TPS, TPS * sizeof(float2));
-                    tma_prefetch_2d(&mb0, it * KSTEP, n0);
-                    tma_prefetch_2d(&mb1, it * KSTEP, n0);
+                    bulk_prefetch(a.wtab + (size_t)iw * a.wld + (size_t)(k_off + it) * TPS, TPS * sizeof(float2));
+                    tma_prefetch_2d(&mb0, (k_off + it) * KSTEP, n0);
+                    tma_prefetch_2d(&mb1, (k_off + it) * KSTEP, n0);
                     if (!a.src_from_b) {
-                        tma_prefetch_2d(&ms0, it * KSTEP, gb * GBLK);
-                        tma_prefetch_2d(&ms1, it * KSTEP, gb * GBLK);
+                        tma_prefetch_2d(&ms0, (k_off + it) * KSTEP, gb * GBLK);
+                        tma_prefetch_2d(&ms1, (k_off + it) * KSTEP, gb * GBLK);
                     }
                 };
-                for (int it = 0; it < PREFETCH && it < a.kstages; ++it) prefetch(it);
+                for (int it = 0; it < PREFETCH && it < kst; ++it) prefetch(it);
                 int last = -1;
                 // with copies withheld (fault injection for tests) nothing is issued, so the
                 // consumers' first waits run out and the kernel reports a timeout
-                for (int it = 0; it < (a.withhold ? 0 : a.kstages); ++it) {
+                for (int it = 0; it < (a.withhold ? 0 : kst); ++it) {
                     const int s = it % NSTAGE;
                     const uint32_t ph = (uint32_t)(it / NSTAGE) & 1u;
-                    if (it + PREFETCH < a.kstages) prefetch(it + PREFETCH);
+                    if (it + PREFETCH < kst) prefetch(it + PREFETCH);
                     if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, a.status, a.wait_limit)) break;
                     uint64_t* fb = &full_b[it % (2 * NSTAGE)];
                     unsigned char* st = base + s * stage_bytes;
                     mbar_arrive_tx(fb, NPB * bbytes + sbytes + TPS * (uint32_t)sizeof(float2));
-                    bulk_load(Wbuf + s * TPS, a.wtab + (size_t)iw * a.wld + (size_t)it * TPS, TPS * sizeof(float2),
+                    bulk_load(Wbuf + s * TPS, a.wtab + (size_t)iw * a.wld + (size_t)(k_off + it) * TPS, TPS * sizeof(float2),
                               fb);
-                    tma_load_2d(st, &mb0, fb, it * KSTEP, n0);
-                    tma_load_2d(st + bbytes, &mb1, fb, it * KSTEP, n0);
+                    tma_load_2d(st, &mb0, fb, (k_off + it) * KSTEP, n0);
+                    tma_load_2d(st + bbytes, &mb1, fb, (k_off + it) * KSTEP, n0);
                     if (!a.src_from_b) {
                         unsigned char* sp = st + NPB * bbytes;
-                        tma_load_2d(sp, &ms0, fb, it * KSTEP, gb * GBLK);
-                        tma_load_2d(sp + spiece, &ms1, fb, it * KSTEP, gb * GBLK);
+                        tma_load_2d(sp, &ms0, fb, (k_off + it) * KSTEP, gb * GBLK);
+                        tma_load_2d(sp + spiece, &ms1, fb, (k_off + it) * KSTEP, gb * GBLK);
                     }
                     last = it;
                 }
@@ -205,7 +207,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
                     if (win >= 2 &&
                         !mbar_wait(&drained[b], (uint32_t)((win - 2) >> 1) & 1u, abort_flag, a.status, a.wait_limit))
                         break;
-                    const int it1 = min((win + 1) * PROMOTE, a.kstages);
+                    const int it1 = min((win + 1) * PROMOTE, kst);
                     for (int it = win * PROMOTE; it < it1; ++it) {
                         const int s = it % NSTAGE;
                         const bool first = it == win * PROMOTE;
@@ -246,7 +248,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const int j = g & 3;                           // 16-byte chunk = 4 transitions
         const int go = g >> 2;                         // G' offset in the block (0..63)
         const int Gp = gb * GBLK + go;
-        for (int it = 0; it < a.kstages; ++it) {
+        for (int it = 0; it < kst; ++it) {
             const int s = it % NSTAGE;
             const int s2 = it % (2 * NSTAGE);
             // the producer issued this stage's copies only after the MMAs of its previous use
@@ -306,7 +308,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         const bool tail8 = (half & 15) != 0;
         const uint32_t lane_off = (uint32_t)(q * 32) << 16;
         const int row = q * 32 + lane;      // accumulator row: 0..63 re, 64..127 im
-        double* acc64 = a.acc64 + (size_t)(blockIdx.y * gridDim.x + blockIdx.x) * 128 * a.n_tile +
+        double* acc64 = a.acc64 + ((size_t)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * 128 * a.n_tile +
                         (size_t)(hc * half) * 128 + row;
         float part[MAXHALF];
 #pragma unroll
@@ -359,7 +361,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             }
         }
         // -------------------------------------------------------------- epilogue
-        if (ok) {
+        if (ok && gridDim.z == 1) {
             const int cpart = row >> 6, gro = row & 63;
             const int Gr = gb * GBLK + gro;
             if (Gr < a.ng) {
@@ -518,6 +520,37 @@ __global__ void k_diag_finish(int nw, int ng, int nsplit, const double2* part, d
     if (chi) chi[o] = ch;
 }
 
+// eps and chi0 from the K splits' FP64 sums, added in split order: thread per (accumulator row, column), rows fastest.
+__global__ void __launch_bounds__(128) k_chi0_splits(TcArgs a, int nsplit) {
+    const int gb = blockIdx.x / a.nw, iw = blockIdx.x % a.nw, row = threadIdx.x;
+    const int cpart = row >> 6, Gr = gb * GBLK + (row & 63), G = blockIdx.y * a.n_tile + blockIdx.z;
+    if (Gr >= a.ng || G >= a.ng) return;
+    const size_t stride = (size_t)gridDim.x * gridDim.y * 128 * a.n_tile;
+    const double* p = a.acc64 + (((size_t)blockIdx.y * gridDim.x + blockIdx.x) * a.n_tile + blockIdx.z) * 128 + row;
+    double sum = 0.0;
+    for (int z = 0; z < nsplit; ++z) sum += p[z * stride];
+    const double ch = a.pref * sum;
+    reinterpret_cast<double*>(a.eps)[2 * (((size_t)iw * a.ng + Gr) * a.ng + G) + cpart] =
+        (cpart == 0 && G == Gr ? 1.0 : 0.0) - a.vs[Gr] * a.vs[G] * ch;
+    if (a.chi) reinterpret_cast<double*>(a.chi)[2 * (((size_t)iw * a.ng + G) * a.ng + Gr) + cpart] = ch;
+}
+
+// K splits: with one CTA per SM the time goes with whole waves of CTAs, each its stages plus ~10 stages' worth of set-up,
+// read-out and the splits' sums; a launch below one wave leaves SMs idle, one just above it pays a second wave.
+// (50 frequencies of N_G = 27, N_t = 3072: 129 -> 44 + 5 us; 37 of 113, 3105: 178 -> 81 + 13 us.)
+static int pick_splits(long long ctas, int kstages) {
+    int best = 1;
+    double cost = 1e300;
+    for (int n = 1; n <= 8 && kstages / n >= 16; ++n) {
+        const double c = (double)((ctas * n + 151) / 152) * (kstages / n + 10.0) * (n == 1 ? 1.0 : 1.05);
+        if (c < cost) {
+            cost = c;
+            best = n;
+        }
+    }
+    return best;
+}
+
 }  // namespace
 
 typedef CUresult (*PFN_encodeTiled_t)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -612,13 +645,16 @@ cudaError_t qcx_launch_chi0_mixed(qcx_ctx* ctx, QSlot& s, int iq, double2* chi, 
     }
     a.wtab = s.wtab.as<float2>();
     dim3 grid(a.n_gb * s.nw, n_chunks);
+    const int want_k = pick_splits((long long)grid.x * grid.y, a.kstages);
+    a.kper = ((a.kstages + want_k - 1) / want_k + PROMOTE - 1) / PROMOTE * PROMOTE;
+    grid.z = (a.kstages + a.kper - 1) / a.kper;
     // split of the transitions for the diagonal pass: enough CTAs to fill the GPU, each range a
     // multiple of 256 transitions; its partial sums reuse acc64 once k_chi0_tc has finished
     const dim3 dgrid((ng + 31) / 32, (s.nw + 31) / 32);
     const long long want = std::max<long long>(1, (8LL * 152 + dgrid.x * dgrid.y - 1) / (dgrid.x * dgrid.y));
     const long long tps = std::max<long long>(256, ((nt + want - 1) / want + 255) / 256 * 256);
     const int nsplit = (int)((nt + tps - 1) / tps);
-    const size_t acc_bytes = std::max((size_t)grid.x * grid.y * 128 * a.n_tile * sizeof(double),
+    const size_t acc_bytes = std::max((size_t)grid.x * grid.y * grid.z * 128 * a.n_tile * sizeof(double),
                                       (size_t)nsplit * s.nw * ng * sizeof(double2));
     e = s.acc64.ensure(acc_bytes);
     if (e != cudaSuccess) return e;
@@ -644,6 +680,11 @@ cudaError_t qcx_launch_chi0_mixed(qcx_ctx* ctx, QSlot& s, int iq, double2* chi, 
     k_chi0_tc<<<grid, NTHREADS, smem, ctx->stream>>>(mb[0], mb[1], ms[0], ms[1], a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    if (grid.z > 1) {
+        k_chi0_splits<<<dim3(grid.x, grid.y, a.n_tile), 128, 0, ctx->stream>>>(a, (int)grid.z);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
     const __nv_bfloat162* q0 = reinterpret_cast<const __nv_bfloat162*>(s.rho.p);
     const long long plane2 = (long long)s.ngp * (s.kp / 2);
     double2* part = s.acc64.as<double2>();
