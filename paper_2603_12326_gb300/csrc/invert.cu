@@ -328,62 +328,85 @@ __global__ void __launch_bounds__(256) k_inv_finish(int n, const cplx<T>* X, con
 
 // FP64 correction of the diagonal of X ~ A^-1 for the blocks with kappa_1 above
 // the threshold (A FP64, X FP32):  d_j = X_jj + sum_k X_jk (delta_kj - sum_l A_kl X_lj).
-// Grid (block, 32-column panel).  The other blocks keep X_jj.
-constexpr int RF_COLS = 32;
-__global__ void __launch_bounds__(256) k_refine_diag(int n, const double2* Aall, const float2* Xall,
-                                                     const int* flags, const double* norms, double kappa_refine,
-                                                     double2* diag_inv, double* L, double* resid) {
-    __shared__ double2 s_d[RF_COLS];
-    const int b = blockIdx.x, j0 = blockIdx.y * RF_COLS;
-    if (flags[b] || j0 >= n) return;
-    const float2* X = Xall + (size_t)b * n * n;
-    if (!(norms[b] * norms[gridDim.x + b] > kappa_refine)) {
-        if (threadIdx.x < RF_COLS && j0 + threadIdx.x < n) {
-            const int j = j0 + threadIdx.x;
-            const float2 x = X[(size_t)j * n + j];
-            diag_inv[(size_t)b * n + j] = make_double2((double)x.x, (double)x.y);
-            L[(size_t)b * n + j] = -(double)x.y;
-        }
-        return;
-    }
+// The other blocks keep X_jj.  A CTA takes 32 rows k and 32 columns j of A X (k_refine_part) and leaves their share of
+// d_j; k_refine_diag adds the shares in row order.  Bound by the FP64 pipe (4 n^3 multiply-adds a block, 1.1 ms at
+// N_G = 531); with all rows k of 32 columns in one CTA a few blocks waited for its serial sums: 5 of 531: 44 -> 5 ms,
+// 84: 143 -> 85 ms.
+constexpr int RF_T = 32, RF_K = 16;
+__global__ void __launch_bounds__(256) k_refine_part(int n, int nw, const double2* Aall, const float2* Xall, const int* flags,
+                                                     const double* norms, double kappa_refine, double2* part) {
+    __shared__ double2 As[RF_K][RF_T + 1];                 // [l][k]
+    __shared__ double2 Xs[RF_K][RF_T];                     // [l][j]
+    __shared__ double2 red[RF_T][17];
+    const int b = blockIdx.x, j0 = blockIdx.y * RF_T, k0 = blockIdx.z * RF_T;
+    if (flags[b] || !(norms[b] * norms[nw + b] > kappa_refine)) return;
     const double2* A = Aall + (size_t)b * n * n;
-    if (threadIdx.x < RF_COLS) s_d[threadIdx.x] = make_double2(0.0, 0.0);
-    __syncthreads();
-    const int jl = threadIdx.x & (RF_COLS - 1);
-    const int j = j0 + jl;
-    double2 part = make_double2(0.0, 0.0);
-    if (j < n) {
-        for (int k = threadIdx.x / RF_COLS; k < n; k += blockDim.x / RF_COLS) {
-            double yr = 0.0, yi = 0.0;          // sum_l A_kl X_lj in FP64
-            for (int l = 0; l < n; ++l) {
-                const double2 av = A[(size_t)k * n + l];
-                const float2 x = X[(size_t)l * n + j];
-                yr = fma(av.x, (double)x.x, yr);
-                yr = fma(-av.y, (double)x.y, yr);
-                yi = fma(av.x, (double)x.y, yi);
-                yi = fma(av.y, (double)x.x, yi);
-            }
-            const double rr = (k == j ? 1.0 : 0.0) - yr, ri = -yi;
-            const float2 xjk = X[(size_t)j * n + k];
-            part.x += (double)xjk.x * rr - (double)xjk.y * ri;
-            part.y += (double)xjk.x * ri + (double)xjk.y * rr;
+    const float2* X = Xall + (size_t)b * n * n;
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;    // rows ty, ty + 16; columns tx, tx + 16
+    double2 acc[2][2];
+#pragma unroll
+    for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) acc[r][c] = make_double2(0.0, 0.0);
+    for (int l0 = 0; l0 < n; l0 += RF_K) {
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+            const int e = threadIdx.x + 256 * v;
+            const int la = e % RF_K, ka = e / RF_K, lx = e / RF_T, jx = e % RF_T;
+            As[la][ka] = l0 + la < n && k0 + ka < n ? A[(size_t)(k0 + ka) * n + l0 + la] : make_double2(0.0, 0.0);
+            const float2 x = l0 + lx < n && j0 + jx < n ? X[(size_t)(l0 + lx) * n + j0 + jx] : make_float2(0.f, 0.f);
+            Xs[lx][jx] = make_double2((double)x.x, (double)x.y);
         }
+        __syncthreads();
+#pragma unroll 4
+        for (int l = 0; l < RF_K; ++l) {
+            const double2 a0 = As[l][ty], a1 = As[l][ty + 16], x0 = Xs[l][tx], x1 = Xs[l][tx + 16];
+            cfma(acc[0][0], a0, x0);
+            cfma(acc[0][1], a0, x1);
+            cfma(acc[1][0], a1, x0);
+            cfma(acc[1][1], a1, x1);
+        }
+        __syncthreads();
     }
-    atomicAdd(&s_d[jl].x, part.x);
-    atomicAdd(&s_d[jl].y, part.y);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int j = j0 + tx + 16 * c;
+        double2 d = make_double2(0.0, 0.0);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const int k = k0 + ty + 16 * r;
+            if (j < n && k < n) {
+                const double2 res = make_double2((k == j ? 1.0 : 0.0) - acc[r][c].x, -acc[r][c].y);
+                const float2 x = X[(size_t)j * n + k];
+                cfma(d, make_double2((double)x.x, (double)x.y), res);
+            }
+        }
+        red[tx + 16 * c][ty] = d;
+    }
     __syncthreads();
-    if (threadIdx.x < RF_COLS && j0 + threadIdx.x < n) {
-        const int jj = j0 + threadIdx.x;
-        const float2 x = X[(size_t)jj * n + jj];
-        const double dr = (double)x.x + s_d[threadIdx.x].x, di = (double)x.y + s_d[threadIdx.x].y;
-        diag_inv[(size_t)b * n + jj] = make_double2(dr, di);
-        L[(size_t)b * n + jj] = -di;
+    if (threadIdx.x < RF_T && j0 + threadIdx.x < n) {
+        double2 d = make_double2(0.0, 0.0);
+        for (int r = 0; r < 16; ++r) d = cadd(d, red[threadIdx.x][r]);
+        part[((size_t)blockIdx.z * nw + b) * n + j0 + threadIdx.x] = d;
+    }
+}
+
+__global__ void __launch_bounds__(128) k_refine_diag(int n, int nw, int nk, const float2* Xall, const int* flags,
+                                                     const double* norms, double kappa_refine, const double2* part,
+                                                     double2* diag_inv, double* L, double* resid) {
+    const int b = blockIdx.x, j = blockIdx.y * 128 + threadIdx.x;
+    if (flags[b] || j >= n) return;
+    const float2 x = Xall[(size_t)b * n * n + (size_t)j * n + j];
+    double2 d = make_double2(0.0, 0.0);
+    if (norms[b] * norms[nw + b] > kappa_refine) {
+        for (int z = 0; z < nk; ++z) d = cadd(d, part[((size_t)z * nw + b) * n + j]);
+        const double dr = (double)x.x + d.x, di = (double)x.y + d.y;
         const double mag = sqrt(dr * dr + di * di);
-        const double rel = mag > 0 ? sqrt(s_d[threadIdx.x].x * s_d[threadIdx.x].x +
-                                          s_d[threadIdx.x].y * s_d[threadIdx.x].y) / mag
-                                   : 0.0;
+        const double rel = mag > 0 ? sqrt(d.x * d.x + d.y * d.y) / mag : 0.0;
         atomicMax(reinterpret_cast<unsigned long long*>(resid + b), (unsigned long long)__double_as_longlong(rel));
     }
+    diag_inv[(size_t)b * n + j] = make_double2((double)x.x + d.x, (double)x.y + d.y);
+    L[(size_t)b * n + j] = -((double)x.y + d.y);
 }
 
 // L_LFE of the mixed path without cancellation: for X = A^-1 (the FP32
@@ -580,10 +603,16 @@ cudaError_t qcx_launch_invert(qcx_ctx* ctx, QSlot& s, qcx_precision prec, double
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(s.resid.p, 0, sizeof(double) * s.nw, ctx->stream);
     if (e != cudaSuccess) return e;
-    dim3 grid(s.nw, (n + RF_COLS - 1) / RF_COLS);
-    k_refine_diag<<<grid, 256, 0, ctx->stream>>>(n, s.eps.as<double2>(), s.work.as<float2>(), s.flags.as<int>(), norms,
-                                                  ctx->kappa_refine, s.diag_inv.as<double2>(), d_loss_out,
-                                                  s.resid.as<double>());
+    const int rt = (n + RF_T - 1) / RF_T;
+    e = s.refine.ensure(sizeof(double2) * (size_t)rt * s.nw * n);
+    if (e != cudaSuccess) return e;
+    k_refine_part<<<dim3(s.nw, rt, rt), 256, 0, ctx->stream>>>(n, s.nw, s.eps.as<double2>(), s.work.as<float2>(),
+                                                               s.flags.as<int>(), norms, ctx->kappa_refine,
+                                                               s.refine.as<double2>());
+    k_refine_diag<<<dim3(s.nw, (n + 127) / 128), 128, 0, ctx->stream>>>(n, s.nw, rt, s.work.as<float2>(), s.flags.as<int>(),
+                                                                        norms, ctx->kappa_refine, s.refine.as<double2>(),
+                                                                        s.diag_inv.as<double2>(), d_loss_out,
+                                                                        s.resid.as<double>());
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int per = inv_group<float2>(n, s.nw);          // B takes the inverse's second copy, group by group

@@ -67,6 +67,7 @@ struct QSlot {
     DevBuf acc64;              // FP64 partial sums of the tensor-core chi0 (one region per CTA)
     DevBuf wtab;               // [nw][kp/2] float2 transition weights of the mixed path
     DevBuf kappa1;             // [2][nw] double |A|_1 and |X|_1 of the mixed inverse (kappa_1 is their product)
+    DevBuf refine;             // shares of the FP64 diagonal correction [row tile][nw][ng] double2
     DevBuf w;                  // [nw] double
     DevBuf diag_inv;           // [nw][ng] double2
     DevBuf eps_diag;           // [nw][ng] double2
