@@ -59,7 +59,8 @@ template <typename T> struct PDArgs {
     // tables (PdTab): one-dimensional factors per (pair, axis, k class, q+G class)
     const cplx<T>* ptab;     // [entries][NCH][4], or null
     const int* kidx;         // [nk][3]
-    const int* gidx;         // [ng][3]
+    const int* gidx;         // [ng][3], G in the tables' order
+    const int* gperm;        // [ng] G of each place in that order
     int nkx[3], nqx[3];
     long long tbase[4];
 };
@@ -482,118 +483,157 @@ __global__ void __launch_bounds__(pdf_maxt<NV>()) k_pair_density_fused(PDArgs<fl
     }
 }
 
-// The pair densities from the tables of PdTab, either precision.  One thread per (G, group a), threads ordered G
-// fastest (a warp reads the entries of one or two pairs, a few hundred bytes each); per group b it adds up the 4 x 4
-// pair block from three table entries per character and multiplies it into its rows of Y = B C_k for NV bands at a
-// time.  Y goes to shared memory (bands padded to a multiple of 4) and rho = C_kq^H Y takes four bands per thread.
+// The pair densities from the tables of PdTab, either precision, in two kernels over a chunk of k points.
 //
-// What bounds it: the FP32 (FP64) pipe: per (k, G, pair) 100 multiply-adds per character for the block and 64 per
-// four bands for Y, where the form with a common factor and unshared y-z products took 192 per character and 96 more.
-// Measured (one q: 512 k x 181 G, 24 groups, 4 x 32 bands): FP32 2.54 -> 1.70 ms; FP64, which formed the lattice
-// sums per (k, G) before, 252 -> 51 ms.
+// k_pd_y: Y = B C_k.  One thread per (G, group a), threads ordered G fastest; per group b it adds up the 4 x 4 pair
+// block from three table entries per character and multiplies it into its rows of Y for NV bands at a time.  The entries
+// of a (k, pair) are ~2 KB for all G, so a CTA takes as many G as it can (up to 192) and few groups a: with 16 G and all
+// groups a, each CTA streamed 1.2 MB of tables from L2 (7.4 GB a call at N_G = 181) and L2 was the bound.  Now bound by
+// the FP32 (FP64) pipe: per (k, G, pair) 100 multiply-adds per character for the block and 64 per four bands for Y.
+// k_pd_rho: rho = C_kq^H Y, 32 conduction bands x 64 G per CTA, 8 G per thread.
+// Measured (one q: 512 k x 181 G, 24 groups, 4 x 32 bands): FP32 2.54 at first, 1.70 as one kernel, 1.46 ms now; FP64,
+// which formed the lattice sums per (k, G) before, 252 -> 51 ms.
 template <typename T, int NV> constexpr int pdt_threads() { return sizeof(T) == 8 ? 192 : pdf_maxt<NV>(); }
 template <typename T, int NCH, int NV>
-__global__ void __launch_bounds__(pdt_threads<T, NV>()) k_pair_density_tab(PDArgs<T> a) {
+__global__ void __launch_bounds__(pdt_threads<T, NV>()) k_pd_y(PDArgs<T> a, int kb, int gc, int ga_per, cplx<T>* Yout) {
     using C = cplx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int nb = a.nb, nv = a.nv, nc = a.nc, gc = a.g_per_cta;
+    const int nb = a.nb, nv = a.nv;
     const int nvp = (nv + NV - 1) / NV * NV;
     C* Cks = reinterpret_cast<C*>(smem_raw);       // [nb][nvp], zero for v >= nv
-    C* Ys = Cks + (size_t)nb * nvp;                // [gc][nb][nvp]
-    C* Ckqs = Ys + (size_t)gc * nb * nvp;          // [nb][nc]
-    const int k = blockIdx.x;
-    const int g0 = blockIdx.y * gc;
-    const int ngl = min(gc, a.ng - g0);
+    const int k = kb + blockIdx.x;
     for (int i = threadIdx.x; i < nb * nvp; i += blockDim.x) {
         const int mu = i / nvp, v = i - mu * nvp;
         Cks[i] = v < nv ? a.Ck[((size_t)k * nb + mu) * nv + v] : mk<T>(0, 0);
     }
-    for (int i = threadIdx.x; i < nb * nc; i += blockDim.x) Ckqs[i] = a.Ckq[(size_t)k * nb * nc + i];
     __syncthreads();
-
-    const int ga = threadIdx.x / gc, gl = threadIdx.x - ga * gc;
-    if (ga < a.ngrp && gl < ngl) {
-        const C* t0[3];
-        int stride[3];
+    const int ga = blockIdx.z * ga_per + threadIdx.x / gc, g = blockIdx.y * gc + threadIdx.x % gc;
+    if (ga >= a.ngrp || g >= a.ng) return;
+    const C* t0[3];
+    int stride[3];
 #pragma unroll
-        for (int x = 0; x < 3; ++x) {
-            stride[x] = a.nkx[x] * a.nqx[x] * (NCH * 4);
-            t0[x] = a.ptab + (a.tbase[x] + ((long long)ga * a.ngrp * a.nkx[x] + a.kidx[3 * k + x]) * a.nqx[x] +
-                              a.gidx[3 * (g0 + gl) + x]) * (NCH * 4);
-        }
-        const int ma = a.grp_mask[ga];
-        const int mu0 = a.grp_mu0[ga] - ((ma & 1) ? 0 : 1);
-        C* yrow = Ys + (size_t)gl * nb * nvp;
-        for (int v0 = 0; v0 < nvp; v0 += NV) {
-            C Y[4][NV];
+    for (int x = 0; x < 3; ++x) {
+        stride[x] = a.nkx[x] * a.nqx[x] * (NCH * 4);
+        t0[x] = a.ptab + (a.tbase[x] + ((long long)ga * a.ngrp * a.nkx[x] + a.kidx[3 * k + x]) * a.nqx[x] +
+                          a.gidx[3 * g + x]) * (NCH * 4);
+    }
+    const int ma = a.grp_mask[ga];
+    const int mu0 = a.grp_mu0[ga] - ((ma & 1) ? 0 : 1);
+    C* yrow = Yout + (size_t)blockIdx.x * nb * nvp * a.ng + g;                // [k][mu][v][G]
+    for (int v0 = 0; v0 < nvp; v0 += NV) {
+        C Y[4][NV];
+#pragma unroll
+        for (int ca = 0; ca < 4; ++ca)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) Y[ca][v] = mk<T>(0, 0);
+        // FP32: the next character's (or pair's) entries are requested before this one's products (three warps per
+        // scheduler do not cover the gathers); FP64 has no registers for it and no need
+        constexpr bool AHEAD = sizeof(T) == 4;
+        C x[4], y[4], z[4];
+        auto fetch = [&](int gb, int ch) {
+            load4(t0[0] + (size_t)gb * stride[0] + 4 * ch, x);
+            load4(t0[1] + (size_t)gb * stride[1] + 4 * ch, y);
+            load4(t0[2] + (size_t)gb * stride[2] + 4 * ch, z);
+        };
+        if (AHEAD) fetch(0, 0);
+        for (int gb = 0; gb < a.ngrp; ++gb) {
+            C B[4][4];
 #pragma unroll
             for (int ca = 0; ca < 4; ++ca)
 #pragma unroll
-                for (int v = 0; v < NV; ++v) Y[ca][v] = mk<T>(0, 0);
-            for (int gb = 0; gb < a.ngrp; ++gb) {
-                C B[4][4];
+                for (int cb = 0; cb < 4; ++cb) B[ca][cb] = mk<T>(0, 0);
 #pragma unroll
-                for (int ca = 0; ca < 4; ++ca)
+            for (int ch = 0; ch < NCH; ++ch) {
+                if (AHEAD) {
+                    C xc[4], yc[4], zc[4];
 #pragma unroll
-                    for (int cb = 0; cb < 4; ++cb) B[ca][cb] = mk<T>(0, 0);
-#pragma unroll
-                for (int ch = 0; ch < NCH; ++ch) {
-                    C x[4], y[4], z[4];
-                    load4(t0[0] + (size_t)gb * stride[0] + 4 * ch, x);
-                    load4(t0[1] + (size_t)gb * stride[1] + 4 * ch, y);
-                    load4(t0[2] + (size_t)gb * stride[2] + 4 * ch, z);
+                    for (int i = 0; i < 4; ++i) {
+                        xc[i] = x[i];
+                        yc[i] = y[i];
+                        zc[i] = z[i];
+                    }
+                    const bool more = ch + 1 < NCH;
+                    fetch(more ? gb : min(gb + 1, a.ngrp - 1), more ? ch + 1 : 0);
+                    add_character(xc, yc, zc, B);
+                } else {
+                    fetch(gb, ch);
                     add_character(x, y, z, B);
                 }
-                const int mb = a.grp_mask[gb];
-                const int nu0 = a.grp_mu0[gb] - ((mb & 1) ? 0 : 1);
+            }
+            const int mb = a.grp_mask[gb];
+            const int nu0 = a.grp_mu0[gb] - ((mb & 1) ? 0 : 1);
 #pragma unroll
-                for (int cb = 0; cb < 4; ++cb) {
-                    if (!(cb == 0 ? (mb & 1) : (mb & 2))) continue;
-                    const C* ck = Cks + (size_t)(nu0 + cb) * nvp + v0;
+            for (int cb = 0; cb < 4; ++cb) {
+                if (!(cb == 0 ? (mb & 1) : (mb & 2))) continue;
+                const C* ck = Cks + (size_t)(nu0 + cb) * nvp + v0;
 #pragma unroll
-                    for (int v = 0; v < NV; v += 4) {
-                        C c[4];
-                        load4(ck + v, c);
+                for (int v = 0; v < NV; v += 4) {
+                    C c[4];
+                    load4(ck + v, c);
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
+                    for (int u = 0; u < 4; ++u)
 #pragma unroll
-                            for (int ca = 0; ca < 4; ++ca) cfma(Y[ca][v + u], B[ca][cb], c[u]);
-                    }
+                        for (int ca = 0; ca < 4; ++ca) cfma(Y[ca][v + u], B[ca][cb], c[u]);
                 }
             }
+        }
 #pragma unroll
-            for (int ca = 0; ca < 4; ++ca) {
-                if (!(ca == 0 ? (ma & 1) : (ma & 2))) continue;
+        for (int ca = 0; ca < 4; ++ca) {
+            if (!(ca == 0 ? (ma & 1) : (ma & 2))) continue;
 #pragma unroll
-                for (int v = 0; v < NV; ++v) yrow[(size_t)(mu0 + ca) * nvp + v0 + v] = Y[ca][v];
-            }
+            for (int v = 0; v < NV; ++v)
+                if (v0 + v < nv) yrow[((size_t)(mu0 + ca) * nvp + v0 + v) * a.ng] = Y[ca][v];
         }
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < ngl * nc * (nvp / 4); i += blockDim.x) {
-        const int c = i % nc, r = i / nc;
-        const int l = r % ngl, v0 = r / ngl * 4;
-        if (v0 >= nv) continue;
-        const C* y = Ys + (size_t)l * nb * nvp + v0;
-        C acc[4];
+}
+
+constexpr int PR_C = 32, PR_G = 64;
+template <typename T>
+__global__ void __launch_bounds__(256) k_pd_rho(PDArgs<T> a, int kb, int nvp, const cplx<T>* Y) {
+    using C = cplx<T>;
+    constexpr int KC = sizeof(T) == 4 ? 48 : 24;   // basis functions staged at a time
+    __shared__ __align__(16) C Ys[KC][PR_G];
+    __shared__ C Cs[KC][PR_C];
+    const int nvb = a.nv, k = kb + blockIdx.z;
+    const int v = blockIdx.y % nvb, c0 = blockIdx.y / nvb * PR_C, g0 = blockIdx.x * PR_G;
+    const int cl = threadIdx.x & 31, gl = threadIdx.x >> 5;    // band, 8 G
+    const C* Yk = Y + ((size_t)blockIdx.z * a.nb * nvp + v) * a.ng;
+    const C* Ckq = a.Ckq + (size_t)k * a.nb * a.nc;
+    C acc[8];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) acc[u] = mk<T>(0, 0);
-        for (int mu = 0; mu < nb; ++mu) {
-            C yv[4];
-            load4(y + (size_t)mu * nvp, yv);
-            const C q = Ckqs[mu * nc + c];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) cfmac(acc[u], q, yv[u]);
+    for (int u = 0; u < 8; ++u) acc[u] = mk<T>(0, 0);
+    for (int m0 = 0; m0 < a.nb; m0 += KC) {
+        const int m = min(KC, a.nb - m0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < m * PR_G; e += 256) {
+            const int mu = e / PR_G, g = e % PR_G;
+            Ys[mu][g] = g0 + g < a.ng ? Yk[(size_t)(m0 + mu) * nvp * a.ng + g0 + g] : mk<T>(0, 0);
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            if (v0 + u >= nv) continue;
-            const long long t = ((long long)k * nv + v0 + u) * nc + c;
-            if constexpr (sizeof(T) == 8)
-                a.R64[(long long)(g0 + l) * a.nt + t] = acc[u];
-            else
-                store_split3(acc[u].x, acc[u].y, a.R0, a.R1, a.R2, (long long)(g0 + l) * a.kp2 + t);
+        for (int e = threadIdx.x; e < m * PR_C; e += 256) {
+            const int mu = e / PR_C, c = e % PR_C;
+            Cs[mu][c] = c0 + c < a.nc ? Ckq[(size_t)(m0 + mu) * a.nc + c0 + c] : mk<T>(0, 0);
         }
+        __syncthreads();
+#pragma unroll 4
+        for (int mu = 0; mu < m; ++mu) {
+            const C q = Cs[mu][cl];
+            C y[8];
+            load4(&Ys[mu][gl * 8], reinterpret_cast<C(&)[4]>(y[0]));
+            load4(&Ys[mu][gl * 8 + 4], reinterpret_cast<C(&)[4]>(y[4]));
+#pragma unroll
+            for (int u = 0; u < 8; ++u) cfmac(acc[u], q, y[u]);
+        }
+    }
+    if (c0 + cl >= a.nc) return;
+    const long long t = ((long long)k * nvb + v) * a.nc + c0 + cl;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        if (g0 + gl * 8 + u >= a.ng) break;
+        const int G = a.gperm[g0 + gl * 8 + u];
+        if constexpr (sizeof(T) == 8)
+            a.R64[(long long)G * a.nt + t] = acc[u];
+        else
+            store_split3(acc[u].x, acc[u].y, a.R0, a.R1, a.R2, (long long)G * a.kp2 + t);
     }
 }
 
@@ -753,21 +793,33 @@ template <int NCH> cudaError_t launch_fused_nv(qcx_ctx* ctx, PDArgs<float>& a, s
     return launch_fused<NCH, 16>(ctx, a, smem, grid, nthr);
 }
 
-// Table kernel with NV bands in registers; cudaErrorInvalidConfiguration when its shared-memory plan does not fit (the
-// caller then takes the kernels without tables).
-template <typename T, int NCH, int NV> cudaError_t launch_tab(qcx_ctx* ctx, PDArgs<T>& a) {
+constexpr size_t PD_Y_BYTES = 512ull << 20;     // Y of one chunk of k points (at least one point)
+// bands held in registers by k_pd_y (FP64: a fifth would spill) and bands padded to that
+template <typename T> int pd_nv(int nv) { return sizeof(T) == 8 || nv <= 4 ? 4 : (nv <= 8 ? 8 : 16); }
+size_t pd_y_per_k(int nb, int nv, int ng, size_t elem) {
+    const int w = elem == 16 ? pd_nv<double>(nv) : pd_nv<float>(nv);
+    return (size_t)nb * ((nv + w - 1) / w * w) * ng * elem;
+}
+
+// The two table kernels over chunks of k; cudaErrorInvalidConfiguration when the basis has more groups than a CTA or C_k
+// does not fit shared memory (the caller then takes the kernels without tables).
+template <typename T, int NCH, int NV> cudaError_t launch_tab(qcx_ctx* ctx, PDArgs<T>& a, const PdTab& t) {
     const int nvp = (a.nv + NV - 1) / NV * NV;
-    int gc = std::min(16, pdt_threads<T, NV>() / a.ngrp);
-    auto need = [&](int g) {
-        return sizeof(cplx<T>) * ((size_t)(g + 1) * a.nb * nvp + (size_t)a.nb * a.nc);
-    };
-    while (gc > 1 && need(gc) > 200 * 1024) --gc;
-    if (gc < 1 || need(gc) > 200 * 1024) return cudaErrorInvalidConfiguration;
-    a.g_per_cta = gc;
-    const cudaError_t e = set_smem<T>((const void*)k_pair_density_tab<T, NCH, NV>, need(gc));
+    const size_t smem = (size_t)a.nb * nvp * sizeof(cplx<T>);
+    if (smem > 200 * 1024) return cudaErrorInvalidConfiguration;
+    const int nch = (a.ng + 191) / 192, gc = (a.ng + nch - 1) / nch;
+    const int ga_per = std::min(a.ngrp, std::max(1, pdt_threads<T, NV>() / gc));
+    cudaError_t e = set_smem<T>((const void*)k_pd_y<T, NCH, NV>, smem);
     if (e != cudaSuccess) return e;
-    k_pair_density_tab<T, NCH, NV><<<dim3(a.nk, (a.ng + gc - 1) / gc), gc * a.ngrp, need(gc), ctx->stream>>>(a);
-    return cudaGetLastError();
+    const int kc = (int)std::min<size_t>({(size_t)a.nk, t.y.bytes / pd_y_per_k(a.nb, a.nv, a.ng, sizeof(cplx<T>)), 65535});
+    cplx<T>* Y = t.y.as<cplx<T>>();
+    for (int k0 = 0; k0 < a.nk; k0 += kc) {
+        const int m = std::min(kc, a.nk - k0);
+        k_pd_y<T, NCH, NV><<<dim3(m, nch, (a.ngrp + ga_per - 1) / ga_per), gc * ga_per, smem, ctx->stream>>>(a, k0, gc, ga_per, Y);
+        k_pd_rho<T><<<dim3((a.ng + PR_G - 1) / PR_G, a.nv * ((a.nc + PR_C - 1) / PR_C), m), 256, 0, ctx->stream>>>(a, k0, nvp, Y);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 template <typename T, int NCH> cudaError_t build_table(qcx_ctx* ctx, PDArgs<T>& a, const PdTab& t) {
@@ -795,19 +847,19 @@ template <typename T, int NCH> cudaError_t build_table(qcx_ctx* ctx, PDArgs<T>& 
     a.ptab = ta.out;
     a.kidx = t.kidx.as<int>();
     a.gidx = t.gidx.as<int>();
+    a.gperm = t.gperm.as<int>();
     k_pd_axis_table<T, NCH><<<(unsigned)((t.tbase[3] + 127) / 128), 128, 0, ctx->stream>>>(ta);
     return cudaGetLastError();
 }
 
-// FP64 keeps four bands in registers (a fifth would spill), FP32 up to sixteen
 template <typename T, int NCH> cudaError_t run_tab(qcx_ctx* ctx, PDArgs<T>& a, const PdTab& t) {
     const cudaError_t e = build_table<T, NCH>(ctx, a, t);
     if (e != cudaSuccess) return e;
     if constexpr (sizeof(T) == 4) {
-        if (a.nv > 8) return launch_tab<T, NCH, 16>(ctx, a);
-        if (a.nv > 4) return launch_tab<T, NCH, 8>(ctx, a);
+        if (pd_nv<T>(a.nv) == 16) return launch_tab<T, NCH, 16>(ctx, a, t);
+        if (pd_nv<T>(a.nv) == 8) return launch_tab<T, NCH, 8>(ctx, a, t);
     }
-    return launch_tab<T, NCH, 4>(ctx, a);
+    return launch_tab<T, NCH, 4>(ctx, a, t);
 }
 template <typename T> cudaError_t run_tab_nch(qcx_ctx* ctx, PDArgs<T>& a, const PdTab& t) {
     switch (ctx->nchar) {
@@ -1011,7 +1063,7 @@ static void axis_classes(const double* v, int n, int x, std::vector<double>& val
 // Classes and buffers of the tables for nk k points and ng values of q+G (host arrays); leaves t invalid when the
 // tables would not save work or exceed their memory budget.
 static cudaError_t tab_prepare(qcx_ctx* ctx, PdTab& t, const double* kpts, int nk, const double* kap, int ng,
-                               size_t elem) {
+                               size_t elem, size_t y_per_k) {
     t.valid = false;
     for (int i = 0; i < 3 * nk; ++i)
         if (!std::isfinite(kpts[i])) return cudaSuccess;
@@ -1030,23 +1082,35 @@ static cudaError_t tab_prepare(qcx_ctx* ctx, PdTab& t, const double* kpts, int n
         t.nqx[x] = (int)qval.size() - t.qofs[x];
         cells += (long long)t.nkx[x] * t.nqx[x];
     }
+    std::vector<int> gperm(ng), gsort(3 * (size_t)ng);
+    for (int g = 0; g < ng; ++g) gperm[g] = g;
+    std::sort(gperm.begin(), gperm.end(), [&](int i, int j) {
+        for (int x = 2; x >= 0; --x)
+            if (gidx[3 * i + x] != gidx[3 * j + x]) return gidx[3 * i + x] < gidx[3 * j + x];
+        return i < j;
+    });
+    for (int g = 0; g < ng; ++g)
+        for (int x = 0; x < 3; ++x) gsort[3 * g + x] = gidx[3 * gperm[g] + x];
     // worth it only when the classes repeat (regular k grids, G shells); bounded memory
     const size_t tab_bytes = (size_t)npair * cells * ctx->nchar * 4 * elem;
     if (4 * cells > 3LL * 3 * nk * ng || tab_bytes > ((size_t)512 << 20)) return cudaSuccess;
     for (int x = 0; x < 3; ++x) t.tbase[x + 1] = t.tbase[x] + (long long)npair * t.nkx[x] * t.nqx[x];
     cudaError_t e;
-    if ((e = t.tab.ensure(tab_bytes)) != cudaSuccess) {
+    const size_t y_bytes = y_per_k * std::min<size_t>(nk, std::max<size_t>(1, PD_Y_BYTES / std::max<size_t>(1, y_per_k)));
+    if ((e = t.tab.ensure(tab_bytes)) != cudaSuccess || (e = t.y.ensure(y_bytes)) != cudaSuccess) {
         if (e != cudaErrorMemoryAllocation) return e;
         cudaGetLastError();                       // no room for the tables: the kernels without them serve
         return cudaSuccess;
     }
     if ((e = t.kidx.ensure(kidx.size() * sizeof(int))) != cudaSuccess) return e;
     if ((e = t.gidx.ensure(gidx.size() * sizeof(int))) != cudaSuccess) return e;
+    if ((e = t.gperm.ensure(gperm.size() * sizeof(int))) != cudaSuccess) return e;
     if ((e = t.kval.ensure(kval.size() * sizeof(double))) != cudaSuccess) return e;
     if ((e = t.qval.ensure(qval.size() * sizeof(double))) != cudaSuccess) return e;
     const cudaMemcpyKind h2d = cudaMemcpyHostToDevice;
     if ((e = cudaMemcpyAsync(t.kidx.p, kidx.data(), kidx.size() * sizeof(int), h2d, ctx->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(t.gidx.p, gidx.data(), gidx.size() * sizeof(int), h2d, ctx->stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(t.gidx.p, gsort.data(), gsort.size() * sizeof(int), h2d, ctx->stream)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(t.gperm.p, gperm.data(), gperm.size() * sizeof(int), h2d, ctx->stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(t.kval.p, kval.data(), kval.size() * sizeof(double), h2d, ctx->stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(t.qval.p, qval.data(), qval.size() * sizeof(double), h2d, ctx->stream)) != cudaSuccess)
         return e;
@@ -1075,8 +1139,8 @@ cudaError_t qcx_pd_tab_prepare(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng
             for (int i = 0; i < 3; ++i) v += G_host[3 * g + i] * 2.0 * M_PI * inv[3 * x + i];
             kap[3 * g + x] = v;
         }
-    return tab_prepare(ctx, s.pdt, ctx->kpts_h.data(), nk, kap.data(), ng,
-                       prec == QCX_FP64 ? sizeof(double2) : sizeof(float2));
+    const size_t elem = prec == QCX_FP64 ? sizeof(double2) : sizeof(float2);
+    return tab_prepare(ctx, s.pdt, ctx->kpts_h.data(), nk, kap.data(), ng, elem, pd_y_per_k(ctx->nb, ctx->nv, ng, elem));
 }
 
 cudaError_t qcx_launch_pair_density(qcx_ctx* ctx, QSlot& s, int iq, qcx_precision prec) {
@@ -1178,7 +1242,7 @@ cudaError_t qcx_launch_overlap(qcx_ctx* ctx, int nk, const double* d_kpts, const
     a.Sout = d_out;
     const double zero[3] = {0.0, 0.0, 0.0};
     if (nk <= 65535) {
-        const cudaError_t e = tab_prepare(ctx, ctx->overlap_tab, k_host, nk, zero, 1, sizeof(double2));
+        const cudaError_t e = tab_prepare(ctx, ctx->overlap_tab, k_host, nk, zero, 1, sizeof(double2), 0);
         if (e != cudaSuccess) return e;
         if (ctx->overlap_tab.valid) {
             const dim3 grid(((ctx->ngrp + 1) / 2 * (ctx->ngrp + 1) + 127) / 128, nk);

@@ -45,8 +45,10 @@ struct PdTab {
     int kofs[3] = {0, 0, 0}, qofs[3] = {0, 0, 0}; // first value of each axis in kval / qval
     long long tbase[4] = {0, 0, 0, 0};            // first entry of each axis (tbase[3] = entries)
     DevBuf kidx, gidx;         // [nk][3], [ng][3] int: class of each point's component
+    DevBuf gperm;              // [ng] int: the G of gidx's rows (ordered by class)
     DevBuf kval, qval;         // values of the classes (axes concatenated)
     DevBuf tab;                // [entries][nchar][4] complex (FP32 or FP64): E(0,0), E(1,0), E(0,1), E(1,1)
+    DevBuf y;                  // Y = B C_k of a chunk of k points (pair densities)
 };
 
 // Per-precision working set of one q.
