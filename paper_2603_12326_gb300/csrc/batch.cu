@@ -167,7 +167,9 @@ struct BatchPlan {
     std::vector<BatchInst> hinst;
     std::vector<int> h_ng;
 
-    DevBuf d_G, d_inst, d_wtab, d_eps, d_work, d_rowmap, d_x, d_r, d_out, d_flags, d_status, d_acc;
+    long long total_n = 0;             // sum of N_G
+    DevBuf d_work2, d_aux;             // mixed: second copy of the matrices, panels and row orders
+    DevBuf d_G, d_inst, d_wtab, d_eps, d_work, d_x, d_r, d_out, d_flags, d_status, d_acc;
     DevBuf d_tiles, d_cta, d_rtask;
     std::vector<CUtensorMap> maps;              // [nslot][3]: the three BF16 planes of each slot
     std::vector<int> grp_tile0, grp_ntile;      // tensor-core tiles per group of <= QCX_BATCH_MAXQ slots
@@ -335,21 +337,22 @@ cudaError_t record(qcx_ctx* ctx, BatchPlan& p) {
     a.cta_ids = p.d_cta.as<int>() + p.lu_grid + 1;
     a.eps = p.d_eps.as<double2>();
     a.work = p.d_work.p;
-    a.rowmap = p.d_rowmap.as<int>();
     a.x = p.d_x.as<double2>();
     a.r = p.d_r.as<double2>();
     a.out = p.d_out.as<double>();
     a.flags = p.d_flags.as<int>();
     a.ninst = p.ninst;
-    if ((e = qcx_launch_lu_head(st, a, p.lu_grid, p.nmax, !mixed, mixed)) != cudaSuccess) return e;
+    if (!mixed) {
+        if ((e = qcx_launch_lu_head(st, a, p.lu_grid, p.nmax)) != cudaSuccess) return e;
+        ++p.launches;
+        return cudaSuccess;
+    }
+    if ((e = qcx_launch_batch_inverse(st, a, p.d_work2.as<float2>(), p.d_aux.p, p.total_n, p.nmax)) != cudaSuccess) return e;
     ++p.launches;
-    if (mixed) {
-        for (int it = 0; it < NREF; ++it) {
-            if ((e = qcx_launch_resid(st, a, p.d_rtask.as<int2>(), p.n_rtask)) != cudaSuccess) return e;
-            if ((e = qcx_launch_lu_correct(st, a, p.lu_grid, p.nmax, it == NREF - 1 ? 1 : 0)) != cudaSuccess)
-                return e;
-            p.launches += 2;
-        }
+    for (int it = 0; it < NREF; ++it) {
+        if ((e = qcx_launch_resid(st, a, p.d_rtask.as<int2>(), p.n_rtask)) != cudaSuccess) return e;
+        if ((e = qcx_launch_batch_correct(st, a, p.nmax, it == NREF - 1 ? 1 : 0)) != cudaSuccess) return e;
+        p.launches += 2;
     }
     return cudaSuccess;
 }
@@ -477,7 +480,11 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
     CUDA_OR_FAIL(p.d_inst.ensure(sizeof(BatchInst) * ninst), "alloc");
     CUDA_OR_FAIL(p.d_eps.ensure(sizeof(double2) * eps_off), "alloc eps");
     CUDA_OR_FAIL(p.d_work.ensure((mixed ? sizeof(float2) : sizeof(double2)) * work_off), "alloc work");
-    CUDA_OR_FAIL(p.d_rowmap.ensure(sizeof(int) * vec_off), "alloc");
+    p.total_n = vec_off;
+    if (mixed) {
+        CUDA_OR_FAIL(p.d_work2.ensure(sizeof(float2) * work_off), "alloc work");
+        CUDA_OR_FAIL(p.d_aux.ensure(qcx_batch_inverse_aux(p.total_n, p.nmax)), "alloc panels");
+    }
     CUDA_OR_FAIL(p.d_x.ensure(sizeof(double2) * vec_off), "alloc");
     CUDA_OR_FAIL(p.d_r.ensure(sizeof(double2) * vec_off), "alloc");
     CUDA_OR_FAIL(p.d_out.ensure(sizeof(double) * 3 * ninst), "alloc");

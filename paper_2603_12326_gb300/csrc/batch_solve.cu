@@ -2,27 +2,21 @@
 // instances: L_LFE = -Im [eps^-1]_{00} (Eq. (eps_LFE)) and L_noLFE =
 // -Im (1/eps_00) (Eq. (eps_noLFE)).
 //
-// Only the head of eps^-1 is needed, so no inverse is formed.  With the head
+// FP64 path: only the head of eps^-1 is needed, so no inverse is formed.  With the head
 // row and column moved last (A' = P^T eps P), [eps^-1]_{00} is the last
 // component of the solution of A' x = e_last; LU elimination with partial
 // pivoting of the augmented matrix [A' | e_last] leaves that component as
-// y_last / u_last,last, with no back substitution.
+// y_last / u_last,last, with no back substitution (k_lu_head: one CTA per instance
+// at a time, instance lists per CTA built on the host, largest first, so the batch is one
+// persistent launch; right-looking blocked LU on a work copy in global memory: rows are
+// never moved, a row map in shared memory records the pivot order; per panel of PB columns
+// the panel is factored in shared memory and the trailing columns, right-hand side included,
+// are processed CW at a time).
 //
-// k_lu_head: one CTA per instance at a time (instance lists per CTA are built
-//   on the host, largest first, so the batch is one persistent launch).
-//   Right-looking blocked LU on a work copy in global memory (L2-resident):
-//   rows are never moved; a row map in shared memory records the pivot order
-//   (logical row -> stored row).  Per panel of PB columns: the panel is
-//   gathered into shared memory and factored there; the trailing columns
-//   (right-hand side included) are processed CW at a time: U12 = L11^-1 A12
-//   through the explicit inverse of the unit lower triangle L11, then the
-//   rank-PB update A22 -= L21 U12 with U12 columns held in registers.
-//   FP64 for the plain path; FP32 for the mixed path, which also back-
-//   substitutes the whole solution x for the refinement.
-// k_resid: r = e_last - A' x in FP64 from the FP64 eps (32 rows per CTA, all
-//   instances at once, so the FP64 work is spread over the whole GPU).
-// k_lu_correct: d = A'^-1 r with the stored FP32 factors (blocked forward
-//   and back substitution), x += d in FP64; the head is x_last.
+// Mixed path: the blocked FP32 inverse of the per-q path over all instances (invert.cu); its
+// head column is x, refined with the FP64 residual r = e_last - A' x (k_resid: 32 rows per CTA,
+// all instances at once, so the FP64 work is spread over the whole GPU) and d = X r.  A CTA per
+// instance left the largest instance's elimination on one SM as the critical path.
 #include "qcx_internal.h"
 #include "cplx.cuh"
 
@@ -32,11 +26,7 @@ constexpr int LU_THREADS = 256;
 constexpr int NWARP = LU_THREADS / 32;
 constexpr int CW = 64;                       // trailing columns per chunk
 constexpr int RG = LU_THREADS / CW;          // row groups of the trailing update
-constexpr double REFINE_TOL = 1.0e-6;        // last relative correction that counts as converged
-
-template <typename T> struct Pb;
-template <> struct Pb<float> { static constexpr int v = 32; };
-template <> struct Pb<double> { static constexpr int v = 16; };
+constexpr int PB = 16;                       // panel columns
 
 // logical index -> index in eps with the head moved last
 __device__ __forceinline__ int head_last(int i, int n, int h) { return i == n - 1 ? h : (i < h ? i : i + 1); }
@@ -66,20 +56,17 @@ template <typename T> __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(LU_THREADS) k_lu_head(BatchSolveArgs a, int nmax, int want_x) {
-    using C = cplx<T>;
-    constexpr int PB = Pb<T>::v;
+__global__ void __launch_bounds__(LU_THREADS) k_lu_head(BatchSolveArgs a, int nmax) {
+    using T = double;
+    using C = double2;
     extern __shared__ __align__(16) unsigned char sm[];
     C* P = reinterpret_cast<C*>(sm);                  // [nmax][PB] panel, logical row order
     C* Li = P + (size_t)nmax * PB;                    // [PB][PB] L11^-1 (then U blocks)
     C* As = Li + PB * PB;                             // [PB][CW] A12 chunk
     C* Ub = As + PB * CW;                             // [PB][CW] U12 chunk
-    C* xs = Ub + PB * CW;                             // [nmax] solution
-    int* rmap = reinterpret_cast<int*>(xs + nmax);    // [nmax]
+    int* rmap = reinterpret_cast<int*>(Ub + PB * CW); // [nmax]
     __shared__ T red_v[NWARP];
     __shared__ int red_i[NWARP];
-    __shared__ C sblk[PB];
     __shared__ int s_p, s_bad;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -247,68 +234,11 @@ __global__ void __launch_bounds__(LU_THREADS) k_lu_head(BatchSolveArgs a, int nm
             __syncthreads();
             continue;
         }
-        if (!want_x) {
-            if (threadIdx.x == 0) {
-                const C* rowp = M + (size_t)rmap[n - 1] * ld;
-                const C xl = cmul(rowp[n], cinv(rowp[n - 1]));
-                a.flags[id] = 0;
-                a.out[id] = -(double)xl.y;
-                a.out[a.ninst + id] = Lno;
-                a.out[2 * a.ninst + id] = 0.0;
-            }
-            __syncthreads();
-            continue;
-        }
-        // back substitution U x = y, PB rows at a time from the bottom
-        for (int bk = ((n - 1) / PB) * PB; bk >= 0; bk -= PB) {
-            const int kb = min(PB, n - bk);
-            for (int i = warp; i < kb; i += NWARP) {
-                const C* rowp = M + (size_t)rmap[bk + i] * ld;
-                T sx = 0, sy = 0;
-                for (int j = bk + kb + lane; j < n; j += 32) {
-                    const C u = rowp[j], xv = xs[j];
-                    sx = fma(u.x, xv.x, fma(-u.y, xv.y, sx));
-                    sy = fma(u.x, xv.y, fma(u.y, xv.x, sy));
-                }
-                sx = warp_sum(sx);
-                sy = warp_sum(sy);
-                if (lane == 0) {
-                    const C y = rowp[n];
-                    C s;
-                    s.x = y.x - sx;
-                    s.y = y.y - sy;
-                    sblk[i] = s;
-                }
-            }
-            for (int e = threadIdx.x; e < kb * kb; e += LU_THREADS) {
-                const int i = e / kb, j = e - i * kb;
-                Li[i * PB + j] = M[(size_t)rmap[bk + i] * ld + bk + j];
-            }
-            __syncthreads();
-            if (warp == 0) {
-                // lane i keeps the running right-hand side of row bk + i
-                C s = lane < kb ? sblk[lane] : czero<C>();
-                for (int i = kb - 1; i >= 0; --i) {
-                    C xi = czero<C>();
-                    if (lane == i) xi = cmul(s, cinv(Li[i * PB + i]));
-                    xi.x = __shfl_sync(0xffffffffu, xi.x, i);
-                    xi.y = __shfl_sync(0xffffffffu, xi.y, i);
-                    if (lane < i) cfms(s, Li[lane * PB + i], xi);
-                    if (lane == i) s = xi;
-                }
-                if (lane < kb) xs[bk + lane] = s;
-            }
-            __syncthreads();
-        }
-        double2* xg = a.x + in.vec_off;
-        int* rg = a.rowmap + in.vec_off;
-        for (int i = threadIdx.x; i < n; i += LU_THREADS) {
-            xg[i] = make_double2((double)xs[i].x, (double)xs[i].y);
-            rg[i] = rmap[i];
-        }
         if (threadIdx.x == 0) {
+            const C* rowp = M + (size_t)rmap[n - 1] * ld;
+            const C xl = cmul(rowp[n], cinv(rowp[n - 1]));
             a.flags[id] = 0;
-            a.out[id] = -(double)xs[n - 1].y;
+            a.out[id] = -(double)xl.y;
             a.out[a.ninst + id] = Lno;
             a.out[2 * a.ninst + id] = 0.0;
         }
@@ -341,166 +271,23 @@ __global__ void __launch_bounds__(256) k_resid(BatchSolveArgs a, const int2* tas
     }
 }
 
-// d = A'^-1 r with the stored FP32 factors; x += d
-__global__ void __launch_bounds__(LU_THREADS) k_lu_correct(BatchSolveArgs a, int nmax, int last) {
-    using C = float2;
-    constexpr int PB = Pb<float>::v;
-    extern __shared__ __align__(16) unsigned char sm[];
-    C* b = reinterpret_cast<C*>(sm);                  // [nmax] right-hand side, stored-row order
-    C* d = b + nmax;                                  // [nmax] forward then backward solution, logical order
-    C* Lt = d + nmax;                                 // [PB][PB] diagonal block
-    int* rmap = reinterpret_cast<int*>(Lt + PB * PB); // [nmax]
-    __shared__ C sblk[PB];
-    __shared__ float s_red[2][NWARP];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
-    for (int ii = a.cta_off[blockIdx.x]; ii < a.cta_off[blockIdx.x + 1]; ++ii) {
-        const int id = a.cta_ids[ii];
-        if (a.flags[id] == 1) continue;
-        const BatchInst in = a.inst[id];
-        const int n = in.ng, ld = n + 1;
-        const C* M = reinterpret_cast<const C*>(a.work) + in.work_off;
-        for (int i = threadIdx.x; i < n; i += LU_THREADS) {
-            const double2 r = a.r[in.vec_off + i];
-            b[i] = make_float2((float)r.x, (float)r.y);
-            rmap[i] = a.rowmap[in.vec_off + i];
-        }
-        __syncthreads();
-        // forward: L y = P b, one panel of PB columns at a time
-        for (int k0 = 0; k0 < n; k0 += PB) {
-            const int kb = min(PB, n - k0);
-            for (int e = threadIdx.x; e < kb * kb; e += LU_THREADS) {
-                const int i = e / kb, l = e - i * kb;
-                Lt[i * PB + l] = M[(size_t)rmap[k0 + i] * ld + k0 + l];
-            }
-            __syncthreads();
-            if (warp == 0) {
-                C s = lane < kb ? b[rmap[k0 + lane]] : czero<C>();
-                for (int l = 0; l < kb; ++l) {
-                    C yl;
-                    yl.x = __shfl_sync(0xffffffffu, s.x, l);
-                    yl.y = __shfl_sync(0xffffffffu, s.y, l);
-                    if (lane > l && lane < kb) cfms(s, Lt[lane * PB + l], yl);
-                }
-                if (lane < kb) d[k0 + lane] = s;
-            }
-            __syncthreads();
-            for (int r = k0 + kb + threadIdx.x; r < n; r += LU_THREADS) {
-                const C* rowp = M + (size_t)rmap[r] * ld + k0;
-                C s = b[rmap[r]];
-                for (int l = 0; l < kb; ++l) cfms(s, rowp[l], d[k0 + l]);
-                b[rmap[r]] = s;
-            }
-            __syncthreads();
-        }
-        // backward: U d = y
-        for (int bk = ((n - 1) / PB) * PB; bk >= 0; bk -= PB) {
-            const int kb = min(PB, n - bk);
-            for (int i = warp; i < kb; i += NWARP) {
-                const C* rowp = M + (size_t)rmap[bk + i] * ld;
-                float sx = 0.f, sy = 0.f;
-                for (int j = bk + kb + lane; j < n; j += 32) {
-                    const C u = rowp[j], xv = d[j];
-                    sx = fmaf(u.x, xv.x, fmaf(-u.y, xv.y, sx));
-                    sy = fmaf(u.x, xv.y, fmaf(u.y, xv.x, sy));
-                }
-                sx = warp_sum(sx);
-                sy = warp_sum(sy);
-                if (lane == 0) sblk[i] = make_float2(d[bk + i].x - sx, d[bk + i].y - sy);
-            }
-            for (int e = threadIdx.x; e < kb * kb; e += LU_THREADS) {
-                const int i = e / kb, j = e - i * kb;
-                Lt[i * PB + j] = M[(size_t)rmap[bk + i] * ld + bk + j];
-            }
-            __syncthreads();
-            if (warp == 0) {
-                C s = lane < kb ? sblk[lane] : czero<C>();
-                for (int i = kb - 1; i >= 0; --i) {
-                    C xi = czero<C>();
-                    if (lane == i) xi = cmul(s, cinv(Lt[i * PB + i]));
-                    xi.x = __shfl_sync(0xffffffffu, xi.x, i);
-                    xi.y = __shfl_sync(0xffffffffu, xi.y, i);
-                    if (lane < i) cfms(s, Lt[lane * PB + i], xi);
-                    if (lane == i) s = xi;
-                }
-                if (lane < kb) d[bk + lane] = s;
-            }
-            __syncthreads();
-        }
-        // x += d; relative size of the correction
-        double2* xg = a.x + in.vec_off;
-        float dmax = 0.f, xmax = 0.f;
-        for (int i = threadIdx.x; i < n; i += LU_THREADS) {
-            double2 xv = xg[i];
-            xv.x += (double)d[i].x;
-            xv.y += (double)d[i].y;
-            xg[i] = xv;
-            dmax = fmaxf(dmax, hypotf(d[i].x, d[i].y));
-            xmax = fmaxf(xmax, (float)hypot(xv.x, xv.y));
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-            xmax = fmaxf(xmax, __shfl_xor_sync(0xffffffffu, xmax, o));
-        }
-        if (lane == 0) {
-            s_red[0][warp] = dmax;
-            s_red[1][warp] = xmax;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float dm = 0.f, xm = 0.f;
-            for (int w = 0; w < NWARP; ++w) {
-                dm = fmaxf(dm, s_red[0][w]);
-                xm = fmaxf(xm, s_red[1][w]);
-            }
-            const double rel = xm > 0.f ? (double)dm / (double)xm : 0.0;
-            const double2 xl = xg[n - 1];
-            a.out[id] = -xl.y;
-            a.out[2 * a.ninst + id] = rel;
-            if (last) a.flags[id] = (rel > REFINE_TOL || !(rel == rel)) ? 2 : 0;
-        }
-        __syncthreads();
-    }
-}
-
-template <typename T> size_t lu_smem(int nmax) {
-    constexpr int PB = Pb<T>::v;
-    return ((size_t)nmax * PB + PB * PB + 2 * PB * CW + nmax) * sizeof(cplx<T>) + nmax * sizeof(int);
+size_t lu_smem(int nmax) {
+    return ((size_t)nmax * PB + PB * PB + 2 * PB * CW) * sizeof(double2) + nmax * sizeof(int);
 }
 
 }  // namespace
 
-cudaError_t qcx_launch_lu_head(cudaStream_t st, const BatchSolveArgs& a, int grid, int nmax, bool fp64, bool want_x) {
+cudaError_t qcx_launch_lu_head(cudaStream_t st, const BatchSolveArgs& a, int grid, int nmax) {
     if (grid < 1 || nmax < 1) return cudaErrorInvalidValue;
-    if (fp64) {
-        const size_t smem = lu_smem<double>(nmax);
-        cudaError_t e = cudaFuncSetAttribute((const void*)k_lu_head<double>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_lu_head<double><<<grid, LU_THREADS, smem, st>>>(a, nmax, want_x ? 1 : 0);
-    } else {
-        const size_t smem = lu_smem<float>(nmax);
-        cudaError_t e = cudaFuncSetAttribute((const void*)k_lu_head<float>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        k_lu_head<float><<<grid, LU_THREADS, smem, st>>>(a, nmax, want_x ? 1 : 0);
-    }
+    const size_t smem = lu_smem(nmax);
+    const cudaError_t e = cudaFuncSetAttribute((const void*)k_lu_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_lu_head<<<grid, LU_THREADS, smem, st>>>(a, nmax);
     return cudaGetLastError();
 }
 
 cudaError_t qcx_launch_resid(cudaStream_t st, const BatchSolveArgs& a, const int2* tasks, int ntask) {
     if (ntask < 1) return cudaErrorInvalidValue;
     k_resid<<<ntask, 256, 0, st>>>(a, tasks);
-    return cudaGetLastError();
-}
-
-cudaError_t qcx_launch_lu_correct(cudaStream_t st, const BatchSolveArgs& a, int grid, int nmax, int last) {
-    if (grid < 1 || nmax < 1) return cudaErrorInvalidValue;
-    constexpr int PB = Pb<float>::v;
-    const size_t smem = (2 * (size_t)nmax + PB * PB) * sizeof(float2) + nmax * sizeof(int);
-    cudaError_t e =
-        cudaFuncSetAttribute((const void*)k_lu_correct, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_lu_correct<<<grid, LU_THREADS, smem, st>>>(a, nmax, last);
     return cudaGetLastError();
 }

@@ -78,6 +78,17 @@ template <> __device__ __forceinline__ void warp_best<double>(unsigned long long
     key = m;
 }
 
+// The matrices of a call: all of order n, or (inst) a batch of uneven ones with their own offsets.  A panel is pb columns;
+// matrix b has ceil(n_b / pb) of them, and the last update lands in the first of the two buffers.
+struct InvShape {
+    int n, pb;
+    const BatchInst* inst;
+    int b0;                                 // first matrix of the launch
+    __device__ int order(int b) const { return inst ? inst[b].ng : n; }
+    __device__ size_t mat(int b) const { return inst ? (size_t)inst[b].work_off : (size_t)b * n * n; }
+    __device__ size_t vec(int b) const { return inst ? (size_t)inst[b].vec_off : (size_t)b * n; }
+};
+
 // FP64 matrices -> work precision; eps_GG, the loss without local fields, |A|_1 (largest column sum) and the
 // starting row order.  Grid (matrix, 64 columns); 64 columns x 4 row groups per CTA.
 template <typename T>
@@ -116,10 +127,15 @@ __global__ void __launch_bounds__(256) k_inv_load(int n, const double2* A, cplx<
 // eliminates in its rows (row, row + 32 RW, ...) and its group's columns.  M[c][i] gets the eliminated panel in the
 // new row order, perm the exchange (new position -> old position), rows the original row of each position.
 template <typename T>
-__global__ void __launch_bounds__(1024) k_inv_panel(int n, int k0, int nb, int RW, int bc, const cplx<T>* src, cplx<T>* M, int* perm, int* rows,
-                            int* flags) {
+__global__ void __launch_bounds__(1024) k_inv_panel(InvShape sh, int p_, int RW, int bc, const cplx<T>* X, const cplx<T>* B2,
+                                                    cplx<T>* M, int* perm, int* rows, int* flags) {
     using C = cplx<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int b = sh.b0 + blockIdx.x, n = sh.order(b), npan = (n + sh.pb - 1) / sh.pb;
+    if (p_ >= npan || flags[b]) return;
+    const int k0 = p_ * sh.pb, nb = min(sh.pb, n - k0);
+    const C* src = ((npan - p_) & 1 ? B2 : X) + sh.mat(b);
+    const size_t vec = sh.vec(b);
     const int ld = n | 1;
     C* xs = reinterpret_cast<C*>(smem_raw);            // [nb][ld]
     C* prow = xs + (size_t)nb * ld;                     // [nb] scaled pivot row (inverse pivot at its own column)
@@ -127,9 +143,6 @@ __global__ void __launch_bounds__(1024) k_inv_panel(int n, int k0, int nb, int R
     int* wrow = reinterpret_cast<int*>(wkey + 32);      // [32]
     int* pos = wrow + 32;                               // [n] position -> row of src
     int* ipos = pos + n;                                // [n] its inverse
-    const int b = blockIdx.x;
-    if (flags[b]) return;
-    src += (size_t)b * n * n;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rw = warp % RW, grp = warp / RW;
     const int stride = 32 * RW;
@@ -224,35 +237,36 @@ __global__ void __launch_bounds__(1024) k_inv_panel(int n, int k0, int nb, int R
         if (threadIdx.x == 0) flags[b] = 1;
         return;
     }
-    M += (size_t)b * nb * n;
+    M += vec * sh.pb;
     for (int c = 0; c < nb; ++c)
         for (int i = threadIdx.x; i < n; i += blockDim.x) M[(size_t)c * n + i] = xs[(size_t)c * ld + pos[i]];
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        perm[(size_t)b * n + i] = pos[i];
-        ipos[i] = rows[(size_t)b * n + pos[i]];
+        perm[vec + i] = pos[i];
+        ipos[i] = rows[vec + pos[i]];
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < n; i += blockDim.x) rows[(size_t)b * n + i] = ipos[i];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) rows[vec + i] = ipos[i];
 }
 
 // The other columns (see above).  Grid (column tile, row tile, matrix); thread (tx, ty) holds rows ty 4 .. + 3 and
 // columns tx + 16 u of a 64 x 64 tile, the panel's multipliers and pivot rows staged once in shared memory.
 template <typename T>
-__global__ void __launch_bounds__(256) k_inv_update(int n, int k0, int nb, const cplx<T>* src, cplx<T>* dst,
-                                                    const cplx<T>* M, const int* perm, const int* rows, int last,
-                                                    const int* flags) {
+__global__ void __launch_bounds__(256) k_inv_update(InvShape sh, int p, cplx<T>* X, cplx<T>* B2, const cplx<T>* M,
+                                                    const int* perm, const int* rows, const int* flags) {
     using C = cplx<T>;
     constexpr int PB = InvCfg<T>::PB;
     __shared__ __align__(16) C ms[PB][UPD];
     __shared__ __align__(16) C rs[PB][UPD];
-    const int b = blockIdx.z;
-    if (flags[b]) return;
-    src += (size_t)b * n * n;
-    dst += (size_t)b * n * n;
-    M += (size_t)b * nb * n;
-    perm += (size_t)b * n;
-    rows += (size_t)b * n;
+    const int b = sh.b0 + blockIdx.z, n = sh.order(b), npan = (n + sh.pb - 1) / sh.pb;
     const int i0 = blockIdx.y * UPD, j0 = blockIdx.x * UPD;
+    if (p >= npan || i0 >= n || j0 >= n || flags[b]) return;
+    const int k0 = p * sh.pb, nb = min(sh.pb, n - k0);
+    const bool from_b = (npan - p) & 1, last = p + 1 == npan;
+    const C* src = (from_b ? B2 : X) + sh.mat(b);
+    C* dst = (from_b ? X : B2) + sh.mat(b);
+    M += sh.vec(b) * sh.pb;
+    perm += sh.vec(b);
+    rows += sh.vec(b);
     for (int e = threadIdx.x; e < nb * UPD; e += 256) {
         const int c = e / UPD, x = e % UPD;
         ms[c][x] = i0 + x < n ? M[(size_t)c * n + i0 + x] : mk<T>(0, 0);
@@ -520,6 +534,36 @@ __global__ void __launch_bounds__(256) k_loss_quadform(int n, const float2* Xall
 
 }  // namespace
 
+// All panels of nmat matrices of order at most n.
+template <typename T>
+static void eliminate(cudaStream_t st, InvShape sh, int n, int nmat, int npan, size_t smem, cplx<T>* X, cplx<T>* B2, cplx<T>* M,
+                      int* perm, int* rows, int* flags) {
+    const int RW = std::min((n + 31) / 32, 32);
+    int groups = 1;
+    while (groups * 2 * RW <= 16 && groups * 2 <= sh.pb) groups *= 2;
+    const int bc = (sh.pb + groups - 1) / groups;
+    for (sh.b0 = 0; sh.b0 < nmat; sh.b0 += 32768) {            // grid limit of the tiles' third dimension
+        const int m = std::min(32768, nmat - sh.b0);
+        const dim3 tiles((n + UPD - 1) / UPD, (n + UPD - 1) / UPD, m);
+        for (int p = 0; p < npan; ++p) {
+            k_inv_panel<T><<<m, 32 * RW * groups, smem, st>>>(sh, p, RW, bc, X, B2, M, perm, rows, flags);
+            k_inv_update<T><<<tiles, 256, 0, st>>>(sh, p, X, B2, M, perm, rows, flags);
+        }
+    }
+}
+
+// Widest panel of order-n matrices that fits shared memory, and its bytes.
+template <typename T> static int panel_width(int n, size_t* smem) {
+    int pb = std::min(InvCfg<T>::PB, n);
+    auto bytes = [&](int w) {
+        return ((size_t)w * (n | 1) + w) * sizeof(cplx<T>) + 32 * (sizeof(unsigned long long) + sizeof(int)) +
+               2 * (size_t)n * sizeof(int);
+    };
+    while (pb > 1 && bytes(pb) > PANEL_SMEM) pb >>= 1;
+    *smem = bytes(pb);
+    return pb;
+}
+
 // Inverse of nmat matrices of order n into X; B2 holds as many for the out-of-place updates, aux the panels and row
 // orders.  norms (mixed path): |A|_1 of every matrix, then |X|_1.
 template <typename T>
@@ -527,34 +571,17 @@ static cudaError_t invert_batch(cudaStream_t st, int n, int nmat, const double2*
                                 double* anorm, double* xnorm, double2* eps_diag, double* L, double* L_nolfe,
                                 double2* diag_inv, int* flags) {
     using C = cplx<T>;
-    int pb = InvCfg<T>::PB;
-    auto smem_of = [&](int w) {
-        return ((size_t)w * (n | 1) + w) * sizeof(C) + 32 * (sizeof(unsigned long long) + sizeof(int)) + 2 * (size_t)n * sizeof(int);
-    };
-    while (pb > 1 && smem_of(pb) > PANEL_SMEM) pb >>= 1;
-    pb = std::min(pb, n);
+    size_t smem = 0;
+    const int pb = panel_width<T>(n, &smem);
     C* M = reinterpret_cast<C*>(aux);
     int* perm = reinterpret_cast<int*>(M + (size_t)nmat * pb * n);
     int* rows = perm + (size_t)nmat * n;
-    const size_t smem = smem_of(pb);
     cudaError_t e = cudaFuncSetAttribute((const void*)k_inv_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int npan = (n + pb - 1) / pb;
-    C* cur = npan & 1 ? B2 : X;                         // the last update lands in X
-    C* nxt = npan & 1 ? X : B2;
     const dim3 cols(nmat, (n + 63) / 64);
-    k_inv_load<T><<<cols, 256, 0, st>>>(n, A, cur, anorm, eps_diag, L_nolfe, rows, flags);
-    const int RW = std::min((n + 31) / 32, 32);
-    int groups = 1;
-    while (groups * 2 * RW <= 16 && groups * 2 <= pb) groups *= 2;
-    const int bc = (pb + groups - 1) / groups;
-    const dim3 tiles((n + UPD - 1) / UPD, (n + UPD - 1) / UPD, nmat);
-    for (int p = 0; p < npan; ++p) {
-        const int k0 = p * pb, nb = std::min(pb, n - k0);
-        k_inv_panel<T><<<nmat, 32 * RW * groups, smem, st>>>(n, k0, nb, RW, bc, cur, M, perm, rows, flags);
-        k_inv_update<T><<<tiles, 256, 0, st>>>(n, k0, nb, cur, nxt, M, perm, rows, p + 1 == npan, flags);
-        std::swap(cur, nxt);
-    }
+    k_inv_load<T><<<cols, 256, 0, st>>>(n, A, npan & 1 ? B2 : X, anorm, eps_diag, L_nolfe, rows, flags);
+    eliminate<T>(st, InvShape{n, pb, nullptr, 0}, n, nmat, npan, smem, X, B2, M, perm, rows, flags);
     k_inv_finish<T><<<cols, 256, 0, st>>>(n, X, flags, xnorm, diag_inv, L);
     return cudaGetLastError();
 }
@@ -629,6 +656,132 @@ cudaError_t qcx_launch_invert(qcx_ctx* ctx, QSlot& s, qcx_precision prec, double
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+// ------------------------------------------------------------------ uneven batches (mixed path)
+namespace {
+
+// FP64 eps of every instance -> FP32, into the buffer its first panel reads; starting row order.  Grid (instance, 64
+// columns).
+__global__ void __launch_bounds__(256) k_batch_load(InvShape sh, const double2* eps, float2* X, float2* B2, int* rows, int* flags) {
+    const int b = blockIdx.x, n = sh.order(b), tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+    const int j = blockIdx.y * 64 + tx;
+    if (blockIdx.y == 0 && threadIdx.x == 0) flags[b] = 0;
+    if (j >= n) return;
+    const int npan = (n + sh.pb - 1) / sh.pb;
+    float2* dst = (npan & 1 ? B2 : X) + sh.mat(b);
+    const double2* A = eps + sh.inst[b].eps_off;
+    for (int i = ty; i < n; i += 4) {
+        const double2 z = A[(size_t)i * n + j];
+        dst[(size_t)i * n + j] = make_float2((float)z.x, (float)z.y);
+    }
+    if (ty == 0) rows[sh.vec(b) + j] = j;
+}
+
+// index of the solution's component i (the head last) in eps
+__device__ __forceinline__ int head_last(int i, int n, int h) { return i == n - 1 ? h : (i < h ? i : i + 1); }
+
+// x = the inverse's head column (head component last), the heads, and zero heads for singular instances
+__global__ void __launch_bounds__(128) k_batch_x(BatchSolveArgs a, const float2* X) {
+    const int id = blockIdx.x;
+    const BatchInst in = a.inst[id];
+    const int n = in.ng, h = in.head;
+    const bool bad = a.flags[id] != 0;
+    if (!bad)
+        for (int i = threadIdx.x; i < n; i += 128) {
+            const float2 z = X[in.work_off + (size_t)head_last(i, n, h) * n + h];
+            a.x[in.vec_off + i] = make_double2((double)z.x, (double)z.y);
+        }
+    if (threadIdx.x == 0) {
+        const double2 e = a.eps[in.eps_off + (size_t)h * n + h];
+        a.out[id] = bad ? 0.0 : -(double)X[in.work_off + (size_t)h * n + h].y;
+        a.out[a.ninst + id] = e.y / (e.x * e.x + e.y * e.y);
+        a.out[2 * a.ninst + id] = 0.0;
+    }
+}
+
+constexpr double REFINE_TOL = 1.0e-6;        // last relative correction that counts as converged
+
+// x += X r (FP32 products of the FP64 residual); one CTA per instance, a row per warp
+__global__ void __launch_bounds__(512) k_batch_correct(BatchSolveArgs a, const float2* Xall, int last) {
+    __shared__ float red[2][16];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    float2* r = reinterpret_cast<float2*>(smem_raw);       // residual in eps order
+    const int id = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (a.flags[id] == 1) return;
+    const BatchInst in = a.inst[id];
+    const int n = in.ng, h = in.head;
+    const float2* X = Xall + in.work_off;
+    for (int i = threadIdx.x; i < n; i += 512) {
+        const double2 z = a.r[in.vec_off + i];
+        r[head_last(i, n, h)] = make_float2((float)z.x, (float)z.y);
+    }
+    __syncthreads();
+    double2* x = a.x + in.vec_off;
+    float dmax = 0.f, xmax = 0.f;
+    for (int i = warp; i < n; i += 16) {
+        const float2* row = X + (size_t)head_last(i, n, h) * n;
+        float2 d = make_float2(0.f, 0.f);
+        for (int j = lane; j < n; j += 32) cfma(d, row[j], r[j]);
+        for (int o = 16; o > 0; o >>= 1) {
+            d.x += __shfl_xor_sync(0xffffffffu, d.x, o);
+            d.y += __shfl_xor_sync(0xffffffffu, d.y, o);
+        }
+        if (lane == 0) {
+            double2 v = x[i];
+            v.x += (double)d.x;
+            v.y += (double)d.y;
+            x[i] = v;
+            dmax = fmaxf(dmax, hypotf(d.x, d.y));
+            xmax = fmaxf(xmax, (float)hypot(v.x, v.y));
+            if (!(d.x == d.x) || !(d.y == d.y)) dmax = INFINITY;
+        }
+    }
+    if (lane == 0) {
+        red[0][warp] = dmax;
+        red[1][warp] = xmax;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float dm = 0.f, xm = 0.f;
+        for (int w = 0; w < 16; ++w) {
+            dm = fmaxf(dm, red[0][w]);
+            xm = fmaxf(xm, red[1][w]);
+        }
+        const double rel = xm > 0.f ? (double)dm / (double)xm : 0.0;
+        a.out[id] = -x[n - 1].y;
+        a.out[2 * a.ninst + id] = rel;
+        if (last) a.flags[id] = (rel > REFINE_TOL || !(rel == rel)) ? 2 : 0;
+    }
+}
+
+}  // namespace
+
+size_t qcx_batch_inverse_aux(long long total_n, int nmax) {
+    size_t smem;
+    return (size_t)total_n * ((size_t)panel_width<float>(nmax, &smem) * sizeof(float2) + 2 * sizeof(int));
+}
+
+cudaError_t qcx_launch_batch_inverse(cudaStream_t st, const BatchSolveArgs& a, float2* B2, void* aux, long long total_n, int nmax) {
+    if (nmax < 1 || nmax > 1024 * PANEL_ROWS) return cudaErrorInvalidValue;
+    size_t smem = 0;
+    const int pb = panel_width<float>(nmax, &smem);
+    float2* M = reinterpret_cast<float2*>(aux);
+    int* perm = reinterpret_cast<int*>(M + (size_t)total_n * pb);
+    int* rows = perm + total_n;
+    cudaError_t e = cudaFuncSetAttribute((const void*)k_inv_panel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const InvShape sh{nmax, pb, a.inst, 0};
+    float2* X = reinterpret_cast<float2*>(a.work);
+    k_batch_load<<<dim3(a.ninst, (nmax + 63) / 64), 256, 0, st>>>(sh, a.eps, X, B2, rows, a.flags);
+    eliminate<float>(st, sh, nmax, a.ninst, (nmax + pb - 1) / pb, smem, X, B2, M, perm, rows, a.flags);
+    k_batch_x<<<a.ninst, 128, 0, st>>>(a, X);
+    return cudaGetLastError();
+}
+
+cudaError_t qcx_launch_batch_correct(cudaStream_t st, const BatchSolveArgs& a, int nmax, int last) {
+    k_batch_correct<<<a.ninst, 512, sizeof(float2) * nmax, st>>>(a, reinterpret_cast<const float2*>(a.work), last);
+    return cudaGetLastError();
 }
 
 extern "C" qcx_status qcx_set_refine_threshold(qcx_ctx* ctx, double kappa1) {

@@ -339,17 +339,19 @@ struct BatchSolveArgs {
     const int* cta_off;        // [grid + 1] instance lists per CTA (CSR)
     const int* cta_ids;
     const double2* eps;        // FP64 eps of every instance
-    void* work;                // LU factors ([ng][ng+1] per instance, FP32 or FP64 complex)
-    int* rowmap;               // [sum ng] pivot order: logical row -> stored row
+    void* work;                // FP64: LU factors ([ng][ng+1] per instance); mixed: FP32 inverses [ng][ng] at the same offsets
     double2* x;                // [sum ng] solution of A' x = e_last (refined in place)
     double2* r;                // [sum ng] FP64 residual
     double* out;               // [3][ninst]: L_LFE head, L_noLFE head, last relative correction
     int* flags;                // [ninst]: 0 ok, 1 zero pivot, 2 refinement not converged
     int ninst;
 };
-cudaError_t qcx_launch_lu_head(cudaStream_t st, const BatchSolveArgs& a, int grid, int nmax, bool fp64, bool want_x);
+cudaError_t qcx_launch_lu_head(cudaStream_t st, const BatchSolveArgs& a, int grid, int nmax);    // FP64
 cudaError_t qcx_launch_resid(cudaStream_t st, const BatchSolveArgs& a, const int2* tasks, int ntask);
-cudaError_t qcx_launch_lu_correct(cudaStream_t st, const BatchSolveArgs& a, int grid, int nmax, int last);
+// mixed (invert.cu): FP32 inverses into a.work with B2 as second copy, x and the heads; x += X r
+size_t qcx_batch_inverse_aux(long long total_n, int nmax);
+cudaError_t qcx_launch_batch_inverse(cudaStream_t st, const BatchSolveArgs& a, float2* B2, void* aux, long long total_n, int nmax);
+cudaError_t qcx_launch_batch_correct(cudaStream_t st, const BatchSolveArgs& a, int nmax, int last);
 
 // inverse + loss (invert.cu)
 cudaError_t qcx_launch_invert(qcx_ctx* ctx, QSlot& s, qcx_precision prec, double* d_loss_out);
