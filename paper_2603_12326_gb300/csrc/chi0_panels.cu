@@ -768,17 +768,18 @@ __global__ void __launch_bounds__(256) k_pn_dyson(int ng, int nw, int nz, const 
                 c.y += v.y;
             }
         }
-        c = make_double2(pref * c.x, pref * c.y);
         t[j][threadIdx.x] = c;
-        if (chi_out) chi_out[o + (size_t)G * ng + H] = c;
+        if (chi_out) chi_out[o + (size_t)G * ng + H] = make_double2(pref * c.x, pref * c.y);
     }
     __syncthreads();
+    // three FP64 operations per element: the pipe, not memory, is what this kernel could be bound by
+    const double vG = G0 + threadIdx.x < ng ? pref * vs[G0 + threadIdx.x] : 0.0;
     for (int j = threadIdx.y; j < 32; j += 8) {
         const int H = H0 + j, G = G0 + threadIdx.x;
         if (G >= ng || H >= ng) continue;
         const double2 c = t[threadIdx.x][j];
-        const double vv = vs[G] * vs[H];
-        eps[o + (size_t)H * ng + G] = make_double2((G == H ? 1.0 : 0.0) - vv * c.x, -vv * c.y);
+        const double vv = vG * vs[H];
+        eps[o + (size_t)H * ng + G] = make_double2(fma(-vv, c.x, G == H ? 1.0 : 0.0), -vv * c.y);
     }
 }
 

@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(pdf_maxt<NV>()) k_pair_density_fused(PDArgs<fl
 // of a (k, pair) are ~2 KB for all G, so a CTA takes as many G as it can (up to 192) and few groups a: with 16 G and all
 // groups a, each CTA streamed 1.2 MB of tables from L2 (7.4 GB a call at N_G = 181) and L2 was the bound.  Now bound by
 // the FP32 (FP64) pipe: per (k, G, pair) 100 multiply-adds per character for the block and 64 per four bands for Y.
-// k_pd_rho: rho = C_kq^H Y, 32 conduction bands x 64 G per CTA, 8 G per thread.
+// k_pd_rho: rho = C_kq^H Y, 32 conduction bands x 64 G per CTA (16 x 128, 8 x 256), 8 G per thread.
 // Measured (one q: 512 k x 181 G, 24 groups, 4 x 32 bands): FP32 2.54 at first, 1.70 as one kernel, 1.46 ms now; FP64,
 // which formed the lattice sums per (k, G) before, 252 -> 51 ms.
 template <typename T, int NV> constexpr int pdt_threads() { return sizeof(T) == 8 ? 192 : pdf_maxt<NV>(); }
@@ -587,16 +587,17 @@ __global__ void __launch_bounds__(pdt_threads<T, NV>()) k_pd_y(PDArgs<T> a, int 
     }
 }
 
-constexpr int PR_C = 32, PR_G = 64;
-template <typename T>
+// PR_C: bands per tile (8, 16 or 32 by nc, so that few lanes idle), 2048 / PR_C G
+template <typename T, int PR_C>
 __global__ void __launch_bounds__(256) k_pd_rho(PDArgs<T> a, int kb, int nvp, const cplx<T>* Y) {
     using C = cplx<T>;
-    constexpr int KC = sizeof(T) == 4 ? 48 : 24;   // basis functions staged at a time
+    constexpr int PR_G = 2048 / PR_C;
+    constexpr int KC = (sizeof(T) == 4 ? 48 : 24) * 64 / PR_G;   // basis functions staged at a time
     __shared__ __align__(16) C Ys[KC][PR_G];
     __shared__ C Cs[KC][PR_C];
     const int nvb = a.nv, k = kb + blockIdx.z;
     const int v = blockIdx.y % nvb, c0 = blockIdx.y / nvb * PR_C, g0 = blockIdx.x * PR_G;
-    const int cl = threadIdx.x & 31, gl = threadIdx.x >> 5;    // band, 8 G
+    const int cl = threadIdx.x % PR_C, gl = threadIdx.x / PR_C;    // band, 8 G
     const C* Yk = Y + ((size_t)blockIdx.z * a.nb * nvp + v) * a.ng;
     const C* Ckq = a.Ckq + (size_t)k * a.nb * a.nc;
     C acc[8];
@@ -801,6 +802,11 @@ size_t pd_y_per_k(int nb, int nv, int ng, size_t elem) {
     return (size_t)nb * ((nv + w - 1) / w * w) * ng * elem;
 }
 
+template <typename T, int PR_C> void launch_rho(qcx_ctx* ctx, PDArgs<T>& a, int k0, int m, int nvp, const cplx<T>* Y) {
+    constexpr int PR_G = 2048 / PR_C;
+    k_pd_rho<T, PR_C><<<dim3((a.ng + PR_G - 1) / PR_G, a.nv * ((a.nc + PR_C - 1) / PR_C), m), 256, 0, ctx->stream>>>(a, k0, nvp, Y);
+}
+
 // The two table kernels over chunks of k; cudaErrorInvalidConfiguration when the basis has more groups than a CTA or C_k
 // does not fit shared memory (the caller then takes the kernels without tables).
 template <typename T, int NCH, int NV> cudaError_t launch_tab(qcx_ctx* ctx, PDArgs<T>& a, const PdTab& t) {
@@ -816,7 +822,12 @@ template <typename T, int NCH, int NV> cudaError_t launch_tab(qcx_ctx* ctx, PDAr
     for (int k0 = 0; k0 < a.nk; k0 += kc) {
         const int m = std::min(kc, a.nk - k0);
         k_pd_y<T, NCH, NV><<<dim3(m, nch, (a.ngrp + ga_per - 1) / ga_per), gc * ga_per, smem, ctx->stream>>>(a, k0, gc, ga_per, Y);
-        k_pd_rho<T><<<dim3((a.ng + PR_G - 1) / PR_G, a.nv * ((a.nc + PR_C - 1) / PR_C), m), 256, 0, ctx->stream>>>(a, k0, nvp, Y);
+        if (a.nc <= 8)
+            launch_rho<T, 8>(ctx, a, k0, m, nvp, Y);
+        else if (a.nc <= 16)
+            launch_rho<T, 16>(ctx, a, k0, m, nvp, Y);
+        else
+            launch_rho<T, 32>(ctx, a, k0, m, nvp, Y);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
