@@ -103,6 +103,24 @@ cudaError_t qcx_copy_out(qcx_ctx* ctx, void* dst, const void* src_dev, size_t by
     return cudaStreamSynchronize(ctx->stream);
 }
 
+cudaError_t qcx_copy_out_all(qcx_ctx* ctx, const char* src, size_t total, const CopyOut* out, int n) {
+    constexpr size_t PIN_MAX = 1 << 20;
+    bool host = total <= PIN_MAX;
+    for (int i = 0; i < n; ++i) host = host && !qcx_is_device_ptr(out[i].dst);
+    cudaError_t e;
+    if (host && ctx->pin.ensure(PIN_MAX) == cudaSuccess) {
+        if ((e = cudaMemcpyAsync(ctx->pin.p, src, total, cudaMemcpyDeviceToHost, ctx->stream)) != cudaSuccess) return e;
+        if ((e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) return e;
+        for (int i = 0; i < n; ++i)
+            if (out[i].dst) std::memcpy(out[i].dst, static_cast<const char*>(ctx->pin.p) + out[i].offset, out[i].bytes);
+        return cudaSuccess;
+    }
+    cudaGetLastError();
+    for (int i = 0; i < n; ++i)
+        if ((e = qcx_copy_out(ctx, out[i].dst, src + out[i].offset, out[i].bytes)) != cudaSuccess) return e;
+    return cudaStreamSynchronize(ctx->stream);
+}
+
 // ===================================================================== ABI
 extern "C" {
 
@@ -273,6 +291,7 @@ qcx_status qcx_set_states(qcx_ctx* ctx, int nk, const double* kpts, int nv, cons
     CUDA_OR_FAIL(cudaGetLastError(), "convert states");
     ++ctx->gen;
     ctx->kpts_h = kh;
+    ctx->kcls = qcx_axis_classes(kh.data(), nk);
     ctx->nk = nk;
     ctx->nv = nv;
     ctx->nc = nc;
@@ -418,6 +437,7 @@ qcx_status qcx_chi0(qcx_ctx* ctx, int iq, int nw, const double* w, double eta, q
     CUDA_OR_FAIL(fetch(ctx, wh, w, nw), "chi0 w");
     if (!finite_all(wh.data(), nw)) return ctx->fail(QCX_ERR_ARG, "chi0: non-finite frequency");
     s.nw = nw;
+    s.wh = wh;
     s.eta = eta;
     s.have_eps = false;
     if (ctx->loss[iq]) ctx->loss[iq]->valid = false;     // the tables of iq belong to the previous chi0
@@ -447,8 +467,8 @@ qcx_status qcx_chi0(qcx_ctx* ctx, int iq, int nw, const double* w, double eta, q
     }
     if (tensor) {
         int st = 0;
-        CUDA_OR_FAIL(cudaMemcpyAsync(&st, s.flags.p, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), "status");
-        CUDA_OR_FAIL(cudaStreamSynchronize(ctx->stream), "sync");
+        const CopyOut out = {&st, 0, sizeof(int)};
+        CUDA_OR_FAIL(qcx_copy_out_all(ctx, s.flags.as<char>(), sizeof(int), &out, 1), "status");
         if (st) return ctx->fail(QCX_ERR_TIMEOUT, "chi0: a pipeline wait in the tensor-core kernel gave up");
     }
     if (out_chi0 && chi != reinterpret_cast<double2*>(out_chi0))
@@ -493,16 +513,14 @@ qcx_status qcx_invert_eps(qcx_ctx* ctx, int iq, qcx_precision prec, qcx_c64* out
     CUDA_OR_FAIL(cudaMemcpyAsync(lt->kvec.p, s.kappa.p, 3 * sizeof(double) * ng, cudaMemcpyDeviceToDevice,
                                  ctx->stream),
                  "copy q+G");
-    lt->w.resize(nw);
-    CUDA_OR_FAIL(cudaMemcpyAsync(lt->w.data(), s.w.p, nw * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream), "w");
+    lt->w = s.wh;
     lt->valid = true;
-    std::vector<int> flags(nw);
-    CUDA_OR_FAIL(cudaMemcpyAsync(flags.data(), s.flags.p, nw * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream),
-                 "flags");
     CUDA_OR_FAIL(qcx_copy_out(ctx, out_diag_inv, s.diag_inv.p, (size_t)nw * ng * sizeof(double2)), "copy out");
     CUDA_OR_FAIL(qcx_copy_out(ctx, out_eps_diag, s.eps_diag.p, (size_t)nw * ng * sizeof(double2)), "copy out");
     CUDA_OR_FAIL(qcx_copy_out(ctx, out_resid, s.resid.p, nw * sizeof(double)), "copy out");
-    CUDA_OR_FAIL(cudaStreamSynchronize(ctx->stream), "sync");
+    std::vector<int> flags(nw);
+    const CopyOut fo = {flags.data(), 0, nw * sizeof(int)};
+    CUDA_OR_FAIL(qcx_copy_out_all(ctx, s.flags.as<char>(), nw * sizeof(int), &fo, 1), "flags");
     int bad = 0;
     for (int f : flags) bad += f != 0;
     if (bad) return ctx->fail(QCX_ERR_SINGULAR, "invert: " + std::to_string(bad) + " singular block(s)");
@@ -576,20 +594,20 @@ qcx_status qcx_bin_loss(qcx_ctx* ctx, int nsel, const int* iq_list, int which, i
     const size_t total = off_c + nbin * sizeof(double);
     CUDA_OR_FAIL(ctx->scratch2.ensure(total), "alloc");
     char* base = ctx->scratch2.as<char>();
-    CUDA_OR_FAIL(cudaMemcpyAsync(base + off_L, Lp.data(), nsel * sizeof(void*), cudaMemcpyHostToDevice, ctx->stream), "copy");
-    CUDA_OR_FAIL(cudaMemcpyAsync(base + off_Q, Qp.data(), nsel * sizeof(void*), cudaMemcpyHostToDevice, ctx->stream), "copy");
-    CUDA_OR_FAIL(cudaMemcpyAsync(base + off_n, ngs.data(), nsel * sizeof(int), cudaMemcpyHostToDevice, ctx->stream), "copy");
-    CUDA_OR_FAIL(cudaMemcpyAsync(base + off_e, ed.data(), (nbin + 1) * sizeof(double), cudaMemcpyHostToDevice, ctx->stream),
-                 "copy");
+    std::vector<char> in(off_o);
+    std::memcpy(in.data() + off_L, Lp.data(), nsel * sizeof(void*));
+    std::memcpy(in.data() + off_Q, Qp.data(), nsel * sizeof(void*));
+    std::memcpy(in.data() + off_n, ngs.data(), nsel * sizeof(int));
+    std::memcpy(in.data() + off_e, ed.data(), (nbin + 1) * sizeof(double));
+    CUDA_OR_FAIL(cudaMemcpyAsync(base, in.data(), in.size(), cudaMemcpyHostToDevice, ctx->stream), "copy");
     CUDA_OR_FAIL(qcx_launch_bin(ctx, nsel, reinterpret_cast<const double* const*>(base + off_L),
                                 reinterpret_cast<const double* const*>(base + off_Q),
                                 reinterpret_cast<const int*>(base + off_n), nw, which, nbin,
                                 reinterpret_cast<const double*>(base + off_e), reinterpret_cast<double*>(base + off_o),
                                 reinterpret_cast<double*>(base + off_c)),
                  "bin kernel");
-    CUDA_OR_FAIL(qcx_copy_out(ctx, out_L, base + off_o, (size_t)nbin * nw * sizeof(double)), "copy out");
-    if (out_count) CUDA_OR_FAIL(qcx_copy_out(ctx, out_count, base + off_c, nbin * sizeof(double)), "copy out");
-    CUDA_OR_FAIL(cudaStreamSynchronize(ctx->stream), "sync");
+    const CopyOut out[2] = {{out_L, 0, (size_t)nbin * nw * sizeof(double)}, {out_count, off_c - off_o, nbin * sizeof(double)}};
+    CUDA_OR_FAIL(qcx_copy_out_all(ctx, base + off_o, total - off_o, out, 2), "copy out");
     return QCX_OK;
 }
 
@@ -609,16 +627,24 @@ qcx_status qcx_rate(qcx_ctx* ctx, int nqbin, const double* qbin, int nw, const d
     const size_t total = oQ + (nQ > 0 ? nQ : 1) * sizeof(double);
     CUDA_OR_FAIL(ctx->scratch2.ensure(total), "alloc");
     char* base = ctx->scratch2.as<char>();
-    CUDA_OR_FAIL(qcx_copy_in(ctx, base + oq, qbin, nqbin * sizeof(double)), "copy");
-    CUDA_OR_FAIL(qcx_copy_in(ctx, base + ow, w, nw * sizeof(double)), "copy");
-    CUDA_OR_FAIL(qcx_copy_in(ctx, base + oL, L, (size_t)nqbin * nw * sizeof(double)), "copy");
+    std::vector<char> in;
+    if (!qcx_is_device_ptr(qbin) && !qcx_is_device_ptr(w) && !qcx_is_device_ptr(L)) {
+        in.resize(oR);
+        std::memcpy(in.data() + oq, qbin, nqbin * sizeof(double));
+        std::memcpy(in.data() + ow, w, nw * sizeof(double));
+        std::memcpy(in.data() + oL, L, (size_t)nqbin * nw * sizeof(double));
+        CUDA_OR_FAIL(cudaMemcpyAsync(base, in.data(), in.size(), cudaMemcpyHostToDevice, ctx->stream), "copy");
+    } else {
+        CUDA_OR_FAIL(qcx_copy_in(ctx, base + oq, qbin, nqbin * sizeof(double)), "copy");
+        CUDA_OR_FAIL(qcx_copy_in(ctx, base + ow, w, nw * sizeof(double)), "copy");
+        CUDA_OR_FAIL(qcx_copy_in(ctx, base + oL, L, (size_t)nqbin * nw * sizeof(double)), "copy");
+    }
     CUDA_OR_FAIL(qcx_launch_rate(ctx, nqbin, reinterpret_cast<double*>(base + oq), nw,
                                  reinterpret_cast<double*>(base + ow), reinterpret_cast<double*>(base + oL), p,
                                  reinterpret_cast<double*>(base + oR), nQ, reinterpret_cast<double*>(base + oQ)),
                  "rate kernel");
-    CUDA_OR_FAIL(qcx_copy_out(ctx, out_dRdw, base + oR, nw * sizeof(double)), "copy out");
-    if (nQ > 0) CUDA_OR_FAIL(qcx_copy_out(ctx, out_dRQ, base + oQ, nQ * sizeof(double)), "copy out");
-    CUDA_OR_FAIL(cudaStreamSynchronize(ctx->stream), "sync");
+    const CopyOut out[2] = {{out_dRdw, 0, nw * sizeof(double)}, {nQ > 0 ? out_dRQ : nullptr, oQ - oR, (size_t)nQ * sizeof(double)}};
+    CUDA_OR_FAIL(qcx_copy_out_all(ctx, base + oR, total - oR, out, 2), "copy out");
     return QCX_OK;
 }
 

@@ -845,8 +845,9 @@ template <typename T, int NCH> cudaError_t build_table(qcx_ctx* ctx, PDArgs<T>& 
     std::memcpy(ta.charre, a.charre, sizeof(ta.charre));
     std::memcpy(ta.charim, a.charim, sizeof(ta.charim));
     std::memcpy(ta.chars, ctx->chars, sizeof(ta.chars));
-    ta.kval = t.kval.as<double>();
-    ta.qval = t.qval.as<double>();
+    const char* meta = t.meta.as<char>();
+    ta.kval = reinterpret_cast<const double*>(meta);
+    ta.qval = reinterpret_cast<const double*>(meta + t.o_qval);
     for (int x = 0; x < 3; ++x) {
         ta.nkx[x] = a.nkx[x] = t.nkx[x];
         ta.nqx[x] = a.nqx[x] = t.nqx[x];
@@ -856,9 +857,9 @@ template <typename T, int NCH> cudaError_t build_table(qcx_ctx* ctx, PDArgs<T>& 
     for (int x = 0; x < 4; ++x) ta.tbase[x] = a.tbase[x] = t.tbase[x];
     ta.out = t.tab.as<cplx<T>>();
     a.ptab = ta.out;
-    a.kidx = t.kidx.as<int>();
-    a.gidx = t.gidx.as<int>();
-    a.gperm = t.gperm.as<int>();
+    a.kidx = reinterpret_cast<const int*>(meta + t.o_kidx);
+    a.gidx = reinterpret_cast<const int*>(meta + t.o_gidx);
+    a.gperm = reinterpret_cast<const int*>(meta + t.o_gperm);
     k_pd_axis_table<T, NCH><<<(unsigned)((t.tbase[3] + 127) / 128), 128, 0, ctx->stream>>>(ta);
     return cudaGetLastError();
 }
@@ -1071,41 +1072,60 @@ static void axis_classes(const double* v, int n, int x, std::vector<double>& val
     }
 }
 
+AxisClasses qcx_axis_classes(const double* v, int n) {
+    AxisClasses c;
+    c.finite = true;
+    for (int i = 0; i < 3 * n; ++i) c.finite = c.finite && std::isfinite(v[i]);
+    if (!c.finite) return c;
+    c.idx.resize(3 * (size_t)n);
+    for (int x = 0; x < 3; ++x) {
+        c.ofs[x] = (int)c.val.size();
+        axis_classes(v, n, x, c.val, c.idx);
+        c.n[x] = (int)c.val.size() - c.ofs[x];
+    }
+    return c;
+}
+
 // Classes and buffers of the tables for nk k points and ng values of q+G (host arrays); leaves t invalid when the
 // tables would not save work or exceed their memory budget.
-static cudaError_t tab_prepare(qcx_ctx* ctx, PdTab& t, const double* kpts, int nk, const double* kap, int ng,
-                               size_t elem, size_t y_per_k) {
+static cudaError_t tab_prepare(qcx_ctx* ctx, PdTab& t, const AxisClasses& kc, int nk, const double* kap, int ng, size_t elem,
+                               size_t y_per_k) {
     t.valid = false;
-    for (int i = 0; i < 3 * nk; ++i)
-        if (!std::isfinite(kpts[i])) return cudaSuccess;
-    for (int i = 0; i < 3 * ng; ++i)
-        if (!std::isfinite(kap[i])) return cudaSuccess;
+    if (!kc.finite) return cudaSuccess;
+    const AxisClasses gc = qcx_axis_classes(kap, ng);
+    if (!gc.finite) return cudaSuccess;
     const int npair = ctx->ngrp * ctx->ngrp;
-    std::vector<double> kval, qval;
-    std::vector<int> kidx(3 * (size_t)nk), gidx(3 * (size_t)ng);
     long long cells = 0;
     for (int x = 0; x < 3; ++x) {
-        t.kofs[x] = (int)kval.size();
-        t.qofs[x] = (int)qval.size();
-        axis_classes(kpts, nk, x, kval, kidx);
-        axis_classes(kap, ng, x, qval, gidx);
-        t.nkx[x] = (int)kval.size() - t.kofs[x];
-        t.nqx[x] = (int)qval.size() - t.qofs[x];
+        t.kofs[x] = kc.ofs[x];
+        t.qofs[x] = gc.ofs[x];
+        t.nkx[x] = kc.n[x];
+        t.nqx[x] = gc.n[x];
         cells += (long long)t.nkx[x] * t.nqx[x];
     }
-    std::vector<int> gperm(ng), gsort(3 * (size_t)ng);
-    for (int g = 0; g < ng; ++g) gperm[g] = g;
-    std::sort(gperm.begin(), gperm.end(), [&](int i, int j) {
-        for (int x = 2; x >= 0; --x)
-            if (gidx[3 * i + x] != gidx[3 * j + x]) return gidx[3 * i + x] < gidx[3 * j + x];
-        return i < j;
-    });
-    for (int g = 0; g < ng; ++g)
-        for (int x = 0; x < 3; ++x) gsort[3 * g + x] = gidx[3 * gperm[g] + x];
     // worth it only when the classes repeat (regular k grids, G shells); bounded memory
     const size_t tab_bytes = (size_t)npair * cells * ctx->nchar * 4 * elem;
     if (4 * cells > 3LL * 3 * nk * ng || tab_bytes > ((size_t)512 << 20)) return cudaSuccess;
     for (int x = 0; x < 3; ++x) t.tbase[x + 1] = t.tbase[x] + (long long)npair * t.nkx[x] * t.nqx[x];
+    std::vector<int> gperm(ng);
+    for (int g = 0; g < ng; ++g) gperm[g] = g;
+    std::sort(gperm.begin(), gperm.end(), [&](int i, int j) {
+        for (int x = 2; x >= 0; --x)
+            if (gc.idx[3 * i + x] != gc.idx[3 * j + x]) return gc.idx[3 * i + x] < gc.idx[3 * j + x];
+        return i < j;
+    });
+    t.o_qval = kc.val.size() * sizeof(double);
+    t.o_kidx = t.o_qval + gc.val.size() * sizeof(double);
+    t.o_gidx = t.o_kidx + kc.idx.size() * sizeof(int);
+    t.o_gperm = t.o_gidx + gc.idx.size() * sizeof(int);
+    std::vector<char> meta(t.o_gperm + gperm.size() * sizeof(int));
+    std::memcpy(meta.data(), kc.val.data(), t.o_qval);
+    std::memcpy(meta.data() + t.o_qval, gc.val.data(), gc.val.size() * sizeof(double));
+    std::memcpy(meta.data() + t.o_kidx, kc.idx.data(), kc.idx.size() * sizeof(int));
+    int* gsort = reinterpret_cast<int*>(meta.data() + t.o_gidx);
+    for (int g = 0; g < ng; ++g)
+        for (int x = 0; x < 3; ++x) gsort[3 * g + x] = gc.idx[3 * gperm[g] + x];
+    std::memcpy(meta.data() + t.o_gperm, gperm.data(), gperm.size() * sizeof(int));
     cudaError_t e;
     const size_t y_bytes = y_per_k * std::min<size_t>(nk, std::max<size_t>(1, PD_Y_BYTES / std::max<size_t>(1, y_per_k)));
     if ((e = t.tab.ensure(tab_bytes)) != cudaSuccess || (e = t.y.ensure(y_bytes)) != cudaSuccess) {
@@ -1113,17 +1133,8 @@ static cudaError_t tab_prepare(qcx_ctx* ctx, PdTab& t, const double* kpts, int n
         cudaGetLastError();                       // no room for the tables: the kernels without them serve
         return cudaSuccess;
     }
-    if ((e = t.kidx.ensure(kidx.size() * sizeof(int))) != cudaSuccess) return e;
-    if ((e = t.gidx.ensure(gidx.size() * sizeof(int))) != cudaSuccess) return e;
-    if ((e = t.gperm.ensure(gperm.size() * sizeof(int))) != cudaSuccess) return e;
-    if ((e = t.kval.ensure(kval.size() * sizeof(double))) != cudaSuccess) return e;
-    if ((e = t.qval.ensure(qval.size() * sizeof(double))) != cudaSuccess) return e;
-    const cudaMemcpyKind h2d = cudaMemcpyHostToDevice;
-    if ((e = cudaMemcpyAsync(t.kidx.p, kidx.data(), kidx.size() * sizeof(int), h2d, ctx->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(t.gidx.p, gsort.data(), gsort.size() * sizeof(int), h2d, ctx->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(t.gperm.p, gperm.data(), gperm.size() * sizeof(int), h2d, ctx->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(t.kval.p, kval.data(), kval.size() * sizeof(double), h2d, ctx->stream)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(t.qval.p, qval.data(), qval.size() * sizeof(double), h2d, ctx->stream)) != cudaSuccess)
+    if ((e = t.meta.ensure(meta.size())) != cudaSuccess ||
+        (e = cudaMemcpyAsync(t.meta.p, meta.data(), meta.size(), cudaMemcpyHostToDevice, ctx->stream)) != cudaSuccess)
         return e;
     t.valid = true;
     return cudaSuccess;
@@ -1151,7 +1162,7 @@ cudaError_t qcx_pd_tab_prepare(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng
             kap[3 * g + x] = v;
         }
     const size_t elem = prec == QCX_FP64 ? sizeof(double2) : sizeof(float2);
-    return tab_prepare(ctx, s.pdt, ctx->kpts_h.data(), nk, kap.data(), ng, elem, pd_y_per_k(ctx->nb, ctx->nv, ng, elem));
+    return tab_prepare(ctx, s.pdt, ctx->kcls, nk, kap.data(), ng, elem, pd_y_per_k(ctx->nb, ctx->nv, ng, elem));
 }
 
 cudaError_t qcx_launch_pair_density(qcx_ctx* ctx, QSlot& s, int iq, qcx_precision prec) {
@@ -1253,7 +1264,7 @@ cudaError_t qcx_launch_overlap(qcx_ctx* ctx, int nk, const double* d_kpts, const
     a.Sout = d_out;
     const double zero[3] = {0.0, 0.0, 0.0};
     if (nk <= 65535) {
-        const cudaError_t e = tab_prepare(ctx, ctx->overlap_tab, k_host, nk, zero, 1, sizeof(double2), 0);
+        const cudaError_t e = tab_prepare(ctx, ctx->overlap_tab, qcx_axis_classes(k_host, nk), nk, zero, 1, sizeof(double2), 0);
         if (e != cudaSuccess) return e;
         if (ctx->overlap_tab.valid) {
             const dim3 grid(((ctx->ngrp + 1) / 2 * (ctx->ngrp + 1) + 127) / 128, nk);

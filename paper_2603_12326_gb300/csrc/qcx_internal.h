@@ -36,6 +36,37 @@ struct DevBuf {
     template <typename T> T* as() const { return reinterpret_cast<T*>(p); }
 };
 
+// Page-locked host staging for the small results of a call (a copy into pageable memory waits twice).  Used only by
+// calls that synchronise their stream before they return.
+struct PinBuf {
+    void* p = nullptr;
+    size_t bytes = 0;
+    PinBuf() = default;
+    PinBuf(const PinBuf&) = delete;
+    PinBuf& operator=(const PinBuf&) = delete;
+    ~PinBuf() {
+        if (p) cudaFreeHost(p);
+    }
+    cudaError_t ensure(size_t n) {
+        if (n <= bytes && p) return cudaSuccess;
+        if (p) cudaFreeHost(p);
+        p = nullptr;
+        bytes = 0;
+        const cudaError_t e = cudaMallocHost(&p, n);
+        if (e == cudaSuccess) bytes = n;
+        return e;
+    }
+};
+
+// Distinct components per axis of a point set (host): values of the classes, axes concatenated, and the class of every
+// point's component.
+struct AxisClasses {
+    int n[3] = {0, 0, 0}, ofs[3] = {0, 0, 0};
+    std::vector<double> val;
+    std::vector<int> idx;      // [points][3]
+    bool finite = false;
+};
+
 // Tables of the pair densities for one q (or of an overlap, q+G = 0): the one-dimensional lattice sums
 // per shell-group pair, axis, distinct k component and distinct (q+G) component, with the axis's share
 // of every factor of the pair, so that the per-(k, G) kernel reads them instead of forming them again.
@@ -44,9 +75,10 @@ struct PdTab {
     int nkx[3] = {0, 0, 0}, nqx[3] = {0, 0, 0};   // distinct k and q+G components per axis
     int kofs[3] = {0, 0, 0}, qofs[3] = {0, 0, 0}; // first value of each axis in kval / qval
     long long tbase[4] = {0, 0, 0, 0};            // first entry of each axis (tbase[3] = entries)
-    DevBuf kidx, gidx;         // [nk][3], [ng][3] int: class of each point's component
-    DevBuf gperm;              // [ng] int: the G of gidx's rows (ordered by class)
-    DevBuf kval, qval;         // values of the classes (axes concatenated)
+    // one upload: kval, qval (values of the classes, axes concatenated; double), then [nk][3] and [ng][3] classes of the
+    // points' components and [ng] the G of each row of the latter (ordered by class; int)
+    DevBuf meta;
+    size_t o_qval = 0, o_kidx = 0, o_gidx = 0, o_gperm = 0;   // byte offsets
     DevBuf tab;                // [entries][nchar][4] complex (FP32 or FP64): E(0,0), E(1,0), E(0,1), E(1,1)
     DevBuf y;                  // Y = B C_k of a chunk of k points (pair densities)
 };
@@ -71,6 +103,7 @@ struct QSlot {
     DevBuf kappa1;             // [2][nw] double |A|_1 and |X|_1 of the mixed inverse (kappa_1 is their product)
     DevBuf refine;             // shares of the FP64 diagonal correction [row tile][nw][ng] double2
     DevBuf w;                  // [nw] double
+    std::vector<double> wh;    // host copy of w
     DevBuf diag_inv;           // [nw][ng] double2
     DevBuf eps_diag;           // [nw][ng] double2
     DevBuf resid;              // [nw] double
@@ -217,6 +250,7 @@ struct qcx_ctx {
     int nk = 0, nv = 0, nc = 0, nq = 0;
     std::vector<double> qpts;  // host copy
     std::vector<double> kpts_h;    // host copy [nk][3]
+    AxisClasses kcls;              // its classes (kept with the states: every q's tables use them)
     DevBuf d_kpts, d_kpts32;   // [nk][3]
     DevBuf d_Ck64, d_Ck32;     // [nk][nb][nv]
     DevBuf d_Ek;               // [nk][nv]
@@ -228,6 +262,7 @@ struct qcx_ctx {
 
     DevBuf scratch;            // host<->device staging for outputs
     DevBuf scratch2;
+    PinBuf pin;                // staging of small results
 
     unsigned long long gen = 0;    // bumped whenever basis or states change
     BatchPlan* batch = nullptr;    // cached plan (and captured graph) of the last batched solve
@@ -283,6 +318,14 @@ cudaError_t qcx_copy_in(qcx_ctx* ctx, void* dst_dev, const void* src, size_t byt
 // copy device memory to a host-or-device destination; host destinations synchronise
 cudaError_t qcx_copy_out(qcx_ctx* ctx, void* dst, const void* src_dev, size_t bytes);
 
+// Device memory [0, total) at src to host destinations (null: skipped), one copy and one wait for all of them; the stream
+// is synchronised either way.  Device destinations and large results are copied directly.
+struct CopyOut {
+    void* dst;
+    size_t offset, bytes;
+};
+cudaError_t qcx_copy_out_all(qcx_ctx* ctx, const char* src, size_t total, const CopyOut* out, int n);
+
 // ---------------------------------------------------------------- launchers
 // pair densities (pair_density.cu)
 cudaError_t qcx_launch_qsetup(qcx_ctx* ctx, QSlot& s, const int* d_G, int ng, const double* q);
@@ -293,6 +336,7 @@ cudaError_t qcx_launch_pair_density(qcx_ctx* ctx, QSlot& s, int iq, qcx_precisio
 cudaError_t qcx_pd_tab_prepare(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng, int iq, qcx_precision prec);
 cudaError_t qcx_launch_overlap(qcx_ctx* ctx, int nk, const double* d_kpts, const double* k_host, double2* d_out);
 cudaError_t qcx_pair_density_configure();
+AxisClasses qcx_axis_classes(const double* v, int n);
 
 // optical limit (optical.cu): momentum elements and the G = 0 row rho~ = -i qhat.p/dE of the
 // slot's pair densities, v^1/2 of that row set to sqrt(4 pi); d_status bit 1: a zero dE

@@ -729,6 +729,7 @@ extern "C" qcx_status qcx_chi0_spectral(qcx_ctx* ctx, int iq, int nw, const doub
     for (double v : wh)
         if (!std::isfinite(v)) return ctx->fail(QCX_ERR_ARG, "chi0_spectral: non-finite frequency");
     s.nw = nw;
+    s.wh = wh;
     s.eta = eta;
     s.have_eps = false;
     if (ctx->loss[iq]) ctx->loss[iq]->valid = false;
