@@ -24,13 +24,13 @@
 //
 // Steps: energy range; stable radix sort of the transitions by panel; plan (segments, 16-transition stages); Lagrange
 // weights; rho~ gathered into stage-contiguous, pre-swizzled tiles (a stage is one plain bulk copy per plane);
-// k_pn_gram; S split into K-major BF16 planes; contraction with W; diagonal; Dyson step.
+// k_pn_gram, which writes S as BF16 planes; contraction with W; diagonal; Dyson step.
 //
 // k_pn_gram is k_chi0_tc (same roles, same stage) made persistent over (segment, G' block, G chunk, node): segments are
 // ~15 stages long, so the drain warps write one item's S while the next one's MMAs run.  A tile holds the columns from
 // its own G' block on, which is what the Hermitian half needs.
-// Measured (one q, 200 w, N_t = 65536, N_G = 181): chi0 14.8 -> 4.1 ms (S 1.5, contraction with
-// W 1.0, split 0.4, gather 0.3); 100 w, N_t = 57344, N_G = 531: 56 -> 34 ms.
+// Measured (one q, 200 w, N_t = 65536, N_G = 181): chi0 14.8 -> 3.5 ms (S 1.5, contraction with W 1.0, gather 0.3);
+// 100 w, N_t = 57344, N_G = 531: 56 -> 24 ms.
 #include "qcx_internal.h"
 #include "tc_ptx.cuh"
 
@@ -45,7 +45,7 @@ constexpr int PN_SEG = 2048;                // transitions per segment (64 accum
 constexpr int PN_TPS = KSTEP / 2;           // transitions per K stage
 constexpr int PN_MAXPANELS = 65536;
 constexpr int PN_CHUNK_NODES = 4096;        // nodes contracted with W in one FP32 chain
-constexpr size_t PN_BYTES = 4ull << 30;     // S and its planes, per chunk of segments
+constexpr size_t PN_BYTES = 4ull << 30;     // S of a chunk of segments
 
 // ------------------------------------------------------------------ energies, sort, plan
 __device__ __forceinline__ unsigned long long order_key(double x) {
@@ -349,9 +349,8 @@ struct PgArgs {
     const float* Lw;                      // [16][ldl]
     long long ldl;
     int npair_row;                        // 32-tiles per row of the pair triangle
-    int nbc;                              // node stride of S
-    float* Sre;                           // [pair][nbc][1024], element (G in 32) 32 + (G' in 32)
-    float* Sim;
+    long long ncol, plane;                // columns of S (2 x 1024 x pairs), elements of a plane
+    __nv_bfloat16* S;                     // three planes [node][ncol], column ((pair 32 + G in 32) 2 + part) 32 + (G' in 32)
     int* status;
     long long wait_limit;
 };
@@ -597,17 +596,27 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(const __grid_constant
                 if (lane == 0) mbar_arrive(&drained[b]);
             }
             if (!ok) break;
-            // S of this item: the warp's 32 rows are one 32-tile of G', lanes contiguous
+            // S of this item in three BF16 terms: the warp's 32 rows are one 32-tile of G'.  Two columns at a time, even
+            // lanes writing the first as pairs of rows, odd lanes the second
             const int gi = m.gb * 2 + (q & 1);                     // G' tile
             if (gi < a.npair_row) {
-                float* S = (q >> 1 ? a.Sim : a.Sre) + ((size_t)m.slot * PN_NODES + m.node) * 1024 + lane;
+                __nv_bfloat16* S = a.S + ((size_t)m.slot * PN_NODES + m.node) * a.ncol + (q >> 1) * 32 + (lane & ~1);
                 const int c0 = m.n0 + hc * half;
 #pragma unroll
-                for (int c = 0; c < PG_MAXHALF; ++c) {
-                    const int G = c0 + c, hi = G >> 5;
-                    if (c < half && hi >= gi) {
+                for (int c = 0; c < PG_MAXHALF; c += 2) {
+                    if (c >= half) break;
+                    const bool odd = lane & 1;
+                    const float other = __shfl_xor_sync(0xffffffffu, odd ? part[c] : part[c + 1], 1);
+                    const float lo = odd ? other : part[c], hi_ = odd ? part[c + 1] : other;
+                    const int G = c0 + c + (odd ? 1 : 0), hi = G >> 5;
+                    if (hi >= gi) {
                         const int p = gi * a.npair_row - gi * (gi - 1) / 2 + hi - gi;
-                        S[(size_t)p * a.nbc * 1024 + (G & 31) * 32] = part[c];
+                        uint32_t s0, s1, s2;
+                        split3(lo, hi_, s0, s1, s2);
+                        uint32_t* o = reinterpret_cast<uint32_t*>(S + (size_t)(p * 32 + (G & 31)) * 64);
+                        o[0] = s0;
+                        o[a.plane / 2] = s1;
+                        o[a.plane] = s2;
                     }
                 }
             }
@@ -618,33 +627,6 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(const __grid_constant
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem, 4 * PG_NMAX);
-    }
-}
-
-// S [pair][nbc][1024] -> three BF16 planes [2 x 1024 x pair][ld], row 2 X + part, column = node in the chunk; zero for
-// nodes >= nb.  Block (32, 8): 32 elements x 64 nodes through shared memory, written as pairs of nodes.
-__global__ void __launch_bounds__(256) k_pn_split(int nbc, int nb, long long ld, const float* Sre, const float* Sim,
-                                                  uint32_t* p0, uint32_t* p1, uint32_t* p2) {
-    __shared__ float t[2][32][65];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const long long X0 = (long long)blockIdx.x * 32;
-    const int b0 = blockIdx.y * 64;
-    const size_t src = ((size_t)(X0 >> 10) * nbc) * 1024 + (X0 & 1023) + tx;
-    for (int j = ty; j < 64; j += 8) {
-        const int b = b0 + j;
-        t[0][tx][j] = b < nb ? Sre[src + (size_t)b * 1024] : 0.f;
-        t[1][tx][j] = b < nb ? Sim[src + (size_t)b * 1024] : 0.f;
-    }
-    __syncthreads();
-    if (b0 + 2 * tx >= ld) return;
-    for (int j = ty; j < 64; j += 8) {
-        const int x = j >> 1, c = j & 1;
-        uint32_t q0, q1, q2;
-        split3(t[c][x][2 * tx], t[c][x][2 * tx + 1], q0, q1, q2);
-        const size_t o = ((size_t)(2 * (X0 + x) + c) * ld + b0) / 2 + tx;
-        p0[o] = q0;
-        p1[o] = q1;
-        p2[o] = q2;
     }
 }
 
@@ -798,7 +780,7 @@ static double panel_us(const QSlot& s, long long nt, double stages, double segs,
     const double T = (s.ng + 31) / 32, pairs = T * (T + 1) / 2, nodes = segs * PN_NODES;
     const double gram = ntile * PN_NODES * (stages * 0.62 + segs * 1.2) / 152.0;
     const double kk = (2.0 * s.nw + 127) / 128 * pairs * 16 * nodes / 32 * 0.65 / 152.0;
-    const double bytes = pairs * 1024 * nodes * 28.0 + (double)nt * s.ngp * 40.0 + 48.0 * s.nw * s.ng * (double)s.ng;
+    const double bytes = pairs * 1024 * nodes * 12.0 + (double)nt * s.ngp * 40.0 + 48.0 * s.nw * s.ng * (double)s.ng;
     return gram + kk + bytes / 3e6 + 200.0;
 }
 
@@ -895,7 +877,7 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
     if (panel_us(s, nt, (double)nst, nseg, ntile) >= 0.8 * direct) return cudaSuccess;
 
     // chunks of segments: nodes per FP32 chain and bytes of S bounded
-    const size_t per_seg = (size_t)PN_NODES * ntp * 1024 * (2 * sizeof(float) + 6 * sizeof(__nv_bfloat16));
+    const size_t per_seg = (size_t)PN_NODES * ntp * 1024 * 6 * sizeof(__nv_bfloat16);
     const int cap = (int)std::max<size_t>(2, std::min<size_t>(PN_CHUNK_NODES / PN_NODES, PN_BYTES / per_seg)) / 2 * 2;
     const int nchunk = (nseg + cap - 1) / cap;
     const int cseg = ((nseg + nchunk - 1) / nchunk + 1) / 2 * 2;                // even: node chunks are multiples of 32
@@ -910,7 +892,7 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
     if (!fits(b.tr, sizeof(int) * (size_t)ldl) || !fits(b.Lw, sizeof(float) * PN_NODES * (size_t)ldl) ||
         !fits(b.tiles, 2 * tile_bytes) || !fits(b.r2, sizeof(float) * (size_t)ldl * ngp) ||
         !fits(b.ktab, sizeof(float4) * (size_t)nw * ldk) || !fits(b.kplanes, 3 * kn * sizeof(__nv_bfloat16)) ||
-        !fits(b.S, 2 * sizeof(float) * (size_t)ntp * nbc * 1024) || !fits(b.splanes, 3 * sn * sizeof(__nv_bfloat16)) ||
+        !fits(b.splanes, 3 * sn * sizeof(__nv_bfloat16)) ||
         !fits(b.Sd, sizeof(float2) * (size_t)nb * ngp) || !fits(b.part, sizeof(double2) * (size_t)nz * nw * ng) ||
         !fits(b.chi, sizeof(double2) * (size_t)nw * ng * ng) || !fits(b.tp, sizeof(int2) * ntp))
         return give_up();
@@ -944,9 +926,9 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
     a.Lw = b.Lw.as<float>();
     a.ldl = ldl;
     a.npair_row = T32;
-    a.nbc = nbc;
-    a.Sre = b.S.as<float>();
-    a.Sim = a.Sre + (size_t)ntp * nbc * 1024;
+    a.ncol = (long long)ntiles * 128;
+    a.plane = a.ncol * nbc;
+    a.S = b.splanes.as<__nv_bfloat16>();
     a.status = d_status;
     a.wait_limit = ctx->wait_limit;
     const size_t smem = 1024 + PG_NSTAGE * (size_t)(2 * (n_max + (with_src ? PG_GBLK : 0)) * ROWB + 3 * PG_ATILE) +
@@ -962,7 +944,7 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
     __nv_bfloat16* sp = b.splanes.as<__nv_bfloat16>();
     for (int i = 0; i < 3; ++i)
         if (!qcx_make_bf16_map(&kmaps[i], kp + i * kn, ldk, mtiles * 128, 128, 32) ||
-            !qcx_make_bf16_map(&smaps[i], sp + i * sn, nbc, ntiles * 128, 128, 32))
+            !qcx_make_bf16_map(&smaps[i], sp + i * sn, ntiles * 128, nbc, 32, 64))
             return cudaErrorInvalidValue;
     for (int c = 0; c < nchunk; ++c) {
         const int s0 = c * cseg, m = std::min(cseg, nseg - s0);
@@ -970,10 +952,12 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
         a.seg = seg + s0;
         a.nseg = m;
         k_pn_gram<<<std::min(152, m * ntile * PN_NODES), PG_THREADS, smem, st>>>(a);
-        k_pn_split<<<dim3(ntp * 32, (nbc + 63) / 64), dim3(32, 8), 0, st>>>(
-            nbc, m * PN_NODES, nbc, a.Sre, a.Sim, reinterpret_cast<uint32_t*>(sp), reinterpret_cast<uint32_t*>(sp + sn),
-            reinterpret_cast<uint32_t*>(sp + 2 * sn));
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        // an odd number of segments leaves 16 points of the last stage
+        for (int i = 0; i < 3 && m * PN_NODES % KSTEP; ++i)
+            if ((e = cudaMemsetAsync(sp + i * sn + (size_t)m * PN_NODES * a.ncol, 0, PN_NODES * a.ncol * sizeof(__nv_bfloat16),
+                                     st)) != cudaSuccess)
+                return e;
         e = qcx_spec_tc_kk(st, kmaps, smaps, mtiles, ntiles, nw, ng, m * PN_NODES, c * nbc, b.tp.as<int2>(), c > 0,
                            b.chi.as<double2>(), d_status, ctx->wait_limit);
         if (e != cudaSuccess) return e;

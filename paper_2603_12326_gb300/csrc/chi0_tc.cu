@@ -571,16 +571,16 @@ static PFN_encodeTiled_t get_encode() {
 }
 
 // 2-D tensor map over one BF16 plane [rows][kp] (row length kp), box {box_k, box_rows} with the
-// swizzle matching the row bytes of the box (32 or 64)
+// swizzle matching the row bytes of the box (32, 64 or 128)
 bool qcx_make_bf16_map(CUtensorMap* m, void* base, long long kp, int rows, int box_rows, int box_k) {
     PFN_encodeTiled_t enc = get_encode();
-    if (!enc || (box_k != 16 && box_k != 32)) return false;
+    if (!enc || (box_k != 16 && box_k != 32 && box_k != 64)) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)kp, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)kp * 2};
     const cuuint32_t box[2] = {(cuuint32_t)box_k, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               box_k == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+               box_k == 16 ? CU_TENSOR_MAP_SWIZZLE_32B : (box_k == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 

@@ -184,7 +184,7 @@ struct PanelBufs {
     DevBuf tr, Lw;             // transition and Lagrange weights of every stage slot
     DevBuf tiles, r2;          // gathered rho~ stage tiles (two planes), |rho|^2
     DevBuf ktab, kplanes;      // W at the nodes: FP32, BF16 planes
-    DevBuf S, splanes, tp;     // S of one chunk, its BF16 planes, 32-tile pairs
+    DevBuf splanes, tp;        // S of one chunk as BF16 planes, 32-tile pairs
     DevBuf Sd, part, chi;      // diagonal of S, its frequency sums; chi0 [nw][ng][ng]
 };
 
@@ -343,17 +343,13 @@ AxisClasses qcx_axis_classes(const double* v, int n);
 cudaError_t qcx_launch_optical(qcx_ctx* ctx, QSlot& s, int iq, int g0, const double qhat[3], qcx_precision prec,
                                int* d_status);
 
-// spectral route on the tensor cores (spectral_tc.cu): K table as three BF16 planes [rows][ld]
-// (row 2 w + r); one chunk's weights [pair][point][32][32] split into three K-major planes and
-// contracted with the K planes into chi (FP64, stored or added)
+// contraction over energies on the tensor cores (spectral_tc.cu): K table as three BF16 planes [rows][ld]
+// (row 2 w + r); weights S as three planes [point][columns], column ((pair 32 + i) 2 + part) 32 + j for element
+// (G = 32 tp.x + i, G' = 32 tp.y + j) of a 32-tile pair, zero rows up to a multiple of 32 points; maps
+// {32, 128} over the K planes (64-byte swizzle) and {64, 32} over the S planes (128-byte swizzle); into chi (FP64,
+// stored or added)
 cudaError_t qcx_spec_tc_ktab(cudaStream_t st, int nw, int rows, long long ld, int nbin, const double* w, double E0,
                              double step, double eta, __nv_bfloat16* planes);
-cudaError_t qcx_spec_tc_contract(cudaStream_t st, const CUtensorMap* kmaps, const CUtensorMap* smaps, int mtiles,
-                                 int ntiles, int nw, int ng, int nbc, int nb, int kb0, long long sld, const float2* S,
-                                 __nv_bfloat16* splanes, const int2* tp, int accumulate, double2* chi, int* status,
-                                 long long wait_limit);
-
-// the contraction alone, on planes already split
 cudaError_t qcx_spec_tc_kk(cudaStream_t st, const CUtensorMap* kmaps, const CUtensorMap* smaps, int mtiles, int ntiles, int nw,
                            int ng, int nb, int kb0, const int2* tp, int accumulate, double2* chi, int* status,
                            long long wait_limit);
@@ -365,7 +361,7 @@ cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0
 cudaError_t qcx_launch_chi0_fp64_tc(qcx_ctx* ctx, QSlot& s, int iq, double pref, double2* chi, int* d_status);
 cudaError_t qcx_launch_chi0_mixed(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out, int* d_status);
 // 2-D tensor map over one BF16 plane [rows][kp], box {box_k, box_rows} (box_k 16: 32-byte
-// swizzle, 32: 64-byte swizzle)
+// swizzle, 32: 64-byte swizzle, 64: 128-byte swizzle)
 bool qcx_make_bf16_map(CUtensorMap* m, void* base, long long kp, int rows, int box_rows, int box_k);
 
 // persistent tensor-core chi0 over a tile list of uneven instances (chi0_tc_batch.cu).

@@ -212,7 +212,9 @@ template <typename R> struct GramArgs {
     long long nt;
     int ng, b0, nbc;
     R pref;
-    cplx<R>* S;                          // [ntp][nbc][32][32]
+    cplx<R>* S;                          // [ntp][nbc][32][32], or null
+    __nv_bfloat16* planes;               // three BF16 planes [nbc][ncol] (spectral_tc.cu), or null
+    long long ncol, plane;               // columns, elements of a plane
 };
 
 // S_b for one upper tile pair and one grid point; thread (tx, ty) holds rows ty, ty + 16 and
@@ -263,13 +265,29 @@ template <typename R> __global__ void __launch_bounds__(256) k_spec_gram(GramArg
     }
     // S_b is Hermitian: its diagonal is real, so the rounding left in the imaginary part there
     // (which Re K would carry into Im chi0_GG) is dropped
-    C* out = a.S + ((size_t)p * a.nbc + bl) * SP_TILE2;
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const bool diag = pr.x == pr.y && ty + 16 * i == tx + 16 * j;
-            out[(ty + 16 * i) * SP_TILE + tx + 16 * j] = mk<R>(a.pref * acc[i][j].x, diag ? (R)0 : a.pref * acc[i][j].y);
+            const int r = ty + 16 * i, c = tx + 16 * j;
+            const bool diag = pr.x == pr.y && r == c;
+            const C v = mk<R>(a.pref * acc[i][j].x, diag ? (R)0 : a.pref * acc[i][j].y);
+            if (a.S) a.S[((size_t)p * a.nbc + bl) * SP_TILE2 + r * SP_TILE + c] = v;
+            if constexpr (sizeof(R) == 4) {
+                if (a.planes) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float x = h ? v.y : v.x;
+                        __nv_bfloat16* q = a.planes + (size_t)bl * a.ncol + ((size_t)(p * 32 + r) * 2 + h) * 32 + c;
+#pragma unroll
+                        for (int u = 0; u < 3; ++u) {
+                            const __nv_bfloat16 t = __float2bfloat16_rn(x);
+                            q[u * a.plane] = t;
+                            x -= __bfloat162float(t);
+                        }
+                    }
+                }
+            }
         }
 }
 
@@ -538,17 +556,23 @@ qcx_status spectral_chi0(qcx_ctx* ctx, QSlot& s, bool mixed, int nw, double E0, 
     CUDA_OR_FAIL(cudaMemcpyAsync(sp.tp.p, tp.data(), sizeof(int2) * ntp, cudaMemcpyHostToDevice, st), "copy tiles");
 
     const long long ldk = (nbin + 31LL) / 32 * 32;
+    if (!mixed || ctx->spec_cuda_cores) {                  // (the tensor-core contraction has its own planes)
     CUDA_OR_FAIL(sp.ktab.ensure(sizeof(C) * (size_t)nw * ldk), "alloc K");
     k_spec_ktab<R><<<nblk((long long)nw * ldk, 256), 256, 0, st>>>(nw, ldk, nbin, s.w.as<double>(), E0, step, s.eta,
                                                                     sp.ktab.as<C>());
     CUDA_OR_FAIL(cudaGetLastError(), "K kernel");
+    }
 
     const size_t per_bin = (size_t)ntp * SP_TILE2 * sizeof(C);
     long long nbc = ctx->spec_chunk_bins > 0 ? ctx->spec_chunk_bins : (long long)(kSpecChunkBytes / per_bin);
     nbc = std::min<long long>(nbc, sizeof(R) == 4 ? KK_F32_CHUNK : 65504);
     nbc = std::max<long long>(32, nbc / 32 * 32);
     nbc = std::min<long long>(nbc, ldk);
-    CUDA_OR_FAIL(sp.S.ensure(per_bin * nbc), "alloc spectral weights");
+    // the mixed route's contraction on the tensor cores reads the weights as BF16 planes, which the weight kernel writes
+    // itself; the complex weights are kept for the other contraction and for export
+    const bool tc = mixed && !ctx->spec_cuda_cores;
+    const bool need_S = !tc || out_S;
+    if (need_S) CUDA_OR_FAIL(sp.S.ensure(per_bin * nbc), "alloc spectral weights");
     CUDA_OR_FAIL(sp.chi.ensure(sizeof(double2) * (size_t)nw * ng * ng), "alloc chi0");
     const bool s_dev = out_S && qcx_is_device_ptr(out_S);
     if (out_S && !s_dev) CUDA_OR_FAIL(sp.Sout.ensure(sizeof(double2) * (size_t)nbc * ng * ng), "alloc");
@@ -558,9 +582,6 @@ qcx_status spectral_chi0(qcx_ctx* ctx, QSlot& s, bool mixed, int nw, double E0, 
                  "contraction smem");
     const R pref = (R)(2.0 / (ctx->nk * cell_volume(ctx)));
     const int nchunk = (int)((nbin + nbc - 1) / nbc);
-    // the mixed route's contraction on the tensor cores: K table and each chunk's weights as
-    // three BF16 planes, K-major over the grid points
-    const bool tc = mixed && !ctx->spec_cuda_cores;
     const int mtiles = (2 * nw + 127) / 128;
     const int ntiles = ntp * 16;                      // 2 x 1024 columns per tile pair, 128 per tile
     CUtensorMap kmaps[3], smaps[3];
@@ -574,7 +595,7 @@ qcx_status spectral_chi0(qcx_ctx* ctx, QSlot& s, bool mixed, int nw, double E0, 
                      "K planes kernel");
         for (int i = 0; i < 3; ++i)
             if (!qcx_make_bf16_map(&kmaps[i], sp.kplanes.as<__nv_bfloat16>() + i * kn, ldk, mtiles * 128, 128, 32) ||
-                !qcx_make_bf16_map(&smaps[i], sp.splanes.as<__nv_bfloat16>() + i * sn, nbc, ntiles * 128, 128, 32))
+                !qcx_make_bf16_map(&smaps[i], sp.splanes.as<__nv_bfloat16>() + i * sn, ntiles * 128, (int)nbc, 32, 64))
                 return ctx->fail(QCX_ERR_CUDA, "chi0_spectral: tensor map encoding failed");
         CUDA_OR_FAIL(cudaMemsetAsync(sp.status.p, 0, sizeof(int), st), "clear");
     }
@@ -595,7 +616,10 @@ qcx_status spectral_chi0(qcx_ctx* ctx, QSlot& s, bool mixed, int nw, double E0, 
         ga.b0 = (int)b0;
         ga.nbc = (int)nbc;
         ga.pref = pref;
-        ga.S = sp.S.as<C>();
+        ga.S = need_S ? sp.S.as<C>() : nullptr;
+        ga.planes = tc ? sp.splanes.as<__nv_bfloat16>() : nullptr;
+        ga.ncol = (long long)ntiles * 128;
+        ga.plane = ga.ncol * nbc;
         k_spec_gram<R><<<dim3(ntp, nb), 256, 0, st>>>(ga);
         CUDA_OR_FAIL(cudaGetLastError(), "spectral weight kernel");
         if (out_S) {
@@ -610,10 +634,14 @@ qcx_status spectral_chi0(qcx_ctx* ctx, QSlot& s, bool mixed, int nw, double E0, 
         }
         CUDA_OR_FAIL(cudaEventRecord(ce[1], st), "event");
         if (tc) {
-            CUDA_OR_FAIL(qcx_spec_tc_contract(st, kmaps, smaps, mtiles, ntiles, nw, ng, (int)nbc, nb, (int)b0, nbc,
-                                              reinterpret_cast<const float2*>(sp.S.p),
-                                              sp.splanes.as<__nv_bfloat16>(), sp.tp.as<int2>(), b0 > 0 ? 1 : 0,
-                                              sp.chi.as<double2>(), sp.status.as<int>(), ctx->wait_limit),
+            // the last stage's points past the chunk's end
+            const int nb32 = (nb + 31) / 32 * 32;
+            for (int i = 0; i < 3 && nb32 > nb; ++i)
+                CUDA_OR_FAIL(cudaMemsetAsync(sp.splanes.as<__nv_bfloat16>() + i * ga.plane + (size_t)nb * ga.ncol, 0,
+                                             (size_t)(nb32 - nb) * ga.ncol * sizeof(__nv_bfloat16), st),
+                             "clear weights");
+            CUDA_OR_FAIL(qcx_spec_tc_kk(st, kmaps, smaps, mtiles, ntiles, nw, ng, nb, (int)b0, sp.tp.as<int2>(),
+                                        b0 > 0 ? 1 : 0, sp.chi.as<double2>(), sp.status.as<int>(), ctx->wait_limit),
                          "tensor-core contraction");
             CUDA_OR_FAIL(cudaEventRecord(ce[2], st), "event");
             continue;

@@ -6,15 +6,17 @@
 // as one real GEMM per chunk of grid points,
 //   D[m][n] = sum_b A[m][b] B[n][b],
 //   m = 2 w + r      A = (Re K, Im K)(w, E_b)                       (r = 0, 1)
-//   n = 2 X + c      B = (Re S, Im S)_b at the upper (G, G') pair X  (c = 0, 1)
-// so that with Ar = D[2w][2X], Bi = D[2w+1][2X+1], Cs = D[2w][2X+1], Dr = D[2w+1][2X]
+//   n = (X, c)        B = (Re S, Im S)_b at the pair X of one triangle  (c = 0, 1)
+// so that with Ar = D[2w][X,0], Bi = D[2w+1][X,1], Cs = D[2w][X,1], Dr = D[2w+1][X,0]
 //   chi0[G][G'] = (Ar - Bi) + i (Cs + Dr),   chi0[G'][G] = (Ar + Bi) + i (Dr - Cs)
 // (S_b is Hermitian; X runs over the 32 x 32 tiles of one triangle, X = p 1024 + 32 r + c).
 //
 // Both operands are split into three BF16 terms (the six products of order <= 2 are
-// accumulated, as in the direct route's kernel) and stored K-major: the K table as
-// [2 N_w (padded)][grid points], the weights of one chunk as [2 x 1024 x tile pairs][chunk
-// points], both loaded by TMA into 64-byte-swizzled stages.  The tensor core's FP32 sums
+// accumulated, as in the direct route's kernel): the K table K-major as
+// [2 N_w (padded)][grid points] (64-byte swizzle), the weights of one chunk MN-major as
+// [chunk points][2 x 1024 x tile pairs] (128-byte swizzle), the order in which the kernels that form
+// them hold them, so that no pass transposes them (that pass took 0.74 ms of the spectral route
+// per mid q, 7.4 ms of the panels' chi0 at N_G = 531).  The tensor core's FP32 sums
 // truncate with every MMA: the leading product has its own accumulator, restarted every two K
 // stages (4 MMAs) and added in FP32 registers, so a chunk is summed in two levels; the five
 // smaller products (2^-8 of it and less) share one for the whole chunk.  Chunks are added into
@@ -39,6 +41,8 @@ constexpr int SK_PROMOTE = 2;               // K stages accumulated in one TMEM 
 constexpr int SK_TILE = SK_M * ROWB;        // one 128-row operand piece (8 KB)
 constexpr int SK_STAGE = 6 * SK_TILE;       // three A pieces and three B pieces
 constexpr int SK_HALF = SK_N / 2;           // columns one drain thread owns
+constexpr int SK_BHALF = KSTEP * 128;       // bytes of 64 columns of a B piece
+static_assert(2 * SK_BHALF == SK_TILE, "two column blocks per B piece");
 
 struct SkArgs {
     int nw, ng;
@@ -104,9 +108,13 @@ __global__ void __launch_bounds__(SK_THREADS, 1)
                 tma_load_2d(st, &ka0, fb, xk, mt * SK_M);
                 tma_load_2d(st + SK_TILE, &ka1, fb, xk, mt * SK_M);
                 tma_load_2d(st + 2 * SK_TILE, &ka2, fb, xk, mt * SK_M);
-                tma_load_2d(st + 3 * SK_TILE, &sb0, fb, xs, nt * SK_N);
-                tma_load_2d(st + 4 * SK_TILE, &sb1, fb, xs, nt * SK_N);
-                tma_load_2d(st + 5 * SK_TILE, &sb2, fb, xs, nt * SK_N);
+                // B: 32 points x 64 columns per box, two boxes per piece
+                for (int h = 0; h < 2; ++h) {
+                    const int x = nt * SK_N + 64 * h;
+                    tma_load_2d(st + 3 * SK_TILE + h * SK_BHALF, &sb0, fb, x, xs);
+                    tma_load_2d(st + 4 * SK_TILE + h * SK_BHALF, &sb1, fb, x, xs);
+                    tma_load_2d(st + 5 * SK_TILE + h * SK_BHALF, &sb2, fb, x, xs);
+                }
                 last = it;
             }
             // let every copy still in flight (at most the last NSTAGE stages) land before the CTA can exit
@@ -118,7 +126,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1)
         // ---------------------------------------------------------------- MMA issuers
         if (lane == 0) {
             const int par = warp == 1 ? 0 : 1;
-            const uint32_t idesc = make_idesc(SK_M, SK_N);
+            const uint32_t idesc = make_idesc(SK_M, SK_N) | IDESC_B_MN;
             bool ok = true;
             for (int win = par; win < nwin && ok; win += 2) {
                 const int b = win & 1;
@@ -141,13 +149,13 @@ __global__ void __launch_bounds__(SK_THREADS, 1)
                     const uint32_t d = tmem + (uint32_t)(b * SK_N), dl = d + 2 * SK_N;
 #pragma unroll
                     for (int kk = 0; kk < KSTEP / 16; ++kk) {
-                        const uint32_t off = kk * 32;
-                        umma_bf16(d, sw64_desc(a0 + off), sw64_desc(b0 + off), idesc, (first && kk == 0) ? 0u : 1u);
-                        umma_bf16(dl, sw64_desc(a0 + off), sw64_desc(b1 + off), idesc, (win < 2 && first && kk == 0) ? 0u : 1u);
-                        umma_bf16(dl, sw64_desc(a1 + off), sw64_desc(b0 + off), idesc, 1u);
-                        umma_bf16(dl, sw64_desc(a0 + off), sw64_desc(b2 + off), idesc, 1u);
-                        umma_bf16(dl, sw64_desc(a1 + off), sw64_desc(b1 + off), idesc, 1u);
-                        umma_bf16(dl, sw64_desc(a2 + off), sw64_desc(b0 + off), idesc, 1u);
+                        const uint32_t off = kk * 32, offb = kk * 16 * 128;
+                        umma_bf16(d, sw64_desc(a0 + off), sw128_mn_desc(b0 + offb, SK_BHALF), idesc, (first && kk == 0) ? 0u : 1u);
+                        umma_bf16(dl, sw64_desc(a0 + off), sw128_mn_desc(b1 + offb, SK_BHALF), idesc, (win < 2 && first && kk == 0) ? 0u : 1u);
+                        umma_bf16(dl, sw64_desc(a1 + off), sw128_mn_desc(b0 + offb, SK_BHALF), idesc, 1u);
+                        umma_bf16(dl, sw64_desc(a0 + off), sw128_mn_desc(b2 + offb, SK_BHALF), idesc, 1u);
+                        umma_bf16(dl, sw64_desc(a1 + off), sw128_mn_desc(b1 + offb, SK_BHALF), idesc, 1u);
+                        umma_bf16(dl, sw64_desc(a2 + off), sw128_mn_desc(b0 + offb, SK_BHALF), idesc, 1u);
                     }
                     umma_commit(&empty[s]);
                 }
@@ -199,18 +207,16 @@ __global__ void __launch_bounds__(SK_THREADS, 1)
             const bool odd = lane & 1;
 #pragma unroll
             for (int xl = 0; xl < SK_HALF / 4; ++xl) {
-                // even lane: pair xl of the thread's 32, odd lane: pair xl + 16; each sends the
-                // partner the two values of its row that the partner's pair needs
-                const int lo = 2 * xl, hi = 2 * (xl + SK_HALF / 4);
-                const float s0 = odd ? part[lo] : part[hi], s1 = odd ? part[lo + 1] : part[hi + 1];
+                // the thread's columns: 32 elements' real parts, then their imaginary parts.  Even lane: element xl,
+                // odd lane: element xl + 16; each sends the partner the two values of its row that the partner needs
+                constexpr int Q = SK_HALF / 4, I = SK_HALF / 2;
+                const float s0 = odd ? part[xl] : part[xl + Q], s1 = odd ? part[I + xl] : part[I + xl + Q];
                 const float r0 = __shfl_xor_sync(0xffffffffu, s0, 1), r1 = __shfl_xor_sync(0xffffffffu, s1, 1);
-                const double Ar = odd ? r0 : part[lo], Cs = odd ? r1 : part[lo + 1];
-                const double Dr = odd ? part[hi] : r0, Bi = odd ? part[hi + 1] : r1;
-                const int xo = odd ? xl + SK_HALF / 4 : xl;
-                const long long P = (long long)nt * (SK_N / 2) + hc * (SK_HALF / 2) + xo;
-                const int p = (int)(P >> 10), X = (int)(P & 1023);
-                const int2 pr = a.tp[p];
-                const int G = pr.x * 32 + (X >> 5), H = pr.y * 32 + (X & 31);
+                const double Ar = odd ? r0 : part[xl], Cs = odd ? r1 : part[I + xl];
+                const double Dr = odd ? part[xl + Q] : r0, Bi = odd ? part[I + xl + Q] : r1;
+                const int row32 = nt * 2 + hc;                    // 32-element rows of the pairs, 64 columns each
+                const int2 pr = a.tp[row32 >> 5];
+                const int G = pr.x * 32 + (row32 & 31), H = pr.y * 32 + (odd ? xl + Q : xl);
                 if (w >= a.nw || G >= a.ng || H >= a.ng) continue;
                 // within a diagonal tile the elements below the diagonal serve both triangles too: with two
                 // roundings of the same S, Re K would carry their difference into the anti-Hermitian part of chi0
@@ -270,40 +276,6 @@ __global__ void k_spec_ktab_split(int nw, int rows, long long ld, int nbin, cons
     }
 }
 
-// weights of one chunk [pair][point][32][32] (FP32 complex) -> three BF16 planes [2 x 1024 x pair][ld]
-// (row 2 X + c, column = point in the chunk); zero for points >= nb.  Block (32, 8): a 32-point x
-// 32-pair tile through shared memory.
-__global__ void __launch_bounds__(256) k_spec_s_split(int nbc, int nb, long long ld, const float2* S,
-                                                      __nv_bfloat16* p0, __nv_bfloat16* p1, __nv_bfloat16* p2) {
-    __shared__ float2 t[32][33];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const long long X0 = (long long)blockIdx.x * 32;     // global pair index p 1024 + X
-    const int b0 = blockIdx.y * 32;
-    const long long p = X0 >> 10;
-    const int xin = (int)(X0 & 1023);
-    for (int j = ty; j < 32; j += 8) {
-        const int b = b0 + j;
-        float2 v = make_float2(0.f, 0.f);
-        if (b < nb) v = S[((size_t)p * nbc + b) * 1024 + xin + tx];
-        t[tx][j] = v;
-    }
-    __syncthreads();
-    for (int j = ty; j < 32; j += 8) {
-        const float2 v = t[j][tx];                       // pair X0 + j, point b0 + tx
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const float x = c ? v.y : v.x;
-            const __nv_bfloat16 h0 = __float2bfloat16_rn(x);
-            const float r1 = x - __bfloat162float(h0);
-            const __nv_bfloat16 h1 = __float2bfloat16_rn(r1);
-            const size_t o = (size_t)(2 * (X0 + j) + c) * ld + b0 + tx;
-            p0[o] = h0;
-            p1[o] = h1;
-            p2[o] = __float2bfloat16_rn(r1 - __bfloat162float(h1));
-        }
-    }
-}
-
 }  // namespace
 
 size_t qcx_spec_tc_smem() { return 1024 + (size_t)SK_NSTAGE * SK_STAGE + (3 * SK_NSTAGE + 5) * 8 + 16; }
@@ -314,18 +286,6 @@ cudaError_t qcx_spec_tc_ktab(cudaStream_t st, int nw, int rows, long long ld, in
     k_spec_ktab_split<<<(int)std::min<long long>((n + 255) / 256, 16384), 256, 0, st>>>(
         nw, rows, ld, nbin, w, E0, step, eta, planes, planes + n, planes + 2 * n);
     return cudaGetLastError();
-}
-
-cudaError_t qcx_spec_tc_contract(cudaStream_t st, const CUtensorMap* kmaps, const CUtensorMap* smaps, int mtiles,
-                                 int ntiles, int nw, int ng, int nbc, int nb, int kb0, long long sld, const float2* S,
-                                 __nv_bfloat16* splanes, const int2* tp, int accumulate, double2* chi, int* status,
-                                 long long wait_limit) {
-    const long long n = (long long)ntiles * SK_N * sld;     // elements per weight plane
-    dim3 sg((unsigned)((long long)ntiles * SK_N / 2 / 32), (unsigned)(sld / 32));
-    k_spec_s_split<<<sg, dim3(32, 8), 0, st>>>(nbc, nb, sld, S, splanes, splanes + n, splanes + 2 * n);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return qcx_spec_tc_kk(st, kmaps, smaps, mtiles, ntiles, nw, ng, nb, kb0, tp, accumulate, chi, status, wait_limit);
 }
 
 cudaError_t qcx_spec_tc_kk(cudaStream_t st, const CUtensorMap* kmaps, const CUtensorMap* smaps, int mtiles, int ntiles, int nw,

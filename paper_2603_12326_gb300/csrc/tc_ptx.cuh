@@ -176,6 +176,17 @@ __device__ __forceinline__ uint64_t sw32_desc(uint32_t saddr) {
 __device__ __forceinline__ uint32_t sw32_off(int r, int j) {
     return (uint32_t)r * 32u + ((uint32_t)(j ^ ((r >> 2) & 1)) << 4);
 }
+// Shared-memory matrix descriptor of a B operand stored MN-major with 128-byte swizzle: rows of 64
+// elements along N per k, 8-row groups along k 1024 bytes apart, blocks of 64 along N `nblock` bytes apart.
+__device__ __forceinline__ uint64_t sw128_mn_desc(uint32_t saddr, uint32_t nblock) {
+    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(nblock >> 4) << 16;  // next 64 elements of N
+    d |= (uint64_t)(1024 >> 4) << 32;    // next 8 k
+    d |= (uint64_t)1 << 46;              // descriptor version
+    d |= (uint64_t)2 << 61;              // 128-byte swizzle
+    return d;
+}
+constexpr uint32_t IDESC_B_MN = 1u << 16;   // instruction descriptor: B is MN-major
 // kind::f16 instruction descriptor: BF16 x BF16 -> FP32 (A and B type fields 1 = BF16), both
 // operands K-major
 __host__ __device__ constexpr uint32_t make_idesc(int M, int N) {
