@@ -289,25 +289,23 @@ __global__ void __launch_bounds__(256) k_pn_gather(int ngp, long long nchunk, co
     }
 }
 
-// W(w; E_b) of every node: a table of FP32 pairs {Re, Im, and what their rounding leaves} [nw][ld], and three BF16 planes [rows][ld], row 2 w + r; zero in the padding
+// W(w; E_b) of every node: FP32 table [nw][ld] and three BF16 planes [rows][ld], row 2 w + r; zero in the padding
 __global__ void k_pn_ktab(int nw, int rows, long long ld, int nb, const double* w, double eta, const int4* seg, double e0,
-                          double width, float4* K, __nv_bfloat16* p0, __nv_bfloat16* p1, __nv_bfloat16* p2) {
+                          double width, float2* K, __nv_bfloat16* p0, __nv_bfloat16* p1, __nv_bfloat16* p2) {
     const long long n = (long long)(rows / 2) * ld;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const int iw = (int)(i / ld);
         const long long b = i - (long long)iw * ld;
-        float2 v = make_float2(0.f, 0.f), lo = v;
+        float2 v = make_float2(0.f, 0.f);
         if (iw < nw && b < nb) {
             const double E = e0 + width * (seg[b / PN_NODES].x + 0.5 + 0.5 * node_x((int)(b % PN_NODES)));
             const double x1 = w[iw] - E, x2 = w[iw] + E;
             const double n1 = x1 * x1 + eta * eta, n2 = x2 * x2 + eta * eta;
             const double r = 1.0 / (n1 * n2);
             const double d1 = n2 * r, d2 = n1 * r;
-            const double re = x1 * d1 - x2 * d2, im = eta * (d2 - d1);
-            v = make_float2((float)re, (float)im);
-            lo = make_float2((float)(re - (double)v.x), (float)(im - (double)v.y));
+            v = make_float2((float)(x1 * d1 - x2 * d2), (float)(eta * (d2 - d1)));
         }
-        if (iw < nw) K[i] = make_float4(v.x, v.y, lo.x, lo.y);
+        if (iw < nw) K[i] = v;
         uint32_t q0, q1, q2;
         split3(v.x, v.y, q0, q1, q2);
         const long long o = 2LL * iw * ld + b;
@@ -631,9 +629,9 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(const __grid_constant
 }
 
 // ------------------------------------------------------------------ diagonal, Dyson step
-// Sd[b][G] = sum_t l_j |rho_t(G)|^2 as an FP32 pair: CTA (segment, 128 G)
+// Sd[b][G] = sum_t l_j |rho_t(G)|^2: CTA (segment, 128 G)
 __global__ void __launch_bounds__(128) k_pn_diag(int ngp, const int4* seg, const float* r2, const float* Lw, long long ldl,
-                                                 float2* Sd) {
+                                                 float* Sd) {
     __shared__ float l[PN_NODES][128];
     const int4 g = seg[blockIdx.x];
     const int G = blockIdx.y * 128 + threadIdx.x;
@@ -666,18 +664,15 @@ __global__ void __launch_bounds__(128) k_pn_diag(int ngp, const int4* seg, const
     }
     if (G < ngp)
 #pragma unroll
-        for (int j = 0; j < PN_NODES; ++j) {
-            const float h = (float)sum[j];
-            Sd[((size_t)blockIdx.x * PN_NODES + j) * ngp + G] = make_float2(h, (float)(sum[j] - (double)h));
-        }
+        for (int j = 0; j < PN_NODES; ++j) Sd[((size_t)blockIdx.x * PN_NODES + j) * ngp + G] = (float)sum[j];
 }
 
-// part[z][w][G] = sum over the nodes of range z of W(w; E_b) Sd[b][G]; CTA 32 w x 32 G, thread 2 x 2.  A few nodes next
-// to w carry most of the sum, so their roundings do not average out: both factors are pairs, sums of 32 in FP32.
-__global__ void __launch_bounds__(256) k_pn_diag_chi(int nw, int ng, int ngp, int nb, int per, const float4* K, long long ld,
-                                                     const float2* Sd, double2* part) {
-    __shared__ float4 Ks[32][33];
-    __shared__ float2 Rs[32][33];
+// part[z][w][G] = sum over the nodes of range z of W(w; E_b) Sd[b][G]; CTA 32 w x 32 G, thread 2 x 2, sums of
+// 32 in FP32 added in FP64 (factors as FP32 pairs changed nothing in the loss).
+__global__ void __launch_bounds__(256) k_pn_diag_chi(int nw, int ng, int ngp, int nb, int per, const float2* K, long long ld,
+                                                     const float* Sd, double2* part) {
+    __shared__ float2 Ks[32][33];
+    __shared__ float Rs[32][33];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int G0 = blockIdx.x * 32, w0 = blockIdx.y * 32;
     const int b_lo = blockIdx.z * per, b_hi = min(nb, b_lo + per);
@@ -690,27 +685,25 @@ __global__ void __launch_bounds__(256) k_pn_diag_chi(int nw, int ng, int ngp, in
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int i = threadIdx.x + 256 * r, a = i & 31, c = i >> 5;
-            Ks[a][c] = b0 + a < b_hi && w0 + c < nw ? K[(long long)(w0 + c) * ld + b0 + a] : make_float4(0.f, 0.f, 0.f, 0.f);
-            Rs[c][a] = b0 + c < b_hi && G0 + a < ng ? Sd[(size_t)(b0 + c) * ngp + G0 + a] : make_float2(0.f, 0.f);
+            Ks[a][c] = b0 + a < b_hi && w0 + c < nw ? K[(long long)(w0 + c) * ld + b0 + a] : make_float2(0.f, 0.f);
+            Rs[c][a] = b0 + c < b_hi && G0 + a < ng ? Sd[(size_t)(b0 + c) * ngp + G0 + a] : 0.f;
         }
         __syncthreads();
-        float2 acc[2][2], low[2][2];
+        float2 acc[2][2];
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
-            for (int j = 0; j < 2; ++j) acc[i][j] = low[i][j] = make_float2(0.f, 0.f);
+            for (int j = 0; j < 2; ++j) acc[i][j] = make_float2(0.f, 0.f);
 #pragma unroll 4
         for (int b = 0; b < 32; ++b) {
-            const float4 k[2] = {Ks[b][ty], Ks[b][ty + 16]};
-            const float2 r[2] = {Rs[b][tx], Rs[b][tx + 16]};
+            const float2 k[2] = {Ks[b][ty], Ks[b][ty + 16]};
+            const float r[2] = {Rs[b][tx], Rs[b][tx + 16]};
 #pragma unroll
             for (int i = 0; i < 2; ++i)
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    acc[i][j].x = fmaf(k[i].x, r[j].x, acc[i][j].x);
-                    acc[i][j].y = fmaf(k[i].y, r[j].x, acc[i][j].y);
-                    low[i][j].x = fmaf(k[i].x, r[j].y, fmaf(k[i].z, r[j].x, low[i][j].x));
-                    low[i][j].y = fmaf(k[i].y, r[j].y, fmaf(k[i].w, r[j].x, low[i][j].y));
+                    acc[i][j].x = fmaf(k[i].x, r[j], acc[i][j].x);
+                    acc[i][j].y = fmaf(k[i].y, r[j], acc[i][j].y);
                 }
         }
         __syncthreads();
@@ -718,8 +711,8 @@ __global__ void __launch_bounds__(256) k_pn_diag_chi(int nw, int ng, int ngp, in
         for (int i = 0; i < 2; ++i)
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-                sum[i][j].x += (double)acc[i][j].x + (double)low[i][j].x;
-                sum[i][j].y += (double)acc[i][j].y + (double)low[i][j].y;
+                sum[i][j].x += (double)acc[i][j].x;
+                sum[i][j].y += (double)acc[i][j].y;
             }
     }
 #pragma unroll
@@ -891,9 +884,9 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
     const int nz = std::max(1, std::min(16, nb / 256)), per = ((nb + nz - 1) / nz + 31) / 32 * 32;
     if (!fits(b.tr, sizeof(int) * (size_t)ldl) || !fits(b.Lw, sizeof(float) * PN_NODES * (size_t)ldl) ||
         !fits(b.tiles, 2 * tile_bytes) || !fits(b.r2, sizeof(float) * (size_t)ldl * ngp) ||
-        !fits(b.ktab, sizeof(float4) * (size_t)nw * ldk) || !fits(b.kplanes, 3 * kn * sizeof(__nv_bfloat16)) ||
+        !fits(b.ktab, sizeof(float2) * (size_t)nw * ldk) || !fits(b.kplanes, 3 * kn * sizeof(__nv_bfloat16)) ||
         !fits(b.splanes, 3 * sn * sizeof(__nv_bfloat16)) ||
-        !fits(b.Sd, sizeof(float2) * (size_t)nb * ngp) || !fits(b.part, sizeof(double2) * (size_t)nz * nw * ng) ||
+        !fits(b.Sd, sizeof(float) * (size_t)nb * ngp) || !fits(b.part, sizeof(double2) * (size_t)nz * nw * ng) ||
         !fits(b.chi, sizeof(double2) * (size_t)nw * ng * ng) || !fits(b.tp, sizeof(int2) * ntp))
         return give_up();
     std::vector<int2> tp;
@@ -910,10 +903,10 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
                                                             s.kp / 2, t0, t0 + tile_bytes, b.r2.as<float>());
     __nv_bfloat16* kp = b.kplanes.as<__nv_bfloat16>();
     k_pn_ktab<<<blocks((long long)mtiles * 64 * ldk, 256), 256, 0, st>>>(nw, mtiles * 128, ldk, nb, s.w.as<double>(), s.eta, seg,
-                                                                         e0, width, b.ktab.as<float4>(), kp, kp + kn, kp + 2 * kn);
-    k_pn_diag<<<dim3(nseg, (ngp + 127) / 128), 128, 0, st>>>(ngp, seg, b.r2.as<float>(), b.Lw.as<float>(), ldl, b.Sd.as<float2>());
-    k_pn_diag_chi<<<dim3((ng + 31) / 32, (nw + 31) / 32, nz), 256, 0, st>>>(nw, ng, ngp, nb, per, b.ktab.as<float4>(), ldk,
-                                                                            b.Sd.as<float2>(), b.part.as<double2>());
+                                                                         e0, width, b.ktab.as<float2>(), kp, kp + kn, kp + 2 * kn);
+    k_pn_diag<<<dim3(nseg, (ngp + 127) / 128), 128, 0, st>>>(ngp, seg, b.r2.as<float>(), b.Lw.as<float>(), ldl, b.Sd.as<float>());
+    k_pn_diag_chi<<<dim3((ng + 31) / 32, (nw + 31) / 32, nz), 256, 0, st>>>(nw, ng, ngp, nb, per, b.ktab.as<float2>(), ldk,
+                                                                            b.Sd.as<float>(), b.part.as<double2>());
     PgArgs a{};
     a.ng = ng;
     a.ngp = ngp;
