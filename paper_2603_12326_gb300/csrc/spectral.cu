@@ -39,6 +39,7 @@
 
 #include <climits>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 namespace {
@@ -68,13 +69,17 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
 // ------------------------------------------------------------------- grid and grouping
-// min and max of dE_t over the transitions of one q (one block)
-__global__ void __launch_bounds__(1024) k_spec_range(long long nt, int nv, int nc, const double* Ek,
-                                                     const double* Ekq, double* out) {
-    __shared__ double lo[1024], hi[1024];
+// min and max of dE_t over the transitions of one q: out[0] = least of the CTAs' order keys, out[1] = greatest (a key
+// orders like its double; one CTA alone took 71 us for 65536 transitions).  NaN energies are passed over, as fmin does.
+__device__ __forceinline__ unsigned long long order_key(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    return b >> 63 ? ~b : b | (1ull << 63);
+}
+__global__ void __launch_bounds__(256) k_spec_range(long long nt, int nv, int nc, const double* Ek,
+                                                    const double* Ekq, unsigned long long* out) {
     double mn = INFINITY, mx = -INFINITY;
     const int nvc = nv * nc;
-    for (long long t = threadIdx.x; t < nt; t += 1024) {
+    for (long long t = blockIdx.x * 256LL + threadIdx.x; t < nt; t += 256LL * gridDim.x) {
         const long long k = t / nvc;
         const int rem = (int)(t - k * nvc);
         const int v = rem / nc, c = rem - v * nc;
@@ -82,19 +87,13 @@ __global__ void __launch_bounds__(1024) k_spec_range(long long nt, int nv, int n
         mn = fmin(mn, dE);
         mx = fmax(mx, dE);
     }
-    lo[threadIdx.x] = mn;
-    hi[threadIdx.x] = mx;
-    __syncthreads();
-    for (int d = 512; d > 0; d >>= 1) {
-        if (threadIdx.x < d) {
-            lo[threadIdx.x] = fmin(lo[threadIdx.x], lo[threadIdx.x + d]);
-            hi[threadIdx.x] = fmax(hi[threadIdx.x], hi[threadIdx.x + d]);
-        }
-        __syncthreads();
+    for (int o = 16; o > 0; o >>= 1) {
+        mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+        mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     }
-    if (threadIdx.x == 0) {
-        out[0] = lo[0];
-        out[1] = hi[0];
+    if ((threadIdx.x & 31) == 0) {
+        atomicMin(out, order_key(mn));
+        atomicMax(out + 1, order_key(mx));
     }
 }
 
@@ -705,13 +704,20 @@ extern "C" qcx_status qcx_spectral_grid(qcx_ctx* ctx, int iq, double step, doubl
     cudaSetDevice(ctx->device);
     const long long nt = (long long)ctx->nk * ctx->nv * ctx->nc;
     CUDA_OR_FAIL(ctx->spec.range.ensure(2 * sizeof(double)), "alloc");
-    k_spec_range<<<1, 1024, 0, ctx->stream>>>(nt, ctx->nv, ctx->nc, ctx->d_Ek.as<double>(),
-                                              ctx->d_Ekq.as<double>() + (size_t)iq * ctx->nk * ctx->nc,
-                                              ctx->spec.range.as<double>());
+    unsigned long long* keys = ctx->spec.range.as<unsigned long long>();
+    CUDA_OR_FAIL(cudaMemsetAsync(keys, 0xff, sizeof(*keys), ctx->stream), "clear");
+    CUDA_OR_FAIL(cudaMemsetAsync(keys + 1, 0, sizeof(*keys), ctx->stream), "clear");
+    k_spec_range<<<nblk(nt, 256, 152), 256, 0, ctx->stream>>>(nt, ctx->nv, ctx->nc, ctx->d_Ek.as<double>(),
+                                                              ctx->d_Ekq.as<double>() + (size_t)iq * ctx->nk * ctx->nc, keys);
     CUDA_OR_FAIL(cudaGetLastError(), "range kernel");
+    unsigned long long got[2];
+    const CopyOut out = {got, 0, sizeof(got)};
+    CUDA_OR_FAIL(qcx_copy_out_all(ctx, ctx->spec.range.as<char>(), sizeof(got), &out, 1), "copy");
     double mm[2];
-    CUDA_OR_FAIL(cudaMemcpyAsync(mm, ctx->spec.range.p, sizeof(mm), cudaMemcpyDeviceToHost, ctx->stream), "copy");
-    CUDA_OR_FAIL(cudaStreamSynchronize(ctx->stream), "sync");
+    for (int i = 0; i < 2; ++i) {
+        const unsigned long long u = got[i] >> 63 ? got[i] & ~(1ull << 63) : ~got[i];
+        std::memcpy(&mm[i], &u, sizeof(u));
+    }
     if (!std::isfinite(mm[0]) || !std::isfinite(mm[1]))
         return ctx->fail(QCX_ERR_ARG, "spectral_grid: non-finite transition energies");
     const double e0 = step * std::floor(mm[0] / step) - step;
