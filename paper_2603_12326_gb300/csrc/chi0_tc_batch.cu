@@ -19,7 +19,7 @@
 // i mod grid), so hundreds of small instances cost one launch.  The shared
 // memory ring and the two TMEM accumulators keep their phases across tile
 // boundaries, so the TMA producer already streams the next tile while the
-// epilogue warps finish the current one.  Every instance of one q reads the
+// drain warps finish the current one.  Every instance of one q reads the
 // same BF16 planes (the pair densities of the union of that q's G sets,
 // sorted by |q+G| so that each instance's set is a prefix); the planes are
 // addressed through one tensor map per q and piece, all passed by value.  B
@@ -31,8 +31,15 @@
 
 namespace {
 
-constexpr int NTHREADS = 384;             // warps: 0 TMA, 1 and 10 MMA, 2-9 A/drain/epilogue, 11 idle
-constexpr int MMA_WARP2 = 10;
+// Roles and register budgets of the per-q kernel: warps 0 TMA, 1 and 2 MMA, 3 idle, 4-11 A generation, 12-19 drain and
+// epilogue (with both in the same eight warps the kernel waited for them: 2.07 -> 1.50 ms for 256 instances of N_G 19-339).
+constexpr int NTHREADS = 640;
+constexpr int LAUNCH_REGS = 96;
+constexpr int REG_CTRL = 40, REG_AGEN = 64, REG_DRAIN = 152;
+static_assert(128 * REG_CTRL + 256 * REG_AGEN + 256 * REG_DRAIN <= NTHREADS * LAUNCH_REGS,
+              "warpgroup register budgets exceed the launch allocation");
+constexpr int MMA_WARP2 = 2;
+constexpr int AGEN_WARP0 = 4, DRAIN_WARP0 = 12;
 constexpr int NSTAGE = 4;
 constexpr int NPA = 3;                    // BF16 terms of the A operand (W rho~)
 constexpr int NPB = 2;                    // BF16 terms of the B operand (rho~ = b0 + b1)
@@ -112,167 +119,119 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_chi0_tc_batch(const __grid_cons
     const uint32_t tmem = *tmem_slot;
     const int nwin = (a.kstages + a.promote - 1) / a.promote;
 
-    if (warp == 0) {
-        // ---------------------------------------------------------- TMA producer
-        if (lane == 0) {
-            int gs = 0;
-            int last = -1;
-            bool ok = true;
-            for (int ti = blockIdx.x; ti < a.ntile && ok; ti += gridDim.x) {
-                const int4 tl = a.tiles[ti];
-                const int nN = tl.w & 0xFFFF, src_b = tl.w >> 16;
-                const int slot = a.inst[tl.x].slot - a.slot0;
-                const int nbox = (nN + GBLK - 1) / GBLK;
-                const uint32_t bytes = (uint32_t)(NPB * nbox * GBLK * ROWB + (src_b ? 0 : NPB * SPIECE) +
-                                                  TPS * (int)sizeof(float2));
-                const float2* wrow = a.wtab + (size_t)tl.x * a.wld;
-                for (int it = 0; it < a.kstages; ++it, ++gs) {
-                    const int s = (int)(gs % NSTAGE);
-                    const uint32_t ph = (uint32_t)(gs / NSTAGE) & 1u;
-                    if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, a.status, a.wait_limit)) {
-                        ok = false;
-                        break;
-                    }
-                    unsigned char* st = base + s * STAGE_BYTES;
-                    uint64_t* fb = &full_b[gs % (2 * NSTAGE)];
-                    mbar_arrive_tx(fb, bytes);
-                    bulk_load(Wbuf + s * TPS, wrow + (size_t)it * TPS, TPS * sizeof(float2), fb);
-                    for (int p = 0; p < NPB; ++p)
-                        for (int r = 0; r < nbox; ++r)
-                            tma_load_2d(st + p * BREG + r * SPIECE, &maps.m[slot][p], fb, it * KSTEP,
-                                        tl.z + r * GBLK);
-                    if (!src_b) {
-                        unsigned char* sp = st + NPB * BREG;
-                        for (int p = 0; p < NPB; ++p)
-                            tma_load_2d(sp + p * SPIECE, &maps.m[slot][p], fb, it * KSTEP, tl.y * GBLK);
-                    }
-                    last = gs;
-                }
-            }
-            // let every copy still in flight (at most the last NSTAGE stages) land before the CTA can exit
-            for (int gs2 = max(0, last - NSTAGE + 1); gs2 <= last; ++gs2)
-                mbar_wait(&full_b[gs2 % (2 * NSTAGE)], (uint32_t)(gs2 / (2 * NSTAGE)) & 1u, abort_flag, a.status,
-                          CLEANUP_WAIT_LIMIT, false);
-        }
-    } else if (warp == 1 || warp == MMA_WARP2) {
-        // ---------------------------------------------------------- MMA issuers
-        // Two issuers take alternate accumulation windows (counted over the CTA's whole
-        // tile sequence), so one waits while the other's MMAs run.
-        if (lane == 0) {
-            const int par = warp == 1 ? 0 : 1;
-            bool ok = true;
-            for (int lt = 0; blockIdx.x + lt * gridDim.x < a.ntile && ok; ++lt) {
-                const int4 tl = a.tiles[blockIdx.x + lt * gridDim.x];
-                const uint32_t idesc = make_idesc(128, tl.w & 0xFFFF);
-                for (int wd = 0; wd < nwin && ok; ++wd) {
-                    const int gw = lt * nwin + wd;
-                    if ((gw & 1) != par) continue;
-                    const int b = gw & 1;
-                    if (gw >= 2 && !mbar_wait(&drained[b], (uint32_t)((gw - 2) >> 1) & 1u, abort_flag, a.status, a.wait_limit)) {
-                        ok = false;
-                        break;
-                    }
-                    const int it1 = min((wd + 1) * a.promote, a.kstages);
-                    for (int it = wd * a.promote; it < it1; ++it) {
-                        const int gs = lt * a.kstages + it;
-                        const int s = gs % NSTAGE;
-                        const bool first = it == wd * a.promote;
-                        // the A warps arrive only after they saw this stage's copies land
-                        if (!mbar_wait(&full_a[gs % (2 * NSTAGE)], (uint32_t)(gs / (2 * NSTAGE)) & 1u, abort_flag,
-                                       a.status, a.wait_limit)) {
+    if (warp < AGEN_WARP0) {
+        regs_dec<REG_CTRL>();
+        if (warp == 0) {
+            // ---------------------------------------------------------- TMA producer
+            if (lane == 0) {
+                int gs = 0;
+                int last = -1;
+                bool ok = true;
+                for (int ti = blockIdx.x; ti < a.ntile && ok; ti += gridDim.x) {
+                    const int4 tl = a.tiles[ti];
+                    const int nN = tl.w & 0xFFFF, src_b = tl.w >> 16;
+                    const int slot = a.inst[tl.x].slot - a.slot0;
+                    const int nbox = (nN + GBLK - 1) / GBLK;
+                    const uint32_t bytes = (uint32_t)(NPB * nbox * GBLK * ROWB + (src_b ? 0 : NPB * SPIECE) +
+                                                      TPS * (int)sizeof(float2));
+                    const float2* wrow = a.wtab + (size_t)tl.x * a.wld;
+                    for (int it = 0; it < a.kstages; ++it, ++gs) {
+                        const int s = (int)(gs % NSTAGE);
+                        const uint32_t ph = (uint32_t)(gs / NSTAGE) & 1u;
+                        if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, a.status, a.wait_limit)) {
                             ok = false;
                             break;
                         }
-                        tc_fence_after();
                         unsigned char* st = base + s * STAGE_BYTES;
-                        const uint32_t b0 = smem_u32(st), b1 = b0 + BREG;
-                        const uint32_t d = tmem + (uint32_t)b * ACC_OFF;
-                        const uint32_t a0 = smem_u32(st + NPB * BREG + NPB * SPIECE), a1 = a0 + ATILE,
-                                       a2 = a1 + ATILE;
-#pragma unroll
-                        for (int kk = 0; kk < KSTEP / 16; ++kk) {
-                            const uint32_t off = kk * 32;
-                            umma_bf16(d, sw64_desc(a0 + off), sw64_desc(b0 + off), idesc,
-                                      (first && kk == 0) ? 0u : 1u);
-                            umma_bf16(d, sw64_desc(a0 + off), sw64_desc(b1 + off), idesc, 1u);
-                            umma_bf16(d, sw64_desc(a1 + off), sw64_desc(b0 + off), idesc, 1u);
-                            umma_bf16(d, sw64_desc(a1 + off), sw64_desc(b1 + off), idesc, 1u);
-                            umma_bf16(d, sw64_desc(a2 + off), sw64_desc(b0 + off), idesc, 1u);
+                        uint64_t* fb = &full_b[gs % (2 * NSTAGE)];
+                        mbar_arrive_tx(fb, bytes);
+                        bulk_load(Wbuf + s * TPS, wrow + (size_t)it * TPS, TPS * sizeof(float2), fb);
+                        for (int p = 0; p < NPB; ++p)
+                            for (int r = 0; r < nbox; ++r)
+                                tma_load_2d(st + p * BREG + r * SPIECE, &maps.m[slot][p], fb, it * KSTEP,
+                                            tl.z + r * GBLK);
+                        if (!src_b) {
+                            unsigned char* sp = st + NPB * BREG;
+                            for (int p = 0; p < NPB; ++p)
+                                tma_load_2d(sp + p * SPIECE, &maps.m[slot][p], fb, it * KSTEP, tl.y * GBLK);
                         }
-                        umma_commit(&empty[s]);
+                        last = gs;
                     }
-                    if (ok) umma_commit(&acc_full[b]);
                 }
+                // let every copy still in flight (at most the last NSTAGE stages) land before the CTA can exit
+                for (int gs2 = max(0, last - NSTAGE + 1); gs2 <= last; ++gs2)
+                    mbar_wait(&full_b[gs2 % (2 * NSTAGE)], (uint32_t)(gs2 / (2 * NSTAGE)) & 1u, abort_flag, a.status,
+                              CLEANUP_WAIT_LIMIT, false);
             }
-            // no MMA of either issuer may still be running when TMEM is freed
-            umma_commit(mma_done);
-            mbar_wait(mma_done, 0, abort_flag, a.status, CLEANUP_WAIT_LIMIT, false);
+        } else if (warp == 1 || warp == MMA_WARP2) {
+            // ---------------------------------------------------------- MMA issuers
+            // Two issuers take alternate accumulation windows (counted over the CTA's whole
+            // tile sequence), so one waits while the other's MMAs run.
+            if (lane == 0) {
+                const int par = warp == 1 ? 0 : 1;
+                bool ok = true;
+                for (int lt = 0; blockIdx.x + lt * gridDim.x < a.ntile && ok; ++lt) {
+                    const int4 tl = a.tiles[blockIdx.x + lt * gridDim.x];
+                    const uint32_t idesc = make_idesc(128, tl.w & 0xFFFF);
+                    for (int wd = 0; wd < nwin && ok; ++wd) {
+                        const int gw = lt * nwin + wd;
+                        if ((gw & 1) != par) continue;
+                        const int b = gw & 1;
+                        if (gw >= 2 && !mbar_wait(&drained[b], (uint32_t)((gw - 2) >> 1) & 1u, abort_flag, a.status, a.wait_limit)) {
+                            ok = false;
+                            break;
+                        }
+                        const int it1 = min((wd + 1) * a.promote, a.kstages);
+                        for (int it = wd * a.promote; it < it1; ++it) {
+                            const int gs = lt * a.kstages + it;
+                            const int s = gs % NSTAGE;
+                            const bool first = it == wd * a.promote;
+                            // the A warps arrive only after they saw this stage's copies land
+                            if (!mbar_wait(&full_a[gs % (2 * NSTAGE)], (uint32_t)(gs / (2 * NSTAGE)) & 1u, abort_flag,
+                                           a.status, a.wait_limit)) {
+                                ok = false;
+                                break;
+                            }
+                            tc_fence_after();
+                            unsigned char* st = base + s * STAGE_BYTES;
+                            const uint32_t b0 = smem_u32(st), b1 = b0 + BREG;
+                            const uint32_t d = tmem + (uint32_t)b * ACC_OFF;
+                            const uint32_t a0 = smem_u32(st + NPB * BREG + NPB * SPIECE), a1 = a0 + ATILE,
+                                           a2 = a1 + ATILE;
+    #pragma unroll
+                            for (int kk = 0; kk < KSTEP / 16; ++kk) {
+                                const uint32_t off = kk * 32;
+                                umma_bf16(d, sw64_desc(a0 + off), sw64_desc(b0 + off), idesc,
+                                          (first && kk == 0) ? 0u : 1u);
+                                umma_bf16(d, sw64_desc(a0 + off), sw64_desc(b1 + off), idesc, 1u);
+                                umma_bf16(d, sw64_desc(a1 + off), sw64_desc(b0 + off), idesc, 1u);
+                                umma_bf16(d, sw64_desc(a1 + off), sw64_desc(b1 + off), idesc, 1u);
+                                umma_bf16(d, sw64_desc(a2 + off), sw64_desc(b0 + off), idesc, 1u);
+                            }
+                            umma_commit(&empty[s]);
+                        }
+                        if (ok) umma_commit(&acc_full[b]);
+                    }
+                }
+                // no MMA of either issuer may still be running when TMEM is freed
+                umma_commit(mma_done);
+                mbar_wait(mma_done, 0, abort_flag, a.status, CLEANUP_WAIT_LIMIT, false);
+            }
         }
-    } else if (warp < MMA_WARP2) {
-        // ------------------------- A generation, accumulator drain, epilogue
-        const int wi = warp - 2;
-        const int g = threadIdx.x - 64;
+    } else if (warp < DRAIN_WARP0) {
+        regs_dec<REG_AGEN>();
+        // ---------------------------------------------------------------- A generation
+        const int g = threadIdx.x - 32 * AGEN_WARP0;
         const int j = g & 3;
         const int go = g >> 2;
-        const int q = warp & 3, hc = wi >> 2;
-        const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-        const int row = q * 32 + lane;
-        float part[MAXHALF];
         bool ok = true;
         // all tiles have kstages stages and nwin windows, so the running stage and
         // window counters of this CTA follow from its local tile number lt
         for (int lt = 0; blockIdx.x + lt * gridDim.x < a.ntile && ok; ++lt) {
-            int nch8, row0, lim;
-            bool src_b;
-            {
-                const int4 tl = a.tiles[blockIdx.x + lt * gridDim.x];
-                src_b = (tl.w >> 16) != 0;
-                nch8 = (tl.w & 0xFFFF) >> 4;
-                lim = a.inst[tl.x].ng - tl.y * GBLK;    // G' rows of this block inside the instance
-                row0 = src_b ? tl.y * GBLK : 0;          // first source row in the staged tile
-            }
-            // register partials restart with every tile (dead across the epilogue)
-#pragma unroll
-            for (int i = 0; i < MAXHALF; ++i) part[i] = 0.0f;
-
-            auto drain = [&](int wd) -> bool {
-                const int gw = lt * nwin + wd;
-                const int b = gw & 1;
-                if (!warp_wait(&acc_full[b], (uint32_t)(gw >> 1) & 1u, abort_flag, a.status, a.wait_limit)) return false;
-                tc_fence_after();
-                const uint32_t tb = tmem + lane_off + (uint32_t)b * ACC_OFF + (uint32_t)(hc * nch8 * 8);
-#pragma unroll
-                for (int grp = 0; grp < MAXHALF / 16; ++grp) {
-                    uint32_t r[2][8];
-#pragma unroll
-                    for (int u = 0; u < 2; ++u)
-                        if (grp * 2 + u < nch8) tmem_ld8(tb + (uint32_t)((grp * 2 + u) * 8), r[u]);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int u = 0; u < 2; ++u)
-                        if (grp * 2 + u < nch8) {
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) part[(grp * 2 + u) * 8 + i] += __uint_as_float(r[u][i]);
-                        }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&drained[b]);
-                if (((wd + 1) * a.promote) % a.flush == 0 || wd + 1 == nwin) {
-                    // the first flush of a tile starts the FP64 sums
-                    const bool flushed = wd >= a.flush / a.promote;
-                    double* acc64 = a.acc64 + (size_t)blockIdx.x * 128 * NMAX + (size_t)(hc * nch8 * 8) * 128 + row;
-#pragma unroll
-                    for (int c = 0; c < MAXHALF; ++c) {
-                        if (c < nch8 * 8) {
-                            acc64[(size_t)c * 128] = (flushed ? acc64[(size_t)c * 128] : 0.0) + (double)part[c];
-                            part[c] = 0.0f;
-                        }
-                    }
-                }
-                return true;
-            };
-
+            const int4 tl = a.tiles[blockIdx.x + lt * gridDim.x];
+            const bool src_b = (tl.w >> 16) != 0;
+            const int lim = a.inst[tl.x].ng - tl.y * GBLK;    // G' rows of this block inside the instance
+            const int row0 = src_b ? tl.y * GBLK : 0;          // first source row in the staged tile
             for (int it = 0; it < a.kstages; ++it) {
                 const int gs = lt * a.kstages + it;
                 const int s = gs % NSTAGE;
@@ -320,35 +279,68 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_chi0_tc_batch(const __grid_cons
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&full_a[s2]);
-                // drain the previous window once this window's A tiles are queued; after the
-                // last stage drain whatever is left (one call site keeps the code compact)
-                int wd0 = nwin, wd1 = -1;
-                if (it % a.promote == a.promote - 1 && it >= a.promote) wd0 = wd1 = it / a.promote - 1;
-                if (it + 1 == a.kstages) {
-                    wd0 = min(wd0, (it % a.promote == a.promote - 1 && it >= a.promote) ? it / a.promote - 1
-                                                                                        : max(nwin - 2, 0));
-                    wd1 = nwin - 1;
+            }
+        }
+    } else {
+        regs_inc<REG_DRAIN>();
+        // ------------------------------------------------- accumulator drain, epilogue
+        const int q = warp & 3, hc = (warp - DRAIN_WARP0) >> 2;
+        const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+        const int row = q * 32 + lane;
+        float part[MAXHALF];
+        bool ok = true;
+        for (int lt = 0; blockIdx.x + lt * gridDim.x < a.ntile && ok; ++lt) {
+            const int4 tl = a.tiles[blockIdx.x + lt * gridDim.x];
+            const int nch8 = (tl.w & 0xFFFF) >> 4, half = nch8 * 8;
+            double* acc64 = a.acc64 + (size_t)blockIdx.x * 128 * NMAX + (size_t)(hc * half) * 128 + row;
+            int flushed = 0;                // the first flush of a tile starts the FP64 sums
+#pragma unroll
+            for (int i = 0; i < MAXHALF; ++i) part[i] = 0.0f;
+            for (int wd = 0; wd < nwin; ++wd) {
+                const int gw = lt * nwin + wd;
+                const int b = gw & 1;
+                if (!(ok = warp_wait(&acc_full[b], (uint32_t)(gw >> 1) & 1u, abort_flag, a.status, a.wait_limit))) break;
+                tc_fence_after();
+                const uint32_t tb = tmem + lane_off + (uint32_t)b * ACC_OFF + (uint32_t)(hc * half);
+#pragma unroll
+                for (int grp = 0; grp < MAXHALF / 16; ++grp) {
+                    uint32_t r[2][8];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+                        if (grp * 2 + u < nch8) tmem_ld8(tb + (uint32_t)((grp * 2 + u) * 8), r[u]);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+                        if (grp * 2 + u < nch8) {
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) part[(grp * 2 + u) * 8 + i] += __uint_as_float(r[u][i]);
+                        }
                 }
-                for (int wd = wd0; wd <= wd1 && ok; ++wd) ok = drain(wd);
-                if (!ok) break;
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&drained[b]);
+                if (((wd + 1) * a.promote) % a.flush == 0 || wd + 1 == nwin) {
+#pragma unroll
+                    for (int c = 0; c < MAXHALF; ++c) {
+                        if (c < half) {
+                            acc64[(size_t)c * 128] = (flushed ? acc64[(size_t)c * 128] : 0.0) + (double)part[c];
+                            part[c] = 0.0f;
+                        }
+                    }
+                    flushed = 1;
+                }
             }
             if (!ok) break;
             // ------------------------------------------------------------ epilogue
-            const int4 tl = a.tiles[blockIdx.x + lt * gridDim.x];
-            const int gb = tl.y, n0 = tl.z, half = (tl.w & 0xFFFF) >> 1, ng = a.inst[tl.x].ng;
-            const int cpart = row >> 6, gro = row & 63;
-            const int Gr = gb * GBLK + gro;
-            const double* acc64 = a.acc64 + (size_t)blockIdx.x * 128 * NMAX + (size_t)(hc * half) * 128 + row;
+            const int ng = a.inst[tl.x].ng, cpart = row >> 6, Gr = tl.y * GBLK + (row & 63);
             if (Gr < ng) {
                 const double* vs = a.inst[tl.x].vs;
-                const double vsp = vs[Gr];
+                const double vsp = vs[Gr] * a.pref;
                 double* plane = reinterpret_cast<double*>(a.eps + a.inst[tl.x].eps_off + (size_t)Gr * ng) + cpart;
-                for (int col = 0; col < half; ++col) {
-                    const int G = n0 + hc * half + col;
-                    if (G < ng) {
-                        const double ch = a.pref * acc64[(size_t)col * 128];
-                        plane[2 * G] = (cpart == 0 && G == Gr ? 1.0 : 0.0) - vsp * vs[G] * ch;
-                    }
+                for (int c = 0; c < half; ++c) {
+                    const int G = tl.z + hc * half + c;
+                    if (G < ng)
+                        plane[2 * G] = fma(-vsp * vs[G], acc64[(size_t)c * 128], cpart == 0 && G == Gr ? 1.0 : 0.0);
                 }
             }
         }
@@ -392,6 +384,10 @@ cudaError_t qcx_launch_chi0_tc_batch(cudaStream_t st, const CUtensorMap* maps, i
     cudaError_t e =
         cudaFuncSetAttribute((const void*)k_chi0_tc_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
     if (e != cudaSuccess) return e;
+    // the register budgets assume this launch allocation (see k_chi0_tc)
+    cudaFuncAttributes fa;
+    if ((e = cudaFuncGetAttributes(&fa, (const void*)k_chi0_tc_batch)) != cudaSuccess) return e;
+    if (fa.numRegs != LAUNCH_REGS) return cudaErrorNotSupported;
     k_chi0_tc_batch<<<grid, NTHREADS, SMEM_BYTES, st>>>(ms, a);
     return cudaGetLastError();
 }
