@@ -708,18 +708,22 @@ static cudaError_t invert_batch(cudaStream_t st, int n, int nmat, const double2*
 }
 
 // Matrices are inverted in groups whose second copy stays within INV_COPY_BYTES (at least one), so that the scratch
-// does not grow with the number of frequencies.
+// does not grow with the number of frequencies; where even that does not fit, in smaller groups.
 constexpr size_t INV_COPY_BYTES = 1ull << 30;
 template <typename C> static int inv_group(int n, int nw) {
     return (int)std::min<size_t>({(size_t)nw, std::max<size_t>(1, INV_COPY_BYTES / ((size_t)n * n * sizeof(C))), 32768});
 }
 
 template <typename T>
-static cudaError_t invert_all(qcx_ctx* ctx, QSlot& s, double* norms, double* L) {
+static cudaError_t invert_all(qcx_ctx* ctx, QSlot& s, double* norms, double* L, int& per) {
     using C = cplx<T>;
     const int n = s.ng, nw = s.nw;
-    const int per = inv_group<C>(n, nw);
-    cudaError_t e = s.work2.ensure((size_t)per * n * n * sizeof(C));
+    cudaError_t e;
+    per = inv_group<C>(n, nw);
+    while ((e = s.work2.ensure((size_t)per * n * n * sizeof(C))) == cudaErrorMemoryAllocation && per > 1) {
+        cudaGetLastError();
+        per /= 2;
+    }
     if (e != cudaSuccess) return e;
     e = s.gjaux.ensure((size_t)per * n * (InvCfg<T>::PB * sizeof(C) + 2 * sizeof(int)));
     if (e != cudaSuccess) return e;
@@ -737,8 +741,9 @@ static cudaError_t invert_all(qcx_ctx* ctx, QSlot& s, double* norms, double* L) 
 
 cudaError_t qcx_launch_invert(qcx_ctx* ctx, QSlot& s, qcx_precision prec, double* d_loss_out) {
     const int n = s.ng;
+    int per = 1;
     if (prec == QCX_FP64) {
-        cudaError_t e = invert_all<double>(ctx, s, nullptr, d_loss_out);
+        cudaError_t e = invert_all<double>(ctx, s, nullptr, d_loss_out, per);
         if (e != cudaSuccess) return e;
         return cudaMemsetAsync(s.resid.p, 0, sizeof(double) * s.nw, ctx->stream);
     }
@@ -747,7 +752,7 @@ cudaError_t qcx_launch_invert(qcx_ctx* ctx, QSlot& s, qcx_precision prec, double
     double* norms = s.kappa1.as<double>();
     e = cudaMemsetAsync(norms, 0, 2 * sizeof(double) * s.nw, ctx->stream);
     if (e != cudaSuccess) return e;
-    e = invert_all<float>(ctx, s, norms, d_loss_out);
+    e = invert_all<float>(ctx, s, norms, d_loss_out, per);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(s.resid.p, 0, sizeof(double) * s.nw, ctx->stream);
     if (e != cudaSuccess) return e;
@@ -763,9 +768,8 @@ cudaError_t qcx_launch_invert(qcx_ctx* ctx, QSlot& s, qcx_precision prec, double
                                                                         s.resid.as<double>());
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int per = inv_group<float2>(n, s.nw);          // B takes the inverse's second copy, group by group
     const int t32 = (n + 31) / 32;
-    for (int w0 = 0; w0 < s.nw; w0 += per) {
+    for (int w0 = 0; w0 < s.nw; w0 += per) {             // B takes the inverse's second copy, group by group
         const int m = std::min(per, s.nw - w0);
         const size_t o = (size_t)w0 * n;
         k_form_b<<<dim3(t32, t32, m), 256, 0, ctx->stream>>>(n, s.eps.as<double2>() + o * n, s.flags.as<int>() + w0, norms + w0,
