@@ -29,7 +29,7 @@
 // k_pn_gram is k_chi0_tc (same roles, same stage) made persistent over (segment, G' block, G chunk, node): segments are
 // ~15 stages long, so the drain warps write one item's S while the next one's MMAs run.  A tile holds the columns from
 // its own G' block on, which is what the Hermitian half needs.
-// Measured (one q, 200 w, N_t = 65536, N_G = 181): chi0 14.8 -> 3.5 ms (S 1.5, contraction with W 1.0, gather 0.3);
+// Measured (one q, 200 w, N_t = 65536, N_G = 181): chi0 14.8 -> 3.5 ms (S 1.5, contraction with W 1.0, gather 0.15);
 // 100 w, N_t = 57344, N_G = 531: 56 -> 24 ms.
 #include "qcx_internal.h"
 #include "tc_ptx.cuh"
@@ -45,6 +45,7 @@ constexpr int PN_SEG = 2048;                // transitions per segment (64 accum
 constexpr int PN_TPS = KSTEP / 2;           // transitions per K stage
 constexpr int PN_MAXPANELS = 65536;
 constexpr int PN_CHUNK_NODES = 4096;        // nodes contracted with W in one FP32 chain
+constexpr size_t GATHER_BYTES = 48ull << 20; // rows of rho~ that the gather reads together (the L2 has 129 MB)
 constexpr size_t PN_BYTES = 4ull << 30;     // S of a chunk of segments
 
 // ------------------------------------------------------------------ energies, sort, plan
@@ -261,15 +262,20 @@ __global__ void __launch_bounds__(128) k_pn_weights(const int4* seg, const int* 
 }
 
 // rho~ (first two planes) into stage tiles [stage][ngp rows][64 bytes], 64-byte swizzle, and |rho|^2 (three planes) as
-// [transition][ngp].  Thread: 4 transitions of one G; a warp covers 8 G, so its writes are contiguous.
-__global__ void __launch_bounds__(256) k_pn_gather(int ngp, long long nchunk, const int* tr, const uint32_t* p0,
+// [transition][ngp].  Thread: 4 transitions of one G; a warp covers 8 G, so its writes are contiguous.  Sorted
+// transitions lie anywhere in a row of rho~, so the 4-byte reads use a sector eight times over the whole pass: G is
+// walked in groups of 2^lg rows whose three planes stay in the L2 while all stages read them.
+// One q, N_t = 65536, N_G = 181: all rows at once 336 us, groups of 32 148 us.
+__global__ void __launch_bounds__(256) k_pn_gather(int ngp, int lg, long long nst, const int* tr, const uint32_t* p0,
                                                    const uint32_t* p1, const uint32_t* p2, long long kp2,
                                                    unsigned char* t0, unsigned char* t1, float* r2) {
-    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < nchunk; i += 256LL * gridDim.x) {
+    const long long per = nst << lg, n = ((ngp + (1 << lg) - 1) >> lg) * per * 4;
+    for (long long i = blockIdx.x * 256LL + threadIdx.x; i < n; i += 256LL * gridDim.x) {
         const int j = (int)(i & 3);
-        const long long row = i >> 2;
-        const int G = (int)(row % ngp);
-        const long long st = row / ngp;
+        const long long grp = (i >> 2) / per, row = (i >> 2) - grp * per;
+        const int G = (int)(grp << lg) + (int)(row & ((1 << lg) - 1));
+        const long long st = row >> lg;
+        if (G >= ngp) continue;
         const int4 t = *reinterpret_cast<const int4*>(tr + st * PN_TPS + 4 * j);
         const int tt[4] = {t.x, t.y, t.z, t.w};
         uint32_t a[4], b[4];
@@ -899,7 +905,10 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
     const uint32_t* p0 = reinterpret_cast<const uint32_t*>(s.rho.p);
     const size_t plane = (size_t)ngp * (s.kp / 2);
     unsigned char* t0 = b.tiles.as<unsigned char>();
-    k_pn_gather<<<blocks(nst * ngp * 4, 256), 256, 0, st>>>(ngp, nst * ngp * 4, b.tr.as<int>(), p0, p0 + plane, p0 + 2 * plane,
+    int lg = 5;                                              // 8 rows at least: a warp's writes stay contiguous
+    while (lg > 3 && (size_t)(s.kp / 2) * 12 << lg > GATHER_BYTES) --lg;
+    const long long grows = (ngp + (1 << lg) - 1) >> lg << lg;
+    k_pn_gather<<<blocks(nst * grows * 4, 256), 256, 0, st>>>(ngp, lg, nst, b.tr.as<int>(), p0, p0 + plane, p0 + 2 * plane,
                                                             s.kp / 2, t0, t0 + tile_bytes, b.r2.as<float>());
     __nv_bfloat16* kp = b.kplanes.as<__nv_bfloat16>();
     k_pn_ktab<<<blocks((long long)mtiles * 64 * ldk, 256), 256, 0, st>>>(nw, mtiles * 128, ldk, nb, s.w.as<double>(), s.eta, seg,
