@@ -27,10 +27,10 @@
 // k_pn_gram, which writes S as BF16 planes; contraction with W; diagonal; Dyson step.
 //
 // k_pn_gram is k_chi0_tc (same roles, same stage) made persistent over (segment, G' block, G chunk, node): segments are
-// ~15 stages long, so the drain warps write one item's S while the next one's MMAs run.  A tile holds the columns from
-// its own G' block on, which is what the Hermitian half needs.
-// Measured (one q, 200 w, N_t = 65536, N_G = 181): chi0 14.8 -> 3.5 ms (S 1.5, contraction with W 1.0, gather 0.15);
-// 100 w, N_t = 57344, N_G = 531: 56 -> 24 ms.
+// ~15 stages long, so the drain warps write one item's S while the next one's MMAs run.  Tiles cover each pair of G'
+// blocks once (pair_cover): a stage's time is the ring's latency, not its MMAs, so fewer and wider tiles win.
+// Measured (one q, 200 w, N_t = 65536, N_G = 181): chi0 14.8 -> 2.9 ms (S 1.2, contraction with W 1.0, gather 0.15);
+// 100 w, N_t = 57344, N_G = 531: 56 -> 21 ms.
 #include "qcx_internal.h"
 #include "tc_ptx.cuh"
 
@@ -333,7 +333,7 @@ constexpr int PG_REG_CTRL = 40, PG_REG_AGEN = 64, PG_REG_DRAIN = 152;
 static_assert(128 * PG_REG_CTRL + 256 * PG_REG_AGEN + 256 * PG_REG_DRAIN <= PG_THREADS * PG_LAUNCH_REGS,
               "warpgroup register budgets exceed the launch allocation");
 constexpr int PG_MMA2 = 2, PG_AGEN0 = 4, PG_DRAIN0 = 12;
-constexpr int PG_NSTAGE = 4;
+constexpr int PG_NSTAGE = 4;                // ring at least; one more stage where the shared memory holds it
 constexpr int PG_PROMOTE = 2;
 constexpr int PG_NMAX = 128;                // columns of a tile at most
 constexpr int PG_MAXHALF = PG_NMAX / 2;
@@ -378,7 +378,7 @@ __device__ __forceinline__ PgItem pg_item(const PgArgs& a, int it) {
     return r;
 }
 
-__global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(const __grid_constant__ PgArgs a) {
+template <int NST> __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(const __grid_constant__ PgArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -386,24 +386,24 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(const __grid_constant
     const uint32_t splane = a.with_src ? (uint32_t)PG_GBLK * ROWB : 0u;
     const uint32_t aoff = 2 * (bplane + splane);
     const uint32_t stage_bytes = aoff + 3 * PG_ATILE;
-    unsigned char* tail = base + PG_NSTAGE * stage_bytes;
-    float* Lbuf = reinterpret_cast<float*>(tail);                 // [NSTAGE][16]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(tail + PG_NSTAGE * PN_TPS * sizeof(float));
-    uint64_t* full_b = bars;                                       // [2 NSTAGE] by stage mod 2 NSTAGE (see k_chi0_tc)
-    uint64_t* full_a = bars + 2 * PG_NSTAGE;                       // [2 NSTAGE]
-    uint64_t* empty = bars + 4 * PG_NSTAGE;                        // [NSTAGE]
-    uint64_t* acc_full = bars + 5 * PG_NSTAGE;                     // [2]
+    unsigned char* tail = base + NST * stage_bytes;
+    float* Lbuf = reinterpret_cast<float*>(tail);                 // [NST][16]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(tail + NST * PN_TPS * sizeof(float));
+    uint64_t* full_b = bars;                                       // [2 NST] by stage mod 2 NST (see k_chi0_tc)
+    uint64_t* full_a = bars + 2 * NST;                       // [2 NST]
+    uint64_t* empty = bars + 4 * NST;                        // [NST]
+    uint64_t* acc_full = bars + 5 * NST;                     // [2]
     uint64_t* drained = acc_full + 2;                              // [2]
     uint64_t* mma_done = drained + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mma_done + 1);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < 2 * PG_NSTAGE; ++s) {
+        for (int s = 0; s < 2 * NST; ++s) {
             mbar_init(&full_b[s], 1);
             mbar_init(&full_a[s], 8);
         }
-        for (int s = 0; s < PG_NSTAGE; ++s) mbar_init(&empty[s], 1);
+        for (int s = 0; s < NST; ++s) mbar_init(&empty[s], 1);
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
             mbar_init(&drained[b], 8);
@@ -429,20 +429,25 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(const __grid_constant
                 for (int im = blockIdx.x; im < nitem && ok; im += gridDim.x) {
                     const PgItem m = pg_item(a, im);
                     const uint32_t bb = (uint32_t)m.n * ROWB;
+                    const uint32_t b1 = (uint32_t)min(m.n, a.ngp - m.n0) * ROWB;   // the columns wrap around ngp
                     const uint32_t sb = m.from_b ? 0u : (uint32_t)min(PG_GBLK, a.ngp - m.gb * PG_GBLK) * ROWB;
                     for (int it = 0; it < m.nst; ++it, ++gs) {
-                        const int s = gs % PG_NSTAGE;
-                        if (!(ok = mbar_wait(&empty[s], ((uint32_t)(gs / PG_NSTAGE) & 1u) ^ 1u, abort_flag, a.status,
+                        const int s = gs % NST;
+                        if (!(ok = mbar_wait(&empty[s], ((uint32_t)(gs / NST) & 1u) ^ 1u, abort_flag, a.status,
                                              a.wait_limit)))
                             break;
-                        uint64_t* fb = &full_b[gs % (2 * PG_NSTAGE)];
+                        uint64_t* fb = &full_b[gs % (2 * NST)];
                         unsigned char* st = base + s * stage_bytes;
                         const size_t stage = (size_t)(m.stage0 + it);
-                        const size_t row = (stage * a.ngp + m.n0) * ROWB;
+                        const size_t top = stage * a.ngp * ROWB, row = top + (size_t)m.n0 * ROWB;
                         mbar_arrive_tx(fb, 2 * (bb + sb) + PN_TPS * (uint32_t)sizeof(float));
                         bulk_load(Lbuf + s * PN_TPS, a.Lw + m.node * a.ldl + stage * PN_TPS, PN_TPS * sizeof(float), fb);
-                        bulk_load(st, a.t0 + row, bb, fb);
-                        bulk_load(st + bplane, a.t1 + row, bb, fb);
+                        bulk_load(st, a.t0 + row, b1, fb);
+                        bulk_load(st + bplane, a.t1 + row, b1, fb);
+                        if (b1 < bb) {
+                            bulk_load(st + b1, a.t0 + top, bb - b1, fb);
+                            bulk_load(st + bplane + b1, a.t1 + top, bb - b1, fb);
+                        }
                         if (sb) {
                             const size_t src = (stage * a.ngp + (size_t)m.gb * PG_GBLK) * ROWB;
                             bulk_load(st + 2 * bplane, a.t0 + src, sb, fb);
@@ -451,8 +456,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(const __grid_constant
                     }
                 }
                 // every copy in flight lands before the CTA can exit
-                for (int it = max(0, gs - PG_NSTAGE); it < gs; ++it)
-                    mbar_wait(&full_b[it % (2 * PG_NSTAGE)], (uint32_t)(it / (2 * PG_NSTAGE)) & 1u, abort_flag, a.status,
+                for (int it = max(0, gs - NST); it < gs; ++it)
+                    mbar_wait(&full_b[it % (2 * NST)], (uint32_t)(it / (2 * NST)) & 1u, abort_flag, a.status,
                               CLEANUP_WAIT_LIMIT, false);
             }
         } else if (warp == 1 || warp == PG_MMA2) {
@@ -476,8 +481,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(const __grid_constant
                         const uint32_t d = tmem + (uint32_t)par * PG_NMAX, dl = d + 2 * PG_NMAX;
                         const bool first = it0 < 2 * PG_PROMOTE;       // this issuer's first window of the item
                         for (int u = 0; u < len; ++u, ++gs) {
-                            const int s = gs % PG_NSTAGE;
-                            if (!(ok = mbar_wait(&full_a[gs % (2 * PG_NSTAGE)], (uint32_t)(gs / (2 * PG_NSTAGE)) & 1u,
+                            const int s = gs % NST;
+                            if (!(ok = mbar_wait(&full_a[gs % (2 * NST)], (uint32_t)(gs / (2 * NST)) & 1u,
                                                  abort_flag, a.status, a.wait_limit)))
                                 break;
                             tc_fence_after();
@@ -515,8 +520,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(const __grid_constant
             const bool on = m.gb * PG_GBLK + go < a.ng;
             const uint32_t src = m.from_b ? 0u : 2 * bplane, src_plane = m.from_b ? bplane : splane;
             for (int it = 0; it < m.nst; ++it, ++gs) {
-                const int s = gs % PG_NSTAGE, s2 = gs % (2 * PG_NSTAGE);
-                if (!(ok = warp_wait(&full_b[s2], (uint32_t)(gs / (2 * PG_NSTAGE)) & 1u, abort_flag, a.status, a.wait_limit)))
+                const int s = gs % NST, s2 = gs % (2 * NST);
+                if (!(ok = warp_wait(&full_b[s2], (uint32_t)(gs / (2 * NST)) & 1u, abort_flag, a.status, a.wait_limit)))
                     break;
                 unsigned char* st = base + s * stage_bytes;
                 uint32_t re0[4] = {0, 0, 0, 0}, re1[4] = {0, 0, 0, 0}, re2[4] = {0, 0, 0, 0};
@@ -600,27 +605,41 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(const __grid_constant
                 if (lane == 0) mbar_arrive(&drained[b]);
             }
             if (!ok) break;
-            // S of this item in three BF16 terms: the warp's 32 rows are one 32-tile of G'.  Two columns at a time, even
-            // lanes writing the first as pairs of rows, odd lanes the second
-            const int gi = m.gb * 2 + (q & 1);                     // G' tile
+            // S of this item in three BF16 terms: the warp's 32 rows are one 32-tile of G'.  Above the diagonal two
+            // columns at a time, even lanes writing the first as pairs of rows, odd lanes the second; below it (another
+            // block's columns, wrapped) the conjugate, eight columns of a row at a time
+            const int gi = m.gb * 2 + (q & 1), part_im = q >> 1;   // G' tile; real or imaginary rows
             if (gi < a.npair_row) {
-                __nv_bfloat16* S = a.S + ((size_t)m.slot * PN_NODES + m.node) * a.ncol + (q >> 1) * 32 + (lane & ~1);
+                __nv_bfloat16* S = a.S + ((size_t)m.slot * PN_NODES + m.node) * a.ncol + part_im * 32;
                 const int c0 = m.n0 + hc * half;
 #pragma unroll
-                for (int c = 0; c < PG_MAXHALF; c += 2) {
+                for (int c = 0; c < PG_MAXHALF; c += 8) {
                     if (c >= half) break;
-                    const bool odd = lane & 1;
-                    const float other = __shfl_xor_sync(0xffffffffu, odd ? part[c] : part[c + 1], 1);
-                    const float lo = odd ? other : part[c], hi_ = odd ? part[c + 1] : other;
-                    const int G = c0 + c + (odd ? 1 : 0), hi = G >> 5;
+                    const int G0 = c0 + c < a.ngp ? c0 + c : c0 + c - a.ngp, hi = G0 >> 5;
                     if (hi >= gi) {
                         const int p = gi * a.npair_row - gi * (gi - 1) / 2 + hi - gi;
-                        uint32_t s0, s1, s2;
-                        split3(lo, hi_, s0, s1, s2);
-                        uint32_t* o = reinterpret_cast<uint32_t*>(S + (size_t)(p * 32 + (G & 31)) * 64);
-                        o[0] = s0;
-                        o[a.plane / 2] = s1;
-                        o[a.plane] = s2;
+                        const bool odd = lane & 1;
+                        uint32_t* o = reinterpret_cast<uint32_t*>(S + (size_t)(p * 32 + (G0 & 31) + (odd ? 1 : 0)) * 64 + (lane & ~1));
+#pragma unroll
+                        for (int u = 0; u < 8; u += 2, o += 64) {
+                            const float other = __shfl_xor_sync(0xffffffffu, odd ? part[c + u] : part[c + u + 1], 1);
+                            uint32_t s0, s1, s2;
+                            split3(odd ? other : part[c + u], odd ? part[c + u + 1] : other, s0, s1, s2);
+                            o[0] = s0;
+                            o[a.plane / 2] = s1;
+                            o[a.plane] = s2;
+                        }
+                    } else if (hi >> 1 != m.gb) {
+                        const int p = hi * a.npair_row - hi * (hi - 1) / 2 + gi - hi;
+                        const float sg = part_im ? -1.0f : 1.0f;
+                        uint32_t s0[4], s1[4], s2[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            split3(sg * part[c + 2 * u], sg * part[c + 2 * u + 1], s0[u], s1[u], s2[u]);
+                        uint4* o = reinterpret_cast<uint4*>(S + (size_t)(p * 32 + lane) * 64 + (G0 & 31));
+                        o[0] = make_uint4(s0[0], s0[1], s0[2], s0[3]);
+                        o[a.plane / 8] = make_uint4(s1[0], s1[1], s1[2], s1[3]);
+                        o[a.plane / 4] = make_uint4(s2[0], s2[1], s2[2], s2[3]);
                     }
                 }
             }
@@ -783,6 +802,26 @@ static double panel_us(const QSlot& s, long long nt, double stages, double segs,
     return gram + kk + bytes / 3e6 + 200.0;
 }
 
+// The pairs of G' blocks as tiles {G' block, first column, columns (wrapping around ngp), A rows from B}: either every
+// block with the columns from its own on (the upper triangle), or with its own and the next floor(blocks / 2) around the
+// circle (the pairs half way around an even circle once).  The time of a tile hardly depends on its width, so the one
+// with fewer tiles: around the circle for 3 blocks (3 against 4: one q, N_G = 181, 1508 -> 1224 us with the deeper ring) and for 7 and 11 or more of
+// an odd number.  Tiles that hold their own rows also need no copy of them, which leaves room for a fifth stage.
+static std::vector<int4> pair_cover(int ng, int ngp) {
+    const int nb = (ng + PG_GBLK - 1) / PG_GBLK;
+    std::vector<int4> cover[2];
+    for (int gb = 0; gb < nb; ++gb)
+        for (int ring = 0; ring < 2; ++ring) {
+            const int up = ring ? nb / 2 - (nb % 2 == 0 && gb >= nb / 2) : nb - 1 - gb;      // further blocks
+            const int end = (gb + up) % nb;                                                  // the last of them
+            const int len = std::min(ngp, (end + 1) * PG_GBLK) - gb * PG_GBLK + (gb + up >= nb ? ngp : 0);
+            const int nch = (len + PG_NMAX - 1) / PG_NMAX, step = ((len + nch - 1) / nch + 15) / 16 * 16;
+            for (int c = 0; c < len; c += step)
+                cover[ring].push_back(make_int4(gb, (gb * PG_GBLK + c) % ngp, std::min(step, len - c), c == 0));
+        }
+    return cover[cover[1].size() < cover[0].size()];
+}
+
 // Tries the panel route.  *used = false (and cudaSuccess) when the direct kernel is to run instead: the estimate above is
 // not better, the energies are not finite or span too many panels, or the work space does not fit.
 cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi, int* d_status, bool* used) {
@@ -794,18 +833,12 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
     if (direct < 600.0 || ctx->withhold_copies) return cudaSuccess;
     const int T32 = (ng + 31) / 32, ntp = T32 * (T32 + 1) / 2;
     if (nw > 65535 || ntp * 16 > 65535) return cudaSuccess;      // grid limits
-    // G' blocks x column chunks of the upper triangle
-    std::vector<int4> tiles;
+    const std::vector<int4> tiles = pair_cover(ng, ngp);
     int n_max = 16;
     bool with_src = false;
-    for (int gb = 0; gb * PG_GBLK < ng; ++gb) {
-        const int len = ngp - gb * PG_GBLK, nch = (len + PG_NMAX - 1) / PG_NMAX;
-        const int step = ((len + nch - 1) / nch + 15) / 16 * 16;
-        for (int c = 0; c < len; c += step) {
-            tiles.push_back(make_int4(gb, gb * PG_GBLK + c, std::min(step, len - c), c == 0));
-            n_max = std::max(n_max, std::min(step, len - c));
-            with_src |= c != 0;
-        }
+    for (const int4& t : tiles) {
+        n_max = std::max(n_max, t.z);
+        with_src |= !t.w;
     }
     const int ntile = (int)tiles.size();
     if (panel_us(s, nt, (double)nt / PN_TPS, 1.0, ntile) >= 0.8 * direct) return cudaSuccess;
@@ -933,14 +966,19 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
     a.S = b.splanes.as<__nv_bfloat16>();
     a.status = d_status;
     a.wait_limit = ctx->wait_limit;
-    const size_t smem = 1024 + PG_NSTAGE * (size_t)(2 * (n_max + (with_src ? PG_GBLK : 0)) * ROWB + 3 * PG_ATILE) +
-                        PG_NSTAGE * PN_TPS * sizeof(float) + (5 * PG_NSTAGE + 5) * sizeof(uint64_t) + 16;
+    auto ring_bytes = [&](size_t nst) {
+        return 1024 + nst * (2 * (n_max + (with_src ? PG_GBLK : 0)) * ROWB + 3 * PG_ATILE + PN_TPS * sizeof(float)) +
+               (5 * nst + 5) * sizeof(uint64_t) + 16;
+    };
+    const bool deep = ring_bytes(PG_NSTAGE + 1) <= PG_SMEM_LIMIT;
+    const size_t smem = ring_bytes(PG_NSTAGE + deep);
+    const auto gram = deep ? k_pn_gram<PG_NSTAGE + 1> : k_pn_gram<PG_NSTAGE>;
     if (smem > PG_SMEM_LIMIT) return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute((const void*)k_pn_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute((const void*)gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
     // the register budgets assume this launch allocation (see k_chi0_tc)
     cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, (const void*)k_pn_gram)) != cudaSuccess) return e;
+    if ((e = cudaFuncGetAttributes(&fa, (const void*)gram)) != cudaSuccess) return e;
     if (fa.numRegs != PG_LAUNCH_REGS) return cudaErrorNotSupported;
     CUtensorMap kmaps[3], smaps[3];
     __nv_bfloat16* sp = b.splanes.as<__nv_bfloat16>();
@@ -953,7 +991,7 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
         if (m <= 0) break;
         a.seg = seg + s0;
         a.nseg = m;
-        k_pn_gram<<<std::min(152, m * ntile * PN_NODES), PG_THREADS, smem, st>>>(a);
+        gram<<<std::min(152, m * ntile * PN_NODES), PG_THREADS, smem, st>>>(a);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         // an odd number of segments leaves 16 points of the last stage
         for (int i = 0; i < 3 && m * PN_NODES % KSTEP; ++i)
