@@ -28,8 +28,10 @@
 //
 // k_pn_gram is k_chi0_tc (same roles, same stage) made persistent over (segment, G' block, G chunk, node): segments are
 // ~15 stages long, so the drain warps write one item's S while the next one's MMAs run.  Tiles cover each pair of G'
-// blocks once (pair_cover): a stage's time is the ring's latency, not its MMAs, so fewer and wider tiles win.
-// Measured (one q, 200 w, N_t = 65536, N_G = 181): chi0 14.8 -> 2.9 ms (S 1.2, contraction with W 1.0, gather 0.15);
+// blocks once (pair_cover).  A stage of 128 columns takes ~1680 cycles: 640 of MMA issue, ~1020 of shared-memory traffic
+// (operands of the MMAs 80 KB, A tiles written 24 KB, copies and reads 24 KB at 128 B per cycle), the rest the ring's
+// hand-overs, so fewer and wider tiles win.
+// Measured (one q, 200 w, N_t = 65536, N_G = 181): chi0 14.8 -> 2.9 ms (S 1.19, contraction with W 1.03, gather 0.15);
 // 100 w, N_t = 57344, N_G = 531: 56 -> 21 ms.
 #include "qcx_internal.h"
 #include "tc_ptx.cuh"
@@ -335,6 +337,7 @@ static_assert(128 * PG_REG_CTRL + 256 * PG_REG_AGEN + 256 * PG_REG_DRAIN <= PG_T
 constexpr int PG_MMA2 = 2, PG_AGEN0 = 4, PG_DRAIN0 = 12;
 constexpr int PG_NSTAGE = 4;                // ring at least; one more stage where the shared memory holds it
 constexpr int PG_PROMOTE = 2;
+constexpr int PG_AWARPS = 4;                // warps that form one stage's A tiles (two such groups)
 constexpr int PG_NMAX = 128;                // columns of a tile at most
 constexpr int PG_MAXHALF = PG_NMAX / 2;
 constexpr int PG_GBLK = 64;
@@ -401,7 +404,7 @@ template <int NST> __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(co
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2 * NST; ++s) {
             mbar_init(&full_b[s], 1);
-            mbar_init(&full_a[s], 8);
+            mbar_init(&full_a[s], PG_AWARPS);
         }
         for (int s = 0; s < NST; ++s) mbar_init(&empty[s], 1);
         for (int b = 0; b < 2; ++b) {
@@ -510,44 +513,49 @@ template <int NST> __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(co
         }
     } else if (warp < PG_DRAIN0) {
         regs_dec<PG_REG_AGEN>();
-        const int g = threadIdx.x - 32 * PG_AGEN0;
-        const int j = g & 3, go = g >> 2;                          // 4 transitions of G' row go
-        const uint32_t coff = sw64_off(go, j), o_re = coff, o_im = sw64_off(64 + go, j);
+        // A stage takes a warp mostly latency (its wait, loads, fence), so two groups of four warps take alternate stages
+        // (eight warps on every stage: 1224 us where this takes 1186, N_G = 181; 10.8 and 10.3 ms, N_G = 531)
+        const int g = threadIdx.x - 32 * PG_AGEN0, group = g / (32 * PG_AWARPS);
+        const int j = g & 3, go = (g >> 2) & 31;                   // 4 transitions of G' rows go and go + 32
         int gs = 0;
         bool ok = true;
         for (int im = blockIdx.x; im < nitem && ok; im += gridDim.x) {
             const PgItem m = pg_item(a, im);
-            const bool on = m.gb * PG_GBLK + go < a.ng;
             const uint32_t src = m.from_b ? 0u : 2 * bplane, src_plane = m.from_b ? bplane : splane;
             for (int it = 0; it < m.nst; ++it, ++gs) {
+                if ((gs & 1) != group) continue;
                 const int s = gs % NST, s2 = gs % (2 * NST);
                 if (!(ok = warp_wait(&full_b[s2], (uint32_t)(gs / (2 * NST)) & 1u, abort_flag, a.status, a.wait_limit)))
                     break;
                 unsigned char* st = base + s * stage_bytes;
-                uint32_t re0[4] = {0, 0, 0, 0}, re1[4] = {0, 0, 0, 0}, re2[4] = {0, 0, 0, 0};
-                uint32_t im0[4] = {0, 0, 0, 0}, im1[4] = {0, 0, 0, 0}, im2[4] = {0, 0, 0, 0};
-                if (on) {
-                    const uint4 h0 = *reinterpret_cast<const uint4*>(st + src + coff);
-                    const uint4 h1 = *reinterpret_cast<const uint4*>(st + src + src_plane + coff);
-                    const float4 l = reinterpret_cast<const float4*>(Lbuf + s * PN_TPS)[j];
-                    const uint32_t v0[4] = {h0.x, h0.y, h0.z, h0.w}, v1[4] = {h1.x, h1.y, h1.z, h1.w};
-                    const float lv[4] = {l.x, l.y, l.z, l.w};
+                const float4 l = reinterpret_cast<const float4*>(Lbuf + s * PN_TPS)[j];
+                const float lv[4] = {l.x, l.y, l.z, l.w};
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float2 f0 = bf2(v0[q]), f1 = bf2(v1[q]);   // rho~ = f0 + f1 is exact in FP32
-                        split3(lv[q] * (f0.x + f1.x), lv[q] * (f0.y + f1.y), re0[q], re1[q], re2[q]);
-                        im0[q] = perm_im(re0[q]);
-                        im1[q] = perm_im(re1[q]);
-                        im2[q] = perm_im(re2[q]);
+                for (int r = 0; r < 2; ++r) {
+                    const int row = go + 32 * r;
+                    uint32_t re0[4] = {0, 0, 0, 0}, re1[4] = {0, 0, 0, 0}, re2[4] = {0, 0, 0, 0};
+                    if (m.gb * PG_GBLK + row < a.ng) {
+                        const uint32_t coff = src + sw64_off(row, j);
+                        const uint4 h0 = *reinterpret_cast<const uint4*>(st + coff);
+                        const uint4 h1 = *reinterpret_cast<const uint4*>(st + src_plane + coff);
+                        const uint32_t v0[4] = {h0.x, h0.y, h0.z, h0.w}, v1[4] = {h1.x, h1.y, h1.z, h1.w};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float2 f0 = bf2(v0[q]), f1 = bf2(v1[q]);   // rho~ = f0 + f1 is exact in FP32
+                            split3(lv[q] * (f0.x + f1.x), lv[q] * (f0.y + f1.y), re0[q], re1[q], re2[q]);
+                        }
                     }
+                    unsigned char* o_re = st + aoff + sw64_off(row, j);
+                    unsigned char* o_im = st + aoff + sw64_off(64 + row, j);
+                    *reinterpret_cast<uint4*>(o_re) = make_uint4(re0[0], re0[1], re0[2], re0[3]);
+                    *reinterpret_cast<uint4*>(o_re + PG_ATILE) = make_uint4(re1[0], re1[1], re1[2], re1[3]);
+                    *reinterpret_cast<uint4*>(o_re + 2 * PG_ATILE) = make_uint4(re2[0], re2[1], re2[2], re2[3]);
+                    *reinterpret_cast<uint4*>(o_im) = make_uint4(perm_im(re0[0]), perm_im(re0[1]), perm_im(re0[2]), perm_im(re0[3]));
+                    *reinterpret_cast<uint4*>(o_im + PG_ATILE) =
+                        make_uint4(perm_im(re1[0]), perm_im(re1[1]), perm_im(re1[2]), perm_im(re1[3]));
+                    *reinterpret_cast<uint4*>(o_im + 2 * PG_ATILE) =
+                        make_uint4(perm_im(re2[0]), perm_im(re2[1]), perm_im(re2[2]), perm_im(re2[3]));
                 }
-                unsigned char* ap = st + aoff;
-                *reinterpret_cast<uint4*>(ap + o_re) = make_uint4(re0[0], re0[1], re0[2], re0[3]);
-                *reinterpret_cast<uint4*>(ap + PG_ATILE + o_re) = make_uint4(re1[0], re1[1], re1[2], re1[3]);
-                *reinterpret_cast<uint4*>(ap + 2 * PG_ATILE + o_re) = make_uint4(re2[0], re2[1], re2[2], re2[3]);
-                *reinterpret_cast<uint4*>(ap + o_im) = make_uint4(im0[0], im0[1], im0[2], im0[3]);
-                *reinterpret_cast<uint4*>(ap + PG_ATILE + o_im) = make_uint4(im1[0], im1[1], im1[2], im1[3]);
-                *reinterpret_cast<uint4*>(ap + 2 * PG_ATILE + o_im) = make_uint4(im2[0], im2[1], im2[2], im2[3]);
                 fence_async_smem();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&full_a[s2]);
