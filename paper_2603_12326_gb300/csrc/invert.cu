@@ -542,7 +542,8 @@ __global__ void __launch_bounds__(128) k_refine_diag(int n, int nw, int nk, cons
 // conj(X_jl).  B being Hermitian, the k tiles above an l tile's own count twice and those
 // below it are left out, half the product.  Bound by the FP32 pipe; with 32 x 32 tiles, all
 // of B and its FP64 source read again by every row block: 200 matrices of 181 660 -> 280 us,
-// 100 of 531 7.0 -> 2.3 ms.
+// 100 of 531 7.0 -> 2.2 ms.  k_form_b is bound by the FP64 pipe (two sums and two conversions per element) and forms only
+// the tiles the form reads.
 constexpr int QF = 64, QK = 16;
 __global__ void __launch_bounds__(256) k_form_b(int n, const double2* Aall, const int* flags, const double* norms,
                                                 const double* xnorms, double kappa_refine, float2* Ball) {
@@ -553,6 +554,7 @@ __global__ void __launch_bounds__(256) k_form_b(int n, const double2* Aall, cons
     float2* B = Ball + (size_t)b * n * n;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     const int k0 = blockIdx.y * 32, l0 = blockIdx.x * 32;
+    if (k0 >= (l0 / QF + 1) * QF) return;                  // below the l tile of the form, which leaves it out
     for (int r = ty; r < 32; r += 8)
         if (l0 + r < n && k0 + tx < n) At[r][tx] = A[(size_t)(l0 + r) * n + k0 + tx];
     __syncthreads();
@@ -560,7 +562,8 @@ __global__ void __launch_bounds__(256) k_form_b(int n, const double2* Aall, cons
         const int k = k0 + r, l = l0 + tx;
         if (k < n && l < n) {
             const double2 akl = A[(size_t)k * n + l], alk = At[tx][r];
-            B[(size_t)k * n + l] = make_float2((float)(0.5 * (akl.y + alk.y)), (float)(-0.5 * (akl.x - alk.x)));
+            // halved after the conversion: exact, and not on the FP64 pipe
+            B[(size_t)k * n + l] = make_float2(0.5f * (float)(akl.y + alk.y), -0.5f * (float)(akl.x - alk.x));
         }
     }
 }
