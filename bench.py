@@ -31,14 +31,6 @@ import numpy as np
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-# DRAM bytes (read + write) of one k_chi0_tc launch over 1 q x 200 w of the mid workload, from one ncu capture
-# of `bench.py --profile-case mid200` (dram__bytes_read.sum + dram__bytes_write.sum), and the commit of the kernel
-# source it was taken at; None once the kernel has changed since.
-CHI0_TRAFFIC = {"bytes": 719207680 + 182851072, "commit": "1fa000c"}
-# Executed FP32 flops of one k_pair_density_fused launch over 1 q of the mid workload (512 k x 181 G), from the
-# ncu thread-instruction counters of `bench.py --profile-case mid` (2 FFMA + FADD + FMUL,
-# smsp__sass_thread_inst_executed_op_{ffma,fadd,fmul}_pred_on.sum), and the commit of the kernel source.
-PD_FP32_FLOPS = {"flops": 2 * 26974224384 + 3570466816 + 10942709760, "commit": "1fa000c"}
 METRIC = "eps^-1 (q,w) blocks/s vs FP64 plain GPU path at <=1e-4 rel err; tensor-pipe %"
 WORKLOAD = ("mid: diamond a=5.43 A, 12 sp shells/atom (N_b=96), 8x8x8 k, N_v=4, N_c=32 (N_t=65536), "
             "N_G=181, 50 q x 200 w on 0-60 eV, eta=0.1 eV")
@@ -130,6 +122,15 @@ def _config(ws, precision, blocks_per_step=10000):
     """The workload both arms report (the reference arm adds its own precision)."""
     return {"workload": WORKLOAD, "blocks_per_step": blocks_per_step, "l2": "inputs larger than L2 (no flush)",
             "precision": precision, "parallelism": f"q shards x {ws}"}
+
+
+def _panel_flops(prob, iq, eta, nw, ng):
+    """Flops that chi0 of one q needs in energy panels (16 nodes on each panel of width 4 eta/3 that holds a
+    transition): one (G <= G') contraction of the transitions per node, one of the nodes per frequency; 4 FMA
+    per complex multiply-add."""
+    dE = (np.asarray(prob.Ekq[iq])[:, None, :] - np.asarray(prob.Ek)[:, :, None]).ravel()
+    nodes = 16 * len(np.unique(np.floor((dE - dE.min()) / (4.0 * eta / 3.0))))
+    return 4.0 * (16.0 * dE.size + float(nw) * nodes) * ng * (ng + 1)
 
 
 def _weak_value(nq, nw, steps, ws, ms_max):
@@ -231,7 +232,8 @@ def run_ours(args, ws, rank, local):
     edges = np.linspace(0.0, 12.0, 121)          # |q+G| bins, bohr^-1
     halo = qcx.halo_params()
     nt = prob.nt
-    pref_flops = 8.0 * nt * ng * ng * nw          # algorithmic chi0 flops per q (one launch)
+    pref_flops = 8.0 * nt * ng * ng * nw          # flops of the direct frequency sum per q
+    pan_flops = float(np.mean([_panel_flops(prob, iq, eta, nw, ng) for iq in range(nq)]))
 
     chi_events = []
     pd_events = []
@@ -295,7 +297,7 @@ def run_ours(args, ws, rank, local):
     chi_avg = float(np.mean(chi_ms))
     pd_avg = float(np.mean([a.elapsed_time(b) for a, b in pd_events]))
     peaks = _peaks()
-    achieved = pref_flops / (chi_avg / 1e3) / 1e12
+    achieved = pan_flops / (chi_avg / 1e3) / 1e12
     peak = peaks.get("bf16_tflops_sustained", 1700.0)
 
     # ------------------------------------------------------ end to end (host buffers)
@@ -392,38 +394,30 @@ def run_ours(args, ws, rank, local):
                "seconds": round(secs, 2)}
 
     if rank == 0:
-        # per q: G setup, the two pair-density tables, pair densities, W table, chi0, chi0 diagonal without
-        # cancellation (two kernels), Gauss-Jordan, FP64 diagonal correction, loss by the quadratic form, |q+G|,
-        # the dielectric values kept for 3-D binning; per step two binnings and two rate + recoil pairs
-        launches_per_step = nq * 13 + 2 + 4
+        # per q (counted with the profiler): pair densities 4 (G setup, tables, Y, rho), chi0 in energy panels 19, inverse
+        # and losses 17 (six panels of the elimination); per step two binnings and two rate + recoil pairs
+        launches_per_step = nq * 40 + 2 + 4
         out = {"metric": METRIC, "value": value, "unit": "blocks/s", "n_gpus": ws, "steps": args.steps,
                "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True, "scaling": "weak",
                "vs_baseline": None, "dtype": "bf16",
                "data": "synthetic (seeded states shaped like the paper's workloads)",
-               "config": _config(ws, "chi0 as split-BF16 tcgen05 products: rho~ (two BF16 terms of the FP32 "
-                                     "pair densities) against W rho~ in three terms, five products, FP32 "
-                                     "accumulation restarted every 20 MMAs and FP64 partial sums, diagonal summed "
-                                     "again in FP32; inverse FP32 + FP64 diagonal correction; rate FP64", nq * nw),
+               "config": _config(ws, "chi0 in energy panels (16 Chebyshev nodes per 4 eta/3) as split-BF16 tcgen05 "
+                                     "products: rho~ (two BF16 terms of the FP32 pair densities) against l rho~ in "
+                                     "three terms, W against S in three terms each; leading product in its own FP32 "
+                                     "accumulator, node chunks added in FP64, diagonal summed again in FP32; inverse "
+                                     "FP32 + FP64 diagonal correction; rate FP64", nq * nw),
                "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                             "frac": achieved / peak,
-                            "traffic": CHI0_TRAFFIC["bytes"] if CHI0_TRAFFIC else None,
-                            "traffic_source": (f"ncu dram__bytes_read.sum + dram__bytes_write.sum of one k_chi0_tc "
-                                               f"launch of 1 q x 200 w at commit {CHI0_TRAFFIC['commit']}"
-                                               if CHI0_TRAFFIC else "not retaken since the kernel changed"),
-                            "kernel": "k_chi0_tc", "flops_per_launch": pref_flops,
+                            "kernel": "qcx_chi0: energy panels (k_pn_gram, k_spec_kk_tc) and the passes around them",
+                            "flops_per_launch": pan_flops,
+                            "flops_note": "needed by the panels' contractions; each multiply-add is five or six BF16 "
+                                          "products on the tensor cores",
+                            "direct_sum_flops": pref_flops,
+                            "direct_sum_equivalent_tflops": pref_flops / (chi_avg / 1e3) / 1e12,
                             "avg_launch_ms": chi_avg,
                             "peak_source": "bf16_tflops_sustained of measured (MEASURED_PEAKS.json)"},
-               "pair_density": {"kernel": "k_pair_density_fused", "avg_launch_ms": pd_avg, "bound": "alu",
-                                "fp32_flops_per_launch": PD_FP32_FLOPS["flops"] if PD_FP32_FLOPS else None,
-                                "fp32_flops_source": (f"ncu FFMA/FADD/FMUL thread-instruction counts of one launch "
-                                                      f"(1 q), kernel at commit {PD_FP32_FLOPS['commit']}"
-                                                      if PD_FP32_FLOPS else "not recounted since the kernel changed"),
-                                "achieved_tflops": (PD_FP32_FLOPS["flops"] / (pd_avg / 1e3) / 1e12
-                                                    if PD_FP32_FLOPS else None),
-                                "fp32_peak_tflops": fma.get("fp32_tflops"),
-                                "frac": (PD_FP32_FLOPS["flops"] / (pd_avg / 1e3) / 1e12 / fma["fp32_tflops"]
-                                         if fma.get("fp32_tflops") and PD_FP32_FLOPS else None),
-                                "peak_source": "FFMA microbenchmark measured in this run (libqcx_peaks)",
+               "pair_density": {"kernel": "k_pd_y, k_pd_rho (k_pd_axis_table before them)", "avg_launch_ms": pd_avg,
+                                "bound": "alu", "fp32_peak_tflops": fma.get("fp32_tflops"),
                                 "algorithmic_bytes": pd_bytes, "achieved_GBs": pd_bytes / (pd_avg / 1e3) / 1e9,
                                 "hbm_peak_GBs": peaks.get("hbm_gbs", 6800.0),
                                 "hbm_frac": pd_bytes / (pd_avg / 1e3) / 1e9 / peaks.get("hbm_gbs", 6800.0),
@@ -433,7 +427,8 @@ def run_ours(args, ws, rank, local):
                "fp64_gpu": {"value": fp64_value, "unit": "blocks/s",
                             "sample": f"1 q: FP64 pair densities amortised over {nw} w + FP64 chi0/inverse "
                                       f"for {nw64} w",
-                            "chi0_kernel": "k_chi0_fp64", "chi0_ms": chi64_ms, "chi0_tflops": chi64_tflops,
+                            "chi0_kernel": "k_oz_gemm (FP64 as integer slices on the tensor cores, so the "
+                                           "rate can pass the DFMA peak)", "chi0_ms": chi64_ms, "chi0_tflops": chi64_tflops,
                             "fp64_peak_tflops": fma.get("fp64_tflops"),
                             "chi0_frac_of_fp64_peak": (chi64_tflops / fma["fp64_tflops"]
                                                        if fma.get("fp64_tflops") else None),
@@ -601,9 +596,9 @@ def spectral_leg(ctx, prob, G, w, eta, stream, fma, nq_spec=10, frac=20, nsample
             "value": nq_spec * nw / (ms / 1e3), "unit": "blocks/s",
             "ms_per_q": ms / nq_spec,
             "precision": "FP32 pair densities and weights; contraction on tcgen05 in three-term split BF16 "
-                         "(FP32 sums restarted every 24 MMAs, chunks added in FP64); grid and K in FP64; inverse as "
+                         "(leading product restarted every 4 MMAs, chunks added in FP64); grid and K in FP64; inverse as "
                          "the mixed direct path",
-            "contraction": {"kernel": "k_spec_kk_tc (with the K-major split of the weights, k_spec_s_split)",
+            "contraction": {"kernel": "k_spec_kk_tc",
                             "bound": "tensor", "ms_per_q": kk / nq_spec,
                             "weights_ms_per_q": float(np.sum(wt_ms)) / nq_spec,
                             "flops": "4 FMA per (w, grid point, G <= G') pair",
@@ -729,6 +724,7 @@ def large_leg(stream, nq=2, nk_oracle=8):
     ms = ev[0].elapsed_time(ev[1])
     chi_ms = float(np.mean([a.elapsed_time(b) for a, b in chi]))
     flops = 8.0 * nt * ng * ng * nw
+    pflops = _panel_flops(p, 0, p.eta, nw, ng)
     peak = _peaks().get("bf16_tflops_sustained", 1700.0)
     edges = np.linspace(0.0, 16.0, 161)
     halo = qcx.halo_params()
@@ -756,9 +752,10 @@ def large_leg(stream, nq=2, nk_oracle=8):
     return {"workload": "large: diamond a=5.43 A, 18 sp shells/atom up to 5000 bohr^-2 (N_b=144), 12x12x12 k, "
                         "N_v=14, N_c=64 (N_t=1548288), N_G=531, 400 w on 0-100 eV, eta=0.05 eV",
             "q_timed": nq, "value": nq * nw / (ms / 1e3), "unit": "blocks/s", "ms_per_q": ms / nq,
-            "chi0": {"kernel": "k_chi0_tc", "avg_launch_ms": chi_ms, "flops_per_launch": flops,
-                     "achieved_tflops": flops / (chi_ms / 1e3) / 1e12, "peak": peak,
-                     "frac": flops / (chi_ms / 1e3) / 1e12 / peak,
+            "chi0": {"kernel": "qcx_chi0: energy panels (k_pn_gram, k_spec_kk_tc)", "avg_launch_ms": chi_ms,
+                     "flops_per_launch": pflops, "achieved_tflops": pflops / (chi_ms / 1e3) / 1e12, "peak": peak,
+                     "frac": pflops / (chi_ms / 1e3) / 1e12 / peak,
+                     "direct_sum_equivalent_tflops": flops / (chi_ms / 1e3) / 1e12,
                      "peak_source": "bf16_tflops_sustained of measured (MEASURED_PEAKS.json)"},
             "recoil_spectrum_events_per_kg_yr": [float(x) for x in dQ],
             "recoil_spectrum_note": f"FP64 rate over the |q+G| bins of the {nq} timed q (heavy mediator, "
