@@ -355,8 +355,10 @@ __global__ void __launch_bounds__(PR_ROWS) k_inv_panel_reg(InvShape sh, int p_, 
 
 // The other columns (see above).  Grid (column tile, row tile, matrix); thread (tx, ty) holds rows ty 4 .. + 3 and
 // columns tx + 16 u of a 64 x 64 tile, the panel's multipliers and pivot rows staged once in shared memory.
+// FP32: four CTAs per SM (64 registers with the loop unrolled by two; three, unrolled by four: 357 us where this takes
+// 332, 200 matrices of N_G = 181).
 template <typename T>
-__global__ void __launch_bounds__(256) k_inv_update(InvShape sh, int p, cplx<T>* X, cplx<T>* B2, const cplx<T>* M,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_inv_update(InvShape sh, int p, cplx<T>* X, cplx<T>* B2, const cplx<T>* M,
                                                     const int* perm, const int* rows, const int* flags) {
     using C = cplx<T>;
     constexpr int PB = InvCfg<T>::PB;
@@ -380,18 +382,11 @@ __global__ void __launch_bounds__(256) k_inv_update(InvShape sh, int p, cplx<T>*
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     C acc[4][4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const int i = i0 + ty * 4 + r;
-        const bool keep = i < n && (i < k0 || i >= k0 + nb);
-        const C* s = src + (keep ? (size_t)perm[i] * n : 0);
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int j = j0 + tx + 16 * u;
-            acc[r][u] = keep && j < n ? s[j] : mk<T>(0, 0);
-        }
-    }
+        for (int u = 0; u < 4; ++u) acc[r][u] = mk<T>(0, 0);
     __syncthreads();
-#pragma unroll 4
+#pragma unroll 2
     for (int c = 0; c < nb; ++c) {
         C m[4], x[4];
 #pragma unroll
@@ -402,6 +397,22 @@ __global__ void __launch_bounds__(256) k_inv_update(InvShape sh, int p, cplx<T>*
         for (int r = 0; r < 4; ++r)
 #pragma unroll
             for (int u = 0; u < 4; ++u) cfma(acc[r][u], m[r], x[u]);
+    }
+    // the products are summed from zero and meet the old element once: one rounding at its size per panel, not nb (the
+    // inverse's part of the loss error 1.23e-6 -> 1.10e-6 and 1.11e-6 -> 0.91e-6 on two q of N_G = 181)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int i = i0 + ty * 4 + r;
+        if (i >= n || (i >= k0 && i < k0 + nb)) continue;
+        const C* s = src + (size_t)perm[i] * n;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = j0 + tx + 16 * u;
+            if (j >= n) continue;
+            const C v = s[j];
+            acc[r][u].x += v.x;
+            acc[r][u].y += v.y;
+        }
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -543,7 +554,7 @@ __global__ void __launch_bounds__(128) k_refine_diag(int n, int nw, int nk, cons
 // below it are left out, half the product.  Bound by the FP32 pipe; with 32 x 32 tiles, all
 // of B and its FP64 source read again by every row block: 200 matrices of 181 660 -> 280 us,
 // 100 of 531 7.0 -> 2.2 ms.  k_form_b is bound by the FP64 pipe (two sums and two conversions per element) and forms only
-// the tiles the form reads.
+// the tiles the form reads (200 of 181: 95 -> 52 us; 100 of 531: 357 -> 160).
 constexpr int QF = 64, QK = 16;
 __global__ void __launch_bounds__(256) k_form_b(int n, const double2* Aall, const int* flags, const double* norms,
                                                 const double* xnorms, double kappa_refine, float2* Ball) {
