@@ -291,7 +291,7 @@ qcx_status qcx_set_states(qcx_ctx* ctx, int nk, const double* kpts, int nv, cons
     CUDA_OR_FAIL(cudaGetLastError(), "convert states");
     ++ctx->gen;
     ctx->kpts_h = kh;
-    ctx->kcls = qcx_axis_classes(kh.data(), nk);
+    for (qcx_precision prec : {QCX_FP64, QCX_MIXED}) ctx->kcls[prec] = qcx_axis_classes(kh.data(), nk, ctx->h, prec);
     ctx->nk = nk;
     ctx->nv = nv;
     ctx->nc = nc;

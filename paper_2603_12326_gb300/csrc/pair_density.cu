@@ -1053,9 +1053,12 @@ cudaError_t qcx_launch_qsetup(qcx_ctx* ctx, QSlot& s, const int* d_G, int ng, co
     return cudaGetLastError();
 }
 
-// Classes of the components v[3 i + x] of n points along axis x: values equal to a class's first
-// value within 1e-9 (relative) share it; idx[3 i + x] receives the class, vals the float values.
-static void axis_classes(const double* v, int n, int x, std::vector<double>& vals, std::vector<int>& idx) {
+// Classes of the components v[3 i + x] of n points along axis x: values that are equal but for rounding share one; idx[3 i + x]
+// receives the class, vals the middle of its values.  A class reaches `width` from its first value, relative to the larger
+// of that value and a full turn's 2 pi/h.  FP64: 8 units in the last place, which holds the rounding of a regular grid's
+// components (sums of three terms; 6 units were enough for 2^3 to 16^3 grids on SC, FCC and BCC, shifted or not, and
+// 600 G), so that no point moves by more than the rounding of its own phase.  FP32: 1e-9, far below its rounding.
+static void axis_classes(const double* v, int n, int x, double h, double width, std::vector<double>& vals, std::vector<int>& idx) {
     std::vector<int> ord(n);
     for (int i = 0; i < n; ++i) ord[i] = i;
     std::sort(ord.begin(), ord.end(), [&](int i, int j) { return v[3 * i + x] < v[3 * j + x]; });
@@ -1063,16 +1066,17 @@ static void axis_classes(const double* v, int n, int x, std::vector<double>& val
     double first = 0.0;
     for (int j = 0; j < n; ++j) {
         const double d = v[3 * ord[j] + x];
-        if (cls < 0 || fabs(d - first) > 1e-9 * fmax(1.0, fabs(d))) {
+        if (cls < 0 || fabs(d - first) > width * fmax(2.0 * M_PI / h, fabs(d))) {
             ++cls;
             first = d;
             vals.push_back(d);
         }
+        vals.back() = first + 0.5 * (d - first);
         idx[3 * ord[j] + x] = cls;
     }
 }
 
-AxisClasses qcx_axis_classes(const double* v, int n) {
+AxisClasses qcx_axis_classes(const double* v, int n, double h, qcx_precision prec) {
     AxisClasses c;
     c.finite = true;
     for (int i = 0; i < 3 * n; ++i) c.finite = c.finite && std::isfinite(v[i]);
@@ -1080,7 +1084,7 @@ AxisClasses qcx_axis_classes(const double* v, int n) {
     c.idx.resize(3 * (size_t)n);
     for (int x = 0; x < 3; ++x) {
         c.ofs[x] = (int)c.val.size();
-        axis_classes(v, n, x, c.val, c.idx);
+        axis_classes(v, n, x, h, prec == QCX_FP64 ? 8.0 * 0x1p-52 : 1e-9, c.val, c.idx);
         c.n[x] = (int)c.val.size() - c.ofs[x];
     }
     return c;
@@ -1088,11 +1092,12 @@ AxisClasses qcx_axis_classes(const double* v, int n) {
 
 // Classes and buffers of the tables for nk k points and ng values of q+G (host arrays); leaves t invalid when the
 // tables would not save work or exceed their memory budget.
-static cudaError_t tab_prepare(qcx_ctx* ctx, PdTab& t, const AxisClasses& kc, int nk, const double* kap, int ng, size_t elem,
-                               size_t y_per_k) {
+static cudaError_t tab_prepare(qcx_ctx* ctx, PdTab& t, const AxisClasses& kc, int nk, const double* kap, int ng,
+                               qcx_precision prec, size_t y_per_k) {
     t.valid = false;
     if (!kc.finite) return cudaSuccess;
-    const AxisClasses gc = qcx_axis_classes(kap, ng);
+    const size_t elem = prec == QCX_FP64 ? sizeof(double2) : sizeof(float2);
+    const AxisClasses gc = qcx_axis_classes(kap, ng, ctx->h, prec);
     if (!gc.finite) return cudaSuccess;
     const int npair = ctx->ngrp * ctx->ngrp;
     long long cells = 0;
@@ -1162,7 +1167,7 @@ cudaError_t qcx_pd_tab_prepare(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng
             kap[3 * g + x] = v;
         }
     const size_t elem = prec == QCX_FP64 ? sizeof(double2) : sizeof(float2);
-    return tab_prepare(ctx, s.pdt, ctx->kcls, nk, kap.data(), ng, elem, pd_y_per_k(ctx->nb, ctx->nv, ng, elem));
+    return tab_prepare(ctx, s.pdt, ctx->kcls[prec], nk, kap.data(), ng, prec, pd_y_per_k(ctx->nb, ctx->nv, ng, elem));
 }
 
 cudaError_t qcx_launch_pair_density(qcx_ctx* ctx, QSlot& s, int iq, qcx_precision prec) {
@@ -1264,7 +1269,7 @@ cudaError_t qcx_launch_overlap(qcx_ctx* ctx, int nk, const double* d_kpts, const
     a.Sout = d_out;
     const double zero[3] = {0.0, 0.0, 0.0};
     if (nk <= 65535) {
-        const cudaError_t e = tab_prepare(ctx, ctx->overlap_tab, qcx_axis_classes(k_host, nk), nk, zero, 1, sizeof(double2), 0);
+        const cudaError_t e = tab_prepare(ctx, ctx->overlap_tab, qcx_axis_classes(k_host, nk, ctx->h, QCX_FP64), nk, zero, 1, QCX_FP64, 0);
         if (e != cudaSuccess) return e;
         if (ctx->overlap_tab.valid) {
             const dim3 grid(((ctx->ngrp + 1) / 2 * (ctx->ngrp + 1) + 127) / 128, nk);

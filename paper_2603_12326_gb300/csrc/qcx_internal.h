@@ -250,7 +250,7 @@ struct qcx_ctx {
     int nk = 0, nv = 0, nc = 0, nq = 0;
     std::vector<double> qpts;  // host copy
     std::vector<double> kpts_h;    // host copy [nk][3]
-    AxisClasses kcls;              // its classes (kept with the states: every q's tables use them)
+    AxisClasses kcls[2];           // its classes by precision (kept with the states: every q's tables use them)
     DevBuf d_kpts, d_kpts32;   // [nk][3]
     DevBuf d_Ck64, d_Ck32;     // [nk][nb][nv]
     DevBuf d_Ek;               // [nk][nv]
@@ -336,7 +336,7 @@ cudaError_t qcx_launch_pair_density(qcx_ctx* ctx, QSlot& s, int iq, qcx_precisio
 cudaError_t qcx_pd_tab_prepare(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng, int iq, qcx_precision prec);
 cudaError_t qcx_launch_overlap(qcx_ctx* ctx, int nk, const double* d_kpts, const double* k_host, double2* d_out);
 cudaError_t qcx_pair_density_configure();
-AxisClasses qcx_axis_classes(const double* v, int n);
+AxisClasses qcx_axis_classes(const double* v, int n, double h, qcx_precision prec);
 
 // optical limit (optical.cu): momentum elements and the G = 0 row rho~ = -i qhat.p/dE of the
 // slot's pair densities, v^1/2 of that row set to sqrt(4 pi); d_status bit 1: a zero dE
