@@ -333,7 +333,9 @@ qcx_status qcx_pair_density(qcx_ctx* ctx, int iq, int ng, const int* G_int, qcx_
     {
         std::vector<int> Gh;
         CUDA_OR_FAIL(fetch(ctx, Gh, G_int, 3 * (size_t)ng), "G list");
-        CUDA_OR_FAIL(qcx_pd_tab_prepare(ctx, s, Gh.data(), ng, iq, prec), "pair-density tables");
+        CUDA_OR_FAIL(qcx_pd_tab_plan(ctx, s, Gh.data(), ng, iq, prec), "pair-density tables");
+        PdTab* tab = &s.pdt;
+        CUDA_OR_FAIL(qcx_pd_tab_alloc(ctx, s.pds, &tab, 1), "pair-density tables");
     }
     if (prec == QCX_FP64) {
         CUDA_OR_FAIL(s.rho.ensure((size_t)ng * nt * sizeof(double2)), "alloc rho");

@@ -171,6 +171,7 @@ struct BatchPlan {
     DevBuf d_work2, d_aux;             // mixed: second copy of the matrices, panels and row orders
     DevBuf d_G, d_inst, d_wtab, d_eps, d_work, d_x, d_r, d_out, d_flags, d_status, d_acc;
     DevBuf d_tiles, d_cta, d_rtask;
+    PdScratch pds;                              // tables and Y of one q at a time
     std::vector<CUtensorMap> maps;              // [nslot][3]: the three BF16 planes of each slot
     std::vector<int> grp_tile0, grp_ntile;      // tensor-core tiles per group of <= QCX_BATCH_MAXQ slots
     int tc_grid = 0, tile_cap = 0, ntile = 0;
@@ -473,10 +474,6 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
     CUDA_OR_FAIL(cudaMemcpyAsync(p.d_G.p, Gflat.data(), sizeof(int) * Gflat.size(), cudaMemcpyHostToDevice,
                                  ctx->stream),
                  "copy G");
-    for (int s = 0; s < p.nslot; ++s)   // tables of the pair densities, planned before the graph is captured
-        CUDA_OR_FAIL(qcx_pd_tab_prepare(ctx, *p.qs[s], Gflat.data() + 3 * p.slot_gofs[s], p.slot_u[s], p.slot_iq[s],
-                                        mixed ? QCX_MIXED : QCX_FP64),
-                     "pair-density tables");
     CUDA_OR_FAIL(p.d_inst.ensure(sizeof(BatchInst) * ninst), "alloc");
     CUDA_OR_FAIL(p.d_eps.ensure(sizeof(double2) * eps_off), "alloc eps");
     CUDA_OR_FAIL(p.d_work.ensure((mixed ? sizeof(float2) : sizeof(double2)) * work_off), "alloc work");
@@ -542,6 +539,14 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
                 if (!qcx_make_bf16_map(&p.maps[3 * s + pc], base + pc * plane, q.kp, q.ngp, 64, 32))
                     return ctx->fail(QCX_ERR_CUDA, "solve_batch: tensor map");
         }
+        // the narrowest caps give the most tiles: size the buffers for them once
+        std::vector<int4> tiles;
+        std::vector<int> g0, gn;
+        const int narrow[3] = {64, 64, 64};
+        make_tc_tiles(p, narrow, tiles, g0, gn);
+        const int grid = (int)std::min<size_t>(tiles.size(), (size_t)nsm);
+        CUDA_OR_FAIL(p.d_tiles.ensure(sizeof(int4) * tiles.size()), "alloc tiles");
+        CUDA_OR_FAIL(p.d_acc.ensure(qcx_chi0_tc_batch_acc_bytes(grid)), "alloc acc");
     } else {
         std::vector<int4> tiles;
         for (int i = 0; i < ninst; ++i) {
@@ -555,6 +560,16 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
                                      ctx->stream),
                      "copy tiles");
     }
+    // tables of the pair densities, planned before the graph is captured; after everything the batch cannot do without,
+    // and one set of buffers for all q (a set per q, each up to 1 GiB, took memory that other batches need)
+    std::vector<PdTab*> tabs;
+    for (int s = 0; s < p.nslot; ++s) {
+        CUDA_OR_FAIL(qcx_pd_tab_plan(ctx, *p.qs[s], Gflat.data() + 3 * p.slot_gofs[s], p.slot_u[s], p.slot_iq[s],
+                                     mixed ? QCX_MIXED : QCX_FP64),
+                     "pair-density tables");
+        tabs.push_back(&p.qs[s]->pdt);
+    }
+    CUDA_OR_FAIL(qcx_pd_tab_alloc(ctx, p.pds, tabs.data(), (int)tabs.size()), "pair-density tables");
     return QCX_OK;
 }
 
@@ -611,18 +626,6 @@ qcx_status prepare(qcx_ctx* ctx, BatchPlan& p) {
         return QCX_OK;
     }
     const bool tune = ctx->batch_tune != 0;
-    {
-        // the narrowest caps give the most tiles: size the buffers for them once
-        size_t most = 0;
-        std::vector<int4> tiles;
-        std::vector<int> g0, gn;
-        const int narrow[3] = {64, 64, 64};
-        make_tc_tiles(p, narrow, tiles, g0, gn);
-        most = tiles.size();
-        const int grid = (int)std::min<size_t>(most, (size_t)sm_count(ctx->device));
-        CUDA_OR_FAIL(p.d_tiles.ensure(sizeof(int4) * most), "alloc tiles");
-        CUDA_OR_FAIL(p.d_acc.ensure(qcx_chi0_tc_batch_acc_bytes(grid)), "alloc acc");
-    }
     // classes present in this batch
     bool present[3] = {false, false, false};
     for (int i = 0; i < p.ninst; ++i) {

@@ -817,8 +817,8 @@ template <typename T, int NCH, int NV> cudaError_t launch_tab(qcx_ctx* ctx, PDAr
     const int ga_per = std::min(a.ngrp, std::max(1, pdt_threads<T, NV>() / gc));
     cudaError_t e = set_smem<T>((const void*)k_pd_y<T, NCH, NV>, smem);
     if (e != cudaSuccess) return e;
-    const int kc = (int)std::min<size_t>({(size_t)a.nk, t.y.bytes / pd_y_per_k(a.nb, a.nv, a.ng, sizeof(cplx<T>)), 65535});
-    cplx<T>* Y = t.y.as<cplx<T>>();
+    const int kc = (int)std::min<size_t>({(size_t)a.nk, t.buf->y.bytes / t.y_per_k, 65535});
+    cplx<T>* Y = t.buf->y.as<cplx<T>>();
     for (int k0 = 0; k0 < a.nk; k0 += kc) {
         const int m = std::min(kc, a.nk - k0);
         k_pd_y<T, NCH, NV><<<dim3(m, nch, (a.ngrp + ga_per - 1) / ga_per), gc * ga_per, smem, ctx->stream>>>(a, k0, gc, ga_per, Y);
@@ -855,7 +855,7 @@ template <typename T, int NCH> cudaError_t build_table(qcx_ctx* ctx, PDArgs<T>& 
         ta.qofs[x] = t.qofs[x];
     }
     for (int x = 0; x < 4; ++x) ta.tbase[x] = a.tbase[x] = t.tbase[x];
-    ta.out = t.tab.as<cplx<T>>();
+    ta.out = t.buf->tab.as<cplx<T>>();
     a.ptab = ta.out;
     a.kidx = reinterpret_cast<const int*>(meta + t.o_kidx);
     a.gidx = reinterpret_cast<const int*>(meta + t.o_gidx);
@@ -1090,9 +1090,9 @@ AxisClasses qcx_axis_classes(const double* v, int n, double h, qcx_precision pre
     return c;
 }
 
-// Classes and buffers of the tables for nk k points and ng values of q+G (host arrays); leaves t invalid when the
+// Classes and sizes of the tables for nk k points and ng values of q+G (host arrays); leaves t invalid when the
 // tables would not save work or exceed their memory budget.
-static cudaError_t tab_prepare(qcx_ctx* ctx, PdTab& t, const AxisClasses& kc, int nk, const double* kap, int ng,
+static cudaError_t tab_plan(qcx_ctx* ctx, PdTab& t, const AxisClasses& kc, int nk, const double* kap, int ng,
                                qcx_precision prec, size_t y_per_k) {
     t.valid = false;
     if (!kc.finite) return cudaSuccess;
@@ -1132,12 +1132,9 @@ static cudaError_t tab_prepare(qcx_ctx* ctx, PdTab& t, const AxisClasses& kc, in
         for (int x = 0; x < 3; ++x) gsort[3 * g + x] = gc.idx[3 * gperm[g] + x];
     std::memcpy(meta.data() + t.o_gperm, gperm.data(), gperm.size() * sizeof(int));
     cudaError_t e;
-    const size_t y_bytes = y_per_k * std::min<size_t>(nk, std::max<size_t>(1, PD_Y_BYTES / std::max<size_t>(1, y_per_k)));
-    if ((e = t.tab.ensure(tab_bytes)) != cudaSuccess || (e = t.y.ensure(y_bytes)) != cudaSuccess) {
-        if (e != cudaErrorMemoryAllocation) return e;
-        cudaGetLastError();                       // no room for the tables: the kernels without them serve
-        return cudaSuccess;
-    }
+    t.tab_bytes = tab_bytes;
+    t.y_per_k = y_per_k;
+    t.buf = nullptr;
     if ((e = t.meta.ensure(meta.size())) != cudaSuccess ||
         (e = cudaMemcpyAsync(t.meta.p, meta.data(), meta.size(), cudaMemcpyHostToDevice, ctx->stream)) != cudaSuccess)
         return e;
@@ -1145,7 +1142,35 @@ static cudaError_t tab_prepare(qcx_ctx* ctx, PdTab& t, const AxisClasses& kc, in
     return cudaSuccess;
 }
 
-cudaError_t qcx_pd_tab_prepare(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng, int iq, qcx_precision prec) {
+cudaError_t qcx_pd_tab_alloc(qcx_ctx* ctx, PdScratch& buf, PdTab* const* tabs, int n) {
+    size_t tab_bytes = 0, y_per_k = 0;
+    for (int i = 0; i < n; ++i)
+        if (tabs[i]->valid) {
+            tab_bytes = std::max(tab_bytes, tabs[i]->tab_bytes);
+            y_per_k = std::max(y_per_k, tabs[i]->y_per_k);
+        }
+    if (!tab_bytes) return cudaSuccess;
+    cudaError_t e = buf.tab.ensure(tab_bytes);
+    if (e == cudaSuccess && y_per_k) {
+        size_t kc = std::min<size_t>(ctx->nk, std::max<size_t>(1, PD_Y_BYTES / y_per_k));
+        while ((e = buf.y.ensure(kc * y_per_k)) == cudaErrorMemoryAllocation && kc > 1) {
+            cudaGetLastError();
+            kc = (kc + 1) / 2;
+        }
+    }
+    if (e != cudaSuccess) {
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();                       // no room for the tables: the kernels without them serve
+        buf.release();
+    }
+    for (int i = 0; i < n; ++i) {
+        tabs[i]->valid = tabs[i]->valid && e == cudaSuccess;
+        tabs[i]->buf = &buf;
+    }
+    return cudaSuccess;
+}
+
+cudaError_t qcx_pd_tab_plan(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng, int iq, qcx_precision prec) {
     s.pdt.valid = false;
     const int nk = ctx->nk;
     if ((int)ctx->kpts_h.size() != 3 * nk || ctx->ngrp < 1) return cudaSuccess;
@@ -1167,7 +1192,7 @@ cudaError_t qcx_pd_tab_prepare(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng
             kap[3 * g + x] = v;
         }
     const size_t elem = prec == QCX_FP64 ? sizeof(double2) : sizeof(float2);
-    return tab_prepare(ctx, s.pdt, ctx->kcls[prec], nk, kap.data(), ng, prec, pd_y_per_k(ctx->nb, ctx->nv, ng, elem));
+    return tab_plan(ctx, s.pdt, ctx->kcls[prec], nk, kap.data(), ng, prec, pd_y_per_k(ctx->nb, ctx->nv, ng, elem));
 }
 
 cudaError_t qcx_launch_pair_density(qcx_ctx* ctx, QSlot& s, int iq, qcx_precision prec) {
@@ -1269,7 +1294,9 @@ cudaError_t qcx_launch_overlap(qcx_ctx* ctx, int nk, const double* d_kpts, const
     a.Sout = d_out;
     const double zero[3] = {0.0, 0.0, 0.0};
     if (nk <= 65535) {
-        const cudaError_t e = tab_prepare(ctx, ctx->overlap_tab, qcx_axis_classes(k_host, nk, ctx->h, QCX_FP64), nk, zero, 1, QCX_FP64, 0);
+        PdTab* tab = &ctx->overlap_tab;
+        cudaError_t e = tab_plan(ctx, *tab, qcx_axis_classes(k_host, nk, ctx->h, QCX_FP64), nk, zero, 1, QCX_FP64, 0);
+        if (e == cudaSuccess) e = qcx_pd_tab_alloc(ctx, ctx->overlap_buf, &tab, 1);
         if (e != cudaSuccess) return e;
         if (ctx->overlap_tab.valid) {
             const dim3 grid(((ctx->ngrp + 1) / 2 * (ctx->ngrp + 1) + 127) / 128, nk);

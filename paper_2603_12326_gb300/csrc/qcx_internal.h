@@ -67,6 +67,16 @@ struct AxisClasses {
     bool finite = false;
 };
 
+// What the tables of one q are formed in and used from, dead once that q's pair densities (or the overlap) exist: the
+// entries and Y = B C_k of a chunk of k points.  The q of a batch run one after another and share one set.
+struct PdScratch {
+    DevBuf tab, y;
+    void release() {
+        tab.release();
+        y.release();
+    }
+};
+
 // Tables of the pair densities for one q (or of an overlap, q+G = 0): the one-dimensional lattice sums
 // per shell-group pair, axis, distinct k component and distinct (q+G) component, with the axis's share
 // of every factor of the pair, so that the per-(k, G) kernel reads them instead of forming them again.
@@ -79,8 +89,9 @@ struct PdTab {
     // points' components and [ng] the G of each row of the latter (ordered by class; int)
     DevBuf meta;
     size_t o_qval = 0, o_kidx = 0, o_gidx = 0, o_gperm = 0;   // byte offsets
-    DevBuf tab;                // [entries][nchar][4] complex (FP32 or FP64): E(0,0), E(1,0), E(0,1), E(1,1)
-    DevBuf y;                  // Y = B C_k of a chunk of k points (pair densities)
+    size_t tab_bytes = 0;      // [entries][nchar][4] complex (FP32 or FP64): E(0,0), E(1,0), E(0,1), E(1,1)
+    size_t y_per_k = 0;        // Y of one k point (pair densities)
+    PdScratch* buf = nullptr;  // where both are
 };
 
 // Per-precision working set of one q.
@@ -112,6 +123,7 @@ struct QSlot {
     long long kp = 0;          // padded K' = 2 nt columns of the BF16 planes
     double eta = 0.0;
     PdTab pdt;                 // tables of the pair-density kernel for this slot's q and G list
+    PdScratch pds;             // their buffers (the slots of a batch share the plan's)
 };
 
 // Loss tables kept per q after qcx_invert_eps.
@@ -245,6 +257,7 @@ struct qcx_ctx {
     DevBuf d_grp_mu0, d_grp_mask;
     PairTables pairs;
     PdTab overlap_tab;         // tables of the last overlap call
+    PdScratch overlap_buf;
 
     // states
     int nk = 0, nv = 0, nc = 0, nq = 0;
@@ -333,7 +346,10 @@ cudaError_t qcx_launch_pair_density(qcx_ctx* ctx, QSlot& s, int iq, qcx_precisio
 // Plan and upload the tables of the pair densities for q number iq and the host G list (outside
 // any stream capture); leaves s.pdt invalid (the kernel then forms every term itself) when the
 // tables would not save work or exceed their memory budget.
-cudaError_t qcx_pd_tab_prepare(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng, int iq, qcx_precision prec);
+cudaError_t qcx_pd_tab_plan(qcx_ctx* ctx, QSlot& s, const int* G_host, int ng, int iq, qcx_precision prec);
+// Buffers for planned tables used one after another (also outside any capture); where there is no room for them the
+// tables become invalid.
+cudaError_t qcx_pd_tab_alloc(qcx_ctx* ctx, PdScratch& buf, PdTab* const* tabs, int n);
 cudaError_t qcx_launch_overlap(qcx_ctx* ctx, int nk, const double* d_kpts, const double* k_host, double2* d_out);
 cudaError_t qcx_pair_density_configure();
 AxisClasses qcx_axis_classes(const double* v, int n, double h, qcx_precision prec);
