@@ -88,6 +88,21 @@ bool qcx_is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+cudaError_t qcx_ensure(qcx_ctx* ctx, DevBuf& b, size_t bytes) {
+    cudaError_t e = b.ensure(bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    ctx->panels.release();
+    ctx->oz.release();
+    ctx->overlap_buf.release();
+    ctx->overlap_tab.valid = false;
+    for (QSlot& s : ctx->slot) {
+        s.pds.release();
+        s.pdt.valid = false;
+    }
+    return b.ensure(bytes);
+}
+
 cudaError_t qcx_copy_in(qcx_ctx* ctx, void* dst_dev, const void* src, size_t bytes) {
     if (!bytes) return cudaSuccess;
     return cudaMemcpyAsync(dst_dev, src, bytes, qcx_is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
@@ -229,8 +244,8 @@ qcx_status qcx_set_basis(qcx_ctx* ctx, const double* lattice, int natom, const d
         ctx->nb = 0;
         return st;
     }
-    CUDA_OR_FAIL(ctx->d_shell_l.ensure(nshell * sizeof(int)), "alloc");
-    CUDA_OR_FAIL(ctx->d_shell_mu0.ensure(nshell * sizeof(int)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->d_shell_l, nshell * sizeof(int)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->d_shell_mu0, nshell * sizeof(int)), "alloc");
     CUDA_OR_FAIL(cudaMemcpy(ctx->d_shell_l.p, sl.data(), nshell * sizeof(int), cudaMemcpyHostToDevice), "copy");
     CUDA_OR_FAIL(cudaMemcpy(ctx->d_shell_mu0.p, mu0.data(), nshell * sizeof(int), cudaMemcpyHostToDevice), "copy");
     return QCX_OK;
@@ -243,13 +258,13 @@ qcx_status qcx_overlap(qcx_ctx* ctx, int nk, const double* kpts, qcx_c64* out_S)
     if (nk < 1 || !kpts || !out_S) return ctx->fail(QCX_ERR_ARG, "overlap: bad arguments");
     cudaSetDevice(ctx->device);
     const size_t nout = (size_t)nk * ctx->nb * ctx->nb * sizeof(double2);
-    CUDA_OR_FAIL(ctx->scratch2.ensure(3 * sizeof(double) * nk), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch2, 3 * sizeof(double) * nk), "alloc");
     CUDA_OR_FAIL(qcx_copy_in(ctx, ctx->scratch2.p, kpts, 3 * sizeof(double) * nk), "copy kpts");
     std::vector<double> kh;
     CUDA_OR_FAIL(fetch(ctx, kh, kpts, 3 * (size_t)nk), "overlap kpts");
     double2* dst = qcx_is_device_ptr(out_S) ? reinterpret_cast<double2*>(out_S) : nullptr;
     if (!dst) {
-        CUDA_OR_FAIL(ctx->scratch.ensure(nout), "alloc");
+        CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch, nout), "alloc");
         dst = ctx->scratch.as<double2>();
     }
     CUDA_OR_FAIL(qcx_launch_overlap(ctx, nk, ctx->scratch2.as<double>(), kh.data(), dst), "overlap kernel");
@@ -272,14 +287,14 @@ qcx_status qcx_set_states(qcx_ctx* ctx, int nk, const double* kpts, int nv, cons
     if (!finite_all(qh.data(), qh.size())) return ctx->fail(QCX_ERR_ARG, "set_states: non-finite q");
     const size_t nb = ctx->nb;
     const size_t nCk = (size_t)nk * nb * nv, nCkq = (size_t)nq * nk * nb * nc;
-    CUDA_OR_FAIL(ctx->d_kpts.ensure(3 * sizeof(double) * nk), "alloc kpts");
-    CUDA_OR_FAIL(ctx->d_kpts32.ensure(3 * sizeof(float) * nk), "alloc kpts");
-    CUDA_OR_FAIL(ctx->d_Ck64.ensure(nCk * sizeof(double2)), "alloc C_k");
-    CUDA_OR_FAIL(ctx->d_Ck32.ensure(nCk * sizeof(float2)), "alloc C_k");
-    CUDA_OR_FAIL(ctx->d_Ek.ensure((size_t)nk * nv * sizeof(double)), "alloc E_k");
-    CUDA_OR_FAIL(ctx->d_Ckq64.ensure(nCkq * sizeof(double2)), "alloc C_kq");
-    CUDA_OR_FAIL(ctx->d_Ckq32.ensure(nCkq * sizeof(float2)), "alloc C_kq");
-    CUDA_OR_FAIL(ctx->d_Ekq.ensure((size_t)nq * nk * nc * sizeof(double)), "alloc E_kq");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->d_kpts, 3 * sizeof(double) * nk), "alloc kpts");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->d_kpts32, 3 * sizeof(float) * nk), "alloc kpts");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->d_Ck64, nCk * sizeof(double2)), "alloc C_k");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->d_Ck32, nCk * sizeof(float2)), "alloc C_k");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->d_Ek, (size_t)nk * nv * sizeof(double)), "alloc E_k");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->d_Ckq64, nCkq * sizeof(double2)), "alloc C_kq");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->d_Ckq32, nCkq * sizeof(float2)), "alloc C_kq");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->d_Ekq, (size_t)nq * nk * nc * sizeof(double)), "alloc E_kq");
     CUDA_OR_FAIL(qcx_copy_in(ctx, ctx->d_kpts.p, kpts, 3 * sizeof(double) * nk), "copy kpts");
     CUDA_OR_FAIL(qcx_copy_in(ctx, ctx->d_Ck64.p, C_k, nCk * sizeof(double2)), "copy C_k");
     CUDA_OR_FAIL(qcx_copy_in(ctx, ctx->d_Ek.p, E_k, (size_t)nk * nv * sizeof(double)), "copy E_k");
@@ -323,26 +338,26 @@ qcx_status qcx_pair_density(qcx_ctx* ctx, int iq, int ng, const int* G_int, qcx_
     s.ng = ng;
     s.ngp = (ng + 15) / 16 * 16;
     s.kp = (2 * nt + 63) / 64 * 64;   // K' = 2 nt padded to the 32-element stage (and 128-byte rows)
-    CUDA_OR_FAIL(s.kappa.ensure(3 * sizeof(double) * ng), "alloc");
-    CUDA_OR_FAIL(s.kappa32.ensure(3 * sizeof(float) * ng), "alloc");
-    CUDA_OR_FAIL(s.vs.ensure(sizeof(double) * ng), "alloc");
-    CUDA_OR_FAIL(s.vs32.ensure(sizeof(float) * ng), "alloc");
-    CUDA_OR_FAIL(ctx->scratch2.ensure(3 * sizeof(int) * ng), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.kappa, 3 * sizeof(double) * ng), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.kappa32, 3 * sizeof(float) * ng), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.vs, sizeof(double) * ng), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.vs32, sizeof(float) * ng), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch2, 3 * sizeof(int) * ng), "alloc");
     CUDA_OR_FAIL(qcx_copy_in(ctx, ctx->scratch2.p, G_int, 3 * sizeof(int) * ng), "copy G");
     CUDA_OR_FAIL(qcx_launch_qsetup(ctx, s, ctx->scratch2.as<int>(), ng, &ctx->qpts[3 * iq]), "q setup");
-    {
+    if (prec == QCX_FP64) {
+        CUDA_OR_FAIL(qcx_ensure(ctx, s.rho, (size_t)ng * nt * sizeof(double2)), "alloc rho");
+    } else {
+        const size_t bytes = 3 * (size_t)s.ngp * s.kp * sizeof(__nv_bfloat16);
+        CUDA_OR_FAIL(qcx_ensure(ctx, s.rho, bytes), "alloc rho");
+        CUDA_OR_FAIL(cudaMemsetAsync(s.rho.p, 0, bytes, ctx->stream), "clear rho");
+    }
+    {   // after rho, which the call cannot do without
         std::vector<int> Gh;
         CUDA_OR_FAIL(fetch(ctx, Gh, G_int, 3 * (size_t)ng), "G list");
         CUDA_OR_FAIL(qcx_pd_tab_plan(ctx, s, Gh.data(), ng, iq, prec), "pair-density tables");
         PdTab* tab = &s.pdt;
         CUDA_OR_FAIL(qcx_pd_tab_alloc(ctx, s.pds, &tab, 1), "pair-density tables");
-    }
-    if (prec == QCX_FP64) {
-        CUDA_OR_FAIL(s.rho.ensure((size_t)ng * nt * sizeof(double2)), "alloc rho");
-    } else {
-        const size_t bytes = 3 * (size_t)s.ngp * s.kp * sizeof(__nv_bfloat16);
-        CUDA_OR_FAIL(s.rho.ensure(bytes), "alloc rho");
-        CUDA_OR_FAIL(cudaMemsetAsync(s.rho.p, 0, bytes, ctx->stream), "clear rho");
     }
     cudaError_t e = qcx_launch_pair_density(ctx, s, iq, prec);
     if (e == cudaErrorInvalidValue)
@@ -352,7 +367,7 @@ qcx_status qcx_pair_density(qcx_ctx* ctx, int iq, int ng, const int* G_int, qcx_
         const size_t nout = (size_t)nt * ng * sizeof(double2);
         double2* dst = qcx_is_device_ptr(out_rho) ? reinterpret_cast<double2*>(out_rho) : nullptr;
         if (!dst) {
-            CUDA_OR_FAIL(ctx->scratch.ensure(nout), "alloc");
+            CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch, nout), "alloc");
             dst = ctx->scratch.as<double2>();
         }
         k_rho_export<<<dim3((unsigned)((nt + 31) / 32), (ng + 31) / 32), 256, 0, ctx->stream>>>(
@@ -398,7 +413,7 @@ qcx_status qcx_pair_density_optical(qcx_ctx* ctx, int iq, int ng, const int* G_i
     QSlot& s = ctx->slot[prec];
     s.have_rho = false;                                 // until the G = 0 row is in place
     OpticalBufs& ob = ctx->optical;
-    CUDA_OR_FAIL(ob.status.ensure(sizeof(int)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ob.status, sizeof(int)), "alloc");
     CUDA_OR_FAIL(cudaMemsetAsync(ob.status.p, 0, sizeof(int), ctx->stream), "clear");
     cudaError_t e = qcx_launch_optical(ctx, s, iq, g0, dir, prec, ob.status.as<int>());
     if (e == cudaErrorInvalidValue)
@@ -413,7 +428,7 @@ qcx_status qcx_pair_density_optical(qcx_ctx* ctx, int iq, int ng, const int* G_i
         const size_t nout = (size_t)nt * ng * sizeof(double2);
         double2* dst = qcx_is_device_ptr(out_rho) ? reinterpret_cast<double2*>(out_rho) : nullptr;
         if (!dst) {
-            CUDA_OR_FAIL(ctx->scratch.ensure(nout), "alloc");
+            CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch, nout), "alloc");
             dst = ctx->scratch.as<double2>();
         }
         k_rho_export<<<dim3((unsigned)((nt + 31) / 32), (ng + 31) / 32), 256, 0, ctx->stream>>>(
@@ -444,19 +459,19 @@ qcx_status qcx_chi0(qcx_ctx* ctx, int iq, int nw, const double* w, double eta, q
     s.have_eps = false;
     if (ctx->loss[iq]) ctx->loss[iq]->valid = false;     // the tables of iq belong to the previous chi0
     const int ng = s.ng;
-    CUDA_OR_FAIL(s.w.ensure(sizeof(double) * nw), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.w, sizeof(double) * nw), "alloc");
     CUDA_OR_FAIL(cudaMemcpyAsync(s.w.p, wh.data(), sizeof(double) * nw, cudaMemcpyHostToDevice, ctx->stream), "copy w");
     const size_t nmat = (size_t)nw * ng * ng;
-    CUDA_OR_FAIL(s.eps.ensure(nmat * sizeof(double2)), "alloc eps");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.eps, nmat * sizeof(double2)), "alloc eps");
     double2* chi = nullptr;
     if (out_chi0) {
         chi = qcx_is_device_ptr(out_chi0) ? reinterpret_cast<double2*>(out_chi0) : nullptr;
         if (!chi) {
-            CUDA_OR_FAIL(ctx->scratch.ensure(nmat * sizeof(double2)), "alloc");
+            CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch, nmat * sizeof(double2)), "alloc");
             chi = ctx->scratch.as<double2>();
         }
     }
-    CUDA_OR_FAIL(s.flags.ensure(sizeof(int) * (nw > 4 ? nw : 4)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.flags, sizeof(int) * (nw > 4 ? nw : 4)), "alloc");
     CUDA_OR_FAIL(cudaMemsetAsync(s.flags.p, 0, sizeof(int), ctx->stream), "clear status");
     bool tensor = prec == QCX_MIXED;
     if (prec == QCX_FP64) {
@@ -489,11 +504,11 @@ qcx_status qcx_invert_eps(qcx_ctx* ctx, int iq, qcx_precision prec, qcx_c64* out
     cudaSetDevice(ctx->device);
     const int ng = s.ng, nw = s.nw;
     const size_t nmat = (size_t)nw * ng * ng;
-    CUDA_OR_FAIL(s.work.ensure(nmat * (prec == QCX_FP64 ? sizeof(double2) : sizeof(float2))), "alloc work");
-    CUDA_OR_FAIL(s.diag_inv.ensure((size_t)nw * ng * sizeof(double2)), "alloc");
-    CUDA_OR_FAIL(s.eps_diag.ensure((size_t)nw * ng * sizeof(double2)), "alloc");
-    CUDA_OR_FAIL(s.resid.ensure(nw * sizeof(double)), "alloc");
-    CUDA_OR_FAIL(s.flags.ensure(nw * sizeof(int)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.work, nmat * (prec == QCX_FP64 ? sizeof(double2) : sizeof(float2))), "alloc work");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.diag_inv, (size_t)nw * ng * sizeof(double2)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.eps_diag, (size_t)nw * ng * sizeof(double2)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.resid, nw * sizeof(double)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.flags, nw * sizeof(int)), "alloc");
     LossTab* lt = ctx->loss[iq];
     if (!lt) {
         lt = new (std::nothrow) LossTab();
@@ -502,13 +517,13 @@ qcx_status qcx_invert_eps(qcx_ctx* ctx, int iq, qcx_precision prec, qcx_c64* out
     }
     lt->ng = ng;
     lt->nw = nw;
-    CUDA_OR_FAIL(lt->L.ensure(2 * (size_t)nw * ng * sizeof(double)), "alloc loss");
-    CUDA_OR_FAIL(lt->qmag.ensure(ng * sizeof(double)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, lt->L, 2 * (size_t)nw * ng * sizeof(double)), "alloc loss");
+    CUDA_OR_FAIL(qcx_ensure(ctx, lt->qmag, ng * sizeof(double)), "alloc");
     k_kmag<<<(ng + 127) / 128, 128, 0, ctx->stream>>>(ng, s.kappa.as<double>(), lt->qmag.as<double>());
     CUDA_OR_FAIL(qcx_launch_invert(ctx, s, prec, lt->L.as<double>()), "invert kernel");
     // the dielectric values of this q kept for the 3-D binning of the composite function
-    CUDA_OR_FAIL(lt->eps.ensure(2 * (size_t)nw * ng * sizeof(double2)), "alloc eps table");
-    CUDA_OR_FAIL(lt->kvec.ensure(3 * sizeof(double) * ng), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, lt->eps, 2 * (size_t)nw * ng * sizeof(double2)), "alloc eps table");
+    CUDA_OR_FAIL(qcx_ensure(ctx, lt->kvec, 3 * sizeof(double) * ng), "alloc");
     CUDA_OR_FAIL(qcx_launch_store_eps(ctx->stream, nw, ng, s.diag_inv.as<double2>(), s.eps_diag.as<double2>(),
                                       lt->L.as<double>(), lt->eps.as<double2>()),
                  "store eps");
@@ -594,7 +609,7 @@ qcx_status qcx_bin_loss(qcx_ctx* ctx, int nsel, const int* iq_list, int which, i
     const size_t off_o = off_e + (nbin + 1) * sizeof(double);
     const size_t off_c = off_o + (size_t)nbin * nw * sizeof(double);
     const size_t total = off_c + nbin * sizeof(double);
-    CUDA_OR_FAIL(ctx->scratch2.ensure(total), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch2, total), "alloc");
     char* base = ctx->scratch2.as<char>();
     std::vector<char> in(off_o);
     std::memcpy(in.data() + off_L, Lp.data(), nsel * sizeof(void*));
@@ -627,7 +642,7 @@ qcx_status qcx_rate(qcx_ctx* ctx, int nqbin, const double* qbin, int nw, const d
     const size_t oq = 0, ow = nqbin * sizeof(double), oL = ow + nw * sizeof(double);
     const size_t oR = oL + (size_t)nqbin * nw * sizeof(double), oQ = oR + nw * sizeof(double);
     const size_t total = oQ + (nQ > 0 ? nQ : 1) * sizeof(double);
-    CUDA_OR_FAIL(ctx->scratch2.ensure(total), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch2, total), "alloc");
     char* base = ctx->scratch2.as<char>();
     std::vector<char> in;
     if (!qcx_is_device_ptr(qbin) && !qcx_is_device_ptr(w) && !qcx_is_device_ptr(L)) {

@@ -452,16 +452,16 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
         q->ng = U;
         q->ngp = std::max(64, (U + 15) / 16 * 16);
         q->kp = p.kp;
-        CUDA_OR_FAIL(q->kappa.ensure(3 * sizeof(double) * U), "alloc");
-        CUDA_OR_FAIL(q->kappa32.ensure(3 * sizeof(float) * U), "alloc");
-        CUDA_OR_FAIL(q->vs.ensure(sizeof(double) * U), "alloc");
-        CUDA_OR_FAIL(q->vs32.ensure(sizeof(float) * U), "alloc");
+        CUDA_OR_FAIL(qcx_ensure(ctx, q->kappa, 3 * sizeof(double) * U), "alloc");
+        CUDA_OR_FAIL(qcx_ensure(ctx, q->kappa32, 3 * sizeof(float) * U), "alloc");
+        CUDA_OR_FAIL(qcx_ensure(ctx, q->vs, sizeof(double) * U), "alloc");
+        CUDA_OR_FAIL(qcx_ensure(ctx, q->vs32, sizeof(float) * U), "alloc");
         if (mixed) {
             const size_t bytes = 3 * (size_t)q->ngp * q->kp * sizeof(__nv_bfloat16);
-            CUDA_OR_FAIL(q->rho.ensure(bytes), "alloc rho");
+            CUDA_OR_FAIL(qcx_ensure(ctx, q->rho, bytes), "alloc rho");
             CUDA_OR_FAIL(cudaMemsetAsync(q->rho.p, 0, bytes, ctx->stream), "clear rho");
         } else {
-            CUDA_OR_FAIL(q->rho.ensure((size_t)U * p.nt * sizeof(double2)), "alloc rho");
+            CUDA_OR_FAIL(qcx_ensure(ctx, q->rho, (size_t)U * p.nt * sizeof(double2)), "alloc rho");
         }
     }
     for (int i = 0; i < ninst; ++i) {
@@ -470,23 +470,23 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
         p.hinst[i].rho64 = mixed ? nullptr : q.rho.as<double2>();
     }
     // device buffers
-    CUDA_OR_FAIL(p.d_G.ensure(sizeof(int) * Gflat.size()), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, p.d_G, sizeof(int) * Gflat.size()), "alloc");
     CUDA_OR_FAIL(cudaMemcpyAsync(p.d_G.p, Gflat.data(), sizeof(int) * Gflat.size(), cudaMemcpyHostToDevice,
                                  ctx->stream),
                  "copy G");
-    CUDA_OR_FAIL(p.d_inst.ensure(sizeof(BatchInst) * ninst), "alloc");
-    CUDA_OR_FAIL(p.d_eps.ensure(sizeof(double2) * eps_off), "alloc eps");
-    CUDA_OR_FAIL(p.d_work.ensure((mixed ? sizeof(float2) : sizeof(double2)) * work_off), "alloc work");
+    CUDA_OR_FAIL(qcx_ensure(ctx, p.d_inst, sizeof(BatchInst) * ninst), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, p.d_eps, sizeof(double2) * eps_off), "alloc eps");
+    CUDA_OR_FAIL(qcx_ensure(ctx, p.d_work, (mixed ? sizeof(float2) : sizeof(double2)) * work_off), "alloc work");
     p.total_n = vec_off;
     if (mixed) {
-        CUDA_OR_FAIL(p.d_work2.ensure(sizeof(float2) * work_off), "alloc work");
-        CUDA_OR_FAIL(p.d_aux.ensure(qcx_batch_inverse_aux(p.total_n, p.nmax)), "alloc panels");
+        CUDA_OR_FAIL(qcx_ensure(ctx, p.d_work2, sizeof(float2) * work_off), "alloc work");
+        CUDA_OR_FAIL(qcx_ensure(ctx, p.d_aux, qcx_batch_inverse_aux(p.total_n, p.nmax)), "alloc panels");
     }
-    CUDA_OR_FAIL(p.d_x.ensure(sizeof(double2) * vec_off), "alloc");
-    CUDA_OR_FAIL(p.d_r.ensure(sizeof(double2) * vec_off), "alloc");
-    CUDA_OR_FAIL(p.d_out.ensure(sizeof(double) * 3 * ninst), "alloc");
-    CUDA_OR_FAIL(p.d_flags.ensure(sizeof(int) * ninst), "alloc");
-    CUDA_OR_FAIL(p.d_status.ensure(sizeof(int)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, p.d_x, sizeof(double2) * vec_off), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, p.d_r, sizeof(double2) * vec_off), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, p.d_out, sizeof(double) * 3 * ninst), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, p.d_flags, sizeof(int) * ninst), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, p.d_status, sizeof(int)), "alloc");
     const int nsm = sm_count(ctx->device);
     // LU instance lists: greedy LPT over cost n^3 + 64 n^2
     p.lu_grid = std::min(ninst, nsm);
@@ -512,7 +512,7 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
             for (int i : lists_c[c]) csr[p.lu_grid + 1 + pos++] = i;
         }
         csr[p.lu_grid] = pos;
-        CUDA_OR_FAIL(p.d_cta.ensure(sizeof(int) * csr.size()), "alloc");
+        CUDA_OR_FAIL(qcx_ensure(ctx, p.d_cta, sizeof(int) * csr.size()), "alloc");
         CUDA_OR_FAIL(cudaMemcpyAsync(p.d_cta.p, csr.data(), sizeof(int) * csr.size(), cudaMemcpyHostToDevice,
                                      ctx->stream),
                      "copy lists");
@@ -523,13 +523,13 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
         for (int i = 0; i < ninst; ++i)
             for (int r0 = 0; r0 < p.h_ng[i]; r0 += 32) rt.push_back(make_int2(i, r0));
         p.n_rtask = (int)rt.size();
-        CUDA_OR_FAIL(p.d_rtask.ensure(sizeof(int2) * rt.size()), "alloc");
+        CUDA_OR_FAIL(qcx_ensure(ctx, p.d_rtask, sizeof(int2) * rt.size()), "alloc");
         CUDA_OR_FAIL(cudaMemcpyAsync(p.d_rtask.p, rt.data(), sizeof(int2) * rt.size(), cudaMemcpyHostToDevice,
                                      ctx->stream),
                      "copy tasks");
     }
     if (mixed) {
-        CUDA_OR_FAIL(p.d_wtab.ensure(sizeof(float2) * (size_t)ninst * (p.kp / 2)), "alloc W");
+        CUDA_OR_FAIL(qcx_ensure(ctx, p.d_wtab, sizeof(float2) * (size_t)ninst * (p.kp / 2)), "alloc W");
         p.maps.resize(3 * p.nslot);
         for (int s = 0; s < p.nslot; ++s) {
             QSlot& q = *p.qs[s];
@@ -545,8 +545,8 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
         const int narrow[3] = {64, 64, 64};
         make_tc_tiles(p, narrow, tiles, g0, gn);
         const int grid = (int)std::min<size_t>(tiles.size(), (size_t)nsm);
-        CUDA_OR_FAIL(p.d_tiles.ensure(sizeof(int4) * tiles.size()), "alloc tiles");
-        CUDA_OR_FAIL(p.d_acc.ensure(qcx_chi0_tc_batch_acc_bytes(grid)), "alloc acc");
+        CUDA_OR_FAIL(qcx_ensure(ctx, p.d_tiles, sizeof(int4) * tiles.size()), "alloc tiles");
+        CUDA_OR_FAIL(qcx_ensure(ctx, p.d_acc, qcx_chi0_tc_batch_acc_bytes(grid)), "alloc acc");
     } else {
         std::vector<int4> tiles;
         for (int i = 0; i < ninst; ++i) {
@@ -555,7 +555,7 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
                 for (int h0 = 0; h0 < ng; h0 += FT) tiles.push_back(make_int4(i, g0, h0, 0));
         }
         p.ntile = (int)tiles.size();
-        CUDA_OR_FAIL(p.d_tiles.ensure(sizeof(int4) * tiles.size()), "alloc");
+        CUDA_OR_FAIL(qcx_ensure(ctx, p.d_tiles, sizeof(int4) * tiles.size()), "alloc");
         CUDA_OR_FAIL(cudaMemcpyAsync(p.d_tiles.p, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice,
                                      ctx->stream),
                      "copy tiles");

@@ -392,8 +392,10 @@ cudaError_t qcx_launch_chi0_fp64_tc(qcx_ctx* ctx, QSlot& s, int iq, double pref,
         (e = b.b.ensure((size_t)NS * 4 * wg * ngp * nt2)) != cudaSuccess ||
         (e = b.w.ensure((size_t)wg * nt * (sizeof(double2) + sizeof(double)))) != cudaSuccess ||
         (e = b.e.ensure(sizeof(int) * (size_t)(ng + wg * ng))) != cudaSuccess ||
-        (e = b.part.ensure(sizeof(double) * (size_t)nsplit * wg * ngp * arows)) != cudaSuccess)
+        (e = b.part.ensure(sizeof(double) * (size_t)nsplit * wg * ngp * arows)) != cudaSuccess) {
+        b.release();
         return e;
+    }
     cudaStream_t st = ctx->stream;
     const double2* R = s.rho.as<double2>();
     double2* W = b.w.as<double2>();

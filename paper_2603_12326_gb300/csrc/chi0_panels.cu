@@ -859,7 +859,10 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
         if (e == cudaErrorMemoryAllocation) cudaGetLastError();
         return e == cudaSuccess;
     };
-    auto give_up = [&]() { return e == cudaErrorMemoryAllocation ? cudaSuccess : e; };
+    auto give_up = [&]() {                       // what did fit would be missing for the direct kernel and the inverse
+        b.release();
+        return e == cudaErrorMemoryAllocation ? cudaSuccess : e;
+    };
     const double* Ek = ctx->d_Ek.as<double>();
     const double* Ekq = ctx->d_Ekq.as<double>() + (size_t)iq * ctx->nk * ctx->nc;
     if (!fits(b.small, 64)) return give_up();

@@ -633,7 +633,7 @@ cudaError_t qcx_launch_chi0_mixed(qcx_ctx* ctx, QSlot& s, int iq, double2* chi, 
     if (smem > SMEM_LIMIT) return cudaErrorNotSupported;
 
     // W table for this q (FP64 dE and w -+ dE, stored FP32)
-    cudaError_t e = s.wtab.ensure((size_t)s.nw * (s.kp / 2) * sizeof(float2));
+    cudaError_t e = qcx_ensure(ctx, s.wtab, (size_t)s.nw * (s.kp / 2) * sizeof(float2));
     if (e != cudaSuccess) return e;
     {
         const long long n = (long long)s.nw * (s.kp / 2);
@@ -654,9 +654,16 @@ cudaError_t qcx_launch_chi0_mixed(qcx_ctx* ctx, QSlot& s, int iq, double2* chi, 
     const long long want = std::max<long long>(1, (8LL * 152 + dgrid.x * dgrid.y - 1) / (dgrid.x * dgrid.y));
     const long long tps = std::max<long long>(256, ((nt + want - 1) / want + 255) / 256 * 256);
     const int nsplit = (int)((nt + tps - 1) / tps);
-    const size_t acc_bytes = std::max((size_t)grid.x * grid.y * grid.z * 128 * a.n_tile * sizeof(double),
-                                      (size_t)nsplit * s.nw * ng * sizeof(double2));
-    e = s.acc64.ensure(acc_bytes);
+    auto acc_bytes = [&]() {
+        return std::max((size_t)grid.x * grid.y * grid.z * 128 * a.n_tile * sizeof(double), (size_t)nsplit * s.nw * ng * sizeof(double2));
+    };
+    e = qcx_ensure(ctx, s.acc64, acc_bytes());
+    if (e == cudaErrorMemoryAllocation && grid.z > 1) {          // no room for the splits' sums
+        cudaGetLastError();
+        a.kper = a.kstages;
+        grid.z = 1;
+        e = qcx_ensure(ctx, s.acc64, acc_bytes());
+    }
     if (e != cudaSuccess) return e;
     a.acc64 = s.acc64.as<double>();
 

@@ -733,14 +733,15 @@ static cudaError_t invert_all(qcx_ctx* ctx, QSlot& s, double* norms, double* L, 
     using C = cplx<T>;
     const int n = s.ng, nw = s.nw;
     cudaError_t e;
-    per = inv_group<C>(n, nw);
-    while ((e = s.work2.ensure((size_t)per * n * n * sizeof(C))) == cudaErrorMemoryAllocation && per > 1) {
+    for (per = inv_group<C>(n, nw);; per /= 2) {
+        e = qcx_ensure(ctx, s.work2, (size_t)per * n * n * sizeof(C));
+        if (e == cudaSuccess) e = qcx_ensure(ctx, s.gjaux, (size_t)per * n * (InvCfg<T>::PB * sizeof(C) + 2 * sizeof(int)));
+        if (e == cudaSuccess) break;
+        if (e != cudaErrorMemoryAllocation || per == 1) return e;
         cudaGetLastError();
-        per /= 2;
+        s.work2.release();
+        s.gjaux.release();
     }
-    if (e != cudaSuccess) return e;
-    e = s.gjaux.ensure((size_t)per * n * (InvCfg<T>::PB * sizeof(C) + 2 * sizeof(int)));
-    if (e != cudaSuccess) return e;
     for (int w0 = 0; w0 < nw; w0 += per) {
         const int m = std::min(per, nw - w0);
         const size_t o = (size_t)w0 * n;
@@ -761,7 +762,9 @@ cudaError_t qcx_launch_invert(qcx_ctx* ctx, QSlot& s, qcx_precision prec, double
         if (e != cudaSuccess) return e;
         return cudaMemsetAsync(s.resid.p, 0, sizeof(double) * s.nw, ctx->stream);
     }
-    cudaError_t e = s.kappa1.ensure(2 * sizeof(double) * s.nw);
+    const int rt = (n + RF_T - 1) / RF_T;
+    cudaError_t e = qcx_ensure(ctx, s.kappa1, 2 * sizeof(double) * s.nw);
+    if (e == cudaSuccess) e = qcx_ensure(ctx, s.refine, sizeof(double2) * (size_t)rt * s.nw * n);
     if (e != cudaSuccess) return e;
     double* norms = s.kappa1.as<double>();
     e = cudaMemsetAsync(norms, 0, 2 * sizeof(double) * s.nw, ctx->stream);
@@ -769,9 +772,6 @@ cudaError_t qcx_launch_invert(qcx_ctx* ctx, QSlot& s, qcx_precision prec, double
     e = invert_all<float>(ctx, s, norms, d_loss_out, per);
     if (e != cudaSuccess) return e;
     e = cudaMemsetAsync(s.resid.p, 0, sizeof(double) * s.nw, ctx->stream);
-    if (e != cudaSuccess) return e;
-    const int rt = (n + RF_T - 1) / RF_T;
-    e = s.refine.ensure(sizeof(double2) * (size_t)rt * s.nw * n);
     if (e != cudaSuccess) return e;
     k_refine_part<<<dim3(s.nw, rt, rt), 256, 0, ctx->stream>>>(n, s.nw, s.eps.as<double2>(), s.work.as<float2>(),
                                                                s.flags.as<int>(), norms, ctx->kappa_refine,

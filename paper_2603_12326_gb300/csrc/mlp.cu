@@ -540,13 +540,13 @@ cudaError_t launch_grad(qcx_ctx* ctx, MlpState& s, int n, int off, int count, in
 }
 
 qcx_status load_data(qcx_ctx* ctx, MlpState& s, int n, const float* X, const float* y, bool identity) {
-    CUDA_OR_FAIL(s.X.ensure(sizeof(float) * NI * (size_t)n), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.X, sizeof(float) * NI * (size_t)n), "alloc");
     CUDA_OR_FAIL(qcx_copy_in(ctx, s.X.p, X, sizeof(float) * NI * (size_t)n), "copy X");
     if (y) {
-        CUDA_OR_FAIL(s.y.ensure(sizeof(float) * (size_t)n), "alloc");
+        CUDA_OR_FAIL(qcx_ensure(ctx, s.y, sizeof(float) * (size_t)n), "alloc");
         CUDA_OR_FAIL(qcx_copy_in(ctx, s.y.p, y, sizeof(float) * (size_t)n), "copy y");
     }
-    CUDA_OR_FAIL(s.idx.ensure(sizeof(int) * (size_t)n), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.idx, sizeof(int) * (size_t)n), "alloc");
     if (identity) {
         std::vector<int> id(n);
         for (int i = 0; i < n; ++i) id[i] = i;
@@ -579,13 +579,13 @@ qcx_status qcx_mlp_set_params(qcx_ctx* ctx, const float* params) {
         if (!ctx->mlp) return ctx->fail(QCX_ERR_ALLOC, "mlp state");
     }
     MlpState& s = *ctx->mlp;
-    CUDA_OR_FAIL(s.theta.ensure(sizeof(float) * NP), "alloc");
-    CUDA_OR_FAIL(s.wbf.ensure(sizeof(__nv_bfloat16) * NP), "alloc");
-    CUDA_OR_FAIL(s.m.ensure(sizeof(float) * NP), "alloc");
-    CUDA_OR_FAIL(s.v.ensure(sizeof(float) * NP), "alloc");
-    CUDA_OR_FAIL(s.tbase.ensure(sizeof(long long)), "alloc");
-    CUDA_OR_FAIL(s.lacc.ensure(sizeof(double)), "alloc");
-    CUDA_OR_FAIL(s.grad.ensure(sizeof(float) * NP), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.theta, sizeof(float) * NP), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.wbf, sizeof(__nv_bfloat16) * NP), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.m, sizeof(float) * NP), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.v, sizeof(float) * NP), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.tbase, sizeof(long long)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.lacc, sizeof(double)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.grad, sizeof(float) * NP), "alloc");
     CUDA_OR_FAIL(qcx_copy_in(ctx, s.theta.p, params, sizeof(float) * NP), "copy params");
     CUDA_OR_FAIL(cudaMemsetAsync(s.m.p, 0, sizeof(float) * NP, ctx->stream), "clear");
     CUDA_OR_FAIL(cudaMemsetAsync(s.v.p, 0, sizeof(float) * NP, ctx->stream), "clear");
@@ -642,8 +642,8 @@ qcx_status qcx_mlp_grad(qcx_ctx* ctx, int n, const float* X, const float* y, flo
     st = load_data(ctx, s, n, X, y, true);
     if (st != QCX_OK) return st;
     const int nslot = (n + S - 1) / S;
-    CUDA_OR_FAIL(s.part.ensure(sizeof(float) * NP * (size_t)nslot), "alloc");
-    CUDA_OR_FAIL(s.ploss.ensure(sizeof(float) * (size_t)nslot), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.part, sizeof(float) * NP * (size_t)nslot), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.ploss, sizeof(float) * (size_t)nslot), "alloc");
     CUDA_OR_FAIL(cudaMemsetAsync(s.lacc.p, 0, sizeof(double), ctx->stream), "clear");
     CUDA_OR_FAIL(launch_grad(ctx, s, n, 0, n, n), "gradient kernel");
     UpdArgs u{};
@@ -685,8 +685,8 @@ qcx_status qcx_mlp_train(qcx_ctx* ctx, int n, const float* X, const float* y, co
     const int batch = std::min(opts->batch, n);
     const int nstep = (n + batch - 1) / batch;
     const int nslot = (batch + S - 1) / S;
-    CUDA_OR_FAIL(s.part.ensure(sizeof(float) * NP * (size_t)nslot), "alloc");
-    CUDA_OR_FAIL(s.ploss.ensure(sizeof(float) * (size_t)nslot), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.part, sizeof(float) * NP * (size_t)nslot), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.ploss, sizeof(float) * (size_t)nslot), "alloc");
     // one epoch as a graph: per step the tile kernel and the reduction + Adam update
     if (!s.exec || s.g_n != n || s.g_batch != batch || s.g_lr != opts->lr || s.g_b1 != opts->beta1 ||
         s.g_b2 != opts->beta2 || s.g_eps != opts->eps || s.g_ptrs != s.ptrs()) {
@@ -770,10 +770,10 @@ qcx_status qcx_mlp_predict(qcx_ctx* ctx, int n, const float* X, float* out_mu, f
     if (n < 1 || n > (1 << 24) || !X || !out_mu || !out_logvar) return ctx->fail(QCX_ERR_ARG, "mlp_predict: bad arguments");
     cudaSetDevice(ctx->device);
     MlpState& s = *ctx->mlp;
-    CUDA_OR_FAIL(s.X.ensure(sizeof(float) * NI * (size_t)n), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.X, sizeof(float) * NI * (size_t)n), "alloc");
     CUDA_OR_FAIL(qcx_copy_in(ctx, s.X.p, X, sizeof(float) * NI * (size_t)n), "copy X");
-    CUDA_OR_FAIL(s.mu.ensure(sizeof(float) * (size_t)n), "alloc");
-    CUDA_OR_FAIL(s.lv.ensure(sizeof(float) * (size_t)n), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.mu, sizeof(float) * (size_t)n), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.lv, sizeof(float) * (size_t)n), "alloc");
     TileArgs a{};
     a.theta = s.theta.as<float>();
     a.wbf = s.wbf.as<__nv_bfloat16>();

@@ -247,11 +247,11 @@ cudaError_t qcx_launch_optical(qcx_ctx* ctx, QSlot& s, int iq, int g0, const dou
                         1;
                 pairs.push_back(pr);
             }
-        e = ob.pairs.ensure(sizeof(MomPair) * pairs.size());
+        e = qcx_ensure(ctx, ob.pairs, sizeof(MomPair) * pairs.size());
         if (e != cudaSuccess) return e;
         e = cudaMemcpyAsync(ob.pairs.p, pairs.data(), sizeof(MomPair) * pairs.size(), cudaMemcpyHostToDevice, st);
         if (e != cudaSuccess) return e;
-        e = ob.P.ensure(sizeof(double2) * (size_t)nk * 3 * nb * nb);
+        e = qcx_ensure(ctx, ob.P, sizeof(double2) * (size_t)nk * 3 * nb * nb);
         if (e != cudaSuccess) return e;
         k_momentum<<<dim3((unsigned)pairs.size(), (nk + 127) / 128), 128, 0, st>>>(
             ob.pairs.as<MomPair>(), Lm[0], Lm[1], Lm[2], Lm[3], Lm[4], Lm[5], Lm[6], Lm[7], Lm[8], nk,
@@ -261,7 +261,7 @@ cudaError_t qcx_launch_optical(qcx_ctx* ctx, QSlot& s, int iq, int g0, const dou
         ob.gen = ctx->gen;
         ob.nk = nk;
     }
-    e = ob.p.ensure(sizeof(double2) * 3 * (size_t)nt);
+    e = qcx_ensure(ctx, ob.p, sizeof(double2) * 3 * (size_t)nt);
     if (e != cudaSuccess) return e;
     const size_t ysm = sizeof(double2) * 3 * (size_t)nb * nv;
     if (ysm > 227 * 1024) return cudaErrorInvalidValue;

@@ -1135,7 +1135,11 @@ static cudaError_t tab_plan(qcx_ctx* ctx, PdTab& t, const AxisClasses& kc, int n
     t.tab_bytes = tab_bytes;
     t.y_per_k = y_per_k;
     t.buf = nullptr;
-    if ((e = t.meta.ensure(meta.size())) != cudaSuccess ||
+    if ((e = t.meta.ensure(meta.size())) == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        return cudaSuccess;
+    }
+    if (e != cudaSuccess ||
         (e = cudaMemcpyAsync(t.meta.p, meta.data(), meta.size(), cudaMemcpyHostToDevice, ctx->stream)) != cudaSuccess)
         return e;
     t.valid = true;

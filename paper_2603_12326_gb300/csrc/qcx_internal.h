@@ -186,6 +186,9 @@ struct OpticalBufs {
 struct OzBufs {
     DevBuf a, b;               // digits of rho and of W rho
     DevBuf w, e, part;         // weights of a group of frequencies, row exponents, FP64 sums per K split
+    void release() {
+        for (DevBuf* d : {&a, &b, &w, &e, &part}) d->release();
+    }
 };
 
 // Work space of the mixed chi0 through energy panels (chi0_panels.cu).
@@ -198,6 +201,10 @@ struct PanelBufs {
     DevBuf ktab, kplanes;      // W at the nodes: FP32, BF16 planes
     DevBuf splanes, tp;        // S of one chunk as BF16 planes, 32-tile pairs
     DevBuf Sd, part, chi;      // diagonal of S, its frequency sums; chi0 [nw][ng][ng]
+    void release() {
+        for (DevBuf* d : {&small, &keys, &perm, &cnt, &seg, &tr, &Lw, &tiles, &r2, &ktab, &kplanes, &splanes, &tp, &Sd, &part, &chi})
+            d->release();
+    }
 };
 
 // Work space of the spectral route to chi0 (one q at a time, either precision).
@@ -325,6 +332,11 @@ template <typename T> cudaError_t fetch(qcx_ctx* ctx, std::vector<T>& out, const
     std::memcpy(out.data(), src, n * sizeof(T));
     return cudaSuccess;
 }
+
+// Grow-only allocation of a buffer that a call cannot do without: where it does not fit, the buffers of the routes that
+// have another to fall back on (chi0 through energy panels or integer slices, pair-density tables), all dead between
+// calls, are given back first.
+cudaError_t qcx_ensure(qcx_ctx* ctx, DevBuf& b, size_t bytes);
 
 // copy `bytes` from a host-or-device source into device memory (stream-ordered)
 cudaError_t qcx_copy_in(qcx_ctx* ctx, void* dst_dev, const void* src, size_t bytes);

@@ -313,7 +313,7 @@ qcx_status qcx_bin_eps3d(qcx_ctx* ctx, int nsel, const int* iq_list, double q_lf
     const size_t off_c = (off_n + nsel * sizeof(int) + 15) / 16 * 16;
     const size_t off_s = (off_c + nbin * sizeof(double) + 15) / 16 * 16;
     const size_t total = off_s + nbin * nw * sizeof(double2);
-    CUDA_OR_FAIL(ctx->scratch2.ensure(total), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch2, total), "alloc");
     char* base = ctx->scratch2.as<char>();
     CUDA_OR_FAIL(cudaMemcpyAsync(base + off_k, kp.data(), nsel * sizeof(void*), cudaMemcpyHostToDevice, ctx->stream),
                  "copy");
@@ -360,7 +360,7 @@ qcx_status qcx_loss_isotropic(qcx_ctx* ctx, int nshell, int n_theta, int n_phi, 
     const size_t oe = 0, oc = nbin * nw * sizeof(double2), ow = oc + nbin * sizeof(double);
     const size_t oL = ow + nw * sizeof(double), on = oL + (size_t)nshell * nw * sizeof(double);
     const size_t total = on + nshell * sizeof(double);
-    CUDA_OR_FAIL(ctx->scratch2.ensure(total), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch2, total), "alloc");
     char* base = ctx->scratch2.as<char>();
     CUDA_OR_FAIL(qcx_copy_in(ctx, base + oe, eps, nbin * nw * sizeof(double2)), "copy eps");
     CUDA_OR_FAIL(qcx_copy_in(ctx, base + oc, count, nbin * sizeof(double)), "copy count");
@@ -397,7 +397,7 @@ qcx_status qcx_rate_general(qcx_ctx* ctx, int nqbin, const double* qbin, int nw,
     const size_t ov = oL + (size_t)nqbin * nw * sizeof(double), of = ov + nv * sizeof(double);
     const size_t oR = of + nv * sizeof(double), oQ = oR + nw * sizeof(double);
     const size_t oX = oQ + (nQ > 0 ? nQ : 1) * sizeof(double), total = oX + (nQ > 0 ? nQ : 1) * sizeof(double);
-    CUDA_OR_FAIL(ctx->scratch2.ensure(total), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch2, total), "alloc");
     char* base = ctx->scratch2.as<char>();
     CUDA_OR_FAIL(qcx_copy_in(ctx, base + oq, qbin, nqbin * sizeof(double)), "copy");
     CUDA_OR_FAIL(qcx_copy_in(ctx, base + ow, w, nw * sizeof(double)), "copy");

@@ -526,8 +526,8 @@ qcx_status spectral_chi0(qcx_ctx* ctx, QSlot& s, bool mixed, int nw, double E0, 
     const int ng = s.ng;
     cudaStream_t st = ctx->stream;
 
-    CUDA_OR_FAIL(sp.rhos.ensure(sizeof(C) * (size_t)ng * nt), "alloc grouped pair densities");
-    CUDA_OR_FAIL(sp.xs.ensure(sizeof(R) * (size_t)nt), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.rhos, sizeof(C) * (size_t)ng * nt), "alloc grouped pair densities");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.xs, sizeof(R) * (size_t)nt), "alloc");
     GatherArgs<R> g{};
     if (mixed) {
         g.p0 = reinterpret_cast<const __nv_bfloat162*>(s.rho.p);
@@ -551,12 +551,12 @@ qcx_status spectral_chi0(qcx_ctx* ctx, QSlot& s, bool mixed, int nw, double E0, 
     tp.reserve(ntp);
     for (int gi = 0; gi < T; ++gi)
         for (int hi = gi; hi < T; ++hi) tp.push_back(make_int2(gi, hi));
-    CUDA_OR_FAIL(sp.tp.ensure(sizeof(int2) * ntp), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.tp, sizeof(int2) * ntp), "alloc");
     CUDA_OR_FAIL(cudaMemcpyAsync(sp.tp.p, tp.data(), sizeof(int2) * ntp, cudaMemcpyHostToDevice, st), "copy tiles");
 
     const long long ldk = (nbin + 31LL) / 32 * 32;
     if (!mixed || ctx->spec_cuda_cores) {                  // (the tensor-core contraction has its own planes)
-    CUDA_OR_FAIL(sp.ktab.ensure(sizeof(C) * (size_t)nw * ldk), "alloc K");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.ktab, sizeof(C) * (size_t)nw * ldk), "alloc K");
     k_spec_ktab<R><<<nblk((long long)nw * ldk, 256), 256, 0, st>>>(nw, ldk, nbin, s.w.as<double>(), E0, step, s.eta,
                                                                     sp.ktab.as<C>());
     CUDA_OR_FAIL(cudaGetLastError(), "K kernel");
@@ -571,10 +571,10 @@ qcx_status spectral_chi0(qcx_ctx* ctx, QSlot& s, bool mixed, int nw, double E0, 
     // itself; the complex weights are kept for the other contraction and for export
     const bool tc = mixed && !ctx->spec_cuda_cores;
     const bool need_S = !tc || out_S;
-    if (need_S) CUDA_OR_FAIL(sp.S.ensure(per_bin * nbc), "alloc spectral weights");
-    CUDA_OR_FAIL(sp.chi.ensure(sizeof(double2) * (size_t)nw * ng * ng), "alloc chi0");
+    if (need_S) CUDA_OR_FAIL(qcx_ensure(ctx, sp.S, per_bin * nbc), "alloc spectral weights");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.chi, sizeof(double2) * (size_t)nw * ng * ng), "alloc chi0");
     const bool s_dev = out_S && qcx_is_device_ptr(out_S);
-    if (out_S && !s_dev) CUDA_OR_FAIL(sp.Sout.ensure(sizeof(double2) * (size_t)nbc * ng * ng), "alloc");
+    if (out_S && !s_dev) CUDA_OR_FAIL(qcx_ensure(ctx, sp.Sout, sizeof(double2) * (size_t)nbc * ng * ng), "alloc");
     const size_t smem = kk_smem_bytes<R>();
     CUDA_OR_FAIL(cudaFuncSetAttribute((const void*)k_spec_kk<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)smem),
@@ -587,8 +587,8 @@ qcx_status spectral_chi0(qcx_ctx* ctx, QSlot& s, bool mixed, int nw, double E0, 
     if (tc) {
         const size_t kn = (size_t)mtiles * 128 * ldk;
         const size_t sn = (size_t)ntiles * 128 * nbc;
-        CUDA_OR_FAIL(sp.kplanes.ensure(3 * kn * sizeof(__nv_bfloat16)), "alloc K planes");
-        CUDA_OR_FAIL(sp.splanes.ensure(3 * sn * sizeof(__nv_bfloat16)), "alloc weight planes");
+        CUDA_OR_FAIL(qcx_ensure(ctx, sp.kplanes, 3 * kn * sizeof(__nv_bfloat16)), "alloc K planes");
+        CUDA_OR_FAIL(qcx_ensure(ctx, sp.splanes, 3 * sn * sizeof(__nv_bfloat16)), "alloc weight planes");
         CUDA_OR_FAIL(qcx_spec_tc_ktab(st, nw, mtiles * 128, ldk, nbin, s.w.as<double>(), E0, step, s.eta,
                                       sp.kplanes.as<__nv_bfloat16>()),
                      "K planes kernel");
@@ -703,7 +703,7 @@ extern "C" qcx_status qcx_spectral_grid(qcx_ctx* ctx, int iq, double step, doubl
         return ctx->fail(QCX_ERR_STATE, "spectral_grid: states of this q not set");
     cudaSetDevice(ctx->device);
     const long long nt = (long long)ctx->nk * ctx->nv * ctx->nc;
-    CUDA_OR_FAIL(ctx->spec.range.ensure(2 * sizeof(double)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, ctx->spec.range, 2 * sizeof(double)), "alloc");
     unsigned long long* keys = ctx->spec.range.as<unsigned long long>();
     CUDA_OR_FAIL(cudaMemsetAsync(keys, 0xff, sizeof(*keys), ctx->stream), "clear");
     CUDA_OR_FAIL(cudaMemsetAsync(keys + 1, 0, sizeof(*keys), ctx->stream), "clear");
@@ -769,21 +769,21 @@ extern "C" qcx_status qcx_chi0_spectral(qcx_ctx* ctx, int iq, int nw, const doub
     if (ctx->loss[iq]) ctx->loss[iq]->valid = false;
     const int ng = s.ng;
     cudaStream_t st = ctx->stream;
-    CUDA_OR_FAIL(s.w.ensure(sizeof(double) * nw), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.w, sizeof(double) * nw), "alloc");
     CUDA_OR_FAIL(cudaMemcpyAsync(s.w.p, wh.data(), sizeof(double) * nw, cudaMemcpyHostToDevice, st), "copy w");
     const size_t nmat = (size_t)nw * ng * ng;
-    CUDA_OR_FAIL(s.eps.ensure(nmat * sizeof(double2)), "alloc eps");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.eps, nmat * sizeof(double2)), "alloc eps");
 
     // grid points of every transition, grouped by grid point
     SpecBufs& sp = ctx->spec;
-    CUDA_OR_FAIL(sp.bin.ensure(sizeof(int) * nt), "alloc");
-    CUDA_OR_FAIL(sp.x.ensure(sizeof(double) * nt), "alloc");
-    CUDA_OR_FAIL(sp.perm0.ensure(sizeof(int) * nt), "alloc");
-    CUDA_OR_FAIL(sp.perm.ensure(sizeof(int) * nt), "alloc");
-    CUDA_OR_FAIL(sp.cnt.ensure(sizeof(int) * (size_t)nbin), "alloc");
-    CUDA_OR_FAIL(sp.fill.ensure(sizeof(int) * (size_t)nbin), "alloc");
-    CUDA_OR_FAIL(sp.off.ensure(sizeof(int) * ((size_t)nbin + 1)), "alloc");
-    CUDA_OR_FAIL(sp.status.ensure(sizeof(int)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.bin, sizeof(int) * nt), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.x, sizeof(double) * nt), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.perm0, sizeof(int) * nt), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.perm, sizeof(int) * nt), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.cnt, sizeof(int) * (size_t)nbin), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.fill, sizeof(int) * (size_t)nbin), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.off, sizeof(int) * ((size_t)nbin + 1)), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, sp.status, sizeof(int)), "alloc");
     CUDA_OR_FAIL(cudaMemsetAsync(sp.cnt.p, 0, sizeof(int) * (size_t)nbin, st), "clear");
     CUDA_OR_FAIL(cudaMemsetAsync(sp.fill.p, 0, sizeof(int) * (size_t)nbin, st), "clear");
     CUDA_OR_FAIL(cudaMemsetAsync(sp.status.p, 0, sizeof(int), st), "clear");
@@ -811,7 +811,7 @@ extern "C" qcx_status qcx_chi0_spectral(qcx_ctx* ctx, int iq, int nw, const doub
     if (out_chi0) {
         chi = qcx_is_device_ptr(out_chi0) ? reinterpret_cast<double2*>(out_chi0) : nullptr;
         if (!chi) {
-            CUDA_OR_FAIL(ctx->scratch.ensure(nmat * sizeof(double2)), "alloc");
+            CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch, nmat * sizeof(double2)), "alloc");
             chi = ctx->scratch.as<double2>();
         }
     }

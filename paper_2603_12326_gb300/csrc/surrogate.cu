@@ -140,7 +140,7 @@ qcx_status qcx_head_nolfe(qcx_ctx* ctx, int iq, int nw, const double* w, double 
     cudaSetDevice(ctx->device);
     // own buffer: the pair-density call below stages its G list in the context's scratch
     DevBuf buf;
-    CUDA_OR_FAIL(buf.ensure(2 * sizeof(double) * nw), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, buf, 2 * sizeof(double) * nw), "alloc");
     double* d_w = buf.as<double>();
     CUDA_OR_FAIL(qcx_copy_in(ctx, d_w, w, sizeof(double) * nw), "copy w");
     qcx_status st = head_nolfe_dev(ctx, iq, nw, d_w, eta, d_w + nw);
@@ -160,7 +160,7 @@ qcx_status qcx_surrogate_features(qcx_ctx* ctx, int n, const double* qvec, const
     const size_t bq = 3 * sizeof(double) * n, bw = sizeof(double) * n, bx = 6 * sizeof(float) * n,
                  by = sizeof(float) * n;
     DevBuf buf;
-    CUDA_OR_FAIL(buf.ensure(bq + 3 * bw + bx + by), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, buf, bq + 3 * bw + bx + by), "alloc");
     char* base = buf.as<char>();
     double* dq = reinterpret_cast<double*>(base);
     double* dw = reinterpret_cast<double*>(base + bq);
@@ -206,13 +206,13 @@ qcx_status qcx_surrogate_heads(qcx_ctx* ctx, int nsel, const int* iq_list, int n
     const size_t n = (size_t)nsel * nw;
     // 1) cheap heads, features, network
     DevBuf d_w, d_L, d_q, d_wall, d_X, d_mu, d_lv;
-    CUDA_OR_FAIL(d_w.ensure(sizeof(double) * nw), "alloc");
-    CUDA_OR_FAIL(d_L.ensure(sizeof(double) * n), "alloc");
-    CUDA_OR_FAIL(d_q.ensure(3 * sizeof(double) * n), "alloc");
-    CUDA_OR_FAIL(d_wall.ensure(sizeof(double) * n), "alloc");
-    CUDA_OR_FAIL(d_X.ensure(6 * sizeof(float) * n), "alloc");
-    CUDA_OR_FAIL(d_mu.ensure(sizeof(float) * n), "alloc");
-    CUDA_OR_FAIL(d_lv.ensure(sizeof(float) * n), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, d_w, sizeof(double) * nw), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, d_L, sizeof(double) * n), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, d_q, 3 * sizeof(double) * n), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, d_wall, sizeof(double) * n), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, d_X, 6 * sizeof(float) * n), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, d_mu, sizeof(float) * n), "alloc");
+    CUDA_OR_FAIL(qcx_ensure(ctx, d_lv, sizeof(float) * n), "alloc");
     CUDA_OR_FAIL(cudaMemcpyAsync(d_w.p, wh.data(), sizeof(double) * nw, cudaMemcpyHostToDevice, ctx->stream), "copy");
     std::vector<double> qall(3 * n), wall(n);
     for (int s = 0; s < nsel; ++s) {
