@@ -167,8 +167,8 @@ struct BatchPlan {
     std::vector<BatchInst> hinst;
     std::vector<int> h_ng;
 
-    long long total_n = 0;             // sum of N_G
-    DevBuf d_work2, d_aux;             // mixed: second copy of the matrices, panels and row orders
+    std::vector<InvGroup> inv_groups;  // mixed: instances inverted together
+    DevBuf d_work2, d_aux;             // second copy of a group's matrices, its panels and row orders
     DevBuf d_G, d_inst, d_wtab, d_eps, d_work, d_x, d_r, d_out, d_flags, d_status, d_acc;
     DevBuf d_tiles, d_cta, d_rtask;
     PdScratch pds;                              // tables and Y of one q at a time
@@ -348,8 +348,8 @@ cudaError_t record(qcx_ctx* ctx, BatchPlan& p) {
         ++p.launches;
         return cudaSuccess;
     }
-    if ((e = qcx_launch_batch_inverse(st, a, p.d_work2.as<float2>(), p.d_aux.p, p.total_n, p.nmax)) != cudaSuccess) return e;
-    ++p.launches;
+    if ((e = qcx_launch_batch_inverse(st, a, p.inv_groups, p.d_work2.as<float2>(), p.d_aux.p, p.nmax, &p.launches)) != cudaSuccess)
+        return e;
     for (int it = 0; it < NREF; ++it) {
         if ((e = qcx_launch_resid(st, a, p.d_rtask.as<int2>(), p.n_rtask)) != cudaSuccess) return e;
         if ((e = qcx_launch_batch_correct(st, a, p.nmax, it == NREF - 1 ? 1 : 0)) != cudaSuccess) return e;
@@ -477,11 +477,6 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
     CUDA_OR_FAIL(qcx_ensure(ctx, p.d_inst, sizeof(BatchInst) * ninst), "alloc");
     CUDA_OR_FAIL(qcx_ensure(ctx, p.d_eps, sizeof(double2) * eps_off), "alloc eps");
     CUDA_OR_FAIL(qcx_ensure(ctx, p.d_work, (mixed ? sizeof(float2) : sizeof(double2)) * work_off), "alloc work");
-    p.total_n = vec_off;
-    if (mixed) {
-        CUDA_OR_FAIL(qcx_ensure(ctx, p.d_work2, sizeof(float2) * work_off), "alloc work");
-        CUDA_OR_FAIL(qcx_ensure(ctx, p.d_aux, qcx_batch_inverse_aux(p.total_n, p.nmax)), "alloc panels");
-    }
     CUDA_OR_FAIL(qcx_ensure(ctx, p.d_x, sizeof(double2) * vec_off), "alloc");
     CUDA_OR_FAIL(qcx_ensure(ctx, p.d_r, sizeof(double2) * vec_off), "alloc");
     CUDA_OR_FAIL(qcx_ensure(ctx, p.d_out, sizeof(double) * 3 * ninst), "alloc");
@@ -559,6 +554,22 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
         CUDA_OR_FAIL(cudaMemcpyAsync(p.d_tiles.p, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice,
                                      ctx->stream),
                      "copy tiles");
+    }
+    // the second copy for the inverse: of as many instances as fit
+    for (size_t copy = QCX_INV_COPY_BYTES; mixed; copy /= 2) {
+        p.inv_groups = qcx_batch_inverse_groups(p.hinst, copy);
+        long long mats = 0, vecs = 0;
+        for (const InvGroup& g : p.inv_groups) {
+            mats = std::max(mats, g.mats);
+            vecs = std::max(vecs, g.vecs);
+        }
+        cudaError_t e = qcx_ensure(ctx, p.d_work2, sizeof(float2) * mats);
+        if (e == cudaSuccess) e = qcx_ensure(ctx, p.d_aux, qcx_batch_inverse_aux(vecs, p.nmax));
+        if (e == cudaSuccess) break;
+        if (e != cudaErrorMemoryAllocation || (int)p.inv_groups.size() == ninst) CUDA_OR_FAIL(e, "alloc inverse copy");
+        cudaGetLastError();
+        p.d_work2.release();
+        p.d_aux.release();
     }
     // tables of the pair densities, planned before the graph is captured; after everything the batch cannot do without,
     // and one set of buffers for all q (a set per q, each up to 1 GiB, took memory that other batches need)

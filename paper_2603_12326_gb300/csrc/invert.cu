@@ -84,9 +84,11 @@ struct InvShape {
     int n, pb;
     const BatchInst* inst;
     int b0;                                 // first matrix of the launch
+    size_t mat0, vec0;                      // where the second copy's matrices and the panels' rows begin
     __device__ int order(int b) const { return inst ? inst[b].ng : n; }
     __device__ size_t mat(int b) const { return inst ? (size_t)inst[b].work_off : (size_t)b * n * n; }
-    __device__ size_t vec(int b) const { return inst ? (size_t)inst[b].vec_off : (size_t)b * n; }
+    __device__ size_t mat2(int b) const { return mat(b) - mat0; }
+    __device__ size_t vec(int b) const { return (inst ? (size_t)inst[b].vec_off : (size_t)b * n) - vec0; }
 };
 
 // FP64 matrices -> work precision; eps_GG, the loss without local fields, |A|_1 (largest column sum) and the
@@ -134,7 +136,7 @@ __global__ void __launch_bounds__(1024) k_inv_panel(InvShape sh, int p_, int RW,
     const int b = sh.b0 + blockIdx.x, n = sh.order(b), npan = (n + sh.pb - 1) / sh.pb;
     if (p_ >= npan || flags[b]) return;
     const int k0 = p_ * sh.pb, nb = min(sh.pb, n - k0);
-    const C* src = ((npan - p_) & 1 ? B2 : X) + sh.mat(b);
+    const C* src = (npan - p_) & 1 ? B2 + sh.mat2(b) : X + sh.mat(b);
     const size_t vec = sh.vec(b);
     const int ld = n | 1;
     C* xs = reinterpret_cast<C*>(smem_raw);            // [nb][ld]
@@ -266,7 +268,7 @@ __global__ void __launch_bounds__(PR_ROWS) k_inv_panel_reg(InvShape sh, int p_, 
     const int b = sh.b0 + blockIdx.x, n = sh.order(b), npan = (n + sh.pb - 1) / sh.pb;
     if (p_ >= npan || flags[b]) return;
     const int k0 = p_ * sh.pb, nb = min(sh.pb, n - k0);
-    const C* src = ((npan - p_) & 1 ? B2 : X) + sh.mat(b);
+    const C* src = (npan - p_) & 1 ? B2 + sh.mat2(b) : X + sh.mat(b);
     const size_t vec = sh.vec(b);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rw = warp % RW, grp = warp / RW;
@@ -369,8 +371,8 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 1) k_inv_update(InvS
     if (p >= npan || i0 >= n || j0 >= n || flags[b]) return;
     const int k0 = p * sh.pb, nb = min(sh.pb, n - k0);
     const bool from_b = (npan - p) & 1, last = p + 1 == npan;
-    const C* src = (from_b ? B2 : X) + sh.mat(b);
-    C* dst = (from_b ? X : B2) + sh.mat(b);
+    const C* src = from_b ? B2 + sh.mat2(b) : X + sh.mat(b);
+    C* dst = from_b ? X + sh.mat(b) : B2 + sh.mat2(b);
     M += sh.vec(b) * sh.pb;
     perm += sh.vec(b);
     rows += sh.vec(b);
@@ -653,10 +655,11 @@ __global__ void __launch_bounds__(256) k_loss_quadform(int n, const float2* Xall
 
 }  // namespace
 
-// All panels of nmat matrices of order at most n.
+// All panels of nmat matrices of order at most n; returns the number of launches.
 template <typename T>
-static void eliminate(cudaStream_t st, InvShape sh, int n, int nmat, int npan, size_t smem, cplx<T>* X, cplx<T>* B2, cplx<T>* M,
-                      int* perm, int* rows, int* flags) {
+static int eliminate(cudaStream_t st, InvShape sh, int n, int nmat, int npan, size_t smem, cplx<T>* X, cplx<T>* B2, cplx<T>* M,
+                     int* perm, int* rows, int* flags) {
+    int launches = 0;
     const int RW = std::min((n + 31) / 32, 32);
     int groups = 1;
     while (groups * 2 * RW <= 16 && groups * 2 <= sh.pb) groups *= 2;
@@ -677,14 +680,16 @@ static void eliminate(cudaStream_t st, InvShape sh, int n, int nmat, int npan, s
         else if constexpr (sizeof(T) == 4)
             k_inv_panel_reg<T, 32><<<m, threads, 0, st>>>(sh, p, RW, X, B2, M, perm, rows, flags);
     };
-    for (sh.b0 = 0; sh.b0 < nmat; sh.b0 += 32768) {            // grid limit of the tiles' third dimension
-        const int m = std::min(32768, nmat - sh.b0);
+    for (const int b1 = sh.b0 + nmat; sh.b0 < b1; sh.b0 += 32768) {    // grid limit of the tiles' third dimension
+        const int m = std::min(32768, b1 - sh.b0);
         const dim3 tiles((n + UPD - 1) / UPD, (n + UPD - 1) / UPD, m);
         for (int p = 0; p < npan; ++p) {
             panel(p, m);
+            launches += 2;
             k_inv_update<T><<<tiles, 256, 0, st>>>(sh, p, X, B2, M, perm, rows, flags);
         }
     }
+    return launches;
 }
 
 // Widest panel of order-n matrices that fits shared memory, and its bytes.
@@ -716,16 +721,15 @@ static cudaError_t invert_batch(cudaStream_t st, int n, int nmat, const double2*
     const int npan = (n + pb - 1) / pb;
     const dim3 cols(nmat, (n + 63) / 64);
     k_inv_load<T><<<cols, 256, 0, st>>>(n, A, npan & 1 ? B2 : X, anorm, eps_diag, L_nolfe, rows, flags);
-    eliminate<T>(st, InvShape{n, pb, nullptr, 0}, n, nmat, npan, smem, X, B2, M, perm, rows, flags);
+    eliminate<T>(st, InvShape{n, pb, nullptr, 0, 0, 0}, n, nmat, npan, smem, X, B2, M, perm, rows, flags);
     k_inv_finish<T><<<cols, 256, 0, st>>>(n, X, flags, xnorm, diag_inv, L);
     return cudaGetLastError();
 }
 
-// Matrices are inverted in groups whose second copy stays within INV_COPY_BYTES (at least one), so that the scratch
+// Matrices are inverted in groups whose second copy stays within QCX_INV_COPY_BYTES (at least one), so that the scratch
 // does not grow with the number of frequencies; where even that does not fit, in smaller groups.
-constexpr size_t INV_COPY_BYTES = 1ull << 30;
 template <typename C> static int inv_group(int n, int nw) {
-    return (int)std::min<size_t>({(size_t)nw, std::max<size_t>(1, INV_COPY_BYTES / ((size_t)n * n * sizeof(C))), 32768});
+    return (int)std::min<size_t>({(size_t)nw, std::max<size_t>(1, QCX_INV_COPY_BYTES / ((size_t)n * n * sizeof(C))), 32768});
 }
 
 template <typename T>
@@ -803,12 +807,12 @@ namespace {
 // FP64 eps of every instance -> FP32, into the buffer its first panel reads; starting row order.  Grid (instance, 64
 // columns).
 __global__ void __launch_bounds__(256) k_batch_load(InvShape sh, const double2* eps, float2* X, float2* B2, int* rows, int* flags) {
-    const int b = blockIdx.x, n = sh.order(b), tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+    const int b = sh.b0 + blockIdx.x, n = sh.order(b), tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
     const int j = blockIdx.y * 64 + tx;
     if (blockIdx.y == 0 && threadIdx.x == 0) flags[b] = 0;
     if (j >= n) return;
     const int npan = (n + sh.pb - 1) / sh.pb;
-    float2* dst = (npan & 1 ? B2 : X) + sh.mat(b);
+    float2* dst = npan & 1 ? B2 + sh.mat2(b) : X + sh.mat(b);
     const double2* A = eps + sh.inst[b].eps_off;
     for (int i = ty; i < n; i += 4) {
         const double2 z = A[(size_t)i * n + j];
@@ -896,24 +900,43 @@ __global__ void __launch_bounds__(512) k_batch_correct(BatchSolveArgs a, const f
 
 }  // namespace
 
-size_t qcx_batch_inverse_aux(long long total_n, int nmax) {
-    size_t smem;
-    return (size_t)total_n * ((size_t)panel_width<float>(nmax, &smem) * sizeof(float2) + 2 * sizeof(int));
+// Consecutive instances whose matrices stay within copy_bytes (at least one instance each).
+std::vector<InvGroup> qcx_batch_inverse_groups(const std::vector<BatchInst>& inst, size_t copy_bytes) {
+    std::vector<InvGroup> groups;
+    for (int b = 0; b < (int)inst.size(); ++b) {
+        const long long mats = (long long)inst[b].ng * (inst[b].ng + 1);
+        if (groups.empty() || (size_t)(groups.back().mats + mats) * sizeof(float2) > copy_bytes)
+            groups.push_back({b, 0, inst[b].work_off, inst[b].vec_off, 0, 0});
+        InvGroup& g = groups.back();
+        ++g.n;
+        g.mats += mats;
+        g.vecs += inst[b].ng;
+    }
+    return groups;
 }
 
-cudaError_t qcx_launch_batch_inverse(cudaStream_t st, const BatchSolveArgs& a, float2* B2, void* aux, long long total_n, int nmax) {
+size_t qcx_batch_inverse_aux(long long vecs, int nmax) {
+    size_t smem;
+    return (size_t)vecs * ((size_t)panel_width<float>(nmax, &smem) * sizeof(float2) + 2 * sizeof(int));
+}
+
+cudaError_t qcx_launch_batch_inverse(cudaStream_t st, const BatchSolveArgs& a, const std::vector<InvGroup>& groups, float2* B2,
+                                     void* aux, int nmax, int* launches) {
     if (nmax < 1 || nmax > 1024 * PANEL_ROWS) return cudaErrorInvalidValue;
     size_t smem = 0;
     const int pb = panel_width<float>(nmax, &smem);
-    float2* M = reinterpret_cast<float2*>(aux);
-    int* perm = reinterpret_cast<int*>(M + (size_t)total_n * pb);
-    int* rows = perm + total_n;
     cudaError_t e = cudaFuncSetAttribute((const void*)k_inv_panel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const InvShape sh{nmax, pb, a.inst, 0};
     float2* X = reinterpret_cast<float2*>(a.work);
-    k_batch_load<<<dim3(a.ninst, (nmax + 63) / 64), 256, 0, st>>>(sh, a.eps, X, B2, rows, a.flags);
-    eliminate<float>(st, sh, nmax, a.ninst, (nmax + pb - 1) / pb, smem, X, B2, M, perm, rows, a.flags);
+    for (const InvGroup& g : groups) {
+        const InvShape sh{nmax, pb, a.inst, g.b0, (size_t)g.mat0, (size_t)g.vec0};
+        float2* M = reinterpret_cast<float2*>(aux);
+        int* perm = reinterpret_cast<int*>(M + (size_t)g.vecs * pb);
+        int* rows = perm + g.vecs;
+        k_batch_load<<<dim3(g.n, (nmax + 63) / 64), 256, 0, st>>>(sh, a.eps, X, B2, rows, a.flags);
+        *launches += 1 + eliminate<float>(st, sh, nmax, g.n, (nmax + pb - 1) / pb, smem, X, B2, M, perm, rows, a.flags);
+    }
+    ++*launches;
     k_batch_x<<<a.ninst, 128, 0, st>>>(a, X);
     return cudaGetLastError();
 }

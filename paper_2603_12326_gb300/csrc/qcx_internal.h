@@ -417,8 +417,17 @@ struct BatchSolveArgs {
 cudaError_t qcx_launch_lu_head(cudaStream_t st, const BatchSolveArgs& a, int grid, int nmax);    // FP64
 cudaError_t qcx_launch_resid(cudaStream_t st, const BatchSolveArgs& a, const int2* tasks, int ntask);
 // mixed (invert.cu): FP32 inverses into a.work with B2 as second copy, x and the heads; x += X r
-size_t qcx_batch_inverse_aux(long long total_n, int nmax);
-cudaError_t qcx_launch_batch_inverse(cudaStream_t st, const BatchSolveArgs& a, float2* B2, void* aux, long long total_n, int nmax);
+// Instances b0 .. b0 + n - 1, inverted together: B2 holds their matrices (from element mat0 of a.work on), aux their rows
+// (from vec0 on, vecs of them).
+constexpr size_t QCX_INV_COPY_BYTES = 1ull << 30;    // second copy of the matrices being inverted at a time
+struct InvGroup {
+    int b0, n;
+    long long mat0, vec0, mats, vecs;
+};
+std::vector<InvGroup> qcx_batch_inverse_groups(const std::vector<BatchInst>& inst, size_t copy_bytes);
+size_t qcx_batch_inverse_aux(long long vecs, int nmax);
+cudaError_t qcx_launch_batch_inverse(cudaStream_t st, const BatchSolveArgs& a, const std::vector<InvGroup>& groups, float2* B2,
+                                     void* aux, int nmax, int* launches);
 cudaError_t qcx_launch_batch_correct(cudaStream_t st, const BatchSolveArgs& a, int nmax, int last);
 
 // inverse + loss (invert.cu)

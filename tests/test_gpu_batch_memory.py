@@ -36,3 +36,29 @@ def test_memory_per_q(prec):
     planes = ng * p.nt * 16 if prec == QCX_FP64 else 3 * ((ng + 15) // 16 * 16) * 2 * p.nt * 2
     assert (used[10] - used[2]) / 8 < planes + (8 << 20)
     assert np.all(np.isfinite(heads[10][0]))
+
+
+def test_inverse_in_groups_of_instances():
+    """2600 instances of N_G = 335: their second copy for the inverse (0.9 MB each) is made for 1 GiB of them at a time.
+    Per instance stay eps and the FP32 matrix, 24 N_G^2 bytes, the weights and vectors; the heads do not depend on the
+    grouping beyond the launches' tiles."""
+    p = synth.make_small(nq=1)
+    ctx = context()
+    used, heads = {}, {}
+    g = np.sqrt(48.0) * 2.0 * np.pi / p.cell.a
+    try:
+        states.load_problem(ctx, p, [0])
+        ctx.batch_autotune(False)
+        for n in (100, 1300, 2600):
+            w = np.linspace(0.2, 1.2, 2600)[:n]
+            ctx.solve_batch(np.zeros(1, np.int32), w[:1], np.full(1, g), p.eta, QCX_MIXED)
+            free = torch.cuda.mem_get_info(0)[0]
+            heads[n] = ctx.solve_batch(np.zeros(n, np.int32), w, np.full(n, g), p.eta, QCX_MIXED)
+            used[n] = free - torch.cuda.mem_get_info(0)[0]
+    finally:
+        ctx.close()
+    ng = int(heads[100][2][0])
+    assert (used[2600] - used[1300]) / 1300 < 24 * ng * (ng + 1) + 8 * p.nt + 256 * ng
+    for n in (100, 1300):
+        for i in range(2):
+            assert np.max(np.abs(heads[2600][i][:n] / heads[n][i] - 1.0)) < 1e-6
