@@ -195,6 +195,20 @@ qcx_status qcx_pair_density_optical(qcx_ctx* ctx, int iq, int ng, const int* G_i
 qcx_status qcx_chi0(qcx_ctx* ctx, int iq, int nw, const double* w, double eta, qcx_precision prec,
                     qcx_c64* out_chi0);
 
+/* How the eps that the context holds in precision prec was formed (no
+ * counterpart in the paper: the routes give the same chi0 to the precision's
+ * error, and qcx_chi0 takes the one it estimates to be fastest and that fits
+ * memory). */
+typedef enum {
+    QCX_ROUTE_NONE = 0,         /* no eps, ctx NULL or a bad precision                   */
+    QCX_ROUTE_FP64_SUM = 1,     /* QCX_FP64: sum over the transitions in FP64            */
+    QCX_ROUTE_FP64_SLICES = 2,  /* QCX_FP64: exact integer slices on the tensor cores    */
+    QCX_ROUTE_DIRECT = 3,       /* QCX_MIXED: one contraction per frequency              */
+    QCX_ROUTE_PANELS = 4,       /* QCX_MIXED: transitions contracted once, by energy     */
+    QCX_ROUTE_SPECTRAL = 5      /* qcx_chi0_spectral                                     */
+} qcx_route;
+qcx_route qcx_chi0_route(const qcx_ctx* ctx, qcx_precision prec);
+
 /* The spectral route to the same chi0 (Eq. (eRPA_spectral): the spectral
  * part of Eq. (RPA), with the principal part from the Kramers-Kronig
  * relations, Section II.D and its footnote).  On the uniform grid

@@ -473,16 +473,15 @@ qcx_status qcx_chi0(qcx_ctx* ctx, int iq, int nw, const double* w, double eta, q
     }
     CUDA_OR_FAIL(qcx_ensure(ctx, s.flags, sizeof(int) * (nw > 4 ? nw : 4)), "alloc");
     CUDA_OR_FAIL(cudaMemsetAsync(s.flags.p, 0, sizeof(int), ctx->stream), "clear status");
-    bool tensor = prec == QCX_MIXED;
     if (prec == QCX_FP64) {
-        CUDA_OR_FAIL(qcx_launch_chi0_fp64(ctx, s, iq, chi, s.flags.as<int>(), &tensor), "chi0 fp64 kernel");
+        CUDA_OR_FAIL(qcx_launch_chi0_fp64(ctx, s, iq, chi, s.flags.as<int>()), "chi0 fp64 kernel");
     } else {
         cudaError_t e = qcx_launch_chi0_mixed(ctx, s, iq, chi, s.flags.as<int>());
         if (e == cudaErrorNotSupported)
             return ctx->fail(QCX_ERR_UNSUPPORTED, "chi0: this G-set size is not handled by the tensor-core kernel");
         CUDA_OR_FAIL(e, "chi0 tensor-core kernel");
     }
-    if (tensor) {
+    if (s.route != QCX_ROUTE_FP64_SUM) {
         int st = 0;
         const CopyOut out = {&st, 0, sizeof(int)};
         CUDA_OR_FAIL(qcx_copy_out_all(ctx, s.flags.as<char>(), sizeof(int), &out, 1), "status");
@@ -492,6 +491,11 @@ qcx_status qcx_chi0(qcx_ctx* ctx, int iq, int nw, const double* w, double eta, q
         CUDA_OR_FAIL(qcx_copy_out(ctx, out_chi0, chi, nmat * sizeof(double2)), "copy out");
     s.have_eps = true;
     return QCX_OK;
+}
+
+qcx_route qcx_chi0_route(const qcx_ctx* ctx, qcx_precision prec) {
+    if (!ctx || (prec != QCX_FP64 && prec != QCX_MIXED) || !ctx->slot[prec].have_eps) return QCX_ROUTE_NONE;
+    return ctx->slot[prec].route;
 }
 
 qcx_status qcx_invert_eps(qcx_ctx* ctx, int iq, qcx_precision prec, qcx_c64* out_diag_inv, qcx_c64* out_eps_diag,

@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(256) k_chi0_fp64(Chi64Args a) {
 
 }  // namespace
 
-cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out, int* d_status, bool* used_tc) {
-    *used_tc = false;
+cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out, int* d_status) {
+    s.route = QCX_ROUTE_FP64_SUM;
     Chi64Args a;
     a.R = s.rho.as<double2>();
     a.nt = (long long)ctx->nk * ctx->nv * ctx->nc;
@@ -155,7 +155,7 @@ cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0
     if (a.nt >= TC_MIN_NT && cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
         const cudaError_t e = qcx_launch_chi0_fp64_tc(ctx, s, iq, a.pref, d_chi0_out, d_status);
         if (e != cudaErrorMemoryAllocation) {
-            *used_tc = true;
+            s.route = QCX_ROUTE_FP64_SLICES;
             return e;
         }
         cudaGetLastError();

@@ -588,6 +588,7 @@ cudaError_t qcx_launch_chi0_mixed(qcx_ctx* ctx, QSlot& s, int iq, double2* chi, 
     bool panels = false;                         // many frequencies: through energy panels
     {
         const cudaError_t ep = qcx_launch_chi0_panels(ctx, s, iq, chi, d_status, &panels);
+        s.route = panels ? QCX_ROUTE_PANELS : QCX_ROUTE_DIRECT;
         if (panels || ep != cudaSuccess) return ep;
     }
     const int ng = s.ng;

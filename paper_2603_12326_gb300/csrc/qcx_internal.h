@@ -101,6 +101,7 @@ struct QSlot {
     int nw = 0;
     bool have_rho = false;
     bool have_eps = false;
+    qcx_route route = QCX_ROUTE_NONE;   // how eps was formed
     DevBuf kappa;              // [ng][3] double, q + G (bohr^-1)
     DevBuf kappa32;            // [ng][3] float
     DevBuf vs;                 // [ng] double, sqrt(4 pi)/|q+G|
@@ -384,8 +385,8 @@ cudaError_t qcx_spec_tc_kk(cudaStream_t st, const CUtensorMap* kmaps, const CUte
 
 // chi0 (chi0_fp64.cu, chi0_tc.cu, chi0_panels.cu)
 cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi, int* d_status, bool* used);
-// FP64: sets *used_tc when the tensor-core route ran (its status word is then to be read)
-cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out, int* d_status, bool* used_tc);
+// both set s.route (a status word is to be read after every route but the plain FP64 sum)
+cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out, int* d_status);
 cudaError_t qcx_launch_chi0_fp64_tc(qcx_ctx* ctx, QSlot& s, int iq, double pref, double2* chi, int* d_status);
 cudaError_t qcx_launch_chi0_mixed(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0_out, int* d_status);
 // 2-D tensor map over one BF16 plane [rows][kp], box {box_k, box_rows} (box_k 16: 32-byte

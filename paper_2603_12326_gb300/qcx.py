@@ -16,6 +16,8 @@ import numpy as np
 
 QCX_FP64 = 0
 QCX_MIXED = 1
+# qcx_route
+ROUTES = (None, "fp64_sum", "fp64_slices", "direct", "panels", "spectral")
 STATUS = {0: "QCX_OK", 1: "QCX_ERR_ARG", 2: "QCX_ERR_ALLOC", 3: "QCX_ERR_CUDA", 4: "QCX_ERR_SINGULAR",
           5: "QCX_ERR_NOT_CONVERGED", 6: "QCX_ERR_TIMEOUT", 7: "QCX_ERR_STATE", 8: "QCX_ERR_UNSUPPORTED"}
 
@@ -74,6 +76,7 @@ _SIGS = {
     "qcx_set_states": (I, [P, I, P, I, P, P, I, P, I, P, P]),
     "qcx_pair_density": (I, [P, I, I, P, I, P]),
     "qcx_chi0": (I, [P, I, I, P, D, I, P]),
+    "qcx_chi0_route": (I, [P, I]),
     "qcx_pair_density_optical": (I, [P, I, I, P, P, I, P]),
     "qcx_chi0_spectral": (I, [P, I, I, P, D, D, D, I, I, P, P]),
     "qcx_spectral_grid": (I, [P, I, D, ct.POINTER(D), ct.POINTER(I)]),
@@ -270,6 +273,10 @@ class Context:
         oa = _Arg(o, np.complex128)
         self._check(qcx_chi0(self.h, iq, nw, wa.ptr, float(eta), prec, oa.ptr))
         return o
+
+    def chi0_route(self, prec=QCX_FP64):
+        """How the eps of `prec` was formed, as a name of ROUTES (None: there is no eps)."""
+        return ROUTES[qcx_chi0_route(self.h, prec)]
 
     def chi0_spectral(self, iq, w, eta, E0, step, nbin, prec=QCX_FP64, want=False, want_S=False, out=None):
         """qcx_chi0_spectral; returns chi0 [nw][ng][ng] (if wanted) and the spectral weights
