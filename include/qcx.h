@@ -304,8 +304,8 @@ qcx_status qcx_set_refine_threshold(qcx_ctx* ctx, double kappa1);
 qcx_status qcx_set_wait_limit(qcx_ctx* ctx, long long cycles);
 
 /* Fault injection for tests of the failure path (no counterpart in the
- * paper): with withhold_copies != 0 the tensor-core kernel of qcx_chi0
- * (QCX_MIXED) issues none of its copies, so its consumers' waits run out after
+ * paper): with withhold_copies != 0 the tensor-core kernels of qcx_chi0
+ * issue none of their copies, so its consumers' waits run out after
  * the limit of qcx_set_wait_limit and the call returns QCX_ERR_TIMEOUT; 0
  * (the default) restores normal operation.  Errors: QCX_ERR_ARG (ctx NULL). */
 qcx_status qcx_set_fault_injection(qcx_ctx* ctx, int withhold_copies);

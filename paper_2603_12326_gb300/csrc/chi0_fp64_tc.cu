@@ -177,6 +177,7 @@ struct OzArgs {
     int accumulate;                   // add to part (later K chunks)
     int* status;
     long long wait_limit;
+    int withhold;                     // fault injection: no copies, so that the consumers' first waits run out
 };
 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     if (warp == 0) {
         if (lane == 0) {
             int last = -1;
-            for (int it = 0; it < nst; ++it) {
+            for (int it = 0; it < (a.withhold ? 0 : nst); ++it) {
                 const int s = it % OZ_NSTAGE;
                 const uint32_t ph = (uint32_t)(it / OZ_NSTAGE) & 1u;
                 if (!mbar_wait(&empty[s], ph ^ 1u, abort_flag, a.status, a.wait_limit)) break;
@@ -413,6 +414,7 @@ cudaError_t qcx_launch_chi0_fp64_tc(qcx_ctx* ctx, QSlot& s, int iq, double pref,
     a.part = b.part.as<double>();
     a.status = d_status;
     a.wait_limit = ctx->wait_limit;
+    a.withhold = ctx->withhold_copies;
     a.kstages = kst;
     a.per_split = per_split;
     a.tmem_cols = 32;

@@ -360,6 +360,7 @@ struct PgArgs {
     __nv_bfloat16* S;                     // three planes [node][ncol], column ((pair 32 + G in 32) 2 + part) 32 + (G' in 32)
     int* status;
     long long wait_limit;
+    int withhold;                         // fault injection: no copies
 };
 
 struct PgItem {
@@ -429,7 +430,8 @@ template <int NST> __global__ void __launch_bounds__(PG_THREADS, 1) k_pn_gram(co
             if (lane == 0) {
                 int gs = 0;
                 bool ok = true;
-                for (int im = blockIdx.x; im < nitem && ok; im += gridDim.x) {
+                // with copies withheld nothing is issued and the consumers' first waits run out
+                for (int im = a.withhold ? nitem : blockIdx.x; im < nitem && ok; im += gridDim.x) {
                     const PgItem m = pg_item(a, im);
                     const uint32_t bb = (uint32_t)m.n * ROWB;
                     const uint32_t b1 = (uint32_t)min(m.n, a.ngp - m.n0) * ROWB;   // the columns wrap around ngp
@@ -838,7 +840,7 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
     const long long nt = (long long)ctx->nk * ctx->nv * ctx->nc;
     const double direct = direct_us(s, nt);
     // below this the host round trips alone would cost what there is to gain
-    if (direct < 600.0 || ctx->withhold_copies) return cudaSuccess;
+    if (direct < 600.0) return cudaSuccess;
     const int T32 = (ng + 31) / 32, ntp = T32 * (T32 + 1) / 2;
     if (nw > 65535 || ntp * 16 > 65535) return cudaSuccess;      // grid limits
     const std::vector<int4> tiles = pair_cover(ng, ngp);
@@ -977,6 +979,7 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
     a.S = b.splanes.as<__nv_bfloat16>();
     a.status = d_status;
     a.wait_limit = ctx->wait_limit;
+    a.withhold = ctx->withhold_copies;
     auto ring_bytes = [&](size_t nst) {
         return 1024 + nst * (2 * (n_max + (with_src ? PG_GBLK : 0)) * ROWB + 3 * PG_ATILE + PN_TPS * sizeof(float)) +
                (5 * nst + 5) * sizeof(uint64_t) + 16;
