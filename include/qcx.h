@@ -23,9 +23,12 @@
  *    with cudaPointerGetAttributes.  Device pointers must belong to the
  *    context's device.
  *  - Outputs are caller-owned.  A NULL output pointer means "not wanted".
- *    When every output of a call is in device memory the call is
- *    asynchronous on the context's stream; a host output makes the call
- *    synchronise before returning.
+ *    qcx_overlap, qcx_pair_density, qcx_chi0 with QCX_FP64 and
+ *    qcx_loss_function are asynchronous on the context's stream when their
+ *    outputs are in device memory (or not wanted) and their small inputs (G
+ *    list, k points, frequencies) in host memory; a host output or a device
+ *    copy of such an input makes them wait for the stream, and so does every
+ *    other call before it returns.
  *  - Complex numbers are qcx_c64 {re, im} (two doubles, interleaved).
  *  - Errors: every call returns a qcx_status; on failure the context keeps
  *    a message (qcx_last_error) and stays usable.  No C++ exception crosses
@@ -191,7 +194,8 @@ qcx_status qcx_pair_density_optical(qcx_ctx* ctx, int iq, int ng, const int* G_i
  * qcx_invert_eps are reset (they belong to the previous chi0).
  * Errors: QCX_ERR_STATE, QCX_ERR_ARG (nw < 1, eta <= 0, non-finite w),
  * QCX_ERR_ALLOC, QCX_ERR_CUDA, QCX_ERR_TIMEOUT (a pipeline wait gave up;
- * results are invalid). */
+ * results are invalid; QCX_FP64 without a host output does not wait for its
+ * kernels: chi0 and eps are then NaN and qcx_invert_eps reports it). */
 qcx_status qcx_chi0(qcx_ctx* ctx, int iq, int nw, const double* w, double eta, qcx_precision prec,
                     qcx_c64* out_chi0);
 
@@ -279,7 +283,8 @@ qcx_status qcx_spectral_timings(qcx_ctx* ctx, double* ms);
  *                          ill-conditioned ones), 0 for the others; 0 for QCX_FP64.
  * and keeps the loss tables of iq in the context.
  * Errors: QCX_ERR_STATE, QCX_ERR_SINGULAR (zero pivot in some block; the
- * other blocks are valid), QCX_ERR_ALLOC, QCX_ERR_CUDA. */
+ * other blocks are valid), QCX_ERR_TIMEOUT (of the qcx_chi0 before it, see
+ * there), QCX_ERR_ALLOC, QCX_ERR_CUDA. */
 qcx_status qcx_invert_eps(qcx_ctx* ctx, int iq, qcx_precision prec, qcx_c64* out_diag_inv,
                           qcx_c64* out_eps_diag, double* out_resid);
 

@@ -471,24 +471,29 @@ qcx_status qcx_chi0(qcx_ctx* ctx, int iq, int nw, const double* w, double eta, q
             chi = ctx->scratch.as<double2>();
         }
     }
-    CUDA_OR_FAIL(qcx_ensure(ctx, s.flags, sizeof(int) * (nw > 4 ? nw : 4)), "alloc");
-    CUDA_OR_FAIL(cudaMemsetAsync(s.flags.p, 0, sizeof(int), ctx->stream), "clear status");
+    CUDA_OR_FAIL(qcx_ensure(ctx, s.flags, sizeof(int) * (nw + 1)), "alloc");
+    s.status_unread = false;
+    int* d_status = s.flags.as<int>() + nw;
+    CUDA_OR_FAIL(cudaMemsetAsync(d_status, 0, sizeof(int), ctx->stream), "clear status");
     if (prec == QCX_FP64) {
-        CUDA_OR_FAIL(qcx_launch_chi0_fp64(ctx, s, iq, chi, s.flags.as<int>()), "chi0 fp64 kernel");
+        CUDA_OR_FAIL(qcx_launch_chi0_fp64(ctx, s, iq, chi, d_status), "chi0 fp64 kernel");
     } else {
-        cudaError_t e = qcx_launch_chi0_mixed(ctx, s, iq, chi, s.flags.as<int>());
+        cudaError_t e = qcx_launch_chi0_mixed(ctx, s, iq, chi, d_status);
         if (e == cudaErrorNotSupported)
             return ctx->fail(QCX_ERR_UNSUPPORTED, "chi0: this G-set size is not handled by the tensor-core kernel");
         CUDA_OR_FAIL(e, "chi0 tensor-core kernel");
     }
-    if (s.route != QCX_ROUTE_FP64_SUM) {
+    // FP64 without host results stays asynchronous: after a wait that gave up the slices leave NaN, and qcx_invert_eps
+    // reads the status
+    const bool host_out = out_chi0 && chi != reinterpret_cast<double2*>(out_chi0);
+    s.status_unread = s.route == QCX_ROUTE_FP64_SLICES && !host_out;
+    if (s.route != QCX_ROUTE_FP64_SUM && !s.status_unread) {
         int st = 0;
         const CopyOut out = {&st, 0, sizeof(int)};
-        CUDA_OR_FAIL(qcx_copy_out_all(ctx, s.flags.as<char>(), sizeof(int), &out, 1), "status");
+        CUDA_OR_FAIL(qcx_copy_out_all(ctx, reinterpret_cast<const char*>(d_status), sizeof(int), &out, 1), "status");
         if (st) return ctx->fail(QCX_ERR_TIMEOUT, "chi0: a pipeline wait in the tensor-core kernel gave up");
     }
-    if (out_chi0 && chi != reinterpret_cast<double2*>(out_chi0))
-        CUDA_OR_FAIL(qcx_copy_out(ctx, out_chi0, chi, nmat * sizeof(double2)), "copy out");
+    if (host_out) CUDA_OR_FAIL(qcx_copy_out(ctx, out_chi0, chi, nmat * sizeof(double2)), "copy out");
     s.have_eps = true;
     return QCX_OK;
 }
@@ -535,13 +540,19 @@ qcx_status qcx_invert_eps(qcx_ctx* ctx, int iq, qcx_precision prec, qcx_c64* out
                                  ctx->stream),
                  "copy q+G");
     lt->w = s.wh;
-    lt->valid = true;
     CUDA_OR_FAIL(qcx_copy_out(ctx, out_diag_inv, s.diag_inv.p, (size_t)nw * ng * sizeof(double2)), "copy out");
     CUDA_OR_FAIL(qcx_copy_out(ctx, out_eps_diag, s.eps_diag.p, (size_t)nw * ng * sizeof(double2)), "copy out");
     CUDA_OR_FAIL(qcx_copy_out(ctx, out_resid, s.resid.p, nw * sizeof(double)), "copy out");
-    std::vector<int> flags(nw);
-    const CopyOut fo = {flags.data(), 0, nw * sizeof(int)};
-    CUDA_OR_FAIL(qcx_copy_out_all(ctx, s.flags.as<char>(), nw * sizeof(int), &fo, 1), "flags");
+    std::vector<int> flags(nw + (s.status_unread ? 1 : 0));
+    const CopyOut fo = {flags.data(), 0, flags.size() * sizeof(int)};
+    CUDA_OR_FAIL(qcx_copy_out_all(ctx, s.flags.as<char>(), flags.size() * sizeof(int), &fo, 1), "flags");
+    if (s.status_unread && flags.back()) {
+        s.have_eps = false;
+        return ctx->fail(QCX_ERR_TIMEOUT, "invert: a pipeline wait in the tensor-core chi0 kernel gave up");
+    }
+    flags.resize(nw);
+    s.status_unread = false;
+    lt->valid = true;
     int bad = 0;
     for (int f : flags) bad += f != 0;
     if (bad) return ctx->fail(QCX_ERR_SINGULAR, "invert: " + std::to_string(bad) + " singular block(s)");

@@ -336,9 +336,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     }
 }
 
-// chi0 = pref x the splits in order; eps = 1 - v^1/2 chi0 v^1/2.  part is [split][nw][ngp (G')][arows (G)].
+// chi0 = pref x the splits in order; eps = 1 - v^1/2 chi0 v^1/2.  part is [split][nw][ngp (G')][arows (G)].  NaN after a wait
+// that gave up, since the host may look at the status later than at the results.
 __global__ void k_oz_finish(int ng, int ngp, int nw, int arows, int nsplit, const double* part, double pref, const double* vs,
-                            double2* eps, double2* chi) {
+                            const int* status, double2* eps, double2* chi) {
     const int G = blockIdx.x * 32 + threadIdx.x, H = blockIdx.y * 8 + threadIdx.y, iw = blockIdx.z;
     __shared__ double2 tile[8][33];
     double2 c = make_double2(0.0, 0.0);
@@ -350,6 +351,7 @@ __global__ void k_oz_finish(int ng, int ngp, int nw, int arows, int nsplit, cons
             c.y += p[64];
         }
     }
+    if (*status) c = make_double2(nan(""), nan(""));
     tile[threadIdx.y][threadIdx.x] = make_double2(pref * c.x, pref * c.y);
     __syncthreads();
     const int id = threadIdx.y * 32 + threadIdx.x, h = id & 7, g = id >> 3;
@@ -445,7 +447,7 @@ cudaError_t qcx_launch_chi0_fp64_tc(qcx_ctx* ctx, QSlot& s, int iq, double pref,
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
         k_oz_finish<<<dim3((ng + 31) / 32, (ng + 7) / 8, m), dim3(32, 8), 0, st>>>(
-            ng, ngp, m, arows, nsplit, a.part, pref, s.vs.as<double>(), s.eps.as<double2>() + (size_t)w0 * ng * ng,
+            ng, ngp, m, arows, nsplit, a.part, pref, s.vs.as<double>(), d_status, s.eps.as<double2>() + (size_t)w0 * ng * ng,
             chi ? chi + (size_t)w0 * ng * ng : nullptr);
     }
     return cudaGetLastError();

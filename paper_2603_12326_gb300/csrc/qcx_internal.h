@@ -102,6 +102,7 @@ struct QSlot {
     bool have_rho = false;
     bool have_eps = false;
     qcx_route route = QCX_ROUTE_NONE;   // how eps was formed
+    bool status_unread = false;         // the status word of chi0's kernels (flags[nw]) is still to be read
     DevBuf kappa;              // [ng][3] double, q + G (bohr^-1)
     DevBuf kappa32;            // [ng][3] float
     DevBuf vs;                 // [ng] double, sqrt(4 pi)/|q+G|
@@ -119,7 +120,7 @@ struct QSlot {
     DevBuf diag_inv;           // [nw][ng] double2
     DevBuf eps_diag;           // [nw][ng] double2
     DevBuf resid;              // [nw] double
-    DevBuf flags;              // [nw] int (singular / error flags)
+    DevBuf flags;              // [nw] int (singular flags), then chi0's status word
     int ngp = 0;               // padded G rows of the BF16 planes (multiple of 16)
     long long kp = 0;          // padded K' = 2 nt columns of the BF16 planes
     double eta = 0.0;

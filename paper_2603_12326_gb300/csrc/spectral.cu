@@ -823,6 +823,7 @@ extern "C" qcx_status qcx_chi0_spectral(qcx_ctx* ctx, int iq, int nw, const doub
         CUDA_OR_FAIL(qcx_copy_out(ctx, out_chi0, chi, nmat * sizeof(double2)), "copy out");
     CUDA_OR_FAIL(cudaStreamSynchronize(st), "sync");
     s.route = QCX_ROUTE_SPECTRAL;
+    s.status_unread = false;
     s.have_eps = true;
     return QCX_OK;
 }
