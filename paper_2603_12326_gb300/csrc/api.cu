@@ -63,6 +63,15 @@ inline int nblocks(size_t n, int t = 256) {
     return (int)(b > 4096 ? 4096 : (b ? b : 1));
 }
 
+constexpr size_t PACK_MAX = 1 << 20;     // arrays of a call that go through the host in one copy
+
+bool is_pageable(const void* p) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) == cudaSuccess) return at.type == cudaMemoryTypeUnregistered;
+    cudaGetLastError();
+    return true;
+}
+
 bool finite_all(const double* p, size_t n) {
     for (size_t i = 0; i < n; ++i)
         if (!std::isfinite(p[i])) return false;
@@ -119,11 +128,10 @@ cudaError_t qcx_copy_out(qcx_ctx* ctx, void* dst, const void* src_dev, size_t by
 }
 
 cudaError_t qcx_copy_out_all(qcx_ctx* ctx, const char* src, size_t total, const CopyOut* out, int n) {
-    constexpr size_t PIN_MAX = 1 << 20;
-    bool host = total <= PIN_MAX;
+    bool host = total <= PACK_MAX;
     for (int i = 0; i < n; ++i) host = host && !qcx_is_device_ptr(out[i].dst);
     cudaError_t e;
-    if (host && ctx->pin.ensure(PIN_MAX) == cudaSuccess) {
+    if (host && ctx->pin.ensure(PACK_MAX) == cudaSuccess) {
         if ((e = cudaMemcpyAsync(ctx->pin.p, src, total, cudaMemcpyDeviceToHost, ctx->stream)) != cudaSuccess) return e;
         if ((e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) return e;
         for (int i = 0; i < n; ++i)
@@ -660,7 +668,8 @@ qcx_status qcx_rate(qcx_ctx* ctx, int nqbin, const double* qbin, int nw, const d
     CUDA_OR_FAIL(qcx_ensure(ctx, ctx->scratch2, total), "alloc");
     char* base = ctx->scratch2.as<char>();
     std::vector<char> in;
-    if (!qcx_is_device_ptr(qbin) && !qcx_is_device_ptr(w) && !qcx_is_device_ptr(L)) {
+    // small pageable arrays in one copy; page-locked ones may still be written by an earlier copy on the stream
+    if (oR <= PACK_MAX && is_pageable(qbin) && is_pageable(w) && is_pageable(L)) {
         in.resize(oR);
         std::memcpy(in.data() + oq, qbin, nqbin * sizeof(double));
         std::memcpy(in.data() + ow, w, nw * sizeof(double));
