@@ -17,7 +17,6 @@ constexpr int TG = 32;   // G tile
 constexpr int TK = 16;   // transitions per stage
 constexpr int TW = 4;    // frequencies per CTA
 constexpr long long TC_MIN_NT = 32;
-constexpr double TC_MIN_ETA = 1e-6;      // Hartree (27 ueV)
 
 struct Chi64Args {
     const double2* R;     // [ng][nt]
@@ -151,12 +150,9 @@ cudaError_t qcx_launch_chi0_fp64(qcx_ctx* ctx, QSlot& s, int iq, double2* d_chi0
     // The tensor-core route, except for a handful of transitions, when its work space does not fit, or while the
     // stream is being captured (the status word could not be read).  This kernel walks the transitions serially
     // at ~5.2 us each whatever N_G and N_w up to a full GPU (measured 425 us at N_t = 80, 15.8 ms at 3072); the
-    // tensor-core route starts at ~120 us for its launches.  Its slices hold W rho to 2^-61 of the largest of a row, up to
-    // 1 / eta, so for a tiny eta the terms away from the resonances lose bits that this kernel keeps: largest error of an
-    // element over sum |rho||W||rho| at eta = 1.8e-2 .. 1.8e-5 Hartree 0.8e-15 .. 1.3e-15 (this kernel 1.2e-15 .. 7e-15),
-    // at 1.8e-7 up to 9e-15 (1e-14), growing with 1 / eta below.
+    // tensor-core route starts at ~120 us for its launches.
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (a.nt >= TC_MIN_NT && s.eta >= TC_MIN_ETA && cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    if (a.nt >= TC_MIN_NT && cudaStreamIsCapturing(ctx->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
         const cudaError_t e = qcx_launch_chi0_fp64_tc(ctx, s, iq, a.pref, d_chi0_out, d_status);
         if (e != cudaErrorMemoryAllocation) {
             s.route = QCX_ROUTE_FP64_SLICES;
