@@ -12,7 +12,11 @@
 // of one order over 128 k stays below 2^24 and is exact in the FP32 accumulator: after each such window the sums are
 // read out as integers and added into two 64-bit integers per element (orders 0-3 and 4-7).  No rounding happens
 // before the final conversion; the K range is split over CTAs and the splits are added in FP64 in a fixed order.
-// Measured against 64-bit sums over the tests' ranges the result is as close as that of the plain FP64 kernel.
+// Bound of an element's error: ~2^-61 of (row maximum of |A|) x (sum of the row of |B|) and the reverse, which is not the
+// plain sum's bound over sum |A||B|: terms far below their row's maximum are held in fewer bits.  Measured over that
+// sum, element by element against sums in extended precision (N_t = 48, 960, 4536; eta = 2e-2 to 2e-12 Hartree,
+// frequencies on and beside resonances): 0.8e-15 to 1.1e-14, the plain kernel 1.2e-15 to 5.8e-14, the slices closer in
+// all 27 cases.
 //
 // What bounds it: the plain kernel is bound by the GB300's FP64 pipe (1.06 TFLOP/s): 42 ms per frequency at N_G =
 // 181, N_t = 65536.  Here a frequency costs 36 BF16 products of the same shape on the tensor cores.  Operand
@@ -47,7 +51,7 @@ __device__ __forceinline__ int exponent_of(unsigned hi) {
     return e == 0x7ff ? OZ_BAD : max(e - 1022, OZ_EMIN);
 }
 __device__ __forceinline__ unsigned hi_abs(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
-__device__ __forceinline__ double pow2(int e) { return e >= OZ_BAD / 2 ? 0.0 : scalbn(1.0, e); }
+__device__ __forceinline__ double pow2(int e) { return scalbn(1.0, e); }    // 0 for a row with OZ_BAD
 
 __device__ __forceinline__ unsigned block_max(unsigned v) {
     __shared__ unsigned red[8];
