@@ -458,7 +458,8 @@ qcx_status qcx_solve_batch(qcx_ctx* ctx, int ninst, const int* inst_q, const dou
 /* Facts about the current batch plan (batching has no counterpart in the
  * paper), written to out[0 .. n-1] (host):
  * [0] tile width cap (columns of G per tensor-core tile), [1] tiles,
- * [2] persistent tensor-core CTAs, [3] solve CTAs, [4] kernels per replay,
+ * [2] persistent tensor-core CTAs, [3] CTAs of the FP64 LU (0 for QCX_MIXED,
+ * whose inverse has a CTA per instance and panel), [4] kernels per replay,
  * [5] 1 if the tile widths were autotuned, [6] distinct q, [7] largest N_G,
  * [8] autotuning time (microseconds), [9] precision, [10..12] the tile width
  * caps of the N_G classes 65-128, 129-192 and above 192 ([0] repeats the last).

@@ -11,10 +11,11 @@
 //  * the mixed path cuts every instance into (64-row G' block, G chunk)
 //    tiles for the persistent tensor-core kernel, largest first; the FP64
 //    path into 32 x 32 tiles for a plain FP64 kernel;
-//  * instance lists per CTA for the LU kernels by greedy longest-processing-
-//    time over the cost N_G^3;
+//  * FP64: instance lists per CTA for the LU kernel by greedy longest-
+//    processing-time over the cost N_G^3; mixed: groups of instances for the
+//    blocked inverse;
 //  * the whole sequence (G set-up, pair densities, W table, chi0 + Dyson,
-//    LU, FP64 residual and correction) is captured once in a CUDA graph and
+//    inverse or LU, FP64 residual and correction) is captured once in a CUDA graph and
 //    replayed per call; only the frequencies are uploaded per call.
 //  * Autotuner: the tile width (columns of G per tensor-core tile) has its own
 //    cap per N_G class (65-128, 129-192, more than 192); on a new plan the
@@ -301,8 +302,9 @@ cudaError_t record(qcx_ctx* ctx, BatchPlan& p) {
         if ((e = qcx_launch_qsetup(ctx, q, p.d_G.as<int>() + 3 * p.slot_gofs[s], p.slot_u[s], &ctx->qpts[3 * iq])) !=
             cudaSuccess)
             return e;
+        const long long before = ctx->pd_launches;
         if ((e = qcx_launch_pair_density(ctx, q, iq, (qcx_precision)p.prec)) != cudaSuccess) return e;
-        p.launches += 2;
+        p.launches += 1 + (int)(ctx->pd_launches - before);
     }
     const BatchInst* dinst = p.d_inst.as<BatchInst>();
     if (mixed) {
@@ -334,8 +336,8 @@ cudaError_t record(qcx_ctx* ctx, BatchPlan& p) {
     }
     BatchSolveArgs a;
     a.inst = dinst;
-    a.cta_off = p.d_cta.as<int>();
-    a.cta_ids = p.d_cta.as<int>() + p.lu_grid + 1;
+    a.cta_off = mixed ? nullptr : p.d_cta.as<int>();
+    a.cta_ids = mixed ? nullptr : p.d_cta.as<int>() + p.lu_grid + 1;
     a.eps = p.d_eps.as<double2>();
     a.work = p.d_work.p;
     a.x = p.d_x.as<double2>();
@@ -483,9 +485,9 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
     CUDA_OR_FAIL(qcx_ensure(ctx, p.d_flags, sizeof(int) * ninst), "alloc");
     CUDA_OR_FAIL(qcx_ensure(ctx, p.d_status, sizeof(int)), "alloc");
     const int nsm = sm_count(ctx->device);
-    // LU instance lists: greedy LPT over cost n^3 + 64 n^2
-    p.lu_grid = std::min(ninst, nsm);
-    {
+    // FP64: LU instance lists, greedy LPT over cost n^3 + 64 n^2
+    if (!mixed) {
+        p.lu_grid = std::min(ninst, nsm);
         std::vector<int> order(ninst);
         std::iota(order.begin(), order.end(), 0);
         auto cost = [&](int i) { const double n = p.h_ng[i]; return n * n * n + 64.0 * n * n; };
@@ -512,8 +514,8 @@ qcx_status build_plan(qcx_ctx* ctx, BatchPlan& p) {
                                      ctx->stream),
                      "copy lists");
     }
-    // residual tasks (32 rows each)
-    {
+    // mixed: residual tasks (32 rows each)
+    if (mixed) {
         std::vector<int2> rt;
         for (int i = 0; i < ninst; ++i)
             for (int r0 = 0; r0 < p.h_ng[i]; r0 += 32) rt.push_back(make_int2(i, r0));

@@ -779,6 +779,7 @@ template <typename T, int NCH> cudaError_t launch_pd(qcx_ctx* ctx, PDArgs<T>& a,
     cudaError_t e = set_smem<T>((const void*)k_pair_density<T, NCH>, smem);
     if (e != cudaSuccess) return e;
     k_pair_density<T, NCH><<<grid, PD_THREADS, smem, ctx->stream>>>(a);
+    ++ctx->pd_launches;
     return cudaGetLastError();
 }
 
@@ -786,6 +787,7 @@ template <int NCH, int NV> cudaError_t launch_fused(qcx_ctx* ctx, PDArgs<float>&
     const cudaError_t e = set_smem<float>((const void*)k_pair_density_fused<NCH, NV>, smem);
     if (e != cudaSuccess) return e;
     k_pair_density_fused<NCH, NV><<<grid, nthr, smem, ctx->stream>>>(a);
+    ++ctx->pd_launches;
     return cudaGetLastError();
 }
 template <int NCH> cudaError_t launch_fused_nv(qcx_ctx* ctx, PDArgs<float>& a, size_t smem, dim3 grid, int nthr) {
@@ -828,6 +830,7 @@ template <typename T, int NCH, int NV> cudaError_t launch_tab(qcx_ctx* ctx, PDAr
             launch_rho<T, 16>(ctx, a, k0, m, nvp, Y);
         else
             launch_rho<T, 32>(ctx, a, k0, m, nvp, Y);
+        ctx->pd_launches += 2;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -861,6 +864,7 @@ template <typename T, int NCH> cudaError_t build_table(qcx_ctx* ctx, PDArgs<T>& 
     a.gidx = reinterpret_cast<const int*>(meta + t.o_gidx);
     a.gperm = reinterpret_cast<const int*>(meta + t.o_gperm);
     k_pd_axis_table<T, NCH><<<(unsigned)((t.tbase[3] + 127) / 128), 128, 0, ctx->stream>>>(ta);
+    ++ctx->pd_launches;
     return cudaGetLastError();
 }
 

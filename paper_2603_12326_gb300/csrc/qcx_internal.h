@@ -286,6 +286,7 @@ struct qcx_ctx {
     DevBuf scratch2;
     PinBuf pin;                // staging of small results
 
+    long long pd_launches = 0;     // kernels launched by qcx_launch_pair_density
     unsigned long long gen = 0;    // bumped whenever basis or states change
     BatchPlan* batch = nullptr;    // cached plan (and captured graph) of the last batched solve
     int batch_tune = 1;            // autotune the batch tiling when a new plan is built
