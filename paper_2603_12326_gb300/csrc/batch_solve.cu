@@ -280,7 +280,7 @@ size_t lu_smem(int nmax) {
 cudaError_t qcx_launch_lu_head(cudaStream_t st, const BatchSolveArgs& a, int grid, int nmax) {
     if (grid < 1 || nmax < 1) return cudaErrorInvalidValue;
     const size_t smem = lu_smem(nmax);
-    const cudaError_t e = cudaFuncSetAttribute((const void*)k_lu_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = qcx_allow_smem((const void*)k_lu_head, 1024);
     if (e != cudaSuccess) return e;
     k_lu_head<<<grid, LU_THREADS, smem, st>>>(a, nmax);
     return cudaGetLastError();

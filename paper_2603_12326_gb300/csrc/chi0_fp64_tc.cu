@@ -426,8 +426,7 @@ cudaError_t qcx_launch_chi0_fp64_tc(qcx_ctx* ctx, QSlot& s, int iq, double pref,
     a.tmem_cols = 32;
     while (a.tmem_cols < (uint32_t)(NS * n_tile)) a.tmem_cols *= 2;
     const size_t smem = 1024 + OZ_NSTAGE * (size_t)NS * (OZ_ATILE + n_tile * ROWB) + (2 * OZ_NSTAGE + 3) * 8 + 16;
-    if ((e = cudaFuncSetAttribute((const void*)k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return e;
+    if ((e = qcx_allow_smem((const void*)k_oz_gemm)) != cudaSuccess) return e;
     k_oz_rowmax<<<ng, 256, 0, st>>>(nt, R, eA);
     CUtensorMap ma, mb;
     if (!qcx_make_bf16_map(&ma, b.a.p, 2LL * nt2, NS * arows, OZ_M, KSTEP)) return cudaErrorInvalidValue;

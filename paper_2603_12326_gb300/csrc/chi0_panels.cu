@@ -988,8 +988,7 @@ cudaError_t qcx_launch_chi0_panels(qcx_ctx* ctx, QSlot& s, int iq, double2* d_ch
     const size_t smem = ring_bytes(PG_NSTAGE + deep);
     const auto gram = deep ? k_pn_gram<PG_NSTAGE + 1> : k_pn_gram<PG_NSTAGE>;
     if (smem > PG_SMEM_LIMIT) return cudaErrorInvalidValue;
-    if ((e = cudaFuncSetAttribute((const void*)gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-        return e;
+    if ((e = qcx_allow_smem((const void*)gram)) != cudaSuccess) return e;
     // the register budgets assume this launch allocation (see k_chi0_tc)
     cudaFuncAttributes fa;
     if ((e = cudaFuncGetAttributes(&fa, (const void*)gram)) != cudaSuccess) return e;

@@ -675,7 +675,7 @@ cudaError_t qcx_launch_chi0_mixed(qcx_ctx* ctx, QSlot& s, int iq, double2* chi, 
         if (!qcx_make_bf16_map(&mb[i], p0 + i * plane, s.kp, s.ngp, a.n_tile, KSTEP) ||
             !qcx_make_bf16_map(&ms[i], p0 + i * plane, s.kp, s.ngp, GBLK, KSTEP))
             return cudaErrorInvalidValue;
-    e = cudaFuncSetAttribute((const void*)k_chi0_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = qcx_allow_smem((const void*)k_chi0_tc);
     if (e != cudaSuccess) return e;
     {
         // the warpgroups' register budgets assume this launch allocation; another one could leave a

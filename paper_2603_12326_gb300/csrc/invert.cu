@@ -716,7 +716,7 @@ static cudaError_t invert_batch(cudaStream_t st, int n, int nmat, const double2*
     C* M = reinterpret_cast<C*>(aux);
     int* perm = reinterpret_cast<int*>(M + (size_t)nmat * pb * n);
     int* rows = perm + (size_t)nmat * n;
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_inv_panel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = qcx_allow_smem((const void*)k_inv_panel<T>);
     if (e != cudaSuccess) return e;
     const int npan = (n + pb - 1) / pb;
     const dim3 cols(nmat, (n + 63) / 64);
@@ -925,7 +925,7 @@ cudaError_t qcx_launch_batch_inverse(cudaStream_t st, const BatchSolveArgs& a, c
     if (nmax < 1 || nmax > 1024 * PANEL_ROWS) return cudaErrorInvalidValue;
     size_t smem = 0;
     const int pb = panel_width<float>(nmax, &smem);
-    cudaError_t e = cudaFuncSetAttribute((const void*)k_inv_panel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = qcx_allow_smem((const void*)k_inv_panel<float>);
     if (e != cudaSuccess) return e;
     float2* X = reinterpret_cast<float2*>(a.work);
     for (const InvGroup& g : groups) {

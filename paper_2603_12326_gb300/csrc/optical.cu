@@ -265,7 +265,7 @@ cudaError_t qcx_launch_optical(qcx_ctx* ctx, QSlot& s, int iq, int g0, const dou
     if (e != cudaSuccess) return e;
     const size_t ysm = sizeof(double2) * 3 * (size_t)nb * nv;
     if (ysm > 227 * 1024) return cudaErrorInvalidValue;
-    e = cudaFuncSetAttribute((const void*)k_momentum_elems, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ysm);
+    e = qcx_allow_smem((const void*)k_momentum_elems);
     if (e != cudaSuccess) return e;
     k_momentum_elems<<<nk, 256, ysm, st>>>(nb, nv, nc, ob.P.as<double2>(), ctx->d_Ck64.as<double2>(),
                                           ctx->d_Ckq64.as<double2>() + (size_t)iq * nk * nb * nc, ob.p.as<double2>());

@@ -771,12 +771,8 @@ template <typename T> int plan_blocks(qcx_ctx* ctx, PDArgs<T>& a, int nv, size_t
     return 0;
 }
 
-template <typename T> cudaError_t set_smem(const void* fn, size_t smem) {
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 template <typename T, int NCH> cudaError_t launch_pd(qcx_ctx* ctx, PDArgs<T>& a, size_t smem, dim3 grid) {
-    cudaError_t e = set_smem<T>((const void*)k_pair_density<T, NCH>, smem);
+    cudaError_t e = qcx_allow_smem((const void*)k_pair_density<T, NCH>);
     if (e != cudaSuccess) return e;
     k_pair_density<T, NCH><<<grid, PD_THREADS, smem, ctx->stream>>>(a);
     ++ctx->pd_launches;
@@ -784,7 +780,7 @@ template <typename T, int NCH> cudaError_t launch_pd(qcx_ctx* ctx, PDArgs<T>& a,
 }
 
 template <int NCH, int NV> cudaError_t launch_fused(qcx_ctx* ctx, PDArgs<float>& a, size_t smem, dim3 grid, int nthr) {
-    const cudaError_t e = set_smem<float>((const void*)k_pair_density_fused<NCH, NV>, smem);
+    const cudaError_t e = qcx_allow_smem((const void*)k_pair_density_fused<NCH, NV>);
     if (e != cudaSuccess) return e;
     k_pair_density_fused<NCH, NV><<<grid, nthr, smem, ctx->stream>>>(a);
     ++ctx->pd_launches;
@@ -817,7 +813,7 @@ template <typename T, int NCH, int NV> cudaError_t launch_tab(qcx_ctx* ctx, PDAr
     if (smem > 200 * 1024) return cudaErrorInvalidConfiguration;
     const int nch = (a.ng + 191) / 192, gc = (a.ng + nch - 1) / nch;
     const int ga_per = std::min(a.ngrp, std::max(1, pdt_threads<T, NV>() / gc));
-    cudaError_t e = set_smem<T>((const void*)k_pd_y<T, NCH, NV>, smem);
+    cudaError_t e = qcx_allow_smem((const void*)k_pd_y<T, NCH, NV>);
     if (e != cudaSuccess) return e;
     const int kc = (int)std::min<size_t>({(size_t)a.nk, t.buf->y.bytes / t.y_per_k, 65535});
     cplx<T>* Y = t.buf->y.as<cplx<T>>();
@@ -886,7 +882,7 @@ template <typename T> cudaError_t run_tab_nch(qcx_ctx* ctx, PDArgs<T>& a, const 
 }
 
 template <typename T, int NCH> cudaError_t launch_ov(qcx_ctx* ctx, PDArgs<T>& a, size_t smem, int nk) {
-    cudaError_t e = set_smem<T>((const void*)k_overlap<T, NCH>, smem);
+    cudaError_t e = qcx_allow_smem((const void*)k_overlap<T, NCH>);
     if (e != cudaSuccess) return e;
     k_overlap<T, NCH><<<nk, PD_THREADS, smem, ctx->stream>>>(a);
     return cudaGetLastError();

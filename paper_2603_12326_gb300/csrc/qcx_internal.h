@@ -321,6 +321,14 @@ struct qcx_ctx {
         }                                                                                       \
     } while (0)
 
+// Dynamic shared memory of a kernel whose launches differ in size.  The attribute belongs to the kernel, not to a launch or
+// a context, so every caller allows the same amount (all of an SM's, less `fixed` bytes of static arrays): allowed by the
+// size of each launch, a context in another thread could lower it between one's call and launch, which then failed.
+constexpr int QCX_SMEM_MAX = 232448;
+inline cudaError_t qcx_allow_smem(const void* kernel, int fixed = 0) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, QCX_SMEM_MAX - fixed);
+}
+
 bool qcx_is_device_ptr(const void* p);
 
 // Host copy of a small host-or-device array (device sources synchronise the stream).
