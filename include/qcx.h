@@ -62,10 +62,14 @@ typedef enum {
 typedef enum {
     QCX_FP64 = 0,   /* plain FP64 throughout                                                    */
     QCX_MIXED = 1   /* FP32 pair densities kept as three BF16 terms; chi0 on the tcgen05
-                       tensor cores with rho~ = the first two terms on one side and W rho~
-                       in three BF16 terms on the other (five products), the FP32
-                       tensor-core sums restarted every 20 MMAs and accumulated in FP64, the
-                       diagonal summed again from the three-term rho in FP32; eps stored in FP64;
+                       tensor cores with rho~ = the first two terms on one side and, on the
+                       other, rho~ times its weight in three BF16 terms (five products): the
+                       weight W per frequency (tensor-core sums restarted every 20 MMAs and
+                       accumulated in FP64) or, for many frequencies, the weights of 16 nodes
+                       per energy panel (leading product restarted every 4 MMAs, sums in FP32),
+                       whose sums then meet W in three-term BF16 (six products, chunks added in
+                       FP64); the diagonal summed again from the three-term rho in FP32; eps
+                       stored in FP64;
                        FP32 Gauss-Jordan inverse with an FP64 residual correction of the diagonal
                        for ill-conditioned blocks (kappa_1 above qcx_set_refine_threshold, 1e4
                        by default) and the other blocks' loss as a quadratic form of the FP64
@@ -230,7 +234,7 @@ qcx_route qcx_chi0_route(const qcx_ctx* ctx, qcx_precision prec);
  * the same precision.  QCX_FP64: FP64 throughout.  QCX_MIXED: FP32 pair
  * densities (the mixed path's), FP32 spectral weights, and the contraction
  * over the grid points on the tcgen05 tensor cores with K and the weights as
- * three-term split BF16 (FP32 sums restarted every 24 MMAs, added in FP32 per
+ * three-term split BF16 (leading product restarted every 4 MMAs, added in FP32 per
  * chunk of at most 4096 points, chunks added in FP64); grid and K in FP64.
  *   out_chi0[nw][ng][ng]  optional, row G, column G' (complex double)
  *   out_S[nbin][ng][ng]   optional spectral weights (complex double); large

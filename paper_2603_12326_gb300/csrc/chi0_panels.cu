@@ -17,10 +17,10 @@
 // accumulator, in windows of 4 MMAs added in FP32 registers (at most 64 windows: longer panels are cut into segments
 // with their own S), and the other four, 2^-8 of it, share one for the whole segment.   (All five in one accumulator
 // with windows of 20: error of the loss 4.2e-6 where the direct kernel has 2.5e-6.)  W and S in three terms, six
-// products (k_spec_kk_tc, the same two accumulators), node chunks added in FP64; the diagonal from the three-term |rho|^2, FP32 sums of 256 added
-// in FP64.  Re W and Im W meet S separately, so the loss is not left over from products of size |Re W||rho|^2 as in the
-// direct kernel: measured error of the loss with
-// local fields 1.4e-6 against the direct kernel's 2.3e-6 (200 w, N_G = 181).
+// products (k_spec_kk_tc, the same two accumulators), node chunks added in FP64.  The diagonal from the three-term
+// |rho|^2: FP32 sums of 128 transitions added in FP64 and rounded to FP32 per node, FP32 sums of 32 nodes added in FP64.
+// Re W and Im W meet S separately, so the loss is not left over from products of size |Re W||rho|^2 as in the
+// direct kernel: measured error of the loss with local fields 1.4e-6 against the direct kernel's 2.3e-6 (200 w, N_G = 181).
 //
 // Steps: energy range; stable radix sort of the transitions by panel; plan (segments, 16-transition stages); Lagrange
 // weights; rho~ gathered into stage-contiguous, pre-swizzled tiles (a stage is one plain bulk copy per plane);
@@ -815,8 +815,9 @@ static double panel_us(const QSlot& s, long long nt, double stages, double segs,
 // The pairs of G' blocks as tiles {G' block, first column, columns (wrapping around ngp), A rows from B}: either every
 // block with the columns from its own on (the upper triangle), or with its own and the next floor(blocks / 2) around the
 // circle (the pairs half way around an even circle once).  The time of a tile hardly depends on its width, so the one
-// with fewer tiles: around the circle for 3 blocks (3 against 4: one q, N_G = 181, 1508 -> 1224 us with the deeper ring) and for 7 and 11 or more of
-// an odd number.  Tiles that hold their own rows also need no copy of them, which leaves room for a fifth stage.
+// with fewer tiles: around the circle for 3 blocks (3 against 4: one q, N_G = 181, 1508 -> 1224 us with the deeper
+// ring) and for 7 and 11 or more of an odd number.  Tiles that hold their own rows also need
+// no copy of them, which leaves room for a fifth stage.
 static std::vector<int4> pair_cover(int ng, int ngp) {
     const int nb = (ng + PG_GBLK - 1) / PG_GBLK;
     std::vector<int4> cover[2];

@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_chi0_tc_batch(const __grid_cons
                             const uint32_t d = tmem + (uint32_t)b * ACC_OFF;
                             const uint32_t a0 = smem_u32(st + NPB * BREG + NPB * SPIECE), a1 = a0 + ATILE,
                                            a2 = a1 + ATILE;
-    #pragma unroll
+#pragma unroll
                             for (int kk = 0; kk < KSTEP / 16; ++kk) {
                                 const uint32_t off = kk * 32;
                                 umma_bf16(d, sw64_desc(a0 + off), sw64_desc(b0 + off), idesc,

@@ -34,15 +34,15 @@ namespace {
 // L2, one CTA per matrix, or through shared memory with a cluster barrier per column); this form touches it
 // n/PB times and spends 8 n^3 flops in a product that the FP32 (FP64) pipe bounds, with tiles of all matrices in
 // one grid.  PB = 32 (FP32) keeps the panel's serial part (two CTA barriers per column, ~0.3 us) below the
-// update's time.  Measured (CUDA events, GB300): 200 matrices of 181: 3.33 -> 0.82 ms; 100 of 531: 177 -> 5.6 ms;
-// FP64, 8 of 181: 10.8 -> 2.0 ms.
+// update's time.  Measured (GB300): 200 matrices of 181: 3.33 -> 0.65 ms; 100 of 531: 177 -> 4.9 ms; FP64, 8 of 181:
+// 10.8 -> 2.0 ms.
 // With P A = rows in pivot order, the eliminated matrix is (P A)^-1, so its column k is the inverse's column
 // row(k): the last update writes its columns there.
 constexpr int UPD = 64;                     // update tile edge
 template <typename T> struct InvCfg;
 template <> struct InvCfg<float> { static constexpr int PB = 32; };
 template <> struct InvCfg<double> { static constexpr int PB = 16; };
-constexpr size_t PANEL_SMEM = 200 * 1024;   // the panel narrows above this (n > 800 in FP32 and FP64)
+constexpr size_t PANEL_SMEM = 200 * 1024;   // the panel narrows above this (from n = 774 on in FP32 and FP64)
 constexpr int PANEL_ROWS = 4;               // rows per thread of the panel at most (n <= 4096)
 
 template <typename T> __device__ __forceinline__ T cabs2(cplx<T> z) { return z.x * z.x + z.y * z.y; }
@@ -254,7 +254,8 @@ __global__ void __launch_bounds__(1024) k_inv_panel(InvShape sh, int p_, int RW,
 // 32-row warps), every group turns its columns by one place per step, so that the current column is always the owning
 // group's place 0 and the loop needs no register indexing; the turn costs nothing, the update writes one place over.
 // Shared memory carries the pivot row, the current column and the row warps' best pivots.  The version above reads and
-// writes its panel in shared memory, a load-store chain per column.  Per panel: 200 matrices of 181 67 -> 32 us, 100 of 531 107 -> 44, a batch of 19-339 93 -> 40.
+// writes its panel in shared memory, a load-store chain per column.  Per panel: 200 matrices of 181 67 -> 32 us, 100 of
+// 531 107 -> 44, a batch of 19-339 93 -> 40.
 constexpr int PR_ROWS = 640;
 template <typename T, int BC>
 __global__ void __launch_bounds__(PR_ROWS) k_inv_panel_reg(InvShape sh, int p_, int RW, const cplx<T>* X, const cplx<T>* B2,

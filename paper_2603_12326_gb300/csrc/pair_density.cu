@@ -639,8 +639,8 @@ __global__ void __launch_bounds__(256) k_pd_rho(PDArgs<T> a, int kb, int nvp, co
 }
 
 // S(k) = B(k; 0) from the tables: one thread per (k, pair of groups a <= b), the block written to both triangles (S is
-// Hermitian).  Bound by the FP64 pipe (200 multiply-adds per 16 elements); measured for 512 k, N_b = 96: 0.08 ms (1.46
-// with the lattice sums formed per k, 0.12 with all pairs).  Pair number p walks rows r and n - 1 - r of the triangle
+// Hermitian).  Bound by the FP64 pipe (200 multiply-adds per 16 elements); measured for 512 k, N_b = 96: 0.08 ms, 0.12 with
+// its tables (1.46 with the lattice sums formed per k).  Pair number p walks rows r and n - 1 - r of the triangle
 // together, n + 1 pairs each.
 template <int NCH> __global__ void __launch_bounds__(128) k_overlap_tab(PDArgs<double> a) {
     const int p = blockIdx.x * 128 + threadIdx.x, k = blockIdx.y, n = a.ngrp;
@@ -805,8 +805,8 @@ template <typename T, int PR_C> void launch_rho(qcx_ctx* ctx, PDArgs<T>& a, int 
     k_pd_rho<T, PR_C><<<dim3((a.ng + PR_G - 1) / PR_G, a.nv * ((a.nc + PR_C - 1) / PR_C), m), 256, 0, ctx->stream>>>(a, k0, nvp, Y);
 }
 
-// The two table kernels over chunks of k; cudaErrorInvalidConfiguration when the basis has more groups than a CTA or C_k
-// does not fit shared memory (the caller then takes the kernels without tables).
+// The two table kernels over chunks of k; cudaErrorInvalidConfiguration when C_k does not fit shared memory (the caller
+// then takes the kernels without tables).
 template <typename T, int NCH, int NV> cudaError_t launch_tab(qcx_ctx* ctx, PDArgs<T>& a, const PdTab& t) {
     const int nvp = (a.nv + NV - 1) / NV * NV;
     const size_t smem = (size_t)a.nb * nvp * sizeof(cplx<T>);

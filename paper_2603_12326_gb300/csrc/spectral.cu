@@ -556,10 +556,10 @@ qcx_status spectral_chi0(qcx_ctx* ctx, QSlot& s, bool mixed, int nw, double E0, 
 
     const long long ldk = (nbin + 31LL) / 32 * 32;
     if (!mixed || ctx->spec_cuda_cores) {                  // (the tensor-core contraction has its own planes)
-    CUDA_OR_FAIL(qcx_ensure(ctx, sp.ktab, sizeof(C) * (size_t)nw * ldk), "alloc K");
-    k_spec_ktab<R><<<nblk((long long)nw * ldk, 256), 256, 0, st>>>(nw, ldk, nbin, s.w.as<double>(), E0, step, s.eta,
-                                                                    sp.ktab.as<C>());
-    CUDA_OR_FAIL(cudaGetLastError(), "K kernel");
+        CUDA_OR_FAIL(qcx_ensure(ctx, sp.ktab, sizeof(C) * (size_t)nw * ldk), "alloc K");
+        k_spec_ktab<R><<<nblk((long long)nw * ldk, 256), 256, 0, st>>>(nw, ldk, nbin, s.w.as<double>(), E0, step, s.eta,
+                                                                        sp.ktab.as<C>());
+        CUDA_OR_FAIL(cudaGetLastError(), "K kernel");
     }
 
     const size_t per_bin = (size_t)ntp * SP_TILE2 * sizeof(C);
