@@ -308,13 +308,14 @@ qcx_status qcx_set_refine_threshold(qcx_ctx* ctx, double kappa1);
  * cycles (default 4e9, about 2 s); the kernel then stops its pipeline, lets its
  * own copies and MMAs finish, frees its tensor memory and returns, and the
  * call reports QCX_ERR_TIMEOUT (for qcx_chi0 with QCX_FP64 see there) with
- * invalid results while the context stays usable.  A short limit makes the waits run out on purpose (tests).
+ * invalid results while the context stays usable.  A short limit makes the
+ * waits run out on purpose (tests).
  * Errors: QCX_ERR_ARG (ctx NULL, cycles < 1). */
 qcx_status qcx_set_wait_limit(qcx_ctx* ctx, long long cycles);
 
 /* Fault injection for tests of the failure path (no counterpart in the
  * paper): with withhold_copies != 0 the tensor-core kernels of qcx_chi0
- * issue none of their copies, so its consumers' waits run out after
+ * issue none of their copies, so their consumers' waits run out after
  * the limit of qcx_set_wait_limit and QCX_ERR_TIMEOUT is reported as there; 0
  * (the default) restores normal operation.  Errors: QCX_ERR_ARG (ctx NULL). */
 qcx_status qcx_set_fault_injection(qcx_ctx* ctx, int withhold_copies);
